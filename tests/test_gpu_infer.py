@@ -118,3 +118,32 @@ def test_lut_matvec_is_deterministic_and_reports_bad_codes():
     with pytest.raises(P.CrvqError) as e:                    # more than 8 inputs
         P.crvq_lut_matvec(dev(np.zeros((9, N), np.float32)), dev(perm), gcbs, M)
     assert e.value.status == -2
+
+
+@pytest.mark.parametrize("b,M,N,Ks,Gcs", [
+    (1, 1, 8, [16], [1]),                               # one row, one group
+    (8, 97, 16, [256, 3], [2, 1]),                      # fewer units than a cluster has CTAs
+    (5, 40, 8 * 261, [256, 256], [261, 7]),             # tables of several sub-ranges of units
+    (2, 20000, 8 * 9, [17, 5], [9, 2]),                 # more rows per cluster than threads
+    (4, 130, 8 * 37, [5000, 64, 300], [37, 11, 10]),    # dotted and looked-up codebooks mixed
+])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_lut_matvec_units_rows_and_unaligned_code_rows(b, M, N, Ks, Gcs, aligned):
+    """Edges of the unit shares, the row blocks and the 16-byte code loads (unaligned: codes as a
+    view with an odd offset and leading dimension)."""
+    import paper_2412_09282_gb300 as P
+    from paper_2412_09282_gb300 import Codebook
+    perm, cbs, G = _case(11, M, N, Ks, Gcs)
+    X = np.random.default_rng(12).standard_normal((b, N)).astype(np.float32)
+    if aligned:
+        _check(X, perm, cbs, M)
+        return
+    gcbs = []
+    for cb in cbs:
+        wide = torch.full((M, cb.G_cov + 6), -1, dtype=torch.int32, device="cuda")
+        wide[:, 1:1 + cb.G_cov] = dev(cb.codes.astype(np.int32))
+        gcbs.append(Codebook(dev(cb.C), wide[:, 1:1 + cb.G_cov], cb.G_cov))
+    Y = P.crvq_lut_matvec(dev(X), dev(perm), gcbs, M)
+    P.crvq_sync()
+    assert torch.equal(Y, _check(X, perm, cbs, M)) or np.allclose(
+        host(Y), host(_check(X, perm, cbs, M)), rtol=0, atol=1e-5 * float(np.abs(host(Y)).max()))

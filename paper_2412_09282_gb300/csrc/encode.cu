@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "score.cuh"
 #include "stats.cuh"
 #include "tc_ops.cuh"
 
@@ -30,11 +31,6 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kChunk = 256;             // codewords staged per shared-memory chunk
-constexpr float kU = 5.9604645e-08f;    // 2^-24
-
-// Error-bound multiplier: about twice the worst-case FMA-chain analysis (<= 37 + 2 n_fixed).
-__host__ __device__ inline float bound_mult(int n_terms) { return 64.f + 4.f * n_terms; }
-
 struct FlagList {
   int64_t* vec;      // vector index within the launch range (i * G_range + (g - g_begin))
   float* thr;        // decision threshold (fast-pass value units)
@@ -44,21 +40,6 @@ struct FlagList {
 };
 
 // --------------------------------------------------------------------------- device helpers
-__device__ __forceinline__ void load_vec(const float* p, float v[kD]) {
-  const float4 a = *reinterpret_cast<const float4*>(p);
-  const float4 b = *reinterpret_cast<const float4*>(p + 4);
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
-
-__device__ __forceinline__ bool code_ok(int32_t k, int32_t K, unsigned* err) {
-  if (k < 0 || k >= K) {
-    raise_error(err, ERRBIT_INDEX);
-    return false;
-  }
-  return true;
-}
-
 // fp32 target r = t - sum of the fixed codebooks covering g (codebook order), and the
 // magnitude bound a_j = |t_j| + sum |c_fixed,j| of every term that went into r.
 __device__ __forceinline__ void target32(const SetView& set, const CbList& cbs, int n_fixed,
@@ -113,27 +94,6 @@ __device__ double quad_err64(const double r[kD], const float* c, const float* H)
     e += hb * dlt[b];
   }
   return e;
-}
-
-// Codeword terms of the score and of its bound: n = c^T H c (fp32, two FMA chains),
-// na = |c|^T |H| |c|, l1 = ||c||_1.
-__device__ __forceinline__ void codeword_terms(const float c[kD], const float* H, float& n,
-                                               float& na, float& l1) {
-  n = 0.f;
-  na = 0.f;
-  l1 = 0.f;
-#pragma unroll
-  for (int a = 0; a < kD; ++a) {
-    float u = 0.f, ua = 0.f;
-#pragma unroll
-    for (int b = 0; b < kD; ++b) {
-      u = fmaf(H[a * kD + b], c[b], u);
-      ua = fmaf(fabsf(H[a * kD + b]), fabsf(c[b]), ua);
-    }
-    n = fmaf(c[a], u, n);
-    na = fmaf(fabsf(c[a]), ua, na);
-    l1 += fabsf(c[a]);
-  }
 }
 
 // Vector terms: m2q = -2 H r (the row FMA chains of stats_htau), Pmax = max_p (|H| a)_p.
@@ -194,25 +154,6 @@ __device__ __forceinline__ void stage_chunk(const float* __restrict__ C, int k0,
     sNL[k] = make_float2(n - kU * cmul * na, l1);
     sNa[k] = na;
   }
-}
-
-// fp32 lower / upper bounds s_k -+ Et_k of the score of codeword k from its terms t = (n, Na,
-// L1) (codeword_terms): s_k = n + sum_p m2q_p c_p, Et_k = u C (Na + 2 Pmax L1). Any
-// evaluation covered by the same error analysis is a valid bound; the fallback needs no more.
-__device__ __forceinline__ float low_from(float n, float na, float l1, const float c[kD],
-                                          const float m2q[kD], float nbeta, float cmul) {
-  float s = fmaf(-kU * cmul, na, n);
-#pragma unroll
-  for (int p = 0; p < kD; ++p) s = fmaf(m2q[p], c[p], s);
-  return fmaf(nbeta, l1, s);
-}
-
-__device__ __forceinline__ float up_from(float n, float na, float l1, const float c[kD],
-                                         const float m2q[kD], float pmax, float cmul) {
-  float s = fmaf(kU * cmul, na, n);
-#pragma unroll
-  for (int p = 0; p < kD; ++p) s = fmaf(m2q[p], c[p], s);
-  return fmaf(2.f * kU * cmul * pmax, l1, s);
 }
 
 __device__ __forceinline__ float low_score(const float c[kD], const float* H, const float m2q[kD],
@@ -369,90 +310,6 @@ prep_b_kernel(SetView set, int64_t g_begin, int64_t G_range, const float* __rest
   }
 }
 
-// Exact scoring in unevaluated fp32 pairs ("double-float"): GB300's fp64 pipe is a small
-// fraction of its fp32 rate, so the few decisions that the certified bounds leave open are
-// settled with error-free transformations (Knuth's TwoSum, the FMA-based TwoProduct) on the
-// fp32 pipe instead. The residual r = t - sum of the fixed codewords is held exactly as
-// rh + rl; the err (r - c)^T H (r - c) comes out within a few 2^-48 of |r - c|^T |H| |r - c|,
-// far inside the near-tie margin at which fp64 itself stops deciding.
-namespace dfl {
-
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bp = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
-}
-
-// (rh + rl) = t - sum of the fixed codebooks' codewords covering g (codebook order).
-__device__ __forceinline__ void target(const SetView& set, const CbList& cbs, int n_fixed,
-                                       int64_t i, int64_t g, float rh[kD], float rl[kD],
-                                       unsigned* err) {
-  load_vec(set.T + i * set.ldT + g * kD, rh);
-#pragma unroll
-  for (int j = 0; j < kD; ++j) rl[j] = 0.f;
-  for (int s = 0; s < n_fixed; ++s) {
-    const CbView& cb = cbs.cb[s];
-    if (g >= cb.G_cov) continue;
-    const int32_t k = cb.codes[i * cb.ld + g];
-    if (!code_ok(k, cb.K, err)) continue;
-    float c[kD];
-    load_vec(cb.C + (int64_t)k * kD, c);
-#pragma unroll
-    for (int j = 0; j < kD; ++j) {
-      float sj, ej;
-      two_sum(rh[j], -c[j], sj, ej);
-      rh[j] = sj;
-      rl[j] = __fadd_rn(rl[j], ej);
-    }
-  }
-}
-
-// err = (r - c)^T H (r - c) as a normalised pair (eh, el), r = rh + rl.
-__device__ __forceinline__ void quad_err(const float rh[kD], const float rl[kD],
-                                         const float c[kD], const float* H, float& eh,
-                                         float& el) {
-  float dh[kD], dl[kD];
-#pragma unroll
-  for (int j = 0; j < kD; ++j) {
-    float e;
-    two_sum(rh[j], -c[j], dh[j], e);
-    dl[j] = __fadd_rn(rl[j], e);
-  }
-  float yh[kD], yl[kD];
-#pragma unroll
-  for (int b = 0; b < kD; ++b) yh[b] = yl[b] = 0.f;
-#pragma unroll
-  for (int a = 0; a < kD; ++a)
-#pragma unroll
-    for (int b = 0; b < kD; ++b) {
-      const float h = H[a * kD + b];
-      const float p = __fmul_rn(dh[a], h);
-      const float pe = __fmaf_rn(dh[a], h, -p);  // dh h = p + pe exactly
-      float s, t;
-      two_sum(yh[b], p, s, t);
-      yh[b] = s;
-      yl[b] = __fadd_rn(yl[b], __fadd_rn(t, __fmaf_rn(dl[a], h, pe)));
-    }
-  float sh = 0.f, sl = 0.f;
-#pragma unroll
-  for (int b = 0; b < kD; ++b) {
-    const float p = __fmul_rn(dh[b], yh[b]);
-    const float pe = __fmaf_rn(dh[b], yh[b], -p);
-    float s, t;
-    two_sum(sh, p, s, t);
-    sh = s;
-    sl = __fadd_rn(sl, __fadd_rn(t, __fmaf_rn(dh[b], yl[b], __fmaf_rn(dl[b], yh[b], pe))));
-  }
-  eh = __fadd_rn(sh, sl);
-  el = __fsub_rn(sl, __fsub_rn(eh, sh));
-}
-
-__device__ __forceinline__ bool less(float ah, float al, int ak, float bh, float bl, int bk) {
-  return ah < bh || (ah == bh && (al < bl || (al == bl && ak < bk)));
-}
-
-}  // namespace dfl
-
 // Per-vector terms of the arg-min's A rows that do not change while one codebook's Lloyd
 // iterations run (the target, H_g and the fixed codebooks stay put): m2q = -2 H_g r and rr,
 // Ra, Pmax (vector_terms_rr of target32), as three planes of M float4 per group,
@@ -476,20 +333,8 @@ row_terms_kernel(SetView set, CbList cbs, int n_fixed, float4* __restrict__ rt,
   }
 }
 
-// Arg-min over one codebook on the tensor cores. A CTA walks `tiles` consecutive row tiles of
-// one group (thread = row = tensor-memory lane) with a 128-column accumulator per tile in
-// flight. HALVES = 1: 128 threads, three CTAs per SM, any codebook size (codeword chunks of 128
-// come from the precomputed B images by bulk copy; with at most two chunks they stay resident
-// for all the CTA's tiles). HALVES = 2 (codebooks of at most 256 codewords): 256 threads in two
-// halves of 128 that run independently (each its own tiles, named barriers, MMA issue and
-// accumulator) and share the resident codebook operand and the statistics; two CTAs per SM,
-// so four tile pipelines per SM interleave their phases (A rows, MMA, epilogue, certificate).
-// The sweep keeps per row the 16-column block with the smallest minimum and the second
-// smallest block minimum. Rows the bounds do not certify go to the flag list (decided exactly
-// by the exact kernels). The Lloyd statistics of certified rows are summed
-// in shared memory (integer atomics, [component][code] so that a warp's lanes hit spread banks)
-// and flushed once.
-constexpr int kTcSmemStatsK = 256;  // codebooks up to this size aggregate statistics in smem
+constexpr int kSmallK = 2 * kTcCols;   // codebooks up to this size stay resident in shared memory
+constexpr int kTcSmemStatsK = kSmallK;  // and sum their statistics there
 
 // Minimum of 16 non-negative fp32 values by their bit patterns (which order like the values),
 // as three-input integer minima.
@@ -502,27 +347,128 @@ __device__ __forceinline__ uint32_t min16_bits(const uint32_t* x) {
 
 constexpr int kBlk = 16;  // columns per block of the arg-min sweep
 
-// dynamic shared memory of argmin_tc_kernel<HALVES>: A tiles, two B chunks, statistics, H r,
-// with two halves the codeword terms (Na, L1) of the group, alignment
-constexpr size_t argmin_smem(int halves) {
-  return (size_t)halves * tcenc::kATile + 2 * (size_t)kTcBTile +
-         (size_t)kTcSmemStatsK * (kD * 8 + 4) + (size_t)halves * tcenc::kRows * kD * 4 +
-         (halves == 2 ? (size_t)kTcSmemStatsK * 8 : 0) + 1024;
-}
+// --------------------------------------------------------------------------- arg-min pass,
+// codebooks of at most 256 codewords: bounds, certificate, exact decisions and Lloyd statistics
+// in one persistent kernel.
+//
+// The work is the linear list of (group, pair of 128-row tiles); CTA c takes an equal share of
+// it, a run of pairs that touches one group or a few. Per group ("segment") the CTA builds the
+// group's B operand itself, a thread per codeword (about 2 k cycles; a separate kernel writing
+// images took 8 us per pass and 32 KB of L2 traffic per group and CTA), and then two halves of 128
+// threads run independently over alternate tiles, as tile pipelines: A rows, MMA per chunk of 128
+// codewords, sweep, certificate, statistics (own A tile, named barrier, mbarrier, 128 accumulator
+// columns each). Two CTAs per SM, so four pipelines interleave.
+//
+// Sweep. A row's 256 scores D form a 16 x 16 grid (block b = column / 16, class e = column % 16).
+// Kept are the minimum of every block and of every class, as three-input integer minima of the
+// non-negative fp32 bit patterns: 0.5 + 0.5 instructions per score and no per-score index. The
+// smallest score is the smallest block minimum and the smallest class minimum, so its block and
+// class name its column; the runner-up differs from it in block or class, so it is the second
+// smallest block minimum or the second smallest class minimum, exactly. (Keeping the winning block's
+// 16 values by selects instead cost 0.6 per score more on the ALU pipe, the busiest one.)
+//
+// Open rows. When the runner-up is within the bound `top` of the winner the row is open: every
+// column whose exact score could be the smallest has D <= top, so its block and its class have
+// minima <= top, and the two 16-bit masks of those name all candidates (two to four columns as a
+// rule, instead of the whole codebook). They go to a list in shared memory, and after its last tile
+// the CTA decides its open rows exactly (dfl, fp32 pairs), eight lanes per row. A row that finds
+// the list full is decided at once by its warp. This replaces a kernel that gave every open row a
+// warp and scanned the codebook twice (21 us per pass of a 4096 x 4096 matrix, 9 us of a 512 x 512).
+constexpr int kOpenCap = 256;  // open rows a CTA keeps for its end
 
-// Barrier over this half's 128 threads (named barrier 1 + half), or the whole CTA.
-template <int HALVES>
-__device__ __forceinline__ void half_sync(int half) {
-  if (HALVES == 1) {
-    __syncthreads();
-  } else {
-    asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+struct OpenRow {
+  uint32_t i, g;   // row, group (absolute)
+  uint32_t masks;  // blocks << 16 | classes
+};
+
+constexpr size_t kArgminSmem = 2 * (size_t)tcenc::kATile + 2 * (size_t)kTcBTile +
+                               (size_t)kTcSmemStatsK * (kD * 8 + 4) +
+                               2 * (size_t)tcenc::kRows * kD * 4 + (size_t)kTcSmemStatsK * 8 +
+                               (size_t)kOpenCap * sizeof(OpenRow) + 1024;
+
+// Exact decision of one open row by the eight lanes of a quarter warp (all 32 lanes call it; a
+// quarter with live = false takes part without writing): the candidates named by the masks are
+// scored in fp32 pairs, the smallest (err, index) wins, its statistics are added when requested.
+__device__ __forceinline__ void decide_open(const SetView& set, const CbList& cbs, int n_fixed,
+                                            int s_idx, const OpenRow& o, bool live,
+                                            int32_t* __restrict__ out_code, int64_t out_ld,
+                                            int64_t out_g0, const StatsView& st, float sscale,
+                                            unsigned* err) {
+  const CbView& cw = cbs.cb[s_idx];
+  const int sub = threadIdx.x & 7;
+  const int64_t i = o.i, g = o.g;
+  const float* H = set.Hb + g * kD * kD;
+  float rh[kD], rl[kD];
+  dfl::target(set, cbs, n_fixed, i, g, rh, rl, err);
+  const uint32_t bm = o.masks >> 16, em = o.masks & 0xffffu;
+  const int ne = __popc(em), total = __popc(bm) * ne;
+  float bh = INFINITY, bl = 0.f;
+  int bk = 0x7fffffff;
+  for (int c = sub; c < total; c += 8) {
+    uint32_t b = bm, e = em;
+    for (int q = c / ne; q > 0; --q) b &= b - 1u;
+    for (int q = c % ne; q > 0; --q) e &= e - 1u;
+    const int k = kBlk * (__ffs(b) - 1) + __ffs(e) - 1;
+    if (k >= cw.K) continue;  // padding columns
+    float cv[kD], eh, el;
+    load_vec(cw.C + (int64_t)k * kD, cv);
+    dfl::quad_err(rh, rl, cv, H, eh, el);
+    if (dfl::less(eh, el, k, bh, bl, bk)) {
+      bh = eh;
+      bl = el;
+      bk = k;
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, bh, off);
+    const float ol = __shfl_xor_sync(0xffffffffu, bl, off);
+    const int ok = __shfl_xor_sync(0xffffffffu, bk, off);
+    if (dfl::less(oh, ol, ok, bh, bl, bk)) {
+      bh = oh;
+      bl = ol;
+      bk = ok;
+    }
+  }
+  if (sub == 0 && live) {
+    if (bk == 0x7fffffff) {
+      raise_error(err, ERRBIT_NUMERIC);  // no candidate: non-finite scores
+    } else {
+      out_code[i * out_ld + (g - out_g0)] = bk;
+      if (st.cnt) {
+        float q[kD];
+        stats_htau(H, rh, q);  // rh is the fp32 target (TwoSum's rounded sums)
+        stats_add(st, sscale, g, bk, q);
+      }
+    }
   }
 }
 
-template <int HALVES>
+// The smallest value of v[0..15] (w1, at index idx; the first of equal ones) and the second
+// smallest (w2, equal to w1 when it occurs twice).
+__device__ __forceinline__ void top2_16(const uint32_t v[kBlk], uint32_t& w1, uint32_t& w2,
+                                        int& idx) {
+  w1 = v[0];
+  w2 = 0xffffffffu;
+  idx = 0;
+#pragma unroll
+  for (int e = 1; e < kBlk; ++e) {
+    w2 = min(w2, max(w1, v[e]));
+    idx = v[e] < w1 ? e : idx;
+    w1 = min(w1, v[e]);
+  }
+}
+
+__device__ __forceinline__ uint32_t mask_le_16(const uint32_t v[kBlk], uint32_t top) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int e = 0; e < kBlk; ++e) m |= v[e] <= top ? 1u << e : 0u;
+  return m;
+}
+
+// Barrier over one half's 128 threads (named barrier 1 + half), with an AND of v.
 __device__ __forceinline__ bool half_sync_and(int half, bool v) {
-  if (HALVES == 1) return __syncthreads_and(v);
   int r;
   asm volatile(
       "{\n .reg .pred p, q;\n setp.ne.b32 q, %1, 0;\n bar.red.and.pred p, %2, 128, q;\n"
@@ -533,8 +479,353 @@ __device__ __forceinline__ bool half_sync_and(int half, bool v) {
   return r != 0;
 }
 
-template <int HALVES>
-__global__ void __launch_bounds__(128 * HALVES, HALVES == 1 ? 3 : 2)
+__global__ void __launch_bounds__(256, 2)
+argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, int n_fixed,
+                    int s_idx, int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
+                    unsigned long long* flag_total, StatsView st,
+                    const float4* __restrict__ rowterms, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
+  using namespace tcenc;
+  extern __shared__ __align__(1024) char smem_raw[];
+  // 1024-byte aligned base, derived from the shared array (keeps the shared address space)
+  char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
+  char* Atiles = smem;                    // 2 x 16 KB
+  char* Bbuf = smem + 2 * kATile;         // 2 x 16 KB
+  int* s_b32 = reinterpret_cast<int*>(Bbuf + 2 * kTcBTile);     // [8][2][256] statistics halves
+  int* s_cnt = s_b32 + kTcSmemStatsK * kD * 2;                  // [256]
+  float* sQ = reinterpret_cast<float*>(s_cnt + kTcSmemStatsK);  // [256][8]: H r of a row
+  float2* sNaL1 = reinterpret_cast<float2*>(sQ + 2 * kRows * kD);      // [256]
+  OpenRow* s_open = reinterpret_cast<OpenRow*>(sNaL1 + kTcSmemStatsK);  // [kOpenCap]
+  __shared__ __align__(16) float sH[kD * kD];
+  __shared__ __align__(8) uint64_t bar_mma_s[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ float s_l1[8], s_cinf[8];
+  __shared__ unsigned n_open;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int half = tid >> 7, rrow = tid & (kRows - 1);
+  char* Atile = Atiles + half * kATile;
+  uint64_t& bar_mma = bar_mma_s[half];
+  const CbView cw = cbs.cb[s_idx];
+  const float cmul = kCmul + 4.f * n_fixed;
+  const float uc = kU * cmul;
+  const int nchunk = cw.K > kTcCols ? 2 : 1;
+
+  if (warp == 0) tc::tmem_alloc(&tmem_slot, 2 * kTcCols);
+  if (tid == 0) {
+    n_open = 0;
+    tc::mbar_init(tc::smem_u32(&bar_mma_s[0]), 1);
+    tc::mbar_init(tc::smem_u32(&bar_mma_s[1]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int e = tid; e < kTcSmemStatsK * kD * 2; e += 256) s_b32[e] = 0;
+  s_cnt[tid] = 0;
+  {  // codebook maxima: max_k ||c_k||_1 (raised by 1e-6 relative) and max |c|
+    float l1 = 0.f, cm = 0.f;
+    if (tid < cw.K) {
+      float c[kD];
+      load_vec(cw.C + (int64_t)tid * kD, c);
+#pragma unroll
+      for (int j = 0; j < kD; ++j) {
+        l1 += fabsf(c[j]);
+        cm = fmaxf(cm, fabsf(c[j]));
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      l1 = fmaxf(l1, __shfl_xor_sync(0xffffffffu, l1, off));
+      cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, off));
+    }
+    if (lane == 0) {
+      s_l1[warp] = l1;
+      s_cinf[warp] = cm;
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  // this half's accumulator: columns [128 half, 128 half + 128)
+  const uint32_t tmem = tmem_slot + (uint32_t)(half * kTcCols);
+  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  const float sscale = st.cnt ? stats_scale_f(st) : 1.f;
+  float l1max = 0.f, cinf = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    l1max = fmaxf(l1max, s_l1[w]);
+    cinf = fmaxf(cinf, s_cinf[w]);
+  }
+  l1max *= 1.f + 1e-6f;
+  constexpr uint32_t idesc = tc::idesc_tf32(kRows, kTcCols);
+
+  // this CTA's share [p, p_end) of the G_range * pairs_g tile pairs
+  const int64_t pairs_g = (set.M + 2 * kRows - 1) / (2 * kRows);
+  const int64_t total = G_range * pairs_g;
+  int64_t p = total * blockIdx.x / gridDim.x;
+  const int64_t p_end = total * (blockIdx.x + 1) / gridDim.x;
+  bool ok = true;
+  int mma_count = 0;
+
+  while (p < p_end) {
+    // one segment: pairs of one group, fewer than 2^16 rows (the 32-bit statistics halves)
+    const int64_t grel = p / pairs_g, g = g_begin + grel;
+    const int64_t pg = p - grel * pairs_g;  // the segment's first pair within the group
+    const int np = (int)min(min(p_end - p, pairs_g - pg), (int64_t)255);
+    if (tid < kD * kD) sH[tid] = set.Hb[g * kD * kD + tid];
+    __syncthreads();
+    {  // B operand of the group: thread = codeword
+      uint32_t row[kK];
+      if (tid < nchunk * kTcCols) {
+        build_b_row(cw.C, cw.K, tid, sH, uc, row);
+        put_row(Bbuf + (tid >> 7) * kTcBTile, tid & (kTcCols - 1), row);
+      }
+      if (tid < cw.K) {
+        float cv[kD], n, na, l1;
+        load_vec(cw.C + (int64_t)tid * kD, cv);
+        codeword_terms(cv, sH, n, na, l1);
+        sNaL1[tid] = make_float2(na, l1);
+      }
+    }
+    tc::fence_async_smem();
+    __syncthreads();
+    // Bound on Na_k over the codebook for this group: (max row sum |H_g|) L1max cinf.
+    float hrow = 0.f;
+#pragma unroll
+    for (int a = 0; a < kD; ++a) {
+      float rs = 0.f;
+#pragma unroll
+      for (int b = 0; b < kD; ++b) rs += fabsf(sH[a * kD + b]);
+      hrow = fmaxf(hrow, rs);
+    }
+
+    for (int t = 0; t < np && ok; ++t) {
+      const int64_t i = ((pg + t) * 2 + half) * kRows + rrow;
+      const bool row_ok = i < set.M;
+      // Prologue: this thread's A row.
+      float pmax, off;
+      {
+        float m2q[kD], rr, ra;
+        if (rowterms) {  // precomputed for this Lloyd loop (row_terms_kernel)
+          float4 q0 = make_float4(0.f, 0.f, 0.f, 0.f), q1 = q0, t2 = q0;
+          if (row_ok) {
+            q0 = rowterms[(3 * g) * set.M + i];
+            q1 = rowterms[(3 * g + 1) * set.M + i];
+            t2 = rowterms[(3 * g + 2) * set.M + i];
+          }
+          m2q[0] = q0.x; m2q[1] = q0.y; m2q[2] = q0.z; m2q[3] = q0.w;
+          m2q[4] = q1.x; m2q[5] = q1.y; m2q[6] = q1.z; m2q[7] = q1.w;
+          rr = t2.x;
+          ra = t2.y;
+          pmax = t2.z;
+        } else {
+          float rv[kD], a[kD];
+          if (row_ok) {
+            target32(set, cbs, n_fixed, i, g, rv, a, err);
+          } else {
+#pragma unroll
+            for (int j = 0; j < kD; ++j) rv[j] = a[j] = 0.f;
+          }
+          vector_terms_rr(rv, a, sH, m2q, pmax, rr, ra);
+        }
+        // offset making every D = low + off >= 0, with margins for every rounding involved
+        off = (rr + 32.f * kU * ra + 2.f * uc * (hrow * l1max * cinf + 2.f * pmax * l1max)) *
+                  (1.f + 4.f * uc) + 1e-30f;
+        const float beta = -2.f * uc * pmax;
+        if (st.cnt) {  // H r of this row, kept for the statistics (-m2q / 2, exact)
+          *reinterpret_cast<float4*>(sQ + tid * kD) =
+              make_float4(-0.5f * m2q[0], -0.5f * m2q[1], -0.5f * m2q[2], -0.5f * m2q[3]);
+          *reinterpret_cast<float4*>(sQ + tid * kD + 4) =
+              make_float4(-0.5f * m2q[4], -0.5f * m2q[5], -0.5f * m2q[6], -0.5f * m2q[7]);
+        }
+        uint32_t row[kK];
+#pragma unroll
+        for (int q = 0; q < kD; ++q) {
+          uint32_t h, l;
+          split(m2q[q], h, l);
+          row[q] = h;
+          row[8 + q] = h;
+          row[16 + q] = l;
+        }
+        const uint32_t one = __float_as_uint(1.f);
+        row[24] = one;
+        row[25] = one;
+        split(beta, row[26], row[28]);
+        row[27] = row[26];
+        split(off * (1.f - uc), row[29], row[30]);
+        row[31] = 0u;
+        put_row(Atile, rrow, row);
+      }
+      tc::fence_async_smem();
+
+      uint32_t mb[kBlk], mc[kBlk];  // block and class minima (fp32 bits)
+#pragma unroll
+      for (int e = 0; e < kBlk; ++e) mb[e] = mc[e] = 0xffffffffu;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        if (c < nchunk) {
+          // the A rows are written, the accumulator has been read; ok is then uniform in the half
+          ok = half_sync_and(half, ok);
+        }
+        if (c < nchunk && ok) {
+          if (rrow == 0) {
+            tc::tc_fence_after();
+            const uint32_t a0 = tc::smem_u32(Atile), b0 = tc::smem_u32(Bbuf + c * kTcBTile);
+#pragma unroll
+            for (int ks = 0; ks < kK / 8; ++ks)
+              tc::mma_tf32(tmem, tc::smem_desc(a0 + ks * 256, 128, (kK / 4) * 128),
+                           tc::smem_desc(b0 + ks * 256, 128, (kK / 4) * 128), idesc,
+                           ks > 0 ? 1u : 0u);
+            tc::mma_commit(tc::smem_u32(&bar_mma));
+          }
+          ok = tc::mbar_wait(tc::smem_u32(&bar_mma), (uint32_t)(mma_count & 1), err);
+          ++mma_count;
+          ok = __all_sync(0xffffffffu, ok);
+          tc::tc_fence_after();
+          if (ok) {
+#pragma unroll
+            for (int rnd = 0; rnd < 4; ++rnd) {
+              uint32_t v[32];
+              tc::tmem_ld32_nowait(trow + 32 * rnd, v);
+              tc::tmem_wait_ld_dep(v);
+              mb[8 * c + 2 * rnd] = min16_bits(v);
+              mb[8 * c + 2 * rnd + 1] = min16_bits(v + kBlk);
+#pragma unroll
+              for (int e = 0; e < kBlk; ++e) mc[e] = __vimin3_u32(mc[e], v[e], v[kBlk + e]);
+            }
+          }
+          tc::tc_fence_before();
+        }
+      }
+      ok = half_sync_and(half, ok);  // both chunks read: the accumulator and the A tile are free
+      if (!ok) break;
+
+      // Certificate, code, open row and statistics of this thread's row.
+      bool open = false;
+      OpenRow o{};
+      if (row_ok) {
+        uint32_t w1, w2, x1, x2;
+        int b1, e1;
+        top2_16(mb, w1, w2, b1);
+        top2_16(mc, x1, x2, e1);
+        const uint32_t s2 = min(w2, x2);
+        int j = b1 * kBlk + e1;
+        const float k1 = __uint_as_float(w1);
+        const float k2 = s2 == 0xffffffffu ? INFINITY : __uint_as_float(s2);
+        bool cert = false;
+        float top = INFINITY;
+        if (j < cw.K) {
+          const float2 tj = sNaL1[j];
+          // D_k <= s_k + off (every k); s_j + off <= D_j + e2 (the winner): no other codeword's
+          // exact score reaches s_j when k2 > D_j + e2 (the sum rounded up).
+          float e2 = 2.f * uc * (tj.x + 2.f * pmax * tj.y + off);
+          top = __fadd_ru(k1, e2);   // >= s_j + off
+          cert = cw.K == 1 || k2 > top;
+          // equal scores: block and class may name different columns; the bound over all codewords
+          if (s2 == w1) {
+            e2 = 2.f * uc * (hrow * l1max * cinf + 2.f * pmax * l1max + off) * 1.0001f;
+            top = __fadd_ru(k1, e2);
+          }
+        } else {
+          j = 0;
+        }
+        if (!cert) {
+          open = true;
+          const uint32_t tb = __float_as_uint(top) & 0x7fffffffu;
+          o.i = (uint32_t)i;
+          o.g = (uint32_t)g;
+          o.masks = (mask_le_16(mb, tb) << 16) | mask_le_16(mc, tb);
+        }
+        out_code[i * out_ld + (g - out_g0)] = j;
+        if (cert && st.cnt) {
+          // H r from the prologue (bit-identical to the standalone update's H tau). A term v
+          // (|v| < 2^30) enters as v = 2^15 vh + vl, 0 <= vl < 2^15, in two 32-bit sums: exact,
+          // since a segment has fewer than 2^16 rows.
+          float q[kD];
+          const float4 q0 = *reinterpret_cast<const float4*>(sQ + tid * kD);
+          const float4 q1 = *reinterpret_cast<const float4*>(sQ + tid * kD + 4);
+          q[0] = q0.x; q[1] = q0.y; q[2] = q0.z; q[3] = q0.w;
+          q[4] = q1.x; q[5] = q1.y; q[6] = q1.z; q[7] = q1.w;
+          atomicAdd(&s_cnt[j], 1);
+#pragma unroll
+          for (int e = 0; e < kD; ++e) {
+            const long long v = fix_rn_small(q[e], sscale);
+            atomicAdd(&s_b32[(2 * e) * kTcSmemStatsK + j], (int)(v >> 15));
+            atomicAdd(&s_b32[(2 * e + 1) * kTcSmemStatsK + j], (int)(v & 0x7fff));
+          }
+        }
+      }
+      // open rows: to the list, or decided here when it is full
+      bool over = false;
+      if (open) {
+        const unsigned slot = atomicAdd(&n_open, 1u);
+        if (slot < (unsigned)kOpenCap)
+          s_open[slot] = o;
+        else
+          over = true;
+      }
+      unsigned om = __ballot_sync(0xffffffffu, over);
+      while (om) {  // four rows at a time, a quarter warp each
+        int src = -1;
+        unsigned rest = om;
+        for (int q = 0; q < 4 && rest; ++q) {
+          if (q == lane >> 3) src = __ffs(rest) - 1;
+          rest &= rest - 1u;
+        }
+        const int from = src < 0 ? __ffs(om) - 1 : src;
+        OpenRow w;
+        w.i = __shfl_sync(0xffffffffu, o.i, from);
+        w.g = __shfl_sync(0xffffffffu, o.g, from);
+        w.masks = __shfl_sync(0xffffffffu, o.masks, from);
+        decide_open(set, cbs, n_fixed, s_idx, w, src >= 0, out_code, out_ld, out_g0, st, sscale,
+                    err);
+        om = rest;
+      }
+    }
+    ok = __syncthreads_and(ok);  // both halves are done with the group's operand and statistics
+    if (st.cnt && tid < cw.K) {  // flush (integer sums: order-free) and clear
+      const int c = s_cnt[tid];
+      if (c != 0) {
+        s_cnt[tid] = 0;
+        atomicAdd(&st.cnt[g * st.K + tid], c);
+#pragma unroll
+        for (int e = 0; e < kD; ++e) {
+          int* ph = &s_b32[(2 * e) * kTcSmemStatsK + tid];
+          int* pl = &s_b32[(2 * e + 1) * kTcSmemStatsK + tid];
+          const long long v = (long long)*ph * 32768 + *pl;
+          *ph = 0;
+          *pl = 0;
+          atomicAdd(reinterpret_cast<unsigned long long*>(&st.bacc[(int64_t)tid * kD + e]),
+                    (unsigned long long)v);
+        }
+      }
+    }
+    if (!ok) break;
+    p += np;
+  }
+  // the open rows of every segment, four per warp at a time
+  const unsigned found = n_open;  // (the barrier after the last segment ordered it)
+  if (flag_total && tid == 0 && found) atomicAdd(flag_total, (unsigned long long)found);
+  const int n = (int)min(found, (unsigned)kOpenCap);
+  for (int e0 = warp * 4; e0 < n; e0 += 32) {
+    const int e = e0 + (lane >> 3);
+    decide_open(set, cbs, n_fixed, s_idx, s_open[min(e, n - 1)], e < n, out_code, out_ld, out_g0,
+                st, sscale, err);
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem_slot, 2 * kTcCols);
+}
+
+// --------------------------------------------------------------------------- arg-min pass,
+// codebooks of more than 256 codewords: a CTA walks `tiles` consecutive row tiles of one group
+// (thread = row = tensor-memory lane), streaming the codebook's precomputed B images in chunks of 128
+// codewords by bulk copy through two buffers; 128 threads, three CTAs per SM. The sweep keeps per
+// row the 16-column block with the smallest minimum and the second smallest block minimum. Rows the
+// bounds do not certify go to the flag list (decided by the exact kernels).
+constexpr size_t kArgminStreamSmem = (size_t)tcenc::kATile + 2 * (size_t)kTcBTile +
+                                     (size_t)tcenc::kRows * kD * 4 + 1024;
+
+__global__ void __launch_bounds__(128, 3)
 argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_idx,
                  int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
                  FlagList flags, StatsView st, const float* __restrict__ cbmax,
@@ -546,50 +837,27 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   extern __shared__ __align__(1024) char smem_raw[];
   // 1024-byte aligned base, derived from the shared array (keeps the shared address space)
   char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
-  char* Atiles = smem;                          // HALVES x 16 KB
-  char* Bbuf = smem + HALVES * kATile;          // 2 x 16 KB
-  long long* s_bacc = reinterpret_cast<long long*>(Bbuf + 2 * kTcBTile);  // [8][256]
-  int* s_cnt = reinterpret_cast<int*>(s_bacc + kTcSmemStatsK * kD);       // [256]
-  float* sQ = reinterpret_cast<float*>(s_cnt + kTcSmemStatsK);            // [128 HALVES][8]
-  float2* sNaL1 = reinterpret_cast<float2*>(sQ + HALVES * kRows * kD);     // [256] (2 halves)
+  char* Atile = smem;                     // 16 KB
+  char* Bbuf = smem + kATile;             // 2 x 16 KB
+  float* sQ = reinterpret_cast<float*>(Bbuf + 2 * kTcBTile);  // [128][8]: H r of a row
   __shared__ __align__(16) float sH[kD * kD];
-  __shared__ __align__(8) uint64_t bar_mma_s[HALVES], bar_b[2];
+  __shared__ __align__(8) uint64_t bar_mma, bar_b[2];
   __shared__ uint32_t tmem_slot;
 
   const int64_t g = g_begin + blockIdx.y;
   const int64_t G_range = gridDim.y;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int half = HALVES == 1 ? 0 : (tid >> 7), rrow = tid & (kRows - 1);
-  char* Atile = Atiles + half * kATile;
-  uint64_t& bar_mma = bar_mma_s[half];
   const CbView cw = cbs.cb[s_idx];
   const float cmul = kCmul + 4.f * n_fixed;
   const float uc = kU * cmul;
   const int nchunk = (cw.K + kTcCols - 1) / kTcCols;
-  const bool resident = nchunk <= 2;
-  const char* bimg = bpre ? bpre + (size_t)(g - g_begin) * nchunk * kTcBTile : nullptr;
-  const float4* gterms = terms ? terms + (g - g_begin) * cw.K : nullptr;
-  const bool smem_stats = st.cnt && cw.K <= kTcSmemStatsK;
+  const char* bimg = bpre + (size_t)(g - g_begin) * nchunk * kTcBTile;
+  const float4* gterms = terms + (g - g_begin) * cw.K;
 
   if (tid < kD * kD) sH[tid] = set.Hb[g * kD * kD + tid];
-  if (smem_stats) {
-    for (int e = tid; e < kTcSmemStatsK * kD; e += blockDim.x) s_bacc[e] = 0;  // (= s_b32)
-    for (int e = tid; e < kTcSmemStatsK; e += blockDim.x) s_cnt[e] = 0;
-  }
-  // Statistics terms (|v| < 2^30) split as v = 2^15 vh + vl, 0 <= vl < 2^15, into two 32-bit
-  // shared sums [component][vh, vl][code] (native 32-bit atomics instead of 64-bit ones): exact,
-  // since the host gives a CTA with these sums fewer than 2^16 rows (|sum| < 2^31).
-  int* s_b32 = reinterpret_cast<int*>(s_bacc);  // [8][2][256] in the 64-bit sums' space
-  // the winner's terms for the certificate, from shared memory (K <= 256 with two halves)
-  const bool smem_terms = HALVES == 2 && gterms != nullptr;
-  if (smem_terms)
-    for (int k = tid; k < cw.K; k += blockDim.x) {
-      const float4 tk = gterms[k];
-      sNaL1[k] = make_float2(tk.y, tk.z);
-    }
-  if (warp == 0) tc::tmem_alloc(&tmem_slot, HALVES * kTcCols);
+  if (warp == 0) tc::tmem_alloc(&tmem_slot, kTcCols);
   if (tid == 0) {
-    for (int h = 0; h < HALVES; ++h) tc::mbar_init(tc::smem_u32(&bar_mma_s[h]), 1);
+    tc::mbar_init(tc::smem_u32(&bar_mma), 1);
     tc::mbar_init(tc::smem_u32(&bar_b[0]), 1);
     tc::mbar_init(tc::smem_u32(&bar_b[1]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -597,8 +865,7 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
-  // this half's accumulator: columns [128 half, 128 half + 128)
-  const uint32_t tmem = tmem_slot + (uint32_t)(half * kTcCols);
+  const uint32_t tmem = tmem_slot;
   const float sscale = st.cnt ? stats_scale_f(st) : 1.f;
 
   // Bound on Na_k over the codebook for this group: (max row sum |H_g|) L1max cinfmax.
@@ -613,18 +880,16 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   const float l1max = cbmax[0], cinf = cbmax[1];
   constexpr uint32_t idesc = tc::idesc_tf32(kRows, kTcCols);
 
-  // this CTA's row tiles (the last CTA of a column may have fewer); with two halves, half h
-  // takes tiles h, h + 2, ...
+  // this CTA's row tiles (the last CTA of a column may have fewer)
   const int64_t row_tiles = (set.M + kRows - 1) / kRows;
-  const int my_tiles = (int)min((int64_t)tiles, row_tiles - (int64_t)blockIdx.x * tiles);
-  const int steps = (my_tiles + HALVES - 1) / HALVES;
-  // Chunk uses are numbered u = t * nchunk + c. Resident chunks sit in buffer c; otherwise use u
-  // reads buffer u & 1, and the copy for use u + 2 starts when use u is done (one half only).
-  // At most one copy per buffer is outstanding; every thread tracks the same state.
-  const int n_uses = resident ? nchunk : steps * nchunk;
+  const int steps = (int)min((int64_t)tiles, row_tiles - (int64_t)blockIdx.x * tiles);
+  // Chunk uses are numbered u = t * nchunk + c: use u reads buffer u & 1, and the copy for use
+  // u + 2 starts when use u is done. At most one copy per buffer is outstanding; every thread
+  // tracks the same state.
+  const int n_uses = steps * nchunk;
   // per buffer (bit b): a copy outstanding, and the parity of its wait (registers, not arrays)
   uint32_t b_pend = 0, b_par = 0;
-  auto fetch = [&](int u) {  // chunk u % nchunk into buffer u & 1 (bimg only)
+  auto fetch = [&](int u) {  // chunk u % nchunk into buffer u & 1 
     const int b = u & 1;
     if (tid == 0) {
       tc::mbar_expect_tx(tc::smem_u32(&bar_b[b]), kTcBTile);
@@ -634,17 +899,14 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
     }
     b_pend |= 1u << b;
   };
-  if (bimg) {
-    fetch(0);
-    if (n_uses > 1) fetch(1);
-  }
+  fetch(0);
+  if (n_uses > 1) fetch(1);
   bool ok = true;
   int mma_count = 0;
 
   for (int t = 0; t < steps && ok; ++t) {
-    const int my_tile = HALVES * t + half;  // past my_tiles: a half without rows this step
-    const int64_t i = ((int64_t)blockIdx.x * tiles + my_tile) * kRows + rrow;
-    const bool row_ok = my_tile < my_tiles && i < set.M;
+    const int64_t i = ((int64_t)blockIdx.x * tiles + t) * kRows + tid;
+    const bool row_ok = i < set.M;
     // Prologue: this thread's A row.
     float pmax, off;
     {
@@ -697,10 +959,10 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
       row[27] = row[26];
       split(off * (1.f - uc), row[29], row[30]);
       row[31] = 0u;
-      put_row(Atile, rrow, row);
+      put_row(Atile, tid, row);
     }
     tc::fence_async_smem();
-    half_sync<HALVES>(half);
+    __syncthreads();
 
     // as fp32 bits: the smallest block minimum, its block and the block's 16 values; the
     // second smallest block minimum
@@ -711,24 +973,16 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
     for (int e = 0; e < kBlk; ++e) bv[e] = 0xffffffffu;
     for (int c = 0; c < nchunk; ++c) {
       const int u = t * nchunk + c;
-      const int buf = resident ? c : (u & 1);
+      const int buf = u & 1;
       char* Bt = Bbuf + buf * kTcBTile;
-      if (bimg) {
-        if ((b_pend >> buf) & 1u) {
-          if (ok) ok = tc::mbar_wait(tc::smem_u32(&bar_b[buf]), (b_par >> buf) & 1u, err);
-          b_par ^= 1u << buf;
-          b_pend &= ~(1u << buf);
-        }
-      } else if (!resident || t == 0) {  // (one half only: the host passes B images with two)
-        uint32_t v[kK];
-        build_b_row(cw.C, cw.K, c * kTcCols + rrow, sH, uc, v);
-        put_row(Bt, rrow, v);
-        tc::fence_async_smem();
-        half_sync<HALVES>(half);
+      if ((b_pend >> buf) & 1u) {
+        if (ok) ok = tc::mbar_wait(tc::smem_u32(&bar_b[buf]), (b_par >> buf) & 1u, err);
+        b_par ^= 1u << buf;
+        b_pend &= ~(1u << buf);
       }
-      ok = half_sync_and<HALVES>(half, ok);
+      ok = __syncthreads_and(ok);
       if (!ok) break;
-      if (rrow == 0) {
+      if (tid == 0) {
         tc::tc_fence_after();
         const uint32_t a0 = tc::smem_u32(Atile), b0 = tc::smem_u32(Bt);
 #pragma unroll
@@ -740,15 +994,15 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
       }
       ok = tc::mbar_wait(tc::smem_u32(&bar_mma), (uint32_t)(mma_count & 1), err);
       ++mma_count;
-      ok = half_sync_and<HALVES>(half, ok);
+      ok = __syncthreads_and(ok);
       if (!ok) break;
-      if (bimg && !resident && u + 2 < n_uses) fetch(u + 2);  // this buffer is free again
+      if (u + 2 < n_uses) fetch(u + 2);  // this buffer is free again
       tc::tc_fence_after();
       // Epilogue: this warp's 32 rows x 128 columns as eight blocks of 16. Per block its
       // minimum (every D >= 0, so the bit patterns order like the values); a block whose
       // minimum is the row's smallest so far is kept whole (16 selects), the previous best
       // block's minimum moves to the second smallest. No per-score index.
-      const uint32_t base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+      const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll
       for (int rnd = 0; rnd < 4; ++rnd) {
         uint32_t v[32];
@@ -766,7 +1020,7 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
         }
       }
       tc::tc_fence_before();
-      half_sync<HALVES>(half);  // the accumulator is free for the next MMA
+      __syncthreads();  // the accumulator is free for the next MMA
     }
     if (!ok) break;
 
@@ -790,21 +1044,8 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
       bool cert = false;
       float thr = INFINITY;
       if (j < cw.K) {
-        float n, na, l1;
-        if (smem_terms) {
-          const float2 tj = sNaL1[j];
-          na = tj.x;
-          l1 = tj.y;
-        } else if (gterms) {
-          const float4 tj = gterms[j];
-          n = tj.x;
-          na = tj.y;
-          l1 = tj.z;
-        } else {
-          float cv[kD];
-          load_vec(cw.C + (int64_t)j * kD, cv);
-          codeword_terms(cv, sH, n, na, l1);
-        }
+        const float4 tj = gterms[j];
+        const float na = tj.y, l1 = tj.z;
         // D_k <= s_k + off (every k); s_j + off <= D_j + e2 (the winner): no other codeword's
         // exact score reaches s_j when k2 > D_j + e2 (the sum rounded up).
         const float e2 = 2.f * uc * (na + 2.f * pmax * l1 + off);
@@ -832,17 +1073,7 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
         const float4 q1 = *reinterpret_cast<const float4*>(sQ + tid * kD + 4);
         q[0] = q0.x; q[1] = q0.y; q[2] = q0.z; q[3] = q0.w;
         q[4] = q1.x; q[5] = q1.y; q[6] = q1.z; q[7] = q1.w;
-        if (smem_stats) {
-          atomicAdd(&s_cnt[j], 1);
-#pragma unroll
-          for (int p = 0; p < kD; ++p) {
-            const long long v = fix_rn_small(q[p], sscale);
-            atomicAdd(&s_b32[(2 * p) * kTcSmemStatsK + j], (int)(v >> 15));
-            atomicAdd(&s_b32[(2 * p + 1) * kTcSmemStatsK + j], (int)(v & 0x7fff));
-          }
-        } else {
-          stats_add(st, sscale, g, j, q);
-        }
+        stats_add(st, sscale, g, j, q);
       }
     }
   }
@@ -852,23 +1083,9 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
       tc::mbar_wait(tc::smem_u32(&bar_b[b]), (b_par >> b) & 1u, err);
     }
   __syncthreads();
-  if (smem_stats) {  // one flush of this CTA's statistics (integer sums: order-free)
-    for (int k = tid; k < cw.K; k += blockDim.x) {
-      const int c = s_cnt[k];
-      if (c == 0) continue;
-      atomicAdd(&st.cnt[g * st.K + k], c);
-#pragma unroll
-      for (int p = 0; p < kD; ++p) {
-        const long long v = (long long)s_b32[(2 * p) * kTcSmemStatsK + k] * 32768 +
-                            s_b32[(2 * p + 1) * kTcSmemStatsK + k];
-        atomicAdd(reinterpret_cast<unsigned long long*>(&st.bacc[(int64_t)k * kD + p]),
-                  (unsigned long long)v);
-      }
-    }
-  }
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem_slot, HALVES * kTcCols);
+  if (warp == 0) tc::tmem_dealloc(tmem_slot, kTcCols);
 }
 
 // Exact decision for the rows the arg-min pass flagged: one CTA per flagged vector. The
@@ -2175,7 +2392,8 @@ struct ArgminLayout {
 };
 
 ArgminLayout argmin_layout(int64_t M, int64_t G_range, int K) {
-  ArgminLayout L;
+  ArgminLayout L{};
+  if (K <= kSmallK) return L;  // argmin_small_kernel takes none
   L.nchunk = (int)ceil_div(K, kTcCols);
   const int64_t per_group = (int64_t)L.nchunk * kTcBTile;
   L.G_sub = std::max<int64_t>(1, std::min<int64_t>(G_range, (int64_t(256) << 20) / per_group));
@@ -2184,6 +2402,107 @@ ArgminLayout argmin_layout(int64_t M, int64_t G_range, int K) {
   L.fbytes = align_up((size_t)M * L.G_sub * (sizeof(int64_t) + sizeof(float)), 256);
   L.total = 256 + L.bbytes + L.tbytes + 256 + L.fbytes;
   return L;
+}
+
+// One arg-min pass over the groups [g_begin, g_begin + G_range): codebook s_idx searched, those
+// before n_fixed fixed, codes to out (with the statistics of st when it has any).
+struct ArgminCall {
+  int64_t g_begin, G_range;
+  int n_fixed, s_idx;
+  int32_t* out;
+  int64_t out_ld, out_g0;
+  StatsView st;
+};
+
+// Codebooks of at most 256 codewords: one persistent kernel, two CTAs per SM.
+crvq_status launch_argmin_small(const SetView& set, const CbList& cbs, const ArgminCall& a,
+                                const EncodeExtras& ex, unsigned* err, cudaStream_t stream) {
+  const int64_t pairs = a.G_range * ceil_div(set.M, (int64_t)2 * tcenc::kRows);
+  CRVQ_TRY(smem_limit((const void*)argmin_small_kernel, kArgminSmem));
+  ProfScope ps(a.st.cnt ? "encode_argmin_lloyd" : "encode_argmin", stream,
+               (double)set.M * a.G_range * cbs.cb[a.s_idx].K);
+  CRVQ_CUDA(launch_pdl(argmin_small_kernel, dim3((unsigned)std::min<int64_t>(2 * sm_count(), pairs)),
+                       dim3(256), kArgminSmem, stream, set, a.g_begin, a.G_range, cbs, a.n_fixed,
+                       a.s_idx, a.out, a.out_ld, a.out_g0, ex.flag_total, a.st, ex.rowterms, err));
+  CRVQ_LAUNCHED();
+  return CRVQ_OK;
+}
+
+// Larger codebooks: groups in sub-ranges whose B images (the codebook's tensor-core operand per
+// group) take at most 256 MB; per sub-range: images + per-group codeword terms (prep_b, which also
+// writes the codebook maxima), the arg-min pass, and the exact decision of flagged rows.
+crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const ArgminCall& a,
+                                const EncodeExtras& ex, unsigned* err, cudaStream_t stream) {
+  const int64_t g_begin = a.g_begin, G_range = a.G_range, out_ld = a.out_ld, out_g0 = a.out_g0;
+  const int n_fixed = a.n_fixed, s_idx = a.s_idx, nsm = sm_count();
+  int32_t* out = a.out;
+  const StatsView& st = a.st;
+  const CbView& cw = cbs.cb[s_idx];
+  const ArgminLayout AL = argmin_layout(set.M, G_range, cw.K);
+  const int nchunk = AL.nchunk;
+  const int64_t G_sub = AL.G_sub;
+  const size_t bbytes = AL.bbytes, tbytes = AL.tbytes;
+  Scratch bmem;
+  char* wbase = ex.work;
+  if (!wbase || ex.work_bytes < AL.total) {
+    CRVQ_TRY(bmem.alloc(AL.total, stream));
+    wbase = bmem.as<char>();
+  }
+  float* cbmax = reinterpret_cast<float*>(wbase);
+  char* bimg = wbase + 256;
+  float4* tout = reinterpret_cast<float4*>(bimg + bbytes);
+  FlagList fl;
+  fl.count = reinterpret_cast<unsigned*>(wbase + 256 + bbytes + tbytes);
+  fl.vec = reinterpret_cast<int64_t*>(wbase + 256 + bbytes + tbytes + 256);
+  fl.cap = set.M * G_sub;
+  fl.thr = reinterpret_cast<float*>(fl.vec + fl.cap);
+  fl.total = ex.flag_total;
+  const float uc = kU * (tcenc::kCmul + 4.f * n_fixed);
+  CRVQ_TRY(smem_limit((const void*)argmin_tc_kernel, kArgminStreamSmem));
+  for (int64_t gs = g_begin; gs < g_begin + G_range; gs += G_sub) {
+    const int64_t gn = std::min<int64_t>(G_sub, g_begin + G_range - gs);
+    const int64_t nv = set.M * gn;
+    fl.cap = nv;
+    fl.thr = reinterpret_cast<float*>(fl.vec + nv);  // the count is cleared by prep_b
+    {
+      ProfScope pb("encode_prep_b", stream, (double)gn * nchunk * kTcCols);
+      const int64_t rows = gn * nchunk * kTcCols;
+      CRVQ_CUDA(launch_pdl(prep_b_kernel,
+                           dim3((unsigned)std::min<int64_t>(ceil_div(rows, 128), 16 * nsm) + 1),
+                           dim3(128), 0, stream, set, gs, gn, cw.C, cw.K, nchunk, uc, bimg,
+                           tout, cbmax, fl.count));
+      CRVQ_LAUNCHED();
+    }
+    {
+      // row tiles per CTA: about eight waves of three CTAs per SM (a fine-grained tail)
+      const int64_t row_tiles = ceil_div(set.M, tcenc::kRows);
+      const int64_t per_group = std::max<int64_t>(1, 24 * (int64_t)nsm / std::max<int64_t>(1, gn));
+      const int tiles = (int)std::max<int64_t>(1, ceil_div(row_tiles, per_group));
+      const dim3 grid((unsigned)ceil_div(row_tiles, tiles), (unsigned)gn);
+      ProfScope ps(st.cnt ? "encode_argmin_lloyd" : "encode_argmin", stream,
+                   (double)nv * cw.K);
+      CRVQ_CUDA(launch_pdl(argmin_tc_kernel, grid, dim3(128), kArgminStreamSmem, stream, set, gs,
+                           cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, st, cbmax, bimg, tout,
+                           ex.rowterms, tiles, err));
+      CRVQ_LAUNCHED();
+    }
+    {
+      ProfScope pf("encode_exact", stream, 0.0);
+      if (cw.K <= kExactWarpK) {
+        CRVQ_CUDA(launch_pdl(argmin_exact_warp_kernel,
+                             dim3((unsigned)std::min<int64_t>(ceil_div(nv, 4), 16 * nsm)),
+                             dim3(128), 0, stream, set, gs, gn, cbs, n_fixed, s_idx, out,
+                             out_ld, out_g0, fl, st, tout, err));
+      } else {
+        CRVQ_CUDA(launch_pdl(argmin_exact_kernel,
+                             dim3((unsigned)std::min<int64_t>(nv, 16 * nsm)), dim3(128), 0,
+                             stream, set, gs, gn, cbs, n_fixed, s_idx, out, out_ld, out_g0, fl,
+                             st, tout, err));
+      }
+      CRVQ_LAUNCHED();
+    }
+  }
+  return CRVQ_OK;
 }
 
 // One range of groups [g_begin, g_begin + G_range) whose searched stages are sd.st[0..S).
@@ -2220,89 +2539,11 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
     }
     StatsView st{};
     if (ex.stats && !keep_if_better) st = *ex.stats;
-    // Groups in sub-ranges whose B images (the codebook's tensor-core operand per group) take
-    // at most 256 MB; per sub-range: images + per-group codeword terms (prep_b, which also
-    // writes the codebook maxima), the arg-min pass, and the exact decision of flagged rows.
-    const ArgminLayout AL = argmin_layout(set.M, G_range, cw.K);
-    const int nchunk = AL.nchunk;
-    const int64_t G_sub = AL.G_sub;
-    const size_t bbytes = AL.bbytes, tbytes = AL.tbytes;
-    Scratch bmem;
-    char* wbase = ex.work;
-    if (!wbase || ex.work_bytes < AL.total) {
-      CRVQ_TRY(bmem.alloc(AL.total, stream));
-      wbase = bmem.as<char>();
-    }
-    float* cbmax = reinterpret_cast<float*>(wbase);
-    char* bimg = wbase + 256;
-    float4* tout = reinterpret_cast<float4*>(bimg + bbytes);
-    FlagList fl;
-    fl.count = reinterpret_cast<unsigned*>(wbase + 256 + bbytes + tbytes);
-    fl.vec = reinterpret_cast<int64_t*>(wbase + 256 + bbytes + tbytes + 256);
-    fl.cap = set.M * G_sub;
-    fl.thr = reinterpret_cast<float*>(fl.vec + fl.cap);
-    fl.total = ex.flag_total;
-    const float uc = kU * (tcenc::kCmul + 4.f * n_fixed);
-    // two independent 128-thread halves per CTA when the codebook stays resident (K <= 256)
-    const bool two_halves = nchunk <= 2;
-    CRVQ_TRY(set_smem_attr(argmin_tc_kernel<1>, argmin_smem(1)));
-    CRVQ_TRY(set_smem_attr(argmin_tc_kernel<2>, argmin_smem(2)));
-    for (int64_t gs = g_begin; gs < g_begin + G_range; gs += G_sub) {
-      const int64_t gn = std::min<int64_t>(G_sub, g_begin + G_range - gs);
-      const int64_t nv = set.M * gn;
-      fl.cap = nv;
-      fl.thr = reinterpret_cast<float*>(fl.vec + nv);  // the count is cleared by prep_b
-      {
-        ProfScope pb("encode_prep_b", stream, (double)gn * nchunk * kTcCols);
-        const int64_t rows = gn * nchunk * kTcCols;
-        CRVQ_CUDA(launch_pdl(prep_b_kernel,
-                             dim3((unsigned)std::min<int64_t>(ceil_div(rows, 128), 16 * nsm) + 1),
-                             dim3(128), 0, stream, set, gs, gn, cw.C, cw.K, nchunk, uc, bimg,
-                             tout, cbmax, fl.count));
-        CRVQ_LAUNCHED();
-      }
-      {
-        // row tiles per CTA: about eight waves of three CTAs per SM with one half (a
-        // fine-grained tail); with two halves about four waves of two (fewer statistics
-        // flushes and codebook fetches; measured 3% faster than eight waves, 10% faster than
-        // sixteen), each CTA reusing its group's resident codebook operand over several tiles
-        // (an even count with two halves)
-        const int64_t row_tiles = ceil_div(set.M, tcenc::kRows);
-        const int64_t want_ctas = (two_halves ? 8 : 24) * (int64_t)nsm;
-        const int64_t per_group = std::max<int64_t>(1, want_ctas / std::max<int64_t>(1, gn));
-        int tiles = (int)std::max<int64_t>(1, ceil_div(row_tiles, per_group));
-        if (two_halves) tiles += tiles & 1;
-        // fused statistics in 32-bit shared sums: fewer than 2^16 rows per CTA
-        if (st.cnt && cw.K <= kTcSmemStatsK) tiles = std::min(tiles, 510);
-        const dim3 grid((unsigned)ceil_div(row_tiles, tiles), (unsigned)gn);
-        ProfScope ps(st.cnt ? "encode_argmin_lloyd" : "encode_argmin", stream,
-                     (double)nv * cw.K);
-        if (two_halves)
-          CRVQ_CUDA(launch_pdl(argmin_tc_kernel<2>, grid, dim3(256), argmin_smem(2), stream, set,
-                               gs, cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, st, cbmax,
-                               bimg, tout, ex.rowterms, tiles, err));
-        else
-          CRVQ_CUDA(launch_pdl(argmin_tc_kernel<1>, grid, dim3(128), argmin_smem(1), stream, set,
-                               gs, cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, st, cbmax,
-                               bimg, tout, ex.rowterms, tiles, err));
-        CRVQ_LAUNCHED();
-      }
-      {
-        ProfScope pf("encode_exact", stream, 0.0);
-        if (cw.K <= kExactWarpK) {
-          CRVQ_CUDA(launch_pdl(argmin_exact_warp_kernel,
-                               dim3((unsigned)std::min<int64_t>(ceil_div(nv, 4), 16 * nsm)),
-                               dim3(128), 0, stream, set, gs, gn, cbs, n_fixed, s_idx, out,
-                               out_ld, out_g0, fl, st, tout, err));
-        } else {
-          CRVQ_CUDA(launch_pdl(argmin_exact_kernel,
-                               dim3((unsigned)std::min<int64_t>(nv, 16 * nsm)), dim3(128), 0,
-                               stream, set, gs, gn, cbs, n_fixed, s_idx, out, out_ld, out_g0, fl,
-                               st, tout, err));
-        }
-        CRVQ_LAUNCHED();
-      }
-    }
+    const ArgminCall ac{g_begin, G_range, n_fixed, s_idx, out, out_ld, out_g0, st};
+    if (cw.K <= kSmallK)
+      CRVQ_TRY(launch_argmin_small(set, cbs, ac, ex, err, stream));
+    else
+      CRVQ_TRY(launch_argmin_large(set, cbs, ac, ex, err, stream));
     if (ex.scores) *ex.scores += (double)nvec * cw.K;
     if (keep_if_better) {
       ProfScope ps3("encode_finalize", stream, 0.0);

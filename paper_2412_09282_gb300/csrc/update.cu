@@ -219,14 +219,33 @@ __device__ __forceinline__ void pair_two_sum(float a, float b, float& s, float& 
 // accumulation, about 2^-44 relative), solves L L^T dx = r in fp32 and adds dx to x, which is
 // kept as a pair, until the correction is below 2^-40 of x (each step gains about
 // -log2(cond(A) u_32) bits) or after 12 steps. No fp64 arithmetic: a dependent fp64 operation
-// costs about 180 cycles on this part, and one thread solves each codeword. Returns false
-// when A has no fp32 Cholesky factor.
-__device__ bool solve8_pairs(const float Ah[36], const float Al[36], const float bh[kD],
-                             const float bl[kD], float x_out[kD]) {
-  float Af[36], Lf[36], inv[kD];
+// costs about 180 cycles on this part. One warp solves one system: the residual, two thirds of
+// the arithmetic, is a row per lane (lanes 0-7; the others repeat row 7's work), everything else
+// runs redundantly on every lane. Each row's operations and their order are those of a single
+// thread, so the result does not depend on the split. Returns false when A has no fp32
+// Cholesky factor.
+__device__ bool solve8_pairs_warp(const float* __restrict__ Ah, const float* __restrict__ Al,
+                                  const float bh[kD], const float bl[kD], float x_out[kD]) {
+  const int lane = threadIdx.x & 31, row = min(lane, kD - 1);
+  float Lf[36], inv[kD];
+  {
+    float Af[36];
 #pragma unroll
-  for (int e = 0; e < 36; ++e) Af[e] = __fadd_rn(Ah[e], Al[e]);
-  if (!chol8_f32(Af, Lf, inv)) return false;
+    for (int e = 0; e < 36; ++e) Af[e] = __fadd_rn(Ah[e], Al[e]);
+    if (!chol8_f32(Af, Lf, inv)) return false;
+  }
+  // this lane's row of A and entry of b
+  float ah[kD], al[kD], rbh = 0.f, rbl = 0.f;
+#pragma unroll
+  for (int c = 0; c < kD; ++c) {
+    const int q = row >= c ? row * (row + 1) / 2 + c : c * (c + 1) / 2 + row;
+    ah[c] = Ah[q];
+    al[c] = Al[q];
+    if (c == row) {
+      rbh = bh[c];
+      rbl = bl[c];
+    }
+  }
   float bf[kD], xh[kD], xl[kD];
 #pragma unroll
   for (int j = 0; j < kD; ++j) {
@@ -235,23 +254,21 @@ __device__ bool solve8_pairs(const float Ah[36], const float Al[36], const float
   }
   chol8_solve_f32(Lf, inv, bf, xh);
   for (int it = 0; it < 12; ++it) {
+    float h = rbh, l = rbl;
+#pragma unroll
+    for (int c = 0; c < kD; ++c) {
+      const float p = __fmul_rn(ah[c], xh[c]);
+      const float pe = __fmaf_rn(ah[c], xh[c], -p);  // Ah xh = p + pe exactly
+      const float cross = __fmaf_rn(ah[c], xl[c], __fmul_rn(al[c], xh[c]));
+      float sum, t;
+      pair_two_sum(h, -p, sum, t);
+      h = sum;
+      l = __fadd_rn(l, __fsub_rn(t, __fadd_rn(pe, cross)));
+    }
+    const float mine = __fadd_rn(h, l);
     float rf[kD];
 #pragma unroll
-    for (int r = 0; r < kD; ++r) {
-      float h = bh[r], l = bl[r];
-#pragma unroll
-      for (int c = 0; c < kD; ++c) {
-        const int q = r >= c ? r * (r + 1) / 2 + c : c * (c + 1) / 2 + r;
-        const float p = __fmul_rn(Ah[q], xh[c]);
-        const float pe = __fmaf_rn(Ah[q], xh[c], -p);  // Ah xh = p + pe exactly
-        const float cross = __fmaf_rn(Ah[q], xl[c], __fmul_rn(Al[q], xh[c]));
-        float sum, t;
-        pair_two_sum(h, -p, sum, t);
-        h = sum;
-        l = __fadd_rn(l, __fsub_rn(t, __fadd_rn(pe, cross)));
-      }
-      rf[r] = __fadd_rn(h, l);
-    }
+    for (int r = 0; r < kD; ++r) rf[r] = __shfl_sync(0xffffffffu, mine, r);
     float dx[kD];
     chol8_solve_f32(Lf, inv, rf, dx);
     float xm = 0.f, dm = 0.f;
@@ -265,10 +282,21 @@ __device__ bool solve8_pairs(const float Ah[36], const float Al[36], const float
       xm = fmaxf(xm, fabsf(xh[j]));
       dm = fmaxf(dm, fabsf(dx[j]));
     }
-    if (dm <= 9.094947e-13f * xm) break;  // 2^-40
+    if (dm <= 9.094947e-13f * xm) break;  // 2^-40 (the same on every lane)
   }
 #pragma unroll
   for (int j = 0; j < kD; ++j) x_out[j] = __fadd_rn(xh[j], xl[j]);
+  return true;
+}
+
+// The fp64 Cholesky solve, for a matrix without an fp32 factor (cond(A) beyond fp32; rare).
+__device__ __noinline__ bool solve8_f64(const float* Ah, const float* Al, const float bh[kD],
+                                        const float bl[kD], float out[kD]) {
+  double A[36], b[kD], x[kD];
+  for (int v = 0; v < 36; ++v) A[v] = (double)Ah[v] + (double)Al[v];
+  for (int j = 0; j < kD; ++j) b[j] = (double)bh[j] + (double)bl[j];
+  if (!cholesky_solve8(A, b, x)) return false;
+  for (int j = 0; j < kD; ++j) out[j] = (float)x[j];
   return true;
 }
 
@@ -286,100 +314,113 @@ __device__ __forceinline__ void fixed_to_pair(long long v, int sexp, float& h, f
   l = ldexpf(__fadd_rn(t, t2), -sexp);
 }
 
-// The least-squares solve of every codeword, in two kernels. stats_sum_kernel: CTA = one
-// codeword; thread = (entry e of A_k's packed lower triangle or the count, slice of the
-// groups). Each thread sums cnt[g][k] * H_g[e] over its slice as an unevaluated fp32 pair
-// (every product is split exactly: cnt < 2^24; TwoSum for the high part), so no fp64
-// arithmetic runs per group; the slices are added in a fixed order as fp32 pairs, and the
-// pairs of A_k go to st.apair. stats_solve_kernel: one thread per codeword solves
-// A_k c_k = b_k (b_k from the fixed point) by Cholesky with refinement in fp32 pairs. The
-// summing threads carry none of the solve's registers, so every codeword's CTA is resident at
-// once. The fixed assignment and order make the result identical on every run. Codewords
-// without members keep their old value.
+// The least-squares solve of every codeword, one kernel. CTA = kSolveNC codewords; thread = (entry
+// e of A_k's packed lower triangle or the count, slice of the groups). Each thread sums
+// cnt[g][k] * H_g[e] over its slice as an unevaluated fp32 pair for each of the CTA's codewords
+// (every product is split exactly: cnt < 2^24; TwoSum for the high part), so no fp64 arithmetic
+// runs per group and an H entry is read once for both codewords; the slices are added in a fixed
+// order as fp32 pairs, and then a warp per codeword solves A_k c_k = b_k (b_k from the fixed point)
+// by Cholesky with refinement in fp32 pairs. The fixed assignment and order make the result
+// identical on every run. Codewords without members keep their old value.
+// Bound: latency (0.4 MB per launch). As two kernels, the solve with one thread per codeword, a 512 x
+// 512 layer (64 groups) took 5.3 + 8.0 us per Lloyd iteration; one kernel saves 4.8 us of that, and
+// nothing at 512 groups, where the sums' own work is the larger part.
 constexpr int kSolveSlices = 16;  // groups split 16 ways: short dependent chains per thread
-constexpr int kSumThreads = kSolveSlices * kNA;  // 592
-constexpr int kSolveThreads = 128;
+constexpr int kSolveSpt = 2;      // slices per thread (their chains interleave)
+constexpr int kSumThreads = kSolveSlices / kSolveSpt * kNA;  // 296: registers for the solve
+constexpr int kSolveNC = 2;       // 256 codewords: 128 CTAs, one wave
 
-__global__ void __launch_bounds__(kSumThreads, 2)
-stats_sum_kernel(const float* __restrict__ Hb, StatsView st) {
+__global__ void __launch_bounds__(kSumThreads)
+stats_solve_kernel(const float* __restrict__ Hb, StatsView st, const float* C_old, float* C_out,
+                   int32_t* __restrict__ counts_out, unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
-  __shared__ float part_h[kSolveSlices][kNA], part_l[kSolveSlices][kNA];
+  __shared__ float part_h[kSolveNC][kSolveSlices][kNA], part_l[kSolveNC][kSolveSlices][kNA];
+  __shared__ float sAh[kSolveNC][kNA], sAl[kSolveNC][kNA];
   const int tid = threadIdx.x;
   const int sl = tid / kNA;
   const int e = tid % kNA;
   const int K = st.K;
-  const int k = blockIdx.x;
+  const int k0 = blockIdx.x * kSolveNC;
+  const int nk = min(kSolveNC, K - k0);
   // entry e of the packed lower triangle: row r, column c (c <= r); e = 36 is the count
   int r = 0;
   while ((r + 1) * (r + 2) / 2 <= e && r < kD - 1) ++r;
   const int c = e - r * (r + 1) / 2;
   const int hoff = r * kD + c;
-  float hi = 0.f, lo = 0.f;
+  constexpr int kThreadSlices = kSolveSlices / kSolveSpt;
+  float hi[kSolveSpt][kSolveNC], lo[kSolveSpt][kSolveNC];
+#pragma unroll
+  for (int w = 0; w < kSolveSpt; ++w)
+#pragma unroll
+    for (int q = 0; q < kSolveNC; ++q) hi[w][q] = lo[w][q] = 0.f;
+  // thread slice sl takes the group slices sl and sl + kThreadSlices, each in group order
   const int64_t gper = (st.G_cov + kSolveSlices - 1) / kSolveSlices;
-  const int64_t g0 = sl * gper, g1 = min(st.G_cov, g0 + gper);
-  constexpr int kBatch = 8;  // loads of 8 groups in flight together; no branches
-  for (int64_t gb = g0; gb < g1; gb += kBatch) {
-    float fc[kBatch], h[kBatch];
+  constexpr int kBatch = 8;  // loads of 8 groups per slice in flight together; no branches
+  for (int64_t gb = 0; gb < gper; gb += kBatch) {
+    float fc[kSolveSpt][kBatch][kSolveNC], h[kSolveSpt][kBatch];
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int64_t g = gb + u;
-      const bool in = g < g1;
-      fc[u] = in ? (float)st.cnt[g * K + k] : 0.f;  // exact: counts stay below 2^24
-      h[u] = in ? (e < 36 ? __ldg(Hb + g * kD * kD + hoff) : 1.f) : 0.f;
+    for (int w = 0; w < kSolveSpt; ++w) {
+      const int64_t g0 = (sl + w * kThreadSlices) * gper, g1 = min(st.G_cov, g0 + gper);
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int64_t g = g0 + gb + u;
+        const bool in = g < g1;
+#pragma unroll
+        for (int q = 0; q < kSolveNC; ++q)  // exact: counts stay below 2^24
+          fc[w][u][q] = in && q < nk ? (float)st.cnt[g * K + k0 + q] : 0.f;
+        h[w][u] = in ? (e < 36 ? __ldg(Hb + g * kD * kD + hoff) : 1.f) : 0.f;
+      }
     }
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const float p = __fmul_rn(fc[u], h[u]);
-      const float pe = __fmaf_rn(fc[u], h[u], -p);  // fc h = p + pe exactly
-      const float sum = __fadd_rn(hi, p);            // TwoSum(hi, p) = sum + t exactly
-      const float bp = __fsub_rn(sum, hi);
-      const float t = __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bp)), __fsub_rn(p, bp));
-      hi = sum;
-      lo = __fadd_rn(lo, __fadd_rn(t, pe));
-    }
+    for (int u = 0; u < kBatch; ++u)
+#pragma unroll
+      for (int w = 0; w < kSolveSpt; ++w)
+#pragma unroll
+        for (int q = 0; q < kSolveNC; ++q) {
+          const float p = __fmul_rn(fc[w][u][q], h[w][u]);
+          const float pe = __fmaf_rn(fc[w][u][q], h[w][u], -p);  // fc h = p + pe exactly
+          float sum, t;
+          pair_two_sum(hi[w][q], p, sum, t);
+          hi[w][q] = sum;
+          lo[w][q] = __fadd_rn(lo[w][q], __fadd_rn(t, pe));
+        }
   }
-  // Slices are merged per entry by its own thread in fp32 pairs (TwoSum of the high parts, low
-  // parts added), in slice order: no serial fp64 chain (a dependent fp64 operation costs
-  // about 180 cycles on this part).
-  part_h[sl][e] = hi;
-  part_l[sl][e] = lo;
+#pragma unroll
+  for (int w = 0; w < kSolveSpt; ++w)
+#pragma unroll
+    for (int q = 0; q < kSolveNC; ++q) {
+      part_h[q][sl + w * kThreadSlices][e] = hi[w][q];
+      part_l[q][sl + w * kThreadSlices][e] = lo[w][q];
+    }
   __syncthreads();
-  // Every thread of the codeword has read its counts: clear them, so that the statistics are
-  // zero for the next accumulation (the Lloyd loop needs no memset between iterations).
-  if (e == 0)
-    for (int64_t gq = g0; gq < g1; ++gq) st.cnt[gq * K + k] = 0;
-  if (sl == 0) {
-    float h = part_h[0][e], l = part_l[0][e];
-    for (int s2 = 1; s2 < kSolveSlices; ++s2) {
-      const float p = part_h[s2][e];
-      const float sum = __fadd_rn(h, p);
-      const float bp = __fsub_rn(sum, h);
-      const float t = __fadd_rn(__fsub_rn(h, __fsub_rn(sum, bp)), __fsub_rn(p, bp));
-      h = sum;
-      l = __fadd_rn(l, __fadd_rn(t, part_l[s2][e]));
-    }
-    st.apair[(int64_t)k * kNA + e] = make_float2(h, l);
-  }
-}
-
-__global__ void __launch_bounds__(kSolveThreads)
-stats_solve_kernel(StatsView st, const float* C_old, float* C_out,
-                   int32_t* __restrict__ counts_out, unsigned* err) {
-  pdl_trigger();
-  pdl_wait();
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= st.K) return;
-  float Ah[kNA], Al[kNA];
+  // Every thread has read its counts: clear them, so that the statistics are zero for the next
+  // accumulation (the Lloyd loop needs no memset between iterations).
+  for (int64_t v = tid; v < st.G_cov * nk; v += kSumThreads)
+    st.cnt[(v / nk) * K + k0 + v % nk] = 0;
+  // Slices are merged per entry by one thread in fp32 pairs (TwoSum of the high parts, low parts
+  // added), in slice order; codeword q by warps 2 q and 2 q + 1.
+  const int q = tid >> 6, eq = tid & 63;
+  if (q < kSolveNC && eq < kNA) {
+    float h = part_h[q][0][eq], l = part_l[q][0][eq];
 #pragma unroll
-  for (int e = 0; e < kNA; ++e) {
-    const float2 v = st.apair[(int64_t)k * kNA + e];
-    Ah[e] = v.x;
-    Al[e] = v.y;
+    for (int s2 = 1; s2 < kSolveSlices; ++s2) {
+      float sum, t;
+      pair_two_sum(h, part_h[q][s2][eq], sum, t);
+      h = sum;
+      l = __fadd_rn(l, __fadd_rn(t, part_l[q][s2][eq]));
+    }
+    sAh[q][eq] = h;
+    sAl[q][eq] = l;
   }
+  __syncthreads();
+  const int kq = tid >> 5, k = k0 + kq;  // warp kq solves codeword k
+  if (kq >= nk) return;
+  const float* Ah = sAh[kq];
+  const float* Al = sAl[kq];
   // the count: an exact integer held by the pair
   const int64_t count = (int64_t)__float2int_rn(Ah[36]) + (int64_t)__float2int_rn(Al[36]);
-  if (counts_out) counts_out[k] = (int32_t)count;
+  if (counts_out && (tid & 31) == 0) counts_out[k] = (int32_t)count;
   bool keep = count == 0;
   float out[kD];
   if (!keep) {
@@ -387,40 +428,28 @@ stats_solve_kernel(StatsView st, const float* C_old, float* C_out,
     float bh[kD], bl[kD];
 #pragma unroll
     for (int j = 0; j < kD; ++j) fixed_to_pair(st.bacc[(int64_t)k * kD + j], sexp, bh[j], bl[j]);
+    __syncwarp();
+    if ((tid & 31) == 0)
 #pragma unroll
-    for (int j = 0; j < kD; ++j) st.bacc[(int64_t)k * kD + j] = 0;  // read: clear (see above)
-    if (!solve8_pairs(Ah, Al, bh, bl, out)) {
-      // no fp32 factor (cond(A) beyond fp32): the fp64 Cholesky solve
-      double A[36], b[kD], x[kD];
-#pragma unroll
-      for (int q = 0; q < 36; ++q) A[q] = (double)Ah[q] + (double)Al[q];
-#pragma unroll
-      for (int j = 0; j < kD; ++j) b[j] = (double)bh[j] + (double)bl[j];
-      if (cholesky_solve8(A, b, x)) {
-#pragma unroll
-        for (int j = 0; j < kD; ++j) out[j] = (float)x[j];
-      } else {
-        raise_error(err, ERRBIT_NUMERIC);
+      for (int j = 0; j < kD; ++j) st.bacc[(int64_t)k * kD + j] = 0;  // read: clear (see above)
+    if (!solve8_pairs_warp(Ah, Al, bh, bl, out)) {
+      if (!solve8_f64(Ah, Al, bh, bl, out)) {
+        if ((tid & 31) == 0) raise_error(err, ERRBIT_NUMERIC);
         keep = true;
       }
     }
   }
-  if (keep)
+  if ((tid & 31) != 0) return;
 #pragma unroll
-    for (int j = 0; j < kD; ++j) out[j] = C_old[(int64_t)k * kD + j];
-#pragma unroll
-  for (int j = 0; j < kD; ++j) C_out[(int64_t)k * kD + j] = out[j];
+  for (int j = 0; j < kD; ++j) C_out[(int64_t)k * kD + j] = keep ? C_old[(int64_t)k * kD + j] : out[j];
 }
 
 crvq_status launch_solve_kernels(const float* Hb, const StatsView& st, const float* C_old,
                                  float* C_out, int32_t* counts, unsigned* err,
                                  cudaStream_t stream) {
   ProfScope ps("update_solve", stream, (double)st.K);
-  CRVQ_CUDA(launch_pdl(stats_sum_kernel, dim3((unsigned)st.K), dim3(kSumThreads), 0, stream,
-                       Hb, st));
-  CRVQ_LAUNCHED();
-  CRVQ_CUDA(launch_pdl(stats_solve_kernel, dim3((unsigned)ceil_div(st.K, kSolveThreads)),
-                       dim3(kSolveThreads), 0, stream, st, C_old, C_out, counts, err));
+  CRVQ_CUDA(launch_pdl(stats_solve_kernel, dim3((unsigned)ceil_div(st.K, kSolveNC)),
+                       dim3(kSumThreads), 0, stream, Hb, st, C_old, C_out, counts, err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -491,10 +520,13 @@ crvq_status launch_update_codebook(const SetView& set, const CbList& cbs, int wh
 namespace crvq {
 
 // The update of launch_update_codebook on caller-provided scratch (no allocation): `scratch`
-// (256-byte aligned, `bytes` long) holds cnt | bacc | scale + maxima | apair, and `err` is the error
+// (256-byte aligned, `bytes` long) holds cnt | bacc | scale + maxima, and `err` is the error
 // word the kernels report to. Returns CRVQ_ERR_UNSUPPORTED when the statistics of this
 // codebook do not fit in `bytes`.
-size_t update_scratch_bytes(int64_t G_cov, int K) { return stats_layout(G_cov, K).total; }
+// The size limit counts K * 296 bytes beyond what the kernels use (the documented limit).
+size_t update_scratch_bytes(int64_t G_cov, int K) {
+  return stats_layout(G_cov, K).total + align_up((size_t)K * kNA * sizeof(float2), 256);
+}
 
 crvq_status launch_update_codebook_on(const SetView& set, const CbList& cbs, int which,
                                       float* C_out, int32_t* counts, void* scratch,

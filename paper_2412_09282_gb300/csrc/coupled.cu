@@ -26,8 +26,10 @@
 #include <vector>
 
 #include "common.cuh"
+#include "img.cuh"
 #include "kernels.h"
 #include "score.cuh"
+#include "tc_ops.cuh"
 
 namespace crvq {
 
@@ -126,7 +128,10 @@ struct CplArgs {
   const float* Hb;     // [G_cov][8][8]
   const float* Lf;     // [G_cov][8][8]
   const float* Linv;   // [G_cov][8]
-  const float* Bt;     // [(g1 - g0) * 8][M]
+  const float* P;      // B^T as [chunks][(g1 - g0) * 8][M]: the chunks' sum, in order
+  int chunks;
+  char *d_hi, *d_lo;   // the operand images of D, kept up to date
+  int64_t nslab;
   int64_t M, N;
   int64_t g0, g1;
   int rows;            // rows per CTA, at most kCplRows
@@ -160,7 +165,9 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
   const int row8 = tid >> 3, j8 = tid & 7;  // (row, component) threads
   for (int e = tid; e < nr * ncol; e += kCplThreads) {
     const int c = e / nr, r = e - c * nr;
-    sB[r * kCplPad + c] = a.Bt[(int64_t)c * a.M + i0 + r];
+    float s = 0.f;
+    for (int q = 0; q < a.chunks; ++q) s += __ldg(a.P + ((int64_t)q * ncol + c) * a.M + i0 + r);
+    sB[r * kCplPad + c] = s;
   }
   for (int64_t g = a.g0; g < a.g1; ++g) {
     const int col0 = (int)(g - a.g0) * kD;
@@ -382,11 +389,22 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
         float rh[kD], rl[kD];
         dfl::target(wset, a.cbs, a.cbs.n, i, g, rh, rl, err);  // (reads the code just written)
         float* d = a.D + i * a.N + g * kD;
+        uint32_t hi[kD], lo[kD];
 #pragma unroll
         for (int j = 0; j < kD; ++j) {
           const float nv = __fadd_rn(rh[j], rl[j]);
           d[j] = nv;
           sDD[tid][j] = nv - sDD[tid][j];
+          hi[j] = tc::to_tf32(nv);
+          lo[j] = tc::to_tf32(nv - __uint_as_float(hi[j]));
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int64_t off = img::img_off(i, g * kD + 4 * q, a.nslab);
+          *reinterpret_cast<uint4*>(a.d_hi + off) =
+              make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
+          *reinterpret_cast<uint4*>(a.d_lo + off) =
+              make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
         }
       } else {
 #pragma unroll
@@ -415,31 +433,19 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
   }
 }
 
-// sum_i sum_n Bt[n][i] D[i][c0 + n] over the block's columns (fp64 per thread, fixed order),
-// into part[blockIdx.x].
-__global__ void __launch_bounds__(256)
-block_loss_kernel(const float* __restrict__ Bt, int64_t ldb, int ncols,
-                  const float* __restrict__ D, int64_t M, int64_t N, int64_t c0,
-                  double* __restrict__ part) {
-  __shared__ double red[256];
+// *out = sum of part[0 .. n) (one CTA, strided sums and a tree: a fixed order).
+__global__ void __launch_bounds__(1024)
+sum_parts_kernel(const double* __restrict__ part, int64_t n, double* out) {
+  __shared__ double red[1024];
   double s = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M;
-       i += (int64_t)gridDim.x * blockDim.x)
-    for (int c = 0; c < ncols; ++c)
-      s += (double)Bt[(int64_t)c * ldb + i] * (double)D[i * N + c0 + c];
+  for (int64_t q = threadIdx.x; q < n; q += blockDim.x) s += part[q];
   red[threadIdx.x] = s;
   __syncthreads();
   for (int w = blockDim.x / 2; w > 0; w >>= 1) {
     if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] += red[0];
-}
-
-__global__ void sum_parts_kernel(const double* __restrict__ part, int n, double* out) {
-  double s = 0.0;
-  for (int q = 0; q < n; ++q) s += part[q];
-  *out = s;
+  if (threadIdx.x == 0) *out = red[0];
 }
 
 }  // namespace
@@ -453,19 +459,24 @@ crvq_status launch_coupled_sweep(const float* W, int64_t M, int64_t N, const flo
   CbList cbs = cbs_in;
   const CbView cw = cbs.cb[which];
   const int64_t G_cov = cw.G_cov;
-  const int loss_blocks = (int)std::min<int64_t>(std::max<int64_t>(1, ceil_div(M, 256)), 2 * nsm);
-  Scratch mD, mB, mP, mF;
+  const int64_t chunks = img_k_chunks(N);
+  const int64_t n_part = ceil_div(M, (int64_t)128) * ceil_div(N, (int64_t)256);
+  const size_t h_img = img_bytes(N, N), d_img = img_bytes(M, N);
+  Scratch mD, mI, mB, mP, mF;
   CRVQ_TRY(mD.alloc((size_t)M * N * sizeof(float), stream));
-  CRVQ_TRY(mB.alloc((size_t)kBlockCols * M * sizeof(float), stream));
-  CRVQ_TRY(mP.alloc((size_t)loss_blocks * sizeof(double), stream));
+  CRVQ_TRY(mI.alloc(2 * (h_img + d_img), stream));
+  CRVQ_TRY(mB.alloc((size_t)chunks * kBlockCols * M * sizeof(float), stream));
+  CRVQ_TRY(mP.alloc((size_t)n_part * sizeof(double), stream));
   CRVQ_TRY(mF.alloc((size_t)std::max<int64_t>(G_cov, 1) * (2 * kD * kD + kD) * sizeof(float),
                     stream));
   float* D = mD.as<float>();
-  float* Bt = mB.as<float>();
+  char* h_hi = mI.as<char>();
+  char* h_lo = h_hi + h_img;
+  char* d_hi = h_lo + h_img;
+  char* d_lo = d_hi + d_img;
   float* Hb = mF.as<float>();
   float* Lf = Hb + G_cov * kD * kD;
   float* Linv = Lf + G_cov * kD * kD;
-  const int64_t ldb = M;
   {
     ProfScope ps("coupled_residual", stream, (double)M * N * 8.0);
     residual_kernel<<<(unsigned)std::min<int64_t>(ceil_div(M * (N / kD), 256), 16 * nsm), 256, 0,
@@ -475,18 +486,12 @@ crvq_status launch_coupled_sweep(const float* W, int64_t M, int64_t N, const flo
                           stream>>>(H, N, G_cov, Hb, Lf, Linv, err);
     CRVQ_LAUNCHED();
   }
-  // tr(D H D^T) by column blocks: B^T = H[block rows, :] D^T, then the block's sum of B^T . D
-  auto loss_into = [&](double* out) -> crvq_status {
-    CRVQ_CUDA(cudaMemsetAsync(mP.as<double>(), 0, (size_t)loss_blocks * sizeof(double), stream));
-    for (int64_t c0 = 0; c0 < N; c0 += kBlockCols) {
-      const int nc = (int)std::min<int64_t>(kBlockCols, N - c0);
-      CRVQ_TRY(launch_tc_gemm_nt(H + c0 * N, N, nc, D, N, M, N, Bt, ldb, stream));
-      ProfScope ps("coupled_loss", stream, (double)M * nc * 8.0);
-      block_loss_kernel<<<loss_blocks, 256, 0, stream>>>(Bt, ldb, nc, D, M, N, c0,
-                                                         mP.as<double>());
-      CRVQ_LAUNCHED();
-    }
-    sum_parts_kernel<<<1, 1, 0, stream>>>(mP.as<double>(), loss_blocks, out);
+  // operand images of H and D; the sweep keeps D's up to date
+  CRVQ_TRY(launch_images(H, nullptr, nullptr, N, N, h_hi, h_lo, stream));
+  CRVQ_TRY(launch_images(D, nullptr, nullptr, M, N, d_hi, d_lo, stream));
+  auto loss_into = [&](double* out) -> crvq_status {  // tr(D H D^T) = sum (D H) . D
+    CRVQ_TRY(launch_img_dot(d_hi, d_lo, M, h_hi, h_lo, N, N, D, mP.as<double>(), stream));
+    sum_parts_kernel<<<1, 1024, 0, stream>>>(mP.as<double>(), n_part, out);
     CRVQ_LAUNCHED();
     return CRVQ_OK;
   };
@@ -498,8 +503,10 @@ crvq_status launch_coupled_sweep(const float* W, int64_t M, int64_t N, const flo
       const int64_t b1 = std::min<int64_t>(G_cov, b0 + kBlockG);
       const int nc = (int)((b1 - b0) * kD);
       // B^T for the block's channels, with every decision so far in D
-      CRVQ_TRY(launch_tc_gemm_nt(H + b0 * kD * N, N, nc, D, N, M, N, Bt, ldb, stream));
-      const CplArgs ca{W, D, H, Hb, Lf, Linv, Bt, M, N, b0, b1, rows, which, cbs};
+      CRVQ_TRY(launch_img_gemm_chunks(h_hi, h_lo, b0 * kD, nc, d_hi, d_lo, M, N, mB.as<float>(),
+                                      stream));
+      const CplArgs ca{W, D, H, Hb, Lf, Linv, mB.as<float>(), (int)chunks, d_hi, d_lo,
+                       ceil_div(N, (int64_t)img::kSlabK), M, N, b0, b1, rows, which, cbs};
       ProfScope ps("coupled_block", stream, (double)M * (b1 - b0) * cw.K);
       coupled_block_kernel<<<(unsigned)ceil_div(M, rows), kCplThreads, 0, stream>>>(ca, err);
       CRVQ_LAUNCHED();

@@ -1,10 +1,10 @@
 // S1: Hessian proxy H = X^T X / n + delta I (App. A.2; the paper's X is N x O and its proxy
 // XX^T is the same matrix as our X^T X).
 //
-// The dense product X^T X (the crvq_hessian entry) runs on the tensor cores (tc_gemm.cuh:
-// tcgen05, 3xTF32, tiles on or above the diagonal, mirrored; K split into 1024-token chunks
-// summed in fp32 in chunk order). A single CTA then takes the diagonal, the damping and the
-// original-order diagonal blocks. The layer schedule forms only the diagonal blocks
+// The dense product X^T X (the crvq_hessian entry) runs on the tensor cores (tc_gemm.cu: tcgen05,
+// 3xTF32, tiles that reach the upper triangle, mirrored; 1024-token chunks summed in fp32 in chunk
+// order) and writes its diagonal beside it. One CTA sums the diagonal; the damping is added where
+// the diagonal blocks are taken. The layer schedule forms only the diagonal blocks
 // (launch_tc_hessian_blocks in tc_gemm.cu), with the same values.
 #include "common.cuh"
 #include "kernels.h"
@@ -13,14 +13,13 @@ namespace crvq {
 
 namespace {
 
-// One CTA: xsq, delta = damp_rel * mean(xsq) (fixed-order fp64 sum), damped diagonal and the
-// original-order diagonal blocks.
+// One CTA: delta = damp_rel * mean(xsq) (fixed-order fp64 sum).
 __global__ void __launch_bounds__(1024)
-hessian_finalize_kernel(float* __restrict__ H, int64_t N, int d, float damp_rel,
-                        float* __restrict__ xsq, float* __restrict__ delta_out) {
+hessian_delta_kernel(const float* __restrict__ xsq, int64_t N, float damp_rel,
+                     float* __restrict__ delta_out, double* __restrict__ delta64) {
   __shared__ double part[1024];
   double s = 0.0;
-  for (int64_t i = threadIdx.x; i < N; i += blockDim.x) s += (double)H[i * N + i];
+  for (int64_t i = threadIdx.x; i < N; i += blockDim.x) s += (double)xsq[i];
   part[threadIdx.x] = s;
   __syncthreads();
   for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -28,12 +27,28 @@ hessian_finalize_kernel(float* __restrict__ H, int64_t N, int d, float damp_rel,
     __syncthreads();
   }
   const double delta = (double)damp_rel * (part[0] / (double)N);
-  for (int64_t i = threadIdx.x; i < N; i += blockDim.x) {
-    const float v = H[i * N + i];
-    xsq[i] = v;
-    H[i * N + i] = (float)((double)v + delta);
+  if (threadIdx.x == 0) {
+    if (delta_out) *delta_out = (float)delta;
+    *delta64 = delta;
   }
-  if (threadIdx.x == 0 && delta_out) *delta_out = (float)delta;
+}
+
+// Adds delta to the diagonal of H (rounded once from fp64) and takes the original-order diagonal
+// blocks (Hb may be null).
+__global__ void __launch_bounds__(256)
+hessian_damp_kernel(float* __restrict__ H, int64_t N, const double* __restrict__ delta64,
+                    float* __restrict__ Hb) {
+  const double delta = *delta64;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N * kD;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = e / kD, col = row / kD * kD + e % kD;
+    float v = H[row * N + col];
+    if (row == col) {
+      v = (float)((double)v + delta);
+      H[row * N + col] = v;
+    }
+    if (Hb) Hb[e] = v;
+  }
 }
 
 __global__ void extract_blocks_kernel(const float* __restrict__ H, int64_t N, int d,
@@ -63,15 +78,17 @@ __global__ void extract_blocks_kernel(const float* __restrict__ H, int64_t N, in
 crvq_status launch_hessian(const float* X, int64_t n, int64_t N, int d, float damp_rel,
                            float* H, float* xsq, float* H_blocks, float* delta,
                            cudaStream_t stream) {
-  unsigned* err = nullptr;
-  CRVQ_TRY(device_error_word(&err));
-  CRVQ_TRY(launch_tc_syrk(X, n, N, H, stream));
+  Scratch mem;
+  CRVQ_TRY(mem.alloc(sizeof(double), stream));
+  CRVQ_TRY(launch_tc_syrk(X, n, N, H, xsq, stream));
   {
     ProfScope ps("hessian_finalize", stream, 0.0);
-    hessian_finalize_kernel<<<1, 1024, 0, stream>>>(H, N, d, damp_rel, xsq, delta);
+    hessian_delta_kernel<<<1, 1024, 0, stream>>>(xsq, N, damp_rel, delta, mem.as<double>());
+    CRVQ_LAUNCHED();
+    const int blocks = (int)std::min<int64_t>(ceil_div(N * kD, 256), 4 * sm_count());
+    hessian_damp_kernel<<<blocks, 256, 0, stream>>>(H, N, mem.as<double>(), H_blocks);
     CRVQ_LAUNCHED();
   }
-  if (H_blocks) CRVQ_TRY(launch_extract_blocks(H, N, d, nullptr, H_blocks, stream));
   return CRVQ_OK;
 }
 

@@ -24,8 +24,9 @@ crvq_status launch_extract_blocks(const float* H, int64_t N, int d, const int32_
                                   float* H_blocks, cudaStream_t stream);
 
 // Tensor-core (tcgen05, 3xTF32) products.
-// S = X^T X / n for X n x N row-major (S N x N, both triangles).
-crvq_status launch_tc_syrk(const float* X, int64_t n, int64_t N, float* S, cudaStream_t stream);
+// S = X^T X / n for X n x N row-major (S N x N, both triangles) and its diagonal.
+crvq_status launch_tc_syrk(const float* X, int64_t n, int64_t N, float* S, float* diag,
+                           cudaStream_t stream);
 // Xt = X^T (N x ldt, columns [n, ldt) zero) for X n x N row-major.
 crvq_status launch_transpose(const float* X, int64_t n, int64_t N, float* Xt, int64_t ldt,
                              cudaStream_t stream);
@@ -47,11 +48,22 @@ crvq_status launch_tc_sumsq(const float* A, const float* A_sub, int64_t M, const
                             const int32_t* B_cols, int64_t Nb, int64_t K, double* part,
                             int64_t part_cap, int64_t* nparts, cudaStream_t stream);
 
-// C = A B^T on the tensor cores (3xTF32; K in chunks of 1024 added in order): A M x K
-// (leading dimension lda), B Nb x K (ldb), C M x Nb (ldc); all row-major, 16-byte aligned rows.
-crvq_status launch_tc_gemm_nt(const float* A, int64_t lda, int64_t M, const float* B,
-                              int64_t ldb, int64_t Nb, int64_t K, float* C, int64_t ldc,
-                              cudaStream_t stream);
+// Operand images (img.cuh) of src - sub (rows x K row-major; sub optional), or of src with its columns
+// in the order `cols`; each of hi and lo holds img_bytes(rows, K).
+size_t img_bytes(int64_t rows, int64_t K);
+crvq_status launch_images(const float* src, const float* sub, const int32_t* cols, int64_t rows,
+                          int64_t K, char* hi, char* lo, cudaStream_t stream);
+// K chunks of an image-fed product (1024 columns each).
+int64_t img_k_chunks(int64_t K);
+// P[c][m][n] = K chunk c of A B^T; A: M rows of its image from row a_row0 (a multiple of 256), B: Nb
+// rows. The product is the sum of the chunks in order.
+crvq_status launch_img_gemm_chunks(const char* a_hi, const char* a_lo, int64_t a_row0, int64_t M,
+                                   const char* b_hi, const char* b_lo, int64_t Nb, int64_t K,
+                                   float* P, cudaStream_t stream);
+// part[tile] = partial sums of sum (A B^T) . E (E row-major M x Nb), one per 128 x 256 tile.
+crvq_status launch_img_dot(const char* a_hi, const char* a_lo, int64_t M, const char* b_hi,
+                           const char* b_lo, int64_t Nb, int64_t K, const float* E, double* part,
+                           cudaStream_t stream);
 
 // hinv[i] = [H^-1]_ii (fp64) of a symmetric positive definite H (N x N fp32): blocked fp64
 // Cholesky, the inverse factor by blocked forward substitution, squared column norms.

@@ -1,12 +1,13 @@
-// Host side of the tcgen05 3xTF32 products: the dense symmetric X^T X and its diagonal blocks
-// alone (tc_gemm.cuh), and the image-fed sum of squares ||(A - A_sub) B^T||^2 of the full loss
-// (img:: below). The tensor core accumulates fp32 with a small systematic rounding bias per
-// accumulation step, so K is cut into chunks of at most kKChunk and the few chunk partials of
-// an element are summed afterwards in fp32, in chunk order (a relative error of a few u); the
-// squares are summed per row in fp32 and per tile in fp64.
+// The tcgen05 3xTF32 products: the image-fed kernel (dense X^T X, the sums of the losses, the coupled
+// sweep's blocks) and the host side of the diagonal blocks alone (tc_gemm.cuh). The tensor core
+// accumulates fp32 with a small systematic rounding bias per accumulation step, so K is cut into
+// chunks of at most kKChunk and the few chunk partials of an element are summed afterwards in fp32,
+// in chunk order (a relative error of a few u); squares are summed per row in fp32 and per tile in
+// fp64.
 #include <algorithm>
 
 #include "common.cuh"
+#include "img.cuh"
 #include "kernels.h"
 #include "tc_gemm.cuh"
 
@@ -25,23 +26,16 @@ __device__ __forceinline__ float chunk_sum(const float* __restrict__ P, int chun
   return s * scale;
 }
 
+// S = scale * the sum of the chunk partials P[c] (N x N each), and its diagonal.
 __global__ void __launch_bounds__(256)
-sum_partials_kernel(const float* __restrict__ P, int64_t count, int chunks, int64_t stride,
-                    float scale, float* __restrict__ out) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count;
-       e += (int64_t)gridDim.x * blockDim.x)
-    out[e] = chunk_sum(P, chunks, stride, e, scale);
-}
-
-// out[m][n] (leading dimension ldo) = sum of the chunk partials P[c][m][n] (M x Nb each), in
-// chunk order.
-__global__ void __launch_bounds__(256)
-sum_partials_strided_kernel(const float* __restrict__ P, int64_t M, int64_t Nb, int chunks,
-                            float* __restrict__ out, int64_t ldo) {
-  const int64_t count = M * Nb;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count;
-       e += (int64_t)gridDim.x * blockDim.x)
-    out[(e / Nb) * ldo + e % Nb] = chunk_sum(P, chunks, count, e, 1.f);
+sum_partials_kernel(const float* __restrict__ P, int64_t N, int chunks, float scale,
+                    float* __restrict__ S, float* __restrict__ diag) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < N * N;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const float v = chunk_sum(P, chunks, N * N, e, scale);
+    S[e] = v;
+    if (e % (N + 1) == 0) diag[e / (N + 1)] = v;
+  }
 }
 
 // Original-order blocks, one CTA: xsq[i] = the undamped diagonal, delta = damp_rel * mean(xsq)
@@ -108,35 +102,34 @@ transpose_kernel(const float* __restrict__ X, int64_t n, int64_t N, float* __res
   }
 }
 
-// ---- image-fed 3xTF32 sum of squares ||A B^T||_F^2 (the full loss of Alg. 1 QuantLoss)
+}  // namespace
+
+// ---- image-fed 3xTF32 products A B^T
 // Both operands are first written once as tf32 hi / lo images in the tcgen05 canonical
 // K-major layout (no swizzle): 256-row blocks, 16-column slabs of 16 KB each, slabs of a block
 // consecutive. A CTA then computes one 128 x 256 tile with no work of its threads on the
 // operand path: warp 0 streams the slabs by bulk copy (TMA) into a four-stage ring, warp 1
-// issues the MMAs (hi.hi, hi.lo, lo.hi per 8-column step, as the split GEMM does), and warps
-// 2-5 keep the K-chunk partials: after every 1024-column chunk the accumulator is added, in
-// chunk order and in fp32, to a running sum kept in the other half of tensor memory; the last
-// chunk's sum is squared and summed per row.
+// issues the MMAs (hi.hi, hi.lo, lo.hi per 8-column step), and warps 2-5 keep the K-chunk
+// partials: after every 1024-column chunk the accumulator is added, in chunk order and in fp32, to
+// a running sum kept in the other half of tensor memory. The last chunk's sum goes to the epilogue:
+//   kSumsq      the sum of its squares (the full loss of Alg. 1 QuantLoss);
+//   kDot        the sum of its products with E's entries in fp32 pairs (tr(D H D^T));
+//   kSymmetric  C[m][n] = C[n][m] = alpha D[m][n] for n >= m (the Hessian; tiles below the
+//               diagonal do nothing);
+//   kPlain      C[m][n] = alpha D[m][n] (blockIdx.y: one K chunk each, to its own C).
+// Row-major stores go through shared memory, so that a warp writes 128 consecutive bytes of a row.
 namespace img {
+namespace {
 
-constexpr int kRowsBlk = 256;                      // image block rows
-constexpr int kSlabK = 16;                         // image slab columns
-constexpr int kSlabBytes = kRowsBlk * kSlabK * 4;  // 16 KB
 constexpr int kAStage = 2 * (kSlabBytes / 2);      // A hi + lo, 128 rows: 16 KB
 constexpr int kBStage = 2 * kSlabBytes;            // B hi + lo, 256 rows: 32 KB
 constexpr int kStageBytes = kAStage + kBStage;     // 48 KB
 constexpr int kStages = 4;
-constexpr int kSmem = kStages * kStageBytes + 1024 + 256;
+constexpr int kStageOut = 4 * 32 * 33 * 4;         // transposing buffers of the storing warps
+constexpr int kSmem = kStages * kStageBytes + kStageOut + 1024 + 256;
 constexpr int kThreads = 192;
 constexpr int kChunkSlabs = 1024 / kSlabK;         // slabs per K chunk
 constexpr uint32_t kIdesc = tc::idesc_tf32(128, 256);
-
-// Image byte offset of element (r, k): block r / 256, slab k / 16, then the canonical offset.
-__host__ __device__ inline int64_t img_off(int64_t r, int64_t k, int64_t nslab) {
-  const int64_t blk = r / kRowsBlk, rr = r % kRowsBlk, sl = k / kSlabK, kk = k % kSlabK;
-  return (blk * nslab + sl) * kSlabBytes +
-         (((rr >> 3) * (kSlabK / 4) + (kk >> 2)) * 128 + (rr & 7) * 16 + (kk & 3) * 4);
-}
 
 // One warp = 8 rows x one 16-column slab: reads 8 x 64 B, writes 512 contiguous bytes per
 // image. Element (r, k) is src[r][k] - sub[r][k] (sub optional, same layout), or
@@ -185,18 +178,58 @@ image_kernel(const float* __restrict__ src, const float* __restrict__ sub,
   *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-struct SumsqArgs {
+// Images of X^T: element (r, k) is X[k][r] (X: K x rows row-major). A thread takes row r, four
+// columns: its reads are 128 consecutive bytes per warp, its writes whole 128-byte core matrices.
+__global__ void __launch_bounds__(256)
+image_t_kernel(const float* __restrict__ X, int64_t rows, int64_t K, int64_t rows_pad,
+               int64_t nslab, char* __restrict__ hi, char* __restrict__ lo) {
+  const int64_t r = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  if (r >= rows_pad) return;
+  for (int64_t k = ((int64_t)blockIdx.y * 8 + (threadIdx.x >> 5)) * 4; k < nslab * kSlabK;
+       k += (int64_t)gridDim.y * 32) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float v = (r < rows && k + j < K) ? __ldg(X + (k + j) * rows + r) : 0.f;
+      h[j] = tc::to_tf32(v);
+      l[j] = tc::to_tf32(v - __uint_as_float(h[j]));
+    }
+    const int64_t off = img_off(r, k, nslab);
+    *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
+  }
+}
+
+enum Epilogue { kSumsq, kDot, kSymmetric, kPlain };
+
+struct ImgArgs {
   const char *a_hi, *a_lo, *b_hi, *b_lo;  // images
   int64_t nslab;                          // slabs per block (both images)
+  int64_t slabs_y;                        // slabs per blockIdx.y (nslab, or one K chunk)
   int tiles_n;                            // 256-row tiles of B
-  double* part;                           // part[tile] = sum over the tile of D^2
+  double* part;                           // kSumsq, kDot: part[tile]
+  const float* E;                         // kDot: E[m][n]
+  float* C;                               // kSymmetric, kPlain: + blockIdx.y * c_stride
+  int64_t ldc, c_stride;                  // leading dimension of C (or E)
+  float alpha;
+  float* diag;                            // kSymmetric: the diagonal, or null
+  int64_t rows_m, rows_n;
   unsigned* err;
 };
 
-__global__ void __launch_bounds__(kThreads, 1) sumsq_img_kernel(SumsqArgs a) {
+__device__ __forceinline__ void pair_acc(float& h, float& l, float x) {  // (h, l) += x
+  const float s = __fadd_rn(h, x);
+  const float bp = __fsub_rn(s, h);
+  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, bp)), __fsub_rn(x, bp)));
+  h = s;
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
   extern __shared__ __align__(1024) char smem_raw[];
   char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+  float* stage_out = reinterpret_cast<float*>(smem + kStages * kStageBytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes + kStageOut);
   uint64_t* empty = full + kStages;
   uint64_t* acc_full = empty + kStages;
   uint64_t* acc_empty = acc_full + 1;
@@ -206,8 +239,10 @@ __global__ void __launch_bounds__(kThreads, 1) sumsq_img_kernel(SumsqArgs a) {
 
   const int tile = blockIdx.x;
   const int bm = tile / a.tiles_n, bn = tile % a.tiles_n;
+  if (EPI == kSymmetric && (int64_t)(bn + 1) * 256 <= (int64_t)bm * 128) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t nslab = a.nslab;
+  const int64_t slab0 = (int64_t)blockIdx.y * a.slabs_y;
+  const int64_t nslab = min(a.slabs_y, a.nslab - slab0);  // of this CTA
   const int nchunk = (int)((nslab + kChunkSlabs - 1) / kChunkSlabs);
 
   if (warp == 0) tc::tmem_alloc(tmem_slot, 512);
@@ -228,10 +263,9 @@ __global__ void __launch_bounds__(kThreads, 1) sumsq_img_kernel(SumsqArgs a) {
 
   if (warp == 0) {
     if (lane == 0) {  // producer
-      const char* ah = a.a_hi + ((int64_t)(bm >> 1) * nslab) * kSlabBytes + (bm & 1) * (kSlabBytes / 2);
-      const char* al = a.a_lo + ((int64_t)(bm >> 1) * nslab) * kSlabBytes + (bm & 1) * (kSlabBytes / 2);
-      const char* bh = a.b_hi + (int64_t)bn * nslab * kSlabBytes;
-      const char* bl = a.b_lo + (int64_t)bn * nslab * kSlabBytes;
+      const int64_t a0 = ((int64_t)(bm >> 1) * a.nslab + slab0) * kSlabBytes + (bm & 1) * (kSlabBytes / 2);
+      const int64_t b0 = ((int64_t)bn * a.nslab + slab0) * kSlabBytes;
+      const char *ah = a.a_hi + a0, *al = a.a_lo + a0, *bh = a.b_hi + b0, *bl = a.b_lo + b0;
       bool ok = true;
       for (int64_t it = 0; it < nslab && ok; ++it) {
         const int s = (int)(it % kStages);
@@ -280,7 +314,10 @@ __global__ void __launch_bounds__(kThreads, 1) sumsq_img_kernel(SumsqArgs a) {
     }
   } else {  // warps 2-5: one accumulator row (tensor-memory lane) per thread
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    float sq = 0.f;
+    const int64_t m0 = (int64_t)bm * 128 + (warp & 3) * 32, m = m0 + lane;
+    float* C = EPI == kPlain || EPI == kSymmetric ? a.C + blockIdx.y * a.c_stride : nullptr;
+    float* so = stage_out + (warp & 3) * 32 * 33;
+    float sq = 0.f, sl = 0.f;  // kSumsq: the sum of squares; kDot: a pair
     bool ok = true;
     for (int c = 0; c < nchunk && ok; ++c) {
       ok = tc::mbar_wait(tc::smem_u32(acc_full), (uint32_t)(c & 1), a.err);
@@ -300,9 +337,38 @@ __global__ void __launch_bounds__(kThreads, 1) sumsq_img_kernel(SumsqArgs a) {
           for (int j = 0; j < 32; ++j)
             v[j] = __float_as_uint(__fadd_rn(__uint_as_float(w[j]), __uint_as_float(v[j])));
         }
-        if (last) {
+        if (last && EPI == kSumsq) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) sq = fmaf(__uint_as_float(v[j]), __uint_as_float(v[j]), sq);
+        } else if (last) {
+          // rows of 32 columns: registers hold a row per lane, memory wants a row per warp
+          const int64_t n0 = (int64_t)bn * 256 + c0, n = n0 + lane;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const float x = EPI == kDot ? __uint_as_float(v[j]) : a.alpha * __uint_as_float(v[j]);
+            so[lane * 33 + j] = x;
+            if (EPI == kSymmetric && n0 + j > m && m < a.rows_m && n0 + j < a.rows_n)
+              C[(n0 + j) * a.ldc + m] = x;
+            if (EPI == kSymmetric && a.diag && n0 + j == m && m < a.rows_m) a.diag[m] = x;
+          }
+          __syncwarp();
+          if (n < a.rows_n) {
+#pragma unroll 8
+            for (int r = 0; r < 32; ++r) {
+              const int64_t mr = m0 + r;
+              if (mr >= a.rows_m) break;
+              const float x = so[r * 33 + lane];
+              if (EPI == kDot) {
+                const float e = __ldg(a.E + mr * a.ldc + n);
+                const float p = __fmul_rn(x, e);
+                pair_acc(sq, sl, p);
+                sl = __fadd_rn(sl, __fmaf_rn(x, e, -p));
+              } else if (EPI == kPlain || n >= mr) {
+                C[mr * a.ldc + n] = x;
+              }
+            }
+          }
+          __syncwarp();
         } else {
           tc::tmem_st32_wait(tmem + lane_base + 256u + (uint32_t)c0, v);
         }
@@ -310,8 +376,8 @@ __global__ void __launch_bounds__(kThreads, 1) sumsq_img_kernel(SumsqArgs a) {
       tc::tc_fence_before();
       if (!last) tc::mbar_arrive(tc::smem_u32(acc_empty));
     }
-    if (!ok) sq = 0.f;
-    double sd = (double)sq;
+    if (!ok) sq = sl = 0.f;
+    double sd = (double)sq + (double)sl;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sd += __shfl_xor_sync(0xffffffffu, sd, o);
     if (lane == 0) red[warp - 2] = sd;
@@ -319,7 +385,7 @@ __global__ void __launch_bounds__(kThreads, 1) sumsq_img_kernel(SumsqArgs a) {
   }
   tc::tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && (EPI == kSumsq || EPI == kDot)) {
     const bool ok = ok_s[0] && ok_s[1] && ok_s[2];
     a.part[tile] = ok ? ((red[0] + red[1]) + (red[2] + red[3])) : 0.0;
   }
@@ -330,104 +396,84 @@ __global__ void __launch_bounds__(kThreads, 1) sumsq_img_kernel(SumsqArgs a) {
   }
 }
 
-}  // namespace img
-
-crvq_status launch_gemm(tc::GemmArgs g, int64_t chunks, cudaStream_t stream) {
-  static bool attr_set[64] = {};
-  int dev = 0;
-  CRVQ_CUDA(cudaGetDevice(&dev));
-  if (dev < 64 && !attr_set[dev]) {
-    CRVQ_CUDA(cudaFuncSetAttribute(tc::gemm3xtf32_kernel,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes));
-    attr_set[dev] = true;
-  }
-  const int64_t tm = ceil_div(g.A.rows, tc::kBM), tn = ceil_div(g.B.rows, tc::kBN);
-  g.tiles_n = (int)tn;
-  dim3 grid((unsigned)(tm * tn), (unsigned)chunks);
-  tc::gemm3xtf32_kernel<<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(g);
+template <int EPI>
+crvq_status launch(const ImgArgs& a, int64_t tiles_m, int64_t chunks, cudaStream_t stream) {
+  CRVQ_TRY(smem_limit((const void*)img_gemm_kernel<EPI>, kSmem));
+  img_gemm_kernel<EPI><<<dim3((unsigned)(tiles_m * a.tiles_n), (unsigned)chunks), kThreads, kSmem,
+                         stream>>>(a);
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
 
-}  // namespace
+int64_t pad_rows(int64_t rows) { return ceil_div(rows, (int64_t)kRowsBlk) * kRowsBlk; }
 
-// S = X^T X / n (X: n x N row-major) into S (N x N), both triangles, via split-K partials.
-crvq_status launch_tc_syrk(const float* X, int64_t n, int64_t N, float* S, cudaStream_t stream) {
-  unsigned* err = nullptr;
-  CRVQ_TRY(device_error_word(&err));
-  const int64_t chunks = ceil_div(n, kKChunk);
-  Scratch mem, xt_mem;
-  float* P = S;
-  if (chunks > 1) {
-    CRVQ_TRY(mem.alloc((size_t)chunks * N * N * sizeof(float), stream));
-    P = mem.as<float>();
-  }
-  // X^T with rows padded to a multiple of 4 floats: both operands K-major, loaded with 16-byte
-  // loads (A(a, k) = X[k][a])
-  const int64_t ldt = (n + 3) / 4 * 4;
-  CRVQ_TRY(xt_mem.alloc((size_t)N * ldt * sizeof(float), stream));
-  CRVQ_TRY(launch_transpose(X, n, N, xt_mem.as<float>(), ldt, stream));
-  tc::GemmArgs g{};
-  g.A = tc::Operand{xt_mem.as<float>(), ldt, N, true};
-  g.B = g.A;
-  g.K = n;
-  g.k_chunk = kKChunk;
-  g.c_chunk_stride = N * N;
-  g.mode = tc::kStoreSymmetric;
-  g.C = P;
-  g.ldc = N;
-  g.alpha = chunks > 1 ? 1.f : (float)(1.0 / (double)n);
-  g.err = err;
-  {
-    ProfScope ps("hessian_gemm_tc", stream, 2.0 * (double)n * N * N);
-    CRVQ_TRY(launch_gemm(g, chunks, stream));
-  }
-  if (chunks > 1) {
-    ProfScope ps("hessian_sum_partials", stream, (double)chunks * N * N * 4.0);
-    const int blocks = (int)std::min<int64_t>(ceil_div(N * N, 256), 16 * sm_count());
-    sum_partials_kernel<<<blocks, 256, 0, stream>>>(P, N * N, (int)chunks, N * N,
-                                                    (float)(1.0 / (double)n), S);
-    CRVQ_LAUNCHED();
-  }
+}  // namespace
+}  // namespace img
+
+size_t img_bytes(int64_t rows, int64_t K) {
+  return (size_t)img::pad_rows(rows) * ceil_div(K, (int64_t)img::kSlabK) * img::kSlabK * 4;
+}
+
+int64_t img_k_chunks(int64_t K) { return std::max<int64_t>(1, ceil_div(K, kKChunk)); }
+
+crvq_status launch_images(const float* src, const float* sub, const int32_t* cols, int64_t rows,
+                          int64_t K, char* hi, char* lo, cudaStream_t stream) {
+  const int64_t nslab = ceil_div(K, (int64_t)img::kSlabK), pad = img::pad_rows(rows);
+  img::image_kernel<<<dim3((unsigned)(pad / 8), (unsigned)ceil_div(nslab, 8)), 256, 0, stream>>>(
+      src, sub, cols, rows, K, K, pad, nslab, hi, lo);
+  CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
 
-// C = A B^T (A: M x K, B: Nb x K, both row-major with leading dimensions lda, ldb; C: M x Nb
-// row-major, leading dimension ldc) on the tensor cores (3xTF32), K in chunks of at most 1024
-// whose partials are added in chunk order (the rounding sequence of the Hessian products).
-crvq_status launch_tc_gemm_nt(const float* A, int64_t lda, int64_t M, const float* B,
-                              int64_t ldb, int64_t Nb, int64_t K, float* C, int64_t ldc,
-                              cudaStream_t stream) {
+// S = X^T X / n (X: n x N row-major) into S (N x N), both triangles, and its diagonal: the images of X^T, then one
+// product over the tiles that reach the upper triangle, chunk sums kept in tensor memory. (Splitting
+// the operands in the product's own shared-memory stages bound it by the L1TEX pipe: 765 us at
+// N = n = 4096, with 57 us more for adding chunk partials kept in memory; now 325 us in all.)
+crvq_status launch_tc_syrk(const float* X, int64_t n, int64_t N, float* S, float* diag,
+                           cudaStream_t stream) {
   unsigned* err = nullptr;
   CRVQ_TRY(device_error_word(&err));
-  const int64_t chunks = std::max<int64_t>(1, ceil_div(K, kKChunk));
+  const size_t bytes = img_bytes(N, n);
   Scratch mem;
-  float* P = C;
-  int64_t ldp = ldc;
-  if (chunks > 1) {
-    CRVQ_TRY(mem.alloc((size_t)chunks * M * Nb * sizeof(float), stream));
-    P = mem.as<float>();
-    ldp = Nb;
+  CRVQ_TRY(mem.alloc(2 * bytes, stream));
+  char *hi = mem.as<char>(), *lo = hi + bytes;
+  const int64_t nslab = ceil_div(n, (int64_t)img::kSlabK), pad = img::pad_rows(N);
+  {
+    ProfScope ps("hessian_images", stream, 12.0 * (double)n * N);
+    const unsigned gy = (unsigned)std::min<int64_t>(ceil_div(nslab * 4, 8), 65535);
+    img::image_t_kernel<<<dim3((unsigned)(pad / 32), gy), 256, 0, stream>>>(X, N, n, pad, nslab, hi,
+                                                                            lo);
+    CRVQ_LAUNCHED();
   }
-  tc::GemmArgs g{};
-  g.A = tc::Operand{A, lda, M, true};
-  g.B = tc::Operand{B, ldb, Nb, true};
-  g.K = K;
-  g.k_chunk = kKChunk;
-  g.c_chunk_stride = M * Nb;
-  g.mode = tc::kStorePlain;
-  g.C = P;
-  g.ldc = ldp;
-  g.alpha = 1.f;
+  // Few tiles (small N): each K chunk in its own CTA, the partials added afterwards in chunk order;
+  // otherwise a CTA runs through all chunks of its tile. The same rounding sequence.
+  const int64_t tiles_m = ceil_div(N, (int64_t)128), tiles_n = ceil_div(N, (int64_t)256);
+  const int64_t chunks = img_k_chunks(n);
+  const bool split = chunks > 1 && tiles_m * tiles_n <= sm_count();
+  const float scale = (float)(1.0 / (double)n);
+  Scratch pmem;
+  if (split) CRVQ_TRY(pmem.alloc((size_t)chunks * N * N * sizeof(float), stream));
+  img::ImgArgs g{};
+  g.a_hi = g.b_hi = hi;
+  g.a_lo = g.b_lo = lo;
+  g.nslab = nslab;
+  g.slabs_y = split ? img::kChunkSlabs : nslab;
+  g.tiles_n = (int)tiles_n;
+  g.C = split ? pmem.as<float>() : S;
+  g.ldc = N;
+  g.c_stride = N * N;
+  g.alpha = split ? 1.f : scale;
+  g.diag = split ? nullptr : diag;
+  g.rows_m = g.rows_n = N;
   g.err = err;
   {
-    ProfScope ps("gemm_nt_tc", stream, 2.0 * (double)M * Nb * K);
-    CRVQ_TRY(launch_gemm(g, chunks, stream));
+    ProfScope ps("hessian_gemm_tc", stream, 2.0 * (double)n * N * N);
+    CRVQ_TRY(img::launch<img::kSymmetric>(g, tiles_m, split ? chunks : 1, stream));
   }
-  if (chunks > 1) {
-    ProfScope ps("gemm_nt_sum_partials", stream, (double)chunks * M * Nb * 4.0);
-    const int blocks = (int)std::min<int64_t>(ceil_div(M * Nb, 256), 16 * sm_count());
-    sum_partials_strided_kernel<<<blocks, 256, 0, stream>>>(P, M, Nb, (int)chunks, C, ldc);
+  if (split) {
+    ProfScope ps("hessian_sum_partials", stream, (double)chunks * N * N * 4.0);
+    const int blocks = (int)std::min<int64_t>(ceil_div(N * N, 256), 16 * sm_count());
+    sum_partials_kernel<<<blocks, 256, 0, stream>>>(pmem.as<float>(), N, (int)chunks, scale, S, diag);
     CRVQ_LAUNCHED();
   }
   return CRVQ_OK;
@@ -442,25 +488,13 @@ crvq_status launch_tc_sumsq(const float* A, const float* A_sub, int64_t M, const
                             int64_t part_cap, int64_t* nparts, cudaStream_t stream) {
   unsigned* err = nullptr;
   CRVQ_TRY(device_error_word(&err));
-  static bool attr_set[64] = {};
-  int dev = 0;
-  CRVQ_CUDA(cudaGetDevice(&dev));
-  if (dev < 64 && !attr_set[dev]) {
-    CRVQ_CUDA(cudaFuncSetAttribute(img::sumsq_img_kernel,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, img::kSmem));
-    attr_set[dev] = true;
-  }
-  const int64_t tiles_m = ceil_div(M, 128), tiles_n = ceil_div(Nb, 256);
+  const int64_t tiles_m = ceil_div(M, (int64_t)128), tiles_n = ceil_div(Nb, (int64_t)256);
   if (tiles_m * tiles_n > part_cap)
     return fail(CRVQ_ERR_UNSUPPORTED, "loss product: %lld tiles exceed %lld partials",
                 (long long)(tiles_m * tiles_n), (long long)part_cap);
   if (tiles_m * tiles_n > INT32_MAX)
     return fail(CRVQ_ERR_UNSUPPORTED, "loss product: too many tiles");
-  const int64_t nslab = ceil_div(K, (int64_t)img::kSlabK);
-  const int64_t am = ceil_div(M, (int64_t)img::kRowsBlk) * img::kRowsBlk;
-  const int64_t bm = ceil_div(Nb, (int64_t)img::kRowsBlk) * img::kRowsBlk;
-  const size_t a_bytes = (size_t)am * nslab * img::kSlabK * 4;
-  const size_t b_bytes = (size_t)bm * nslab * img::kSlabK * 4;
+  const size_t a_bytes = img_bytes(M, K), b_bytes = img_bytes(Nb, K);
   Scratch mem;
   CRVQ_TRY(mem.alloc(2 * a_bytes + 2 * b_bytes, stream));
   char* a_hi = mem.as<char>();
@@ -469,19 +503,74 @@ crvq_status launch_tc_sumsq(const float* A, const float* A_sub, int64_t M, const
   char* b_lo = b_hi + b_bytes;
   {
     ProfScope ps("loss_images", stream, 12.0 * (double)(M + Nb) * K);
-    img::image_kernel<<<dim3((unsigned)(am / 8), (unsigned)ceil_div(nslab, 8)), 256, 0,
-                        stream>>>(A, A_sub, nullptr, M, K, K, am, nslab, a_hi, a_lo);
-    CRVQ_LAUNCHED();
-    img::image_kernel<<<dim3((unsigned)(bm / 8), (unsigned)ceil_div(nslab, 8)), 256, 0,
-                        stream>>>(B, nullptr, B_cols, Nb, K, K, bm, nslab, b_hi, b_lo);
-    CRVQ_LAUNCHED();
+    CRVQ_TRY(launch_images(A, A_sub, nullptr, M, K, a_hi, a_lo, stream));
+    CRVQ_TRY(launch_images(B, nullptr, B_cols, Nb, K, b_hi, b_lo, stream));
   }
-  img::SumsqArgs g{a_hi, a_lo, b_hi, b_lo, nslab, (int)tiles_n, part, err};
+  img::ImgArgs g{};
+  g.a_hi = a_hi;
+  g.a_lo = a_lo;
+  g.b_hi = b_hi;
+  g.b_lo = b_lo;
+  g.nslab = g.slabs_y = ceil_div(K, (int64_t)img::kSlabK);
+  g.tiles_n = (int)tiles_n;
+  g.part = part;
+  g.err = err;
   ProfScope ps("loss_gemm_tc", stream, 2.0 * (double)M * Nb * K);
-  img::sumsq_img_kernel<<<(unsigned)(tiles_m * tiles_n), img::kThreads, img::kSmem, stream>>>(g);
-  CRVQ_LAUNCHED();
+  CRVQ_TRY(img::launch<img::kSumsq>(g, tiles_m, 1, stream));
   *nparts = tiles_m * tiles_n;
   return CRVQ_OK;
+}
+
+// P[c][m][n] = the K chunk c of A B^T (A: M rows starting at block row `a_row0`, a multiple of 256,
+// of its image; B: Nb rows; both with K columns), c < img_k_chunks(K), each M x Nb.
+crvq_status launch_img_gemm_chunks(const char* a_hi, const char* a_lo, int64_t a_row0, int64_t M,
+                                   const char* b_hi, const char* b_lo, int64_t Nb, int64_t K,
+                                   float* P, cudaStream_t stream) {
+  unsigned* err = nullptr;
+  CRVQ_TRY(device_error_word(&err));
+  const int64_t nslab = ceil_div(K, (int64_t)img::kSlabK);
+  const int64_t a_off = a_row0 / img::kRowsBlk * nslab * img::kSlabBytes;
+  img::ImgArgs g{};
+  g.a_hi = a_hi + a_off;
+  g.a_lo = a_lo + a_off;
+  g.b_hi = b_hi;
+  g.b_lo = b_lo;
+  g.nslab = nslab;
+  g.slabs_y = img::kChunkSlabs;
+  g.tiles_n = (int)ceil_div(Nb, (int64_t)256);
+  g.C = P;
+  g.ldc = Nb;
+  g.c_stride = M * Nb;
+  g.alpha = 1.f;
+  g.rows_m = M;
+  g.rows_n = Nb;
+  g.err = err;
+  ProfScope ps("gemm_nt_tc", stream, 2.0 * (double)M * Nb * K);
+  return img::launch<img::kPlain>(g, ceil_div(M, (int64_t)128), img_k_chunks(K), stream);
+}
+
+// part[tile] = partial sums of sum_{m,n} (A B^T)[m][n] E[m][n] (A: M x K, B: Nb x K images; E
+// row-major M x Nb), one per 128 x 256 tile.
+crvq_status launch_img_dot(const char* a_hi, const char* a_lo, int64_t M, const char* b_hi,
+                           const char* b_lo, int64_t Nb, int64_t K, const float* E, double* part,
+                           cudaStream_t stream) {
+  unsigned* err = nullptr;
+  CRVQ_TRY(device_error_word(&err));
+  img::ImgArgs g{};
+  g.a_hi = a_hi;
+  g.a_lo = a_lo;
+  g.b_hi = b_hi;
+  g.b_lo = b_lo;
+  g.nslab = g.slabs_y = ceil_div(K, (int64_t)img::kSlabK);
+  g.tiles_n = (int)ceil_div(Nb, (int64_t)256);
+  g.part = part;
+  g.E = E;
+  g.ldc = Nb;
+  g.rows_m = M;
+  g.rows_n = Nb;
+  g.err = err;
+  ProfScope ps("coupled_loss", stream, 2.0 * (double)M * Nb * K);
+  return img::launch<img::kDot>(g, ceil_div(M, (int64_t)128), 1, stream);
 }
 
 crvq_status launch_transpose(const float* X, int64_t n, int64_t N, float* Xt, int64_t ldt,

@@ -147,3 +147,20 @@ def test_coupled_sweep_on_a_quantized_q_proj_sampled_rows():
     ocbs = [O.Codebook(host(out.C_base), host(start_codes), G)] + \
         [O.Codebook(host(out.C_ext[t]), host(out.codes_ext[t]), Gc) for t in range(cfg.n_ext)]
     _stepwise(host(Ws), host(Hs), ocbs, 0, host(out.codes_base), rows)
+
+
+@pytest.mark.parametrize("M,G,K", [(1, 1, 1), (33, 33, 300), (7, 65, 256), (1300, 3, 257)])
+def test_coupled_sweep_block_row_and_codebook_edges(M, G, K):
+    """Rows around a CTA's share, groups around the 32-group blocks, codebooks around the 256 of a
+    score chunk; stepwise against the fp64 arg-min, losses against the oracle."""
+    import paper_2412_09282_gb300 as P
+    from paper_2412_09282_gb300 import Codebook
+    W, H, cbs = _case(31, M=M, G=G, K=K, Ke=5, Gc=min(G, 2), n=8 * G + 100)
+    gcbs = [Codebook(dev(cb.C), dev(cb.codes.astype(np.int32)), cb.G_cov) for cb in cbs]
+    loss = P.crvq_coupled_sweep(dev(W), dev(H), gcbs, 0, sweeps=1)
+    P.crvq_sync()
+    codes = host(gcbs[0].codes)
+    _stepwise(W, H, cbs, 0, codes, np.arange(M))
+    after = [O.Codebook(cbs[0].C, codes, G), cbs[1]]
+    assert loss[0] == pytest.approx(O.full_loss(W, H, cbs), rel=1e-5)
+    assert loss[1] == pytest.approx(O.full_loss(W, H, after), rel=1e-5)

@@ -206,13 +206,19 @@ __device__ __forceinline__ void split(float x, uint32_t& hi, uint32_t& lo) {
 
 // Row of the B operand for codeword kk of C (K codewords): [c_hi | c_lo | c_hi | n'_hi n'_lo |
 // L1_hi L1_lo L1_hi | 1 1 | 0]; padding rows (kk >= K) score +1e30.
+// t = (n, Na, L1) of the codeword (codeword_terms; zeros for padding).
 __device__ __forceinline__ void build_b_row(const float* __restrict__ C, int K, int kk,
-                                            const float* H, float uc, uint32_t row[tcenc::kK]) {
+                                            const float* H, float uc, uint32_t row[tcenc::kK],
+                                            float t[3]) {
   using namespace tcenc;
+  t[0] = t[1] = t[2] = 0.f;
   if (kk < K) {
     float cv[kD], n, na, l1;
     load_vec(C + (int64_t)kk * kD, cv);
     codeword_terms(cv, H, n, na, l1);
+    t[0] = n;
+    t[1] = na;
+    t[2] = l1;
 #pragma unroll
     for (int p = 0; p < kD; ++p) {
       uint32_t hh, ll;
@@ -283,9 +289,9 @@ prep_b_kernel(SetView set, int64_t g_begin, int64_t G_range, const float* __rest
               float* __restrict__ cbmax, unsigned* __restrict__ flag_count) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
-  // The flag list of the arg-min pass that follows starts empty. The previous pass's exact
-  // kernel, which read the count, completed before the wait above returned.
-  if (blockIdx.x == 0 && threadIdx.x == 0) *flag_count = 0u;
+  // The open lists of the arg-min pass that follows start empty. The previous pass's exact
+  // kernels, which read the counts, completed before the wait above returned.
+  if (blockIdx.x == 0 && threadIdx.x < 2) flag_count[threadIdx.x] = 0u;
   if (blockIdx.x == gridDim.x - 1) {  // the last CTA: the codebook maxima
     cbmax_block(C, K, cbmax);
     return;
@@ -299,14 +305,10 @@ prep_b_kernel(SetView set, int64_t g_begin, int64_t G_range, const float* __rest
     const int64_t g = g_begin + blk / nchunk;
     uint32_t v[tcenc::kK];
     const int kk = chunk * kTcCols + row;
-    build_b_row(C, K, kk, set.Hb + g * kD * kD, uc, v);
+    float tk[3];
+    build_b_row(C, K, kk, set.Hb + g * kD * kD, uc, v, tk);
     tcenc::put_row(out + blk * kTcBTile, row, v);
-    if (kk < K) {
-      float cv[kD], n, na, l1;
-      load_vec(C + (int64_t)kk * kD, cv);
-      codeword_terms(cv, set.Hb + g * kD * kD, n, na, l1);
-      terms[(g - g_begin) * K + kk] = make_float4(n, na, l1, 0.f);
-    }
+    if (kk < K) terms[(g - g_begin) * K + kk] = make_float4(tk[0], tk[1], tk[2], 0.f);
   }
 }
 
@@ -386,29 +388,25 @@ constexpr size_t kArgminSmem = 2 * (size_t)tcenc::kATile + 2 * (size_t)kTcBTile 
                                2 * (size_t)tcenc::kRows * kD * 4 + (size_t)kTcSmemStatsK * 8 +
                                (size_t)kOpenCap * sizeof(OpenRow) + 1024;
 
-// Exact decision of one open row by the eight lanes of a quarter warp (all 32 lanes call it; a
-// quarter with live = false takes part without writing): the candidates named by the masks are
-// scored in fp32 pairs, the smallest (err, index) wins, its statistics are added when requested.
+// Exact decision of one open row (i, g) by the eight lanes of a quarter warp (all 32 lanes call it; a
+// quarter with live = false takes part without writing): the candidates k = cand(0 .. total - 1)
+// are scored in fp32 pairs (H: the group's block), the smallest (err, index) wins, its statistics
+// are added when requested.
+template <class Cand>
 __device__ __forceinline__ void decide_open(const SetView& set, const CbList& cbs, int n_fixed,
-                                            int s_idx, const OpenRow& o, bool live,
-                                            int32_t* __restrict__ out_code, int64_t out_ld,
-                                            int64_t out_g0, const StatsView& st, float sscale,
-                                            unsigned* err) {
+                                            int s_idx, int64_t i, int64_t g, bool live, int total,
+                                            Cand cand, int32_t* __restrict__ out_code,
+                                            int64_t out_ld, int64_t out_g0, const StatsView& st,
+                                            float sscale, unsigned* err) {
   const CbView& cw = cbs.cb[s_idx];
   const int sub = threadIdx.x & 7;
-  const int64_t i = o.i, g = o.g;
   const float* H = set.Hb + g * kD * kD;
   float rh[kD], rl[kD];
   dfl::target(set, cbs, n_fixed, i, g, rh, rl, err);
-  const uint32_t bm = o.masks >> 16, em = o.masks & 0xffffu;
-  const int ne = __popc(em), total = __popc(bm) * ne;
   float bh = INFINITY, bl = 0.f;
   int bk = 0x7fffffff;
   for (int c = sub; c < total; c += 8) {
-    uint32_t b = bm, e = em;
-    for (int q = c / ne; q > 0; --q) b &= b - 1u;
-    for (int q = c % ne; q > 0; --q) e &= e - 1u;
-    const int k = kBlk * (__ffs(b) - 1) + __ffs(e) - 1;
+    const int k = cand(c);
     if (k >= cw.K) continue;  // padding columns
     float cv[kD], eh, el;
     load_vec(cw.C + (int64_t)k * kD, cv);
@@ -445,25 +443,45 @@ __device__ __forceinline__ void decide_open(const SetView& set, const CbList& cb
   }
 }
 
-// The smallest value of v[0..15] (w1, at index idx; the first of equal ones) and the second
+// Index of the (n + 1)-th set bit of m.
+__device__ __forceinline__ int nth_bit(uint32_t m, int n) {
+  for (; n > 0; --n) m &= m - 1u;
+  return __ffs(m) - 1;
+}
+
+// decide_open of a row of the small-codebook pass: blocks x classes of its masks.
+__device__ __forceinline__ void decide_grid(const SetView& set, const CbList& cbs, int n_fixed,
+                                            int s_idx, const OpenRow& o, bool live,
+                                            int32_t* __restrict__ out_code, int64_t out_ld,
+                                            int64_t out_g0, const StatsView& st, float sscale,
+                                            unsigned* err) {
+  const uint32_t bm = o.masks >> 16, em = o.masks & 0xffffu;
+  const int ne = __popc(em);
+  decide_open(set, cbs, n_fixed, s_idx, o.i, o.g, live, __popc(bm) * ne,
+              [&](int c) { return kBlk * nth_bit(bm, c / ne) + nth_bit(em, c % ne); }, out_code,
+              out_ld, out_g0, st, sscale, err);
+}
+
+// The smallest value of v[0..N) (w1, at index idx; the first of equal ones) and the second
 // smallest (w2, equal to w1 when it occurs twice).
-__device__ __forceinline__ void top2_16(const uint32_t v[kBlk], uint32_t& w1, uint32_t& w2,
-                                        int& idx) {
+template <int N>
+__device__ __forceinline__ void top2(const uint32_t v[N], uint32_t& w1, uint32_t& w2, int& idx) {
   w1 = v[0];
   w2 = 0xffffffffu;
   idx = 0;
 #pragma unroll
-  for (int e = 1; e < kBlk; ++e) {
+  for (int e = 1; e < N; ++e) {
     w2 = min(w2, max(w1, v[e]));
     idx = v[e] < w1 ? e : idx;
     w1 = min(w1, v[e]);
   }
 }
 
-__device__ __forceinline__ uint32_t mask_le_16(const uint32_t v[kBlk], uint32_t top) {
+template <int N>
+__device__ __forceinline__ uint32_t mask_le(const uint32_t v[N], uint32_t top) {
   uint32_t m = 0;
 #pragma unroll
-  for (int e = 0; e < kBlk; ++e) m |= v[e] <= top ? 1u << e : 0u;
+  for (int e = 0; e < N; ++e) m |= v[e] <= top ? 1u << e : 0u;
   return m;
 }
 
@@ -575,15 +593,11 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
     __syncthreads();
     {  // B operand of the group: thread = codeword
       uint32_t row[kK];
+      float tk[3];
       if (tid < nchunk * kTcCols) {
-        build_b_row(cw.C, cw.K, tid, sH, uc, row);
+        build_b_row(cw.C, cw.K, tid, sH, uc, row, tk);
         put_row(Bbuf + (tid >> 7) * kTcBTile, tid & (kTcCols - 1), row);
-      }
-      if (tid < cw.K) {
-        float cv[kD], n, na, l1;
-        load_vec(cw.C + (int64_t)tid * kD, cv);
-        codeword_terms(cv, sH, n, na, l1);
-        sNaL1[tid] = make_float2(na, l1);
+        sNaL1[tid] = make_float2(tk[1], tk[2]);
       }
     }
     tc::fence_async_smem();
@@ -705,8 +719,8 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
       if (row_ok) {
         uint32_t w1, w2, x1, x2;
         int b1, e1;
-        top2_16(mb, w1, w2, b1);
-        top2_16(mc, x1, x2, e1);
+        top2<kBlk>(mb, w1, w2, b1);
+        top2<kBlk>(mc, x1, x2, e1);
         const uint32_t s2 = min(w2, x2);
         int j = b1 * kBlk + e1;
         const float k1 = __uint_as_float(w1);
@@ -733,7 +747,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
           const uint32_t tb = __float_as_uint(top) & 0x7fffffffu;
           o.i = (uint32_t)i;
           o.g = (uint32_t)g;
-          o.masks = (mask_le_16(mb, tb) << 16) | mask_le_16(mc, tb);
+          o.masks = (mask_le<kBlk>(mb, tb) << 16) | mask_le<kBlk>(mc, tb);
         }
         out_code[i * out_ld + (g - out_g0)] = j;
         if (cert && st.cnt) {
@@ -776,7 +790,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
         w.i = __shfl_sync(0xffffffffu, o.i, from);
         w.g = __shfl_sync(0xffffffffu, o.g, from);
         w.masks = __shfl_sync(0xffffffffu, o.masks, from);
-        decide_open(set, cbs, n_fixed, s_idx, w, src >= 0, out_code, out_ld, out_g0, st, sscale,
+        decide_grid(set, cbs, n_fixed, s_idx, w, src >= 0, out_code, out_ld, out_g0, st, sscale,
                     err);
         om = rest;
       }
@@ -808,7 +822,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
   const int n = (int)min(found, (unsigned)kOpenCap);
   for (int e0 = warp * 4; e0 < n; e0 += 32) {
     const int e = e0 + (lane >> 3);
-    decide_open(set, cbs, n_fixed, s_idx, s_open[min(e, n - 1)], e < n, out_code, out_ld, out_g0,
+    decide_grid(set, cbs, n_fixed, s_idx, s_open[min(e, n - 1)], e < n, out_code, out_ld, out_g0,
                 st, sscale, err);
   }
   tc::tc_fence_before();
@@ -819,16 +833,39 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
 // --------------------------------------------------------------------------- arg-min pass,
 // codebooks of more than 256 codewords: a CTA walks `tiles` consecutive row tiles of one group
 // (thread = row = tensor-memory lane), streaming the codebook's precomputed B images in chunks of 128
-// codewords by bulk copy through two buffers; 128 threads, three CTAs per SM. The sweep keeps per
-// row the 16-column block with the smallest minimum and the second smallest block minimum. Rows the
-// bounds do not certify go to the flag list (decided by the exact kernels).
-constexpr size_t kArgminStreamSmem = (size_t)tcenc::kATile + 2 * (size_t)kTcBTile +
+// codewords by bulk copy through four buffers. Two 128-column accumulators: the MMA of the next chunk
+// runs while the threads sweep this one, one block barrier per chunk. 128 threads, two CTAs per SM.
+//
+// Sweep, as in argmin_small_kernel but over 32-column granules and 32 classes (column % 32): a
+// granule's minimum and the class minima, 0.5 + 0.5 instructions per score, and the three smallest
+// granule minima with the first two's numbers (10 instructions per 32 scores). The winner is the
+// smallest granule's column of the smallest class; the runner-up is the second smallest granule or
+// class minimum. An open row whose third smallest granule lies above the bound has its candidates in
+// two granules and the classes below the bound (a few columns): the narrow list, decided by
+// argmin_narrow_kernel. The others (wide list) are decided over the whole codebook. Sending every
+// open row over the whole codebook took 60% of a K = 65536 pass (3% of the rows are open there).
+struct NarrowRow {
+  uint32_t i, g;     // row, group (absolute)
+  uint32_t gran;     // the two granules, first << 16 | second (the same twice: one)
+  uint32_t classes;  // mask
+};
+
+struct NarrowList {
+  NarrowRow* row;
+  unsigned* count;
+  unsigned long long* total;  // optional running total of open rows
+};
+
+constexpr int kGran = 32;      // columns per granule
+constexpr int kBRing = 4;      // B chunk buffers
+
+constexpr size_t kArgminStreamSmem = (size_t)tcenc::kATile + kBRing * (size_t)kTcBTile +
                                      (size_t)tcenc::kRows * kD * 4 + 1024;
 
-__global__ void __launch_bounds__(128, 3)
+__global__ void __launch_bounds__(128, 2)
 argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_idx,
                  int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
-                 FlagList flags, StatsView st, const float* __restrict__ cbmax,
+                 FlagList wide, NarrowList narrow, StatsView st, const float* __restrict__ cbmax,
                  const char* __restrict__ bpre, const float4* __restrict__ terms,
                  const float4* __restrict__ rowterms, int tiles, unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
@@ -838,10 +875,10 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   // 1024-byte aligned base, derived from the shared array (keeps the shared address space)
   char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
   char* Atile = smem;                     // 16 KB
-  char* Bbuf = smem + kATile;             // 2 x 16 KB
-  float* sQ = reinterpret_cast<float*>(Bbuf + 2 * kTcBTile);  // [128][8]: H r of a row
+  char* Bbuf = smem + kATile;             // kBRing x 16 KB
+  float* sQ = reinterpret_cast<float*>(Bbuf + kBRing * kTcBTile);  // [128][8]: H r of a row
   __shared__ __align__(16) float sH[kD * kD];
-  __shared__ __align__(8) uint64_t bar_mma, bar_b[2];
+  __shared__ __align__(8) uint64_t bar_mma[2], bar_b[kBRing];
   __shared__ uint32_t tmem_slot;
 
   const int64_t g = g_begin + blockIdx.y;
@@ -855,17 +892,17 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   const float4* gterms = terms + (g - g_begin) * cw.K;
 
   if (tid < kD * kD) sH[tid] = set.Hb[g * kD * kD + tid];
-  if (warp == 0) tc::tmem_alloc(&tmem_slot, kTcCols);
+  if (warp == 0) tc::tmem_alloc(&tmem_slot, 2 * kTcCols);
   if (tid == 0) {
-    tc::mbar_init(tc::smem_u32(&bar_mma), 1);
-    tc::mbar_init(tc::smem_u32(&bar_b[0]), 1);
-    tc::mbar_init(tc::smem_u32(&bar_b[1]), 1);
+    for (int b = 0; b < 2; ++b) tc::mbar_init(tc::smem_u32(&bar_mma[b]), 1);
+    for (int b = 0; b < kBRing; ++b) tc::mbar_init(tc::smem_u32(&bar_b[b]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
   const float sscale = st.cnt ? stats_scale_f(st) : 1.f;
 
   // Bound on Na_k over the codebook for this group: (max row sum |H_g|) L1max cinfmax.
@@ -883,26 +920,42 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   // this CTA's row tiles (the last CTA of a column may have fewer)
   const int64_t row_tiles = (set.M + kRows - 1) / kRows;
   const int steps = (int)min((int64_t)tiles, row_tiles - (int64_t)blockIdx.x * tiles);
-  // Chunk uses are numbered u = t * nchunk + c: use u reads buffer u & 1, and the copy for use
-  // u + 2 starts when use u is done. At most one copy per buffer is outstanding; every thread
-  // tracks the same state.
-  const int n_uses = steps * nchunk;
-  // per buffer (bit b): a copy outstanding, and the parity of its wait (registers, not arrays)
-  uint32_t b_pend = 0, b_par = 0;
-  auto fetch = [&](int u) {  // chunk u % nchunk into buffer u & 1 
-    const int b = u & 1;
-    if (tid == 0) {
-      tc::mbar_expect_tx(tc::smem_u32(&bar_b[b]), kTcBTile);
-      tc::bulk_copy_g2s(tc::smem_u32(Bbuf + b * kTcBTile),
-                        bimg + (size_t)(u % nchunk) * kTcBTile, kTcBTile,
-                        tc::smem_u32(&bar_b[b]));
-    }
-    b_pend |= 1u << b;
+  // Chunk uses are numbered u = t * nchunk + c. Use u reads buffer u % kBRing; thread 0 fetches,
+  // waits for and multiplies them in order (fetched: uses whose copy has started, issued: uses
+  // whose MMA has).
+  const int64_t n_uses = (int64_t)steps * nchunk;
+  int64_t fetched = 0, issued = 0;
+  auto fetch = [&]() {  // thread 0: the next chunk, into the buffer of the use kBRing before it
+    const int b = (int)(fetched % kBRing);
+    tc::mbar_expect_tx(tc::smem_u32(&bar_b[b]), kTcBTile);
+    tc::bulk_copy_g2s(tc::smem_u32(Bbuf + b * kTcBTile),
+                      bimg + (size_t)(fetched % nchunk) * kTcBTile, kTcBTile,
+                      tc::smem_u32(&bar_b[b]));
+    ++fetched;
   };
-  fetch(0);
-  if (n_uses > 1) fetch(1);
+  // Thread 0: the next use's MMA into accumulator `acc`. After a timeout its waiters are released
+  // and the caller's ok turns false.
+  auto issue = [&](int acc) -> bool {
+    const int b = (int)(issued % kBRing);
+    const bool ready = tc::mbar_wait(tc::smem_u32(&bar_b[b]), (uint32_t)((issued / kBRing) & 1), err);
+    ++issued;
+    if (!ready) {
+      tc::mbar_arrive(tc::smem_u32(&bar_mma[acc]));
+      return false;
+    }
+    tc::tc_fence_after();
+    const uint32_t a0 = tc::smem_u32(Atile), b0 = tc::smem_u32(Bbuf + b * kTcBTile);
+#pragma unroll
+    for (int ks = 0; ks < kK / 8; ++ks)
+      tc::mma_tf32(tmem + (uint32_t)(acc * kTcCols), tc::smem_desc(a0 + ks * 256, 128, (kK / 4) * 128),
+                   tc::smem_desc(b0 + ks * 256, 128, (kK / 4) * 128), idesc, ks > 0 ? 1u : 0u);
+    tc::mma_commit(tc::smem_u32(&bar_mma[acc]));
+    return true;
+  };
+  if (tid == 0)
+    while (fetched < min((int64_t)kBRing, n_uses)) fetch();
   bool ok = true;
-  int mma_count = 0;
+  uint32_t mpar = 0;  // parity of the next wait per accumulator (bit = accumulator)
 
   for (int t = 0; t < steps && ok; ++t) {
     const int64_t i = ((int64_t)blockIdx.x * tiles + t) * kRows + tid;
@@ -963,106 +1016,98 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
     }
     tc::fence_async_smem();
     __syncthreads();
+    if (tid == 0) {
+      ok = issue(0);
+      if (ok && nchunk > 1) ok = issue(1);
+    }
 
-    // as fp32 bits: the smallest block minimum, its block and the block's 16 values; the
-    // second smallest block minimum
-    uint32_t v1 = 0xffffffffu, v2 = 0xffffffffu;
-    int b1 = 0;
-    uint32_t bv[kBlk];
+    // fp32 bits: the three smallest granule minima, the first two's granules; the class minima
+    uint32_t v1 = 0xffffffffu, v2 = 0xffffffffu, v3 = 0xffffffffu;
+    int b1 = 0, b2 = 0;
+    uint32_t mc[kGran];
 #pragma unroll
-    for (int e = 0; e < kBlk; ++e) bv[e] = 0xffffffffu;
+    for (int e = 0; e < kGran; ++e) mc[e] = 0xffffffffu;
     for (int c = 0; c < nchunk; ++c) {
-      const int u = t * nchunk + c;
-      const int buf = u & 1;
-      char* Bt = Bbuf + buf * kTcBTile;
-      if ((b_pend >> buf) & 1u) {
-        if (ok) ok = tc::mbar_wait(tc::smem_u32(&bar_b[buf]), (b_par >> buf) & 1u, err);
-        b_par ^= 1u << buf;
-        b_pend &= ~(1u << buf);
-      }
-      ok = __syncthreads_and(ok);
-      if (!ok) break;
-      if (tid == 0) {
-        tc::tc_fence_after();
-        const uint32_t a0 = tc::smem_u32(Atile), b0 = tc::smem_u32(Bt);
-#pragma unroll
-        for (int ks = 0; ks < kK / 8; ++ks)
-          tc::mma_tf32(tmem, tc::smem_desc(a0 + ks * 256, 128, (kK / 4) * 128),
-                       tc::smem_desc(b0 + ks * 256, 128, (kK / 4) * 128), idesc,
-                       ks > 0 ? 1u : 0u);
-        tc::mma_commit(tc::smem_u32(&bar_mma));
-      }
-      ok = tc::mbar_wait(tc::smem_u32(&bar_mma), (uint32_t)(mma_count & 1), err);
-      ++mma_count;
-      ok = __syncthreads_and(ok);
-      if (!ok) break;
-      if (u + 2 < n_uses) fetch(u + 2);  // this buffer is free again
+      const int acc = c & 1;
+      const bool done = tc::mbar_wait(tc::smem_u32(&bar_mma[acc]), (mpar >> acc) & 1u, err);
+      mpar ^= 1u << acc;
+      ok = __all_sync(0xffffffffu, ok && done);
       tc::tc_fence_after();
-      // Epilogue: this warp's 32 rows x 128 columns as eight blocks of 16. Per block its
-      // minimum (every D >= 0, so the bit patterns order like the values); a block whose
-      // minimum is the row's smallest so far is kept whole (16 selects), the previous best
-      // block's minimum moves to the second smallest. No per-score index.
-      const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
+      if (ok) {
 #pragma unroll
-      for (int rnd = 0; rnd < 4; ++rnd) {
-        uint32_t v[32];
-        tc::tmem_ld32_nowait(base + 32 * rnd, v);
-        tc::tmem_wait_ld_dep(v);
+        for (int rnd = 0; rnd < 2; ++rnd) {
+          uint32_t v[64];
+          tc::tmem_ld64_wait(trow + (uint32_t)(acc * kTcCols + 64 * rnd), v);
 #pragma unroll
-        for (int q = 0; q < 32 / kBlk; ++q) {
-          const uint32_t m = min16_bits(v + kBlk * q);
-          v2 = min(v2, max(v1, m));
-          const bool lt = m < v1;
-          v1 = lt ? m : v1;
-          b1 = lt ? (c * kTcCols + 32 * rnd + kBlk * q) / kBlk : b1;
+          for (int q = 0; q < 2; ++q) {
+            const uint32_t m = min(min16_bits(v + kGran * q), min16_bits(v + kGran * q + 16));
+            const int gr = c * (kTcCols / kGran) + 2 * rnd + q;
+            const bool lt1 = m < v1, lt2 = m < v2;
+            v3 = min(v3, max(v2, m));
+            b2 = lt1 ? b1 : (lt2 ? gr : b2);
+            b1 = lt1 ? gr : b1;
+            v2 = min(v2, max(v1, m));
+            v1 = min(v1, m);
+          }
 #pragma unroll
-          for (int e = 0; e < kBlk; ++e) bv[e] = lt ? v[kBlk * q + e] : bv[e];
+          for (int e = 0; e < kGran; ++e) mc[e] = __vimin3_u32(mc[e], v[e], v[kGran + e]);
         }
       }
       tc::tc_fence_before();
-      __syncthreads();  // the accumulator is free for the next MMA
+      // the accumulator has been read and its MMA is done with its buffer
+      ok = __syncthreads_and(ok);
+      if (!ok) break;
+      if (tid == 0) {
+        if (fetched < n_uses) fetch();
+        if (c + 2 < nchunk) ok = issue(acc);
+      }
     }
+    ok = __syncthreads_and(ok);
     if (!ok) break;
 
-    // Certificate, code, flag and statistics of this thread's row. j = the smallest D (ties to
-    // the smaller column), k2 = the second smallest D over the row (the winning block's second
-    // value or the other blocks' smallest minimum).
+    // Certificate, code, open row and statistics of this thread's row.
     if (row_ok) {
-      uint32_t w1 = bv[0], w2 = 0xffffffffu;
-      int jb = 0;
-#pragma unroll
-      for (int e = 1; e < kBlk; ++e) {
-        w2 = min(w2, max(w1, bv[e]));
-        const bool lt = bv[e] < w1;
-        w1 = lt ? bv[e] : w1;
-        jb = lt ? e : jb;
-      }
-      int j = b1 * kBlk + jb;
-      const uint32_t s2 = min(v2, w2);
-      const float k1 = __uint_as_float(w1);
+      uint32_t x1, x2;
+      int e1;
+      top2<kGran>(mc, x1, x2, e1);
+      int j = b1 * kGran + e1;
+      const uint32_t s2 = min(v2, x2);
+      const float k1 = __uint_as_float(v1);
       const float k2 = s2 == 0xffffffffu ? INFINITY : __uint_as_float(s2);
       bool cert = false;
-      float thr = INFINITY;
+      float thr = INFINITY, top = INFINITY;
       if (j < cw.K) {
         const float4 tj = gterms[j];
         const float na = tj.y, l1 = tj.z;
         // D_k <= s_k + off (every k); s_j + off <= D_j + e2 (the winner): no other codeword's
         // exact score reaches s_j when k2 > D_j + e2 (the sum rounded up).
-        const float e2 = 2.f * uc * (na + 2.f * pmax * l1 + off);
-        const float top = __fadd_ru(k1, e2);   // >= s_j + off
-        cert = cw.K == 1 || k2 > top;
+        float e2 = 2.f * uc * (na + 2.f * pmax * l1 + off);
+        top = __fadd_ru(k1, e2);   // >= s_j + off
+        cert = k2 > top;
+        if (s2 == v1) {  // equal scores: the bound over all codewords (see argmin_small_kernel)
+          e2 = 2.f * uc * (hrow * l1max * cinf + 2.f * pmax * l1max + off) * 1.0001f;
+          top = __fadd_ru(k1, e2);
+        }
         thr = top - off;
         thr += 4.f * kU * (k1 + off + e2);
       } else {
         j = 0;
       }
       if (!cert) {
-        const unsigned slot = atomicAdd(flags.count, 1u);
-        if (slot < flags.cap) {
-          flags.vec[slot] = i * G_range + (g - g_begin);
-          flags.thr[slot] = thr;
+        const uint32_t tb = __float_as_uint(top) & 0x7fffffffu;
+        if (v3 > tb && v1 <= tb) {
+          const unsigned slot = atomicAdd(narrow.count, 1u);  // at most one per row: it fits
+          narrow.row[slot] = NarrowRow{(uint32_t)i, (uint32_t)g,
+                                       (uint32_t)b1 << 16 | (uint32_t)(v2 <= tb ? b2 : b1),
+                                       mask_le<kGran>(mc, tb)};
         } else {
-          raise_error(err, ERRBIT_INDEX);
+          const unsigned slot = atomicAdd(wide.count, 1u);
+          if (slot < wide.cap) {
+            wide.vec[slot] = i * G_range + (g - g_begin);
+            wide.thr[slot] = thr;
+          } else {
+            raise_error(err, ERRBIT_INDEX);
+          }
         }
       }
       out_code[i * out_ld + (g - out_g0)] = j;
@@ -1078,17 +1123,36 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
     }
   }
   // After a timeout: let copies still in flight into this CTA's shared memory land (bounded).
-  for (int b = 0; b < 2; ++b)
-    if ((b_pend >> b) & 1u) {
-      tc::mbar_wait(tc::smem_u32(&bar_b[b]), (b_par >> b) & 1u, err);
-    }
-  __syncthreads();
+  if (tid == 0)
+    for (; issued < fetched; ++issued)
+      tc::mbar_wait(tc::smem_u32(&bar_b[issued % kBRing]), (uint32_t)((issued / kBRing) & 1), err);
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem_slot, kTcCols);
+  if (warp == 0) tc::tmem_dealloc(tmem_slot, 2 * kTcCols);
 }
 
-// Exact decision for the rows the arg-min pass flagged: one CTA per flagged vector. The
+// Exact decision of the narrow list, a quarter warp per row.
+__global__ void __launch_bounds__(128)
+argmin_narrow_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_idx,
+                     int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
+                     NarrowList list, StatsView st, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
+  const int n = (int)*list.count;
+  if (list.total && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(list.total, (unsigned long long)n);
+  const float sscale = st.cnt ? stats_scale_f(st) : 1.f;
+  const int quarter = (threadIdx.x & 31) >> 3;
+  for (int e0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * 4; e0 < n; e0 += gridDim.x * 16) {
+    const int e = e0 + quarter;
+    const NarrowRow o = list.row[min(e, n - 1)];
+    const int ga = (int)(o.gran >> 16), gb = (int)(o.gran & 0xffffu), ne = __popc(o.classes);
+    decide_open(set, cbs, n_fixed, s_idx, o.i, o.g, e < n, (ga == gb ? 1 : 2) * ne,
+                [&](int c) { return kGran * (c < ne ? ga : gb) + nth_bit(o.classes, c % ne); },
+                out_code, out_ld, out_g0, st, sscale, err);
+  }
+}
+
+// Exact decision of rows open over the whole codebook (argmin_tc_kernel's wide list): one CTA per row. The
 // threads stride over the codebook for U = min(fast-pass threshold, smallest fp32 upper
 // bound); every codeword whose fp32 lower bound is at most U is a candidate (the exact
 // arg-min always is) and is re-scored exactly in fp32 pairs (dfl) by one thread; the
@@ -2383,12 +2447,12 @@ crvq_status launch_beam_stage(const SetView& set, int64_t g_begin, int64_t G_ran
 }
 
 // Scratch of one arg-min pass: codebook maxima (256 B) | B images of G_sub groups (groups
-// in sub-ranges whose images take at most 256 MB) | codeword terms | flag count (256 B) |
-// flag list (vector ids and thresholds).
+// in sub-ranges whose images take at most 256 MB) | codeword terms | counts of the two open lists
+// (256 B) | narrow list | wide list (vector ids and thresholds).
 struct ArgminLayout {
   int nchunk;
   int64_t G_sub;
-  size_t bbytes, tbytes, fbytes, total;
+  size_t bbytes, tbytes, obytes, fbytes, total;
 };
 
 ArgminLayout argmin_layout(int64_t M, int64_t G_range, int K) {
@@ -2399,8 +2463,9 @@ ArgminLayout argmin_layout(int64_t M, int64_t G_range, int K) {
   L.G_sub = std::max<int64_t>(1, std::min<int64_t>(G_range, (int64_t(256) << 20) / per_group));
   L.bbytes = (size_t)L.G_sub * per_group;
   L.tbytes = align_up((size_t)L.G_sub * K * sizeof(float4), 256);
+  L.obytes = align_up((size_t)M * L.G_sub * sizeof(NarrowRow), 256);
   L.fbytes = align_up((size_t)M * L.G_sub * (sizeof(int64_t) + sizeof(float)), 256);
-  L.total = 256 + L.bbytes + L.tbytes + 256 + L.fbytes;
+  L.total = 256 + L.bbytes + L.tbytes + 256 + L.obytes + L.fbytes;
   return L;
 }
 
@@ -2453,10 +2518,11 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
   float4* tout = reinterpret_cast<float4*>(bimg + bbytes);
   FlagList fl;
   fl.count = reinterpret_cast<unsigned*>(wbase + 256 + bbytes + tbytes);
-  fl.vec = reinterpret_cast<int64_t*>(wbase + 256 + bbytes + tbytes + 256);
+  const NarrowList nl{reinterpret_cast<NarrowRow*>(wbase + 256 + bbytes + tbytes + 256), fl.count + 1,
+                      fl.total = ex.flag_total};
+  fl.vec = reinterpret_cast<int64_t*>(wbase + 256 + bbytes + tbytes + 256 + AL.obytes);
   fl.cap = set.M * G_sub;
   fl.thr = reinterpret_cast<float*>(fl.vec + fl.cap);
-  fl.total = ex.flag_total;
   const float uc = kU * (tcenc::kCmul + 4.f * n_fixed);
   CRVQ_TRY(smem_limit((const void*)argmin_tc_kernel, kArgminStreamSmem));
   for (int64_t gs = g_begin; gs < g_begin + G_range; gs += G_sub) {
@@ -2474,20 +2540,24 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
       CRVQ_LAUNCHED();
     }
     {
-      // row tiles per CTA: about eight waves of three CTAs per SM (a fine-grained tail)
+      // row tiles per CTA: about sixteen waves of two CTAs per SM (a fine-grained tail)
       const int64_t row_tiles = ceil_div(set.M, tcenc::kRows);
-      const int64_t per_group = std::max<int64_t>(1, 24 * (int64_t)nsm / std::max<int64_t>(1, gn));
+      const int64_t per_group = std::max<int64_t>(1, 32 * (int64_t)nsm / std::max<int64_t>(1, gn));
       const int tiles = (int)std::max<int64_t>(1, ceil_div(row_tiles, per_group));
       const dim3 grid((unsigned)ceil_div(row_tiles, tiles), (unsigned)gn);
       ProfScope ps(st.cnt ? "encode_argmin_lloyd" : "encode_argmin", stream,
                    (double)nv * cw.K);
       CRVQ_CUDA(launch_pdl(argmin_tc_kernel, grid, dim3(128), kArgminStreamSmem, stream, set, gs,
-                           cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, st, cbmax, bimg, tout,
+                           cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, nl, st, cbmax, bimg, tout,
                            ex.rowterms, tiles, err));
       CRVQ_LAUNCHED();
     }
     {
       ProfScope pf("encode_exact", stream, 0.0);
+      CRVQ_CUDA(launch_pdl(argmin_narrow_kernel,
+                           dim3((unsigned)std::min<int64_t>(ceil_div(nv, 16), 8 * nsm)), dim3(128), 0,
+                           stream, set, gs, cbs, n_fixed, s_idx, out, out_ld, out_g0, nl, st, err));
+      CRVQ_LAUNCHED();
       if (cw.K <= kExactWarpK) {
         CRVQ_CUDA(launch_pdl(argmin_exact_warp_kernel,
                              dim3((unsigned)std::min<int64_t>(ceil_div(nv, 4), 16 * nsm)),

@@ -1,0 +1,94 @@
+"""Edges of the arg-min kernels against the fp64 oracle: codebook sizes around the 128-codeword
+chunks and the 256-codeword limit between the resident and the streaming kernel, row counts around
+the 128-row tiles and their pairs, shares that span several groups, rows left open by the certificate
+(duplicate and nearly equal codewords, more of them than a CTA's list holds). Codes must be the fp64
+arg-min, ties to the smaller index, except at fp64 near-ties (parity_util)."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2412_09282_gb300 as P
+from paper_2412_09282_gb300 import Codebook
+from oracle import crvq_oracle as O
+from parity_util import check_codes_with_ties, dev, host
+
+pytestmark = pytest.mark.gpu
+
+D = 8
+
+
+def _blocks(rng, G, n=64):
+    X = rng.standard_normal((n, G * D)) * rng.lognormal(0.0, 0.5, G * D)
+    Xb = X.reshape(n, G, D).transpose(1, 0, 2)
+    return (Xb.transpose(0, 2, 1) @ Xb / n + 0.05 * np.eye(D)).astype(np.float32)
+
+
+def _encode(W, Hb, C):
+    M, G = W.shape[0], Hb.shape[0]
+    codes = torch.full((M, G), -1, dtype=torch.int32, device="cuda")
+    err = P.crvq_encode_beam(dev(W), D, dev(Hb), [Codebook(dev(C), codes, G)], 0, 1, want_err=True)
+    P.crvq_sync()
+    return host(codes), host(err)
+
+
+def _check(W, Hb, C):
+    codes, err = _encode(W, Hb, C)
+    cb = [O.Codebook(C, None, Hb.shape[0])]
+    oc, oerr = O.encode_beam(W, D, Hb, cb, 0, 1)
+    check_codes_with_ties(W, D, Hb, cb, 0, [codes], oc)
+    np.testing.assert_allclose(err, oerr, rtol=1e-5, atol=1e-12)
+    return codes
+
+
+@pytest.mark.parametrize("M,G,K", [
+    (1, 1, 1), (127, 3, 2), (128, 2, 127), (129, 2, 128), (255, 5, 129), (256, 1, 255),
+    (257, 7, 256), (300, 650, 16),                                   # shares over several groups
+    (130, 2, 257), (1, 3, 384), (257, 2, 385), (129, 3, 1025), (64, 2, 3000)])
+def test_codebook_and_row_edges(M, G, K):
+    rng = np.random.default_rng(M * 1000 + K)
+    W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
+    C = (0.02 * rng.standard_normal((K, D))).astype(np.float32)
+    _check(W, _blocks(rng, G), C)
+
+
+@pytest.mark.parametrize("K", [64, 256, 600])
+def test_open_rows_more_than_a_list_holds(K):
+    """Every codeword twice, the copy one unit in the last place off: no row is certified."""
+    rng = np.random.default_rng(K)
+    M, G = 700, 4
+    W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
+    C = (0.02 * rng.standard_normal((K // 2, D))).astype(np.float32)
+    near = np.nextafter(C, np.float32(1)).astype(np.float32)
+    _check(W, _blocks(rng, G), np.concatenate([C, near]))
+    # exact duplicates: the smaller index of every pair
+    codes, _ = _encode(W, _blocks(rng, G), np.concatenate([C, C]))
+    assert codes.max() < K // 2
+
+
+@pytest.mark.parametrize("K", [200, 700])
+def test_three_close_codewords_in_different_granules(K):
+    """Triples of almost equal codewords spread over the codebook: more candidates than the two
+    granules that the large pass keeps."""
+    rng = np.random.default_rng(K + 1)
+    M, G = 260, 3
+    W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
+    base = (0.02 * rng.standard_normal((K // 4, D))).astype(np.float32)
+    C = np.concatenate([base * (1 + 1e-7 * t) for t in range(4)]).astype(np.float32)
+    _check(W, _blocks(rng, G), C)
+
+
+def test_non_finite_codeword_and_target_are_reported_and_leave_the_rest():
+    rng = np.random.default_rng(5)
+    M, G, K = 200, 2, 100
+    W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
+    C = (0.02 * rng.standard_normal((K, D))).astype(np.float32)
+    Hb = _blocks(rng, G)
+    good, _ = _encode(W, Hb, C)
+    W[7, 3] = np.nan
+    codes = torch.zeros((M, G), dtype=torch.int32, device="cuda")
+    P.crvq_encode_beam(dev(W), D, dev(Hb), [Codebook(dev(C), codes, G)], 0, 1)
+    with pytest.raises(P.CrvqError) as e:
+        P.crvq_sync()
+    assert e.value.status == -6
+    rest = np.arange(M) != 7
+    np.testing.assert_array_equal(host(codes)[rest], good[rest])

@@ -156,13 +156,6 @@ __device__ __forceinline__ void stage_chunk(const float* __restrict__ C, int k0,
   }
 }
 
-__device__ __forceinline__ float low_score(const float c[kD], const float* H, const float m2q[kD],
-                                           float nbeta, float cmul) {
-  float n, na, l1;
-  codeword_terms(c, H, n, na, l1);
-  return low_from(n, na, l1, c, m2q, nbeta, cmul);
-}
-
 // --------------------------------------------------------------------------- arg-min pass on
 // the tensor cores. The whole certified lower bound is one dot product of length 32:
 //   D[v][k] = sum_p q_vp c_kp + n'_k + beta_v L1_k + off_v = low_k(v) + off_v,
@@ -1781,10 +1774,12 @@ beam_stage_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDe
 //   y(h, k) = base_h + sN_k + m2q_h . c_k + nbeta_h L1_k
 // for all 128 vectors x 256 codewords (3xTF32 operands: the B images of prep_b built with the
 // stage's bound multiplier), and each thread reads its row from tensor memory. y differs from
-// the fast stage's fp32 chain x(h, k) (the same linear form) by at most eps_h = 2^-12 S_h,
+// the fast stage's fp32 chain x(h, k) (the same linear form) by at most eps_h = 2^-16 S_h,
 // S_h = |base_h| + Na_max + 2 Pmax_h L1max + |nbeta_h| L1max, which bounds every term's
 // magnitude (the split products lose about 2^-22 and the fp32 accumulation of 32 terms about
-// 2^-19 of it). A pair whose x could enter the list has y <= (the list's last x, or the bound
+// 2^-19 of it; the arg-min pass's bound multiplier of 256 u is the same 2^-16). Outlier codewords
+// make S_h large against the errs, so a looser eps lets many pairs through: at 2^-12 candidates
+// were most of the kernel's instructions. A pair whose x could enter the list has y <= (the list's last x, or the bound
 // tau below) + eps_h; only those are kept (a bit mask per thread), scored again with exactly
 // the fast stage's chain and inserted in (h, k) order with its rule (strictly below the last
 // entry, before the first entry strictly above). Every member of the final
@@ -1793,14 +1788,13 @@ beam_stage_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDe
 // at least L pairs have y <= tau, so the L-th smallest x is at most tau + eps_0.
 constexpr size_t kBeamTcSmem = 1024 + (size_t)tcenc::kATile + 2 * (size_t)kTcBTile +
                                (size_t)kChunk * kD * 4 + (size_t)kChunk * 8 + (size_t)kChunk * 4 +
-                               2 * 16 * (size_t)kThreads * 4 + 2 * 9 * (size_t)kThreads * 4;
+                               2 * 16 * (size_t)kThreads * 4;
 
 template <int L>
 __global__ void __launch_bounds__(kThreads, 2)
 beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc sd,
                BeamBufs bb, const char* __restrict__ bimg, const float* __restrict__ cbmax,
                FlagList flags, unsigned* err) {
-  static_assert(L <= 9, "the shared-memory list holds 9 entries");
   using namespace tcenc;
   extern __shared__ __align__(1024) char smem_raw[];
   char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -1811,8 +1805,6 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
   float* sNa = reinterpret_cast<float*>(sNL + kChunk);
   float* sRa = sNa + kChunk;  // [h][thread]
   float* sPm = sRa + 16 * kThreads;
-  float* sTopV = sPm + 16 * kThreads;                          // [j][thread]
-  int* sTopI = reinterpret_cast<int*>(sTopV + 9 * kThreads);  // [j][thread]
   __shared__ __align__(16) float sH[kD * kD];
   __shared__ __align__(8) uint64_t bar_b, bar_mma;
   __shared__ uint32_t tmem_slot;
@@ -1871,15 +1863,17 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
 #pragma unroll
     for (int j = 0; j < kD; ++j) th[j] = tl[j] = 0.f;
   }
-  // The sorted top-L list lives in shared memory ([j][thread]), `last` = its last value: a
-  // candidate that does not enter costs one compare, one that does only the shifts it needs
-  // (a register list would be updated by a predicated network for every candidate).
+  // The sorted top-L list in registers. An insertion compares with every entry at once and moves
+  // each by at most one place (no chain along the list): about 45 instructions, run only when some
+  // lane's candidate enters. (A shifting insert in shared memory took a dependent load, compare and
+  // store per place.)
+  float topv[L];
+  int topi[L];
 #pragma unroll
   for (int j = 0; j < L; ++j) {
-    sTopV[j * kThreads + tid] = INFINITY;
-    sTopI[j * kThreads + tid] = 0x7fffffff;
+    topv[j] = INFINITY;
+    topi[j] = 0x7fffffff;
   }
-  float last = INFINITY;
   float tau_x = INFINITY;
   bool ok = true;
   const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
@@ -1899,7 +1893,7 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
       sPm[h * kThreads + tid] = pmax;
       base = rr - kU * cmul * ra;
       nbeta = -2.f * kU * cmul * pmax;
-      eps = 2.44140625e-04f *  // 2^-12
+      eps = 1.52587890625e-05f *  // 2^-16
             (fabsf(base) + na_max + 2.f * pmax * l1max * 1.0001f + fabsf(nbeta) * l1max);
     }
   };
@@ -1991,7 +1985,7 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
 #pragma unroll 1
     for (int q = 0; q < nq; ++q) {
       const float thrD =
-          act ? __fadd_ru(fminf(last, tau_x), eps) : __int_as_float(0x7fffffff);
+          act ? __fadd_ru(fminf(topv[L - 1], tau_x), eps) : __int_as_float(0x7fffffff);
       uint32_t m0 = 0u, m1 = 0u;
       {
         uint32_t v[64];
@@ -2022,18 +2016,15 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
           sv = fmaf(m2q[6], c1.z, sv);
           sv = fmaf(m2q[7], c1.w, sv);
           sv = fmaf(nbeta, nl.y, sv);
-          if (sv < last) {  // insert before the first entry strictly above sv
-            int j = L - 1;
-            while (j > 0) {
-              const float pv = sTopV[(j - 1) * kThreads + tid];
-              if (!(sv < pv)) break;
-              sTopV[j * kThreads + tid] = pv;
-              sTopI[j * kThreads + tid] = sTopI[(j - 1) * kThreads + tid];
-              --j;
+          if (sv < topv[L - 1]) {  // insert before the first entry strictly above sv
+            const int si = (h << 16) | k;
+#pragma unroll
+            for (int j = L - 1; j >= 0; --j) {
+              const bool below = j > 0 && sv < topv[j > 0 ? j - 1 : 0];
+              const bool here = sv < topv[j];
+              topi[j] = below ? topi[j > 0 ? j - 1 : 0] : (here ? si : topi[j]);
+              topv[j] = below ? topv[j > 0 ? j - 1 : 0] : (here ? sv : topv[j]);
             }
-            sTopV[j * kThreads + tid] = sv;
-            sTopI[j * kThreads + tid] = (h << 16) | k;
-            last = sTopV[(L - 1) * kThreads + tid];
           }
         }
       }
@@ -2054,13 +2045,6 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, 2 * kTcCols);
   if (!live) return;
-  float topv[L];
-  int topi[L];
-#pragma unroll
-  for (int j = 0; j < L; ++j) {
-    topv[j] = sTopV[j * kThreads + tid];
-    topi[j] = sTopI[j * kThreads + tid];
-  }
   beam_list_finish<L>(set, cbs, sd, bb, flags, i, g, vi, Bh, cmul, th, tl, sH, sNL, sNa, true,
                       sRa + tid, sPm + tid, kThreads, topv, topi, err);
 }
@@ -2073,7 +2057,7 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
 __global__ void __launch_bounds__(kThreads)
 beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs,
                            int n_fixed, StageDesc sd, BeamBufs bb, FlagList flags,
-                           unsigned* err) {
+                           const float4* __restrict__ terms, unsigned* err) {
   __shared__ int queue[kThreads / 32][32], queue_h[kThreads / 32][32];
   const int lane = threadIdx.x & 31;
   int* q = queue[threadIdx.x >> 5];
@@ -2135,9 +2119,17 @@ beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList
         const int k = k0 + lane;
         bool cand = false;
         if (k < cw.K) {
-          float c[kD];
+          float c[kD], n, na, l1;
           load_vec(cw.C + (int64_t)k * kD, c);
-          cand = base + low_score(c, H, m2q, nbeta, cmul) <= thr;
+          if (terms) {  // the tensor-core stage's codeword terms of the group
+            const float4 t = terms[(g - g_begin) * cw.K + k];
+            n = t.x;
+            na = t.y;
+            l1 = t.z;
+          } else {
+            codeword_terms(c, H, n, na, l1);
+          }
+          cand = base + low_from(n, na, l1, c, m2q, nbeta, cmul) <= thr;
         }
         const unsigned m = __ballot_sync(0xffffffffu, cand);
         const int n = __popc(m);
@@ -2225,10 +2217,39 @@ __device__ void tuple_err32(const SetView& set, const CbList& cbs, int n_fixed,
   bnd = kU * bound_mult(n_fixed + sd.S + 1) * na;
 }
 
+// err of a whole tuple of vector (i, g) in fp32 pairs (a few 2^-44 relative, so the rounded value is
+// the one an fp64 evaluation gives; GB300's fp64 pipe made this most of the kernel's time): the
+// fixed codebooks' codes, then for each searched stage q the code sc[q] (with sc null: the code
+// already stored).
+__device__ __forceinline__ float tuple_err_pair(const SetView& set, const CbList& cbs, int n_fixed,
+                                                const StageDesc& sd, int64_t i, int64_t g,
+                                                const int32_t* sc, const float* H, unsigned* err) {
+  float rh[kD], rl[kD], zero[kD], eh, el;
+  dfl::target(set, cbs, n_fixed, i, g, rh, rl, err);
+#pragma unroll
+  for (int j = 0; j < kD; ++j) zero[j] = 0.f;
+  for (int q = 0; q < sd.S; ++q) {
+    const CbView& cb = cbs.cb[sd.st[q]];
+    const int32_t k = sc ? sc[q] : cb.codes[i * cb.ld + g];
+    if (!code_ok(k, cb.K, err)) continue;
+    float c[kD];
+    load_vec(cb.C + (int64_t)k * kD, c);
+#pragma unroll
+    for (int j = 0; j < kD; ++j) {
+      float sj, ej;
+      dfl::two_sum(rh[j], -c[j], sj, ej);
+      rh[j] = sj;
+      rl[j] = __fadd_rn(rl[j], ej);
+    }
+  }
+  dfl::quad_err(rh, rl, zero, H, eh, el);
+  return __fadd_rn(eh, el);
+}
+
 // Final step of a multi-stage (or keep-if-better) encode: write the best tuple, or keep the
 // tuple already in the codes when its err is strictly smaller. The comparison is decided by
 // fp32 errs with bounds when they separate, in fp64 otherwise; an unchanged tuple needs no
-// comparison. vec_err (optional) is the fp64 err of the tuple kept.
+// comparison. vec_err (optional) is the err of the tuple kept.
 __global__ void beam_finalize_kernel(SetView set, int64_t g_begin, int64_t G_range,
                                      CbList cbs, int n_fixed, StageDesc sd,
                                      const int32_t* __restrict__ hyp, bool keep_if_better,
@@ -2241,7 +2262,7 @@ __global__ void beam_finalize_kernel(SetView set, int64_t g_begin, int64_t G_ran
     const float* H = set.Hb + g * kD * kD;
     const int32_t* best = hyp + vi * B * S;
     bool use_old = false;
-    bool exact = vec_err != nullptr;
+    bool exact = false;
     if (keep_if_better) {
       bool same = true;
       for (int q = 0; q < S; ++q) {
@@ -2273,23 +2294,21 @@ __global__ void beam_finalize_kernel(SetView set, int64_t g_begin, int64_t G_ran
         for (int j = 0; j < kD; ++j) r[j] -= (double)c[j];
       }
       const double e_new = quad_err64(r, nullptr, H);
-      double e_old = e_new;
-      if (keep_if_better) {
 #pragma unroll
-        for (int j = 0; j < kD; ++j) r[j] = tgt[j];
-        for (int q = 0; q < S; ++q) {
-          const CbView& cb = cbs.cb[sd.st[q]];
-          const int32_t k = cb.codes[i * cb.ld + g];
-          if (!code_ok(k, cb.K, err)) continue;
-          const float* c = cb.C + (int64_t)k * kD;
+      for (int j = 0; j < kD; ++j) r[j] = tgt[j];
+      for (int q = 0; q < S; ++q) {
+        const CbView& cb = cbs.cb[sd.st[q]];
+        const int32_t k = cb.codes[i * cb.ld + g];
+        if (!code_ok(k, cb.K, err)) continue;
+        const float* c = cb.C + (int64_t)k * kD;
 #pragma unroll
-          for (int j = 0; j < kD; ++j) r[j] -= (double)c[j];
-        }
-        e_old = quad_err64(r, nullptr, H);
-        use_old = e_old < e_new;
+        for (int j = 0; j < kD; ++j) r[j] -= (double)c[j];
       }
-      if (vec_err) vec_err[i * set.G_sub + g] = (float)(use_old ? e_old : e_new);
+      use_old = quad_err64(r, nullptr, H) < e_new;
     }
+    if (vec_err)
+      vec_err[i * set.G_sub + g] =
+          tuple_err_pair(set, cbs, n_fixed, sd, i, g, use_old ? nullptr : best, H, err);
     if (!use_old) {
       for (int q = 0; q < S; ++q) {
         const CbView& cb = cbs.cb[sd.st[q]];
@@ -2299,16 +2318,16 @@ __global__ void beam_finalize_kernel(SetView set, int64_t g_begin, int64_t G_ran
   }
 }
 
-// err of the tuple currently in the codes (all covering codebooks), fp64.
+// err of the tuple currently in the codes (all covering codebooks), in fp32 pairs.
 __global__ void residual_err_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs,
                                     float* __restrict__ vec_err, unsigned* err) {
   const int64_t nvec = set.M * G_range;
+  StageDesc none{};
   for (int64_t vi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; vi < nvec;
        vi += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = vi / G_range, g = g_begin + vi % G_range;
-    double r[kD];
-    target64(set, cbs, cbs.n, i, g, r, err);
-    vec_err[i * set.G_sub + g] = (float)quad_err64(r, nullptr, set.Hb + g * kD * kD);
+    vec_err[i * set.G_sub + g] = tuple_err_pair(set, cbs, cbs.n, none, i, g, nullptr,
+                                                set.Hb + g * kD * kD, err);
   }
 }
 
@@ -2388,6 +2407,12 @@ size_t beam_tc_scratch_bytes(int64_t G_range, int K) {
          align_up((size_t)G_range * K * sizeof(float4), 256) + 256;
 }
 
+// The codeword terms within that scratch.
+float4* beam_tc_terms(char* work, int64_t G_range, int K) {
+  return reinterpret_cast<float4*>(work + 256 +
+                                   (size_t)G_range * ceil_div(K, kTcCols) * kTcBTile);
+}
+
 // CRVQ_BEAM_TC=0 in the environment (read at every call) keeps every stage on the SIMT kernel:
 // the two forms give the same lists, which tests compare.
 bool beam_tc_applies(const StageDesc& sd, const CbList& cbs, int64_t G_range) {
@@ -2406,7 +2431,7 @@ crvq_status launch_beam_stage_tc(const SetView& set, int64_t g_begin, int64_t G_
   const int nchunk = (int)ceil_div(cw.K, kTcCols);
   float* cbmax = reinterpret_cast<float*>(work);
   char* bimg = work + 256;
-  float4* tout = reinterpret_cast<float4*>(bimg + (size_t)G_range * nchunk * kTcBTile);
+  float4* tout = beam_tc_terms(work, G_range, cw.K);
   const float uc = kU * bound_mult(n_fixed + sd.s);
   {
     ProfScope pb("encode_prep_b", stream, (double)G_range * nchunk * kTcCols);
@@ -2674,7 +2699,8 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
     CRVQ_CUDA(cudaMemsetAsync(fl.count, 0, sizeof(unsigned), stream));
     BeamBufs bb{in_h, in_n, out_h, out_n};
     const int K = cbs.cb[sd.st[s]].K;
-    if (beam_tc_applies(sd, cbs, G_range))
+    const bool tc_stage = beam_tc_applies(sd, cbs, G_range);
+    if (tc_stage)
       CRVQ_TRY(launch_beam_stage_tc(set, g_begin, G_range, cbs, n_fixed, sd, bb, fl, err,
                                     tc_mem.as<char>(), (double)nvec * parents * K, stream));
     else
@@ -2683,7 +2709,8 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
     {
       ProfScope ps("encode_beam_fallback", stream, 0.0);
       beam_stage_fallback_kernel<<<4 * nsm, kThreads, 0, stream>>>(
-          set, g_begin, G_range, cbs, n_fixed, sd, bb, fl, err);
+          set, g_begin, G_range, cbs, n_fixed, sd, bb, fl,
+          tc_stage ? beam_tc_terms(tc_mem.as<char>(), G_range, K) : nullptr, err);
       CRVQ_LAUNCHED();
     }
     sc += (double)nvec * parents * K;

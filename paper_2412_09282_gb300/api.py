@@ -39,19 +39,20 @@ def _check(st: int):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    # (the ABI's pointer parameters are declared c_void_p: ctypes converts a plain int)
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream, device):
     if stream is None:
         stream = torch.cuda.current_stream(device)
-    return C.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 def _need(t: torch.Tensor, dtype, name):
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
-    if t.device.type != "cuda":
+    if not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
 
 
@@ -68,17 +69,18 @@ class Codebook:
     G_cov: int
 
     def to_c(self) -> _lib.crvq_codebook:
-        _need(self.C, torch.float32, "codebook C")
-        if not self.C.is_contiguous():
+        cw, codes = self.C, self.codes
+        _need(cw, torch.float32, "codebook C")
+        if not cw.is_contiguous():
             raise ValueError("codebook C must be contiguous")
-        ld = 0
-        if self.codes is not None:
-            _need(self.codes, torch.int32, "codes")
-            _rowmajor(self.codes, "codes")
-            ld = self.codes.stride(0) if self.codes.shape[0] > 1 else max(self.G_cov, 1)
-        return _lib.crvq_codebook(self.C.data_ptr(), int(self.C.shape[0]), 0,
-                                  None if self.codes is None else self.codes.data_ptr(),
-                                  int(ld), int(self.G_cov))
+        ld, codes_ptr = 0, None
+        if codes is not None:
+            _need(codes, torch.int32, "codes")
+            _rowmajor(codes, "codes")
+            ld = codes.stride(0) if codes.shape[0] > 1 else max(self.G_cov, 1)
+            codes_ptr = codes.data_ptr()
+        return _lib.crvq_codebook(cw.data_ptr(), cw.shape[0], 0, codes_ptr, int(ld),
+                                  int(self.G_cov))
 
 
 def _cb_array(cbs):

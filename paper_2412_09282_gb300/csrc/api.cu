@@ -45,19 +45,72 @@ void clear_last_error() { t_last_error.clear(); }
 namespace {
 std::mutex g_mu;
 std::vector<unsigned*> g_err_words;  // per device
+std::vector<cudaMemPool_t> g_pools;  // per device (null: the device's default pool)
 std::vector<int> g_sm;               // per device
 }  // namespace
+
+// Scratch comes from a pool of the library's own. The device's default pool gives everything back
+// whenever a stream is synchronized, so a call after a synchronization paid for mapping its scratch
+// again (0.25 ms for a few MB, 0.7 ms for the 330 MB of a 4096 x 4096 reconstruction). This pool keeps
+// at most kPoolKeep of what is free; the rest goes back at the next synchronization, and all of
+// it when an allocation fails. Freed memory is reused in stream order by any stream or thread.
+namespace {
+constexpr uint64_t kPoolKeep = uint64_t(1) << 30;
+
+// The current device's pool, created on first use (called with g_mu held).
+cudaMemPool_t make_pool(int dev) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  uint64_t keep = kPoolKeep;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess)
+    cudaGetLastError();
+  return pool;
+}
+}  // namespace
+
+crvq_status scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  unsigned* word = nullptr;
+  CRVQ_TRY(device_error_word(&word));  // (creates the pool beside the error word)
+  int dev = 0;
+  CRVQ_CUDA(cudaGetDevice(&dev));
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    pool = g_pools[dev];
+  }
+  if (!pool) {
+    CRVQ_CUDA(cudaMallocAsync(p, bytes, s));
+    return CRVQ_OK;
+  }
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  if (e == cudaErrorMemoryAllocation) {  // give back what is kept free and try once more
+    cudaGetLastError();
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  }
+  CRVQ_CUDA(e);
+  return CRVQ_OK;
+}
 
 crvq_status device_error_word(unsigned** out) {
   int dev = 0;
   CRVQ_CUDA(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_mu);
   if ((int)g_err_words.size() <= dev) g_err_words.resize(dev + 1, nullptr);
+  if ((int)g_pools.size() <= dev) g_pools.resize(dev + 1, nullptr);
   if (!g_err_words[dev]) {
     unsigned* p = nullptr;
     CRVQ_CUDA(cudaMalloc(&p, sizeof(unsigned)));
     CRVQ_CUDA(cudaMemset(p, 0, sizeof(unsigned)));
     g_err_words[dev] = p;
+    g_pools[dev] = make_pool(dev);
   }
   *out = g_err_words[dev];
   return CRVQ_OK;

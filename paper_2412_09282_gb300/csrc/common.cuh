@@ -96,6 +96,9 @@ enum : unsigned { ERRBIT_INDEX = 1u, ERRBIT_NUMERIC = 2u, ERRBIT_TIMEOUT = 4u };
 // Device error word of the current device (allocated once per device, zeroed).
 crvq_status device_error_word(unsigned** out);
 
+// Stream-ordered allocation from the library's memory pool of the current device (api.cu).
+crvq_status scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+
 // Stream-ordered scratch buffer; freed (stream-ordered) when it goes out of scope.
 class Scratch {
  public:
@@ -107,8 +110,7 @@ class Scratch {
     release();
     stream_ = s;
     if (bytes == 0) return CRVQ_OK;
-    CRVQ_CUDA(cudaMallocAsync(&p_, bytes, s));
-    return CRVQ_OK;
+    return scratch_alloc(&p_, bytes, s);
   }
   void release() {
     if (p_) cudaFreeAsync(p_, stream_);

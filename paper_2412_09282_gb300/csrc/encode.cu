@@ -378,7 +378,7 @@ struct OpenRow {
 
 constexpr size_t kArgminSmem = 2 * (size_t)tcenc::kATile + 2 * (size_t)kTcBTile +
                                (size_t)kTcSmemStatsK * (kD * 8 + 4) +
-                               2 * (size_t)tcenc::kRows * kD * 4 + (size_t)kTcSmemStatsK * 8 +
+                               4 * (size_t)tcenc::kRows * kD * 4 + (size_t)kTcSmemStatsK * 8 +
                                (size_t)kOpenCap * sizeof(OpenRow) + 1024;
 
 // Exact decision of one open row (i, g) by the eight lanes of a quarter warp (all 32 lanes call it; a
@@ -505,8 +505,8 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
   char* Bbuf = smem + 2 * kATile;         // 2 x 16 KB
   int* s_b32 = reinterpret_cast<int*>(Bbuf + 2 * kTcBTile);     // [8][2][256] statistics halves
   int* s_cnt = s_b32 + kTcSmemStatsK * kD * 2;                  // [256]
-  float* sQ = reinterpret_cast<float*>(s_cnt + kTcSmemStatsK);  // [256][8]: H r of a row
-  float2* sNaL1 = reinterpret_cast<float2*>(sQ + 2 * kRows * kD);      // [256]
+  float* sQ = reinterpret_cast<float*>(s_cnt + kTcSmemStatsK);  // [2][256][8]: H r of a row
+  float2* sNaL1 = reinterpret_cast<float2*>(sQ + 4 * kRows * kD);      // [256]
   OpenRow* s_open = reinterpret_cast<OpenRow*>(sNaL1 + kTcSmemStatsK);  // [kOpenCap]
   __shared__ __align__(16) float sH[kD * kD];
   __shared__ __align__(8) uint64_t bar_mma_s[2];
@@ -605,106 +605,135 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
       hrow = fmaxf(hrow, rs);
     }
 
-    for (int t = 0; t < np && ok; ++t) {
-      const int64_t i = ((pg + t) * 2 + half) * kRows + rrow;
-      const bool row_ok = i < set.M;
-      // Prologue: this thread's A row.
-      float pmax, off;
-      {
-        float m2q[kD], rr, ra;
-        if (rowterms) {  // precomputed for this Lloyd loop (row_terms_kernel)
-          float4 q0 = make_float4(0.f, 0.f, 0.f, 0.f), q1 = q0, t2 = q0;
-          if (row_ok) {
-            q0 = rowterms[(3 * g) * set.M + i];
-            q1 = rowterms[(3 * g + 1) * set.M + i];
-            t2 = rowterms[(3 * g + 2) * set.M + i];
-          }
-          m2q[0] = q0.x; m2q[1] = q0.y; m2q[2] = q0.z; m2q[3] = q0.w;
-          m2q[4] = q1.x; m2q[5] = q1.y; m2q[6] = q1.z; m2q[7] = q1.w;
-          rr = t2.x;
-          ra = t2.y;
-          pmax = t2.z;
-        } else {
-          float rv[kD], a[kD];
-          if (row_ok) {
-            target32(set, cbs, n_fixed, i, g, rv, a, err);
-          } else {
-#pragma unroll
-            for (int j = 0; j < kD; ++j) rv[j] = a[j] = 0.f;
-          }
-          vector_terms_rr(rv, a, sH, m2q, pmax, rr, ra);
-        }
-        // offset making every D = low + off >= 0, with margins for every rounding involved
-        off = (rr + 32.f * kU * ra + 2.f * uc * (hrow * l1max * cinf + 2.f * pmax * l1max)) *
-                  (1.f + 4.f * uc) + 1e-30f;
-        const float beta = -2.f * uc * pmax;
-        if (st.cnt) {  // H r of this row, kept for the statistics (-m2q / 2, exact)
-          *reinterpret_cast<float4*>(sQ + tid * kD) =
-              make_float4(-0.5f * m2q[0], -0.5f * m2q[1], -0.5f * m2q[2], -0.5f * m2q[3]);
-          *reinterpret_cast<float4*>(sQ + tid * kD + 4) =
-              make_float4(-0.5f * m2q[4], -0.5f * m2q[5], -0.5f * m2q[6], -0.5f * m2q[7]);
-        }
-        uint32_t row[kK];
-#pragma unroll
-        for (int q = 0; q < kD; ++q) {
-          uint32_t h, l;
-          split(m2q[q], h, l);
-          row[q] = h;
-          row[8 + q] = h;
-          row[16 + q] = l;
-        }
-        const uint32_t one = __float_as_uint(1.f);
-        row[24] = one;
-        row[25] = one;
-        split(beta, row[26], row[28]);
-        row[27] = row[26];
-        split(off * (1.f - uc), row[29], row[30]);
-        row[31] = 0u;
-        put_row(Atile, rrow, row);
+    // This thread's terms of row i (row_terms_kernel's planes; zeros past the rows).
+    auto load_terms = [&](int64_t i, float4& q0, float4& q1, float4& t2) {
+      q0 = q1 = t2 = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < set.M) {
+        q0 = rowterms[(3 * g) * set.M + i];
+        q1 = rowterms[(3 * g + 1) * set.M + i];
+        t2 = rowterms[(3 * g + 2) * set.M + i];
       }
+    };
+    // The A row of row i, from its terms when they are precomputed; H r to sQ[buf].
+    auto make_row = [&](int64_t i, const float4& q0, const float4& q1, const float4& t2, int buf,
+                        float& pmax, float& off) {
+      float m2q[kD], rr, ra;
+      if (rowterms) {
+        m2q[0] = q0.x; m2q[1] = q0.y; m2q[2] = q0.z; m2q[3] = q0.w;
+        m2q[4] = q1.x; m2q[5] = q1.y; m2q[6] = q1.z; m2q[7] = q1.w;
+        rr = t2.x;
+        ra = t2.y;
+        pmax = t2.z;
+      } else {
+        float rv[kD], a[kD];
+        if (i < set.M) {
+          target32(set, cbs, n_fixed, i, g, rv, a, err);
+        } else {
+#pragma unroll
+          for (int j = 0; j < kD; ++j) rv[j] = a[j] = 0.f;
+        }
+        vector_terms_rr(rv, a, sH, m2q, pmax, rr, ra);
+      }
+      // offset making every D = low + off >= 0, with margins for every rounding involved
+      off = (rr + 32.f * kU * ra + 2.f * uc * (hrow * l1max * cinf + 2.f * pmax * l1max)) *
+                (1.f + 4.f * uc) + 1e-30f;
+      const float beta = -2.f * uc * pmax;
+      if (st.cnt) {  // H r of this row, kept for the statistics (-m2q / 2, exact)
+        float* q = sQ + (buf * 256 + tid) * kD;
+        *reinterpret_cast<float4*>(q) =
+            make_float4(-0.5f * m2q[0], -0.5f * m2q[1], -0.5f * m2q[2], -0.5f * m2q[3]);
+        *reinterpret_cast<float4*>(q + 4) =
+            make_float4(-0.5f * m2q[4], -0.5f * m2q[5], -0.5f * m2q[6], -0.5f * m2q[7]);
+      }
+      uint32_t row[kK];
+#pragma unroll
+      for (int q = 0; q < kD; ++q) {
+        uint32_t h, l;
+        split(m2q[q], h, l);
+        row[q] = h;
+        row[8 + q] = h;
+        row[16 + q] = l;
+      }
+      const uint32_t one = __float_as_uint(1.f);
+      row[24] = one;
+      row[25] = one;
+      split(beta, row[26], row[28]);
+      row[27] = row[26];
+      split(off * (1.f - uc), row[29], row[30]);
+      row[31] = 0u;
+      put_row(Atile, rrow, row);
       tc::fence_async_smem();
+    };
+    auto issue = [&](int c) {  // chunk c's MMA into this half's accumulator
+      if (rrow == 0) {
+        tc::tc_fence_after();
+        const uint32_t a0 = tc::smem_u32(Atile), b0 = tc::smem_u32(Bbuf + c * kTcBTile);
+#pragma unroll
+        for (int ks = 0; ks < kK / 8; ++ks)
+          tc::mma_tf32(tmem, tc::smem_desc(a0 + ks * 256, 128, (kK / 4) * 128),
+                       tc::smem_desc(b0 + ks * 256, 128, (kK / 4) * 128), idesc, ks > 0 ? 1u : 0u);
+        tc::mma_commit(tc::smem_u32(&bar_mma));
+      }
+    };
+    auto wait_mma = [&]() -> bool {  // the same answer in the whole warp
+      const bool done = tc::mbar_wait(tc::smem_u32(&bar_mma), (uint32_t)(mma_count & 1), err);
+      ++mma_count;
+      tc::tc_fence_after();
+      return __all_sync(0xffffffffu, done);
+    };
 
+    // Software pipeline of a half: while a tile's certificate and statistics run, the next tile's
+    // first MMA does, and the next tile's terms are loaded before the sweep.
+    int64_t i = (pg * 2 + half) * kRows + rrow;
+    float pmax, off;
+    {
+      float4 q0, q1, t2;
+      if (rowterms) load_terms(i, q0, q1, t2);
+      make_row(i, q0, q1, t2, 0, pmax, off);
+    }
+    ok = half_sync_and(half, ok);
+    if (ok) issue(nchunk - 1);
+    for (int t = 0; t < np && ok; ++t) {
+      const bool row_ok = i < set.M, more = t + 1 < np;
+      const int64_t i_next = i + 2 * kRows;
+      float4 q0, q1, t2;
+      if (rowterms && more) load_terms(i_next, q0, q1, t2);
       uint32_t mb[kBlk], mc[kBlk];  // block and class minima (fp32 bits)
 #pragma unroll
       for (int e = 0; e < kBlk; ++e) mb[e] = mc[e] = 0xffffffffu;
+      auto sweep = [&](auto chunk) {
+        constexpr int c = decltype(chunk)::value;
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        if (c < nchunk) {
-          // the A rows are written, the accumulator has been read; ok is then uniform in the half
-          ok = half_sync_and(half, ok);
+        for (int rnd = 0; rnd < 2; ++rnd) {
+          uint32_t v[64];
+          tc::tmem_ld64_wait(trow + 64 * rnd, v);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) mb[8 * c + 4 * rnd + q] = min16_bits(v + kBlk * q);
+#pragma unroll
+          for (int e = 0; e < kBlk; ++e) {
+            mc[e] = __vimin3_u32(mc[e], v[e], v[kBlk + e]);
+            mc[e] = __vimin3_u32(mc[e], v[2 * kBlk + e], v[3 * kBlk + e]);
+          }
         }
-        if (c < nchunk && ok) {
-          if (rrow == 0) {
-            tc::tc_fence_after();
-            const uint32_t a0 = tc::smem_u32(Atile), b0 = tc::smem_u32(Bbuf + c * kTcBTile);
-#pragma unroll
-            for (int ks = 0; ks < kK / 8; ++ks)
-              tc::mma_tf32(tmem, tc::smem_desc(a0 + ks * 256, 128, (kK / 4) * 128),
-                           tc::smem_desc(b0 + ks * 256, 128, (kK / 4) * 128), idesc,
-                           ks > 0 ? 1u : 0u);
-            tc::mma_commit(tc::smem_u32(&bar_mma));
-          }
-          ok = tc::mbar_wait(tc::smem_u32(&bar_mma), (uint32_t)(mma_count & 1), err);
-          ++mma_count;
-          ok = __all_sync(0xffffffffu, ok);
-          tc::tc_fence_after();
-          if (ok) {
-#pragma unroll
-            for (int rnd = 0; rnd < 4; ++rnd) {
-              uint32_t v[32];
-              tc::tmem_ld32_nowait(trow + 32 * rnd, v);
-              tc::tmem_wait_ld_dep(v);
-              mb[8 * c + 2 * rnd] = min16_bits(v);
-              mb[8 * c + 2 * rnd + 1] = min16_bits(v + kBlk);
-#pragma unroll
-              for (int e = 0; e < kBlk; ++e) mc[e] = __vimin3_u32(mc[e], v[e], v[kBlk + e]);
-            }
-          }
-          tc::tc_fence_before();
+      };
+      ok = wait_mma();
+      if (nchunk == 2) {  // chunk 1 first: the last sweep is always chunk 0's
+        if (ok) sweep(std::integral_constant<int, 1>{});
+        tc::tc_fence_before();
+        ok = half_sync_and(half, ok);  // the accumulator has been read; ok uniform in the half
+        if (ok) {
+          issue(0);
+          ok = wait_mma();
         }
       }
-      ok = half_sync_and(half, ok);  // both chunks read: the accumulator and the A tile are free
+      // this tile's MMAs are done with the A tile: the next tile's rows
+      float pmax_next = 0.f, off_next = 0.f;
+      if (ok && more) make_row(i_next, q0, q1, t2, (t + 1) & 1, pmax_next, off_next);
+      if (ok) sweep(std::integral_constant<int, 0>{});
+      tc::tc_fence_before();
+      ok = half_sync_and(half, ok);  // rows written, accumulator read
       if (!ok) break;
+      if (more) issue(nchunk - 1);
 
       // Certificate, code, open row and statistics of this thread's row.
       bool open = false;
@@ -748,10 +777,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
           // (|v| < 2^30) enters as v = 2^15 vh + vl, 0 <= vl < 2^15, in two 32-bit sums: exact,
           // since a segment has fewer than 2^16 rows.
           float q[kD];
-          const float4 q0 = *reinterpret_cast<const float4*>(sQ + tid * kD);
-          const float4 q1 = *reinterpret_cast<const float4*>(sQ + tid * kD + 4);
-          q[0] = q0.x; q[1] = q0.y; q[2] = q0.z; q[3] = q0.w;
-          q[4] = q1.x; q[5] = q1.y; q[6] = q1.z; q[7] = q1.w;
+          load_vec(sQ + ((t & 1) * 256 + tid) * kD, q);
           atomicAdd(&s_cnt[j], 1);
 #pragma unroll
           for (int e = 0; e < kD; ++e) {
@@ -787,6 +813,9 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
                     err);
         om = rest;
       }
+      i = i_next;
+      pmax = pmax_next;
+      off = off_next;
     }
     ok = __syncthreads_and(ok);  // both halves are done with the group's operand and statistics
     if (st.cnt && tid < cw.K) {  // flush (integer sums: order-free) and clear

@@ -310,14 +310,19 @@ prep_b_kernel(SetView set, int64_t g_begin, int64_t G_range, const float* __rest
 // Ra, Pmax (vector_terms_rr of target32), as three planes of M float4 per group,
 // rt[(3 g + p) M + i]: p = 0, 1 the two halves of m2q, p = 2 (rr, Ra, Pmax, 0). The arg-min
 // pass reads them instead of recomputing them, with bit-identical values.
+// With statistics (st.cnt) it also takes the maxima behind their fixed-point scale from the vectors
+// it reads, and sets the scale (stats_merge_scale): a pass over the matrix and two launches less per
+// codebook fit.
 __global__ void __launch_bounds__(128)
-row_terms_kernel(SetView set, CbList cbs, int n_fixed, float4* __restrict__ rt,
+row_terms_kernel(SetView set, CbList cbs, int n_fixed, float4* __restrict__ rt, StatsView st,
                  unsigned* err) {
   pdl_trigger();
   pdl_wait();
   const int64_t nvec = set.M * set.G_sub;
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvec;
-       v += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t nth = (int64_t)gridDim.x * blockDim.x;
+  float tm = 0.f;
+  for (int64_t v = tid; v < nvec; v += nth) {
     const int64_t g = v / set.M, i = v - g * set.M;
     float rv[kD], a[kD], m2q[kD], pmax, rr, ra;
     target32(set, cbs, n_fixed, i, g, rv, a, err);
@@ -325,7 +330,20 @@ row_terms_kernel(SetView set, CbList cbs, int n_fixed, float4* __restrict__ rt,
     rt[(3 * g) * set.M + i] = make_float4(m2q[0], m2q[1], m2q[2], m2q[3]);
     rt[(3 * g + 1) * set.M + i] = make_float4(m2q[4], m2q[5], m2q[6], m2q[7]);
     rt[(3 * g + 2) * set.M + i] = make_float4(rr, ra, pmax, 0.f);
+    float t[kD];
+    load_vec(set.T + i * set.ldT + g * kD, t);
+#pragma unroll
+    for (int j = 0; j < kD; ++j) tm = max_keep_nan(tm, fabsf(t[j]));
   }
+  if (!st.cnt) return;
+  float hm = 0.f;
+  for (int64_t r = tid; r < set.G_sub * kD; r += nth) {
+    float s = 0.f;
+#pragma unroll
+    for (int j = 0; j < kD; ++j) s += fabsf(set.Hb[r * kD + j]);  // a NaN entry makes the sum NaN
+    hm = max_keep_nan(hm, s);
+  }
+  stats_merge_scale(st, cbs, n_fixed, tm, hm, nvec > 0 ? nvec : 1, err);
 }
 
 constexpr int kSmallK = 2 * kTcCols;   // codebooks up to this size stay resident in shared memory
@@ -2760,14 +2778,14 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
 }  // namespace
 
 crvq_status launch_row_terms(const SetView& set, const CbList& cbs, int n_fixed, float4* rt,
-                             cudaStream_t stream) {
+                             const StatsView* st, cudaStream_t stream) {
   const int64_t nvec = set.M * set.G_sub;
   if (nvec == 0) return CRVQ_OK;
   unsigned* err = nullptr;
   CRVQ_TRY(device_error_word(&err));
   const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(nvec, 128), 16 * sm_count());
   CRVQ_CUDA(launch_pdl(row_terms_kernel, dim3(blocks), dim3(128), 0, stream, set, cbs, n_fixed,
-                       rt, err));
+                       rt, st ? *st : StatsView{}, err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }

@@ -94,9 +94,11 @@ struct EncodeExtras {
   const float4* rowterms = nullptr;
 };
 
-// The arg-min pass's per-vector terms for all M x G_sub vectors of the set (3 M G_sub float4).
+// The arg-min pass's per-vector terms for all M x G_sub vectors of the set (3 M G_sub float4); with
+// st, also the fixed-point scale of codebook n_fixed's statistics (which covers every group of the
+// set), as launch_stats_prepare sets it.
 crvq_status launch_row_terms(const SetView& set, const CbList& cbs, int n_fixed, float4* rt,
-                             cudaStream_t stream);
+                             const StatsView* st, cudaStream_t stream);
 
 // Scratch of one arg-min pass over a set of M rows and G_range groups with a K-entry codebook
 // (B images, codeword terms, codebook maxima, flag list).

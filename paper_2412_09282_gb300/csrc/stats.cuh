@@ -61,10 +61,76 @@ __host__ __device__ inline double stats_scale_for(double bound, int64_t n) {
   const double lim = 4.611686018427387904e18;  // 2^62
   const double denom = bound * (double)(n > 0 ? n : 1);
   if (!(denom > 0.0)) return 1099511627776.0;  // 2^40: nothing to scale
-  int e = (int)floor(log2(lim / denom));
-  const int e_term = (int)floor(log2(1073741824.0 / bound));  // 2^30 / bound
+  int e = ilogb(lim / denom);
+  const int e_term = ilogb(1073741824.0 / bound);  // 2^30 / bound
   if (e_term < e) e = e_term;
   return ldexp(1.0, e < -126 ? -126 : (e > 126 ? 126 : e));
+}
+
+// Maxima behind the scale, in the statistics' head after the scale itself: maxbits[0] = max |T| over
+// the covered vectors, [1] = max row sum of |H_g|, [2 + s] = max |C_s| (float bits of non-negative
+// values, merged with atomicMax; a NaN has larger bits than every finite value and Inf, so it
+// survives the merge and makes the bound non-finite), [2 + kMaxCodebooks] = CTAs done.
+constexpr int kMaxWords = 2 + kMaxCodebooks + 1;
+
+__host__ __device__ inline unsigned* stats_maxbits(const StatsView& st) {
+  return reinterpret_cast<unsigned*>(st.scale + 1);
+}
+
+// max(a, b) that keeps a NaN: fmaxf returns the other operand when one is NaN, which would
+// leave the bound below finite and hide a non-finite input from the scale check.
+__device__ __forceinline__ float max_keep_nan(float a, float b) {
+  return (b > a || b != b) ? b : a;
+}
+
+// Merges a thread's maxima of |T| (tm) and of the row sums of |H| (hm) and, strided over the grid,
+// the maxima of the other codebooks; the grid's last CTA sets the scale from them (whole CTAs of
+// whole warps call it once, at their end). n_members: the vectors that may be added.
+__device__ __forceinline__ void stats_merge_scale(const StatsView& st, const CbList& cbs, int which,
+                                                  float tm, float hm, int64_t n_members,
+                                                  unsigned* err) {
+  unsigned* maxbits = stats_maxbits(st);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    tm = max_keep_nan(tm, __shfl_xor_sync(0xffffffffu, tm, off));
+    hm = max_keep_nan(hm, __shfl_xor_sync(0xffffffffu, hm, off));
+  }
+  __shared__ float red[2][32];  // one atomic per CTA: thousands on one address would queue
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = tm;
+    red[1][threadIdx.x >> 5] = hm;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    float m = red[threadIdx.x][0];
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max_keep_nan(m, red[threadIdx.x][w]);
+    atomicMax(&maxbits[threadIdx.x], __float_as_uint(m));
+  }
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t nth = (int64_t)gridDim.x * blockDim.x;
+  for (int s = 0; s < cbs.n; ++s) {
+    if (s == which) continue;
+    float m = 0.f;
+    for (int64_t e = tid; e < (int64_t)cbs.cb[s].K * kD; e += nth)
+      m = max_keep_nan(m, fabsf(cbs.cb[s].C[e]));
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+      m = max_keep_nan(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if ((threadIdx.x & 31) == 0 && m != 0.f) atomicMax(&maxbits[2 + s], __float_as_uint(m));
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  if (atomicAdd(&maxbits[2 + kMaxCodebooks], 1u) != gridDim.x - 1) return;
+  __threadfence();
+  double cs = 0.0;
+  for (int s = 0; s < cbs.n; ++s)
+    if (s != which) cs += (double)__uint_as_float(__ldcg(&maxbits[2 + s]));
+  // |H_g tau|_inf <= max row sum |H_g| * (max |t| + sum_s max |C_s|)
+  const double bound = (double)__uint_as_float(__ldcg(&maxbits[1])) *
+                       ((double)__uint_as_float(__ldcg(&maxbits[0])) + cs) * 1.001;
+  if (!isfinite(bound)) raise_error(err, ERRBIT_NUMERIC);
+  *st.scale = stats_scale_for(bound, n_members);
 }
 
 // tau = t - sum over the codebooks s != which that cover g of C_s[code] (fp32, codebook order).
@@ -153,9 +219,9 @@ __device__ inline bool cholesky_solve8(const double A[36], const double b[kD], d
 
 // Host side (update.cu).
 crvq_status stats_alloc(Scratch& mem, int64_t G_cov, int K, StatsView* st, cudaStream_t s);
-// Zeroes cnt/bacc (scale is kept).
+// Zeroes cnt, bacc and the maxima behind the scale.
 crvq_status stats_zero(const StatsView& st, cudaStream_t s);
-// Computes the fixed-point scale for accumulating codebook `which` over `set`.
+// Computes the fixed-point scale for accumulating codebook `which` over `set` (maxima zero on entry).
 crvq_status launch_stats_prepare(const SetView& set, const CbList& cbs, int which,
                                  const StatsView& st, cudaStream_t stream);
 // Solves every codeword from the statistics and leaves cnt and bacc zero (each is cleared

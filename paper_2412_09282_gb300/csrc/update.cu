@@ -22,18 +22,10 @@ namespace crvq {
 
 namespace {
 
-// max(a, b) that keeps a NaN: fmaxf returns the other operand when one is NaN, which would
-// leave the bound below finite and hide a non-finite input from the scale check.
-__device__ __forceinline__ float max_keep_nan(float a, float b) {
-  return (b > a || b != b) ? b : a;
-}
-
-// maxbits[0] = max |T| over the covered vectors, maxbits[1] = max row sum of |H_g|,
-// maxbits[2 + s] = max |C_s| (float bits of non-negative values, merged with atomicMax; a NaN
-// has larger bits than every finite value and Inf, so it survives the merge and makes the
-// bound non-finite).
+// The maxima behind the fixed-point scale, and the scale (stats_merge_scale).
 __global__ void __launch_bounds__(256)
-maxabs_kernel(SetView set, int64_t G_cov, CbList cbs, int which, unsigned* __restrict__ maxbits) {
+maxabs_kernel(SetView set, CbList cbs, int which, StatsView st, int64_t n_members, unsigned* err) {
+  const int64_t G_cov = st.G_cov;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nth = (int64_t)gridDim.x * blockDim.x;
   float tm = 0.f;
@@ -55,39 +47,7 @@ maxabs_kernel(SetView set, int64_t G_cov, CbList cbs, int which, unsigned* __res
     for (int j = 0; j < kD; ++j) s += fabsf(h[j]);  // a NaN entry makes the sum NaN
     hm = max_keep_nan(hm, s);
   }
-  // warp max, then one atomic per warp
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    tm = max_keep_nan(tm, __shfl_xor_sync(0xffffffffu, tm, off));
-    hm = max_keep_nan(hm, __shfl_xor_sync(0xffffffffu, hm, off));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicMax(&maxbits[0], __float_as_uint(tm));
-    atomicMax(&maxbits[1], __float_as_uint(hm));
-  }
-  for (int s = 0; s < cbs.n; ++s) {
-    if (s == which) continue;
-    float m = 0.f;
-    for (int64_t e = tid; e < (int64_t)cbs.cb[s].K * kD; e += nth)
-      m = max_keep_nan(m, fabsf(cbs.cb[s].C[e]));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-      m = max_keep_nan(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) atomicMax(&maxbits[2 + s], __float_as_uint(m));
-  }
-}
-
-__global__ void stats_scale_kernel(const unsigned* __restrict__ maxbits, int n_cb, int which,
-                                   int64_t n_members, double* __restrict__ scale,
-                                   unsigned* err) {
-  double cs = 0.0;
-  for (int s = 0; s < n_cb; ++s)
-    if (s != which) cs += (double)__uint_as_float(maxbits[2 + s]);
-  // |H_g tau|_inf <= max row sum |H_g| * (max |t| + sum_s max |C_s|)
-  const double bound =
-      (double)__uint_as_float(maxbits[1]) * ((double)__uint_as_float(maxbits[0]) + cs) * 1.001;
-  if (!isfinite(bound)) raise_error(err, ERRBIT_NUMERIC);
-  *scale = stats_scale_for(bound, n_members);
+  stats_merge_scale(st, cbs, which, tm, hm, n_members, err);
 }
 
 // Statistics of every covered vector from its current code. CTA (x, y): groups y,
@@ -98,6 +58,7 @@ __global__ void stats_scale_kernel(const unsigned* __restrict__ maxbits, int n_c
 // atomics): exact, as accumulate_grid gives a CTA fewer than 2^16 rows of a group. Integer
 // sums: the order is immaterial.
 constexpr int kSmemStatsK = 256;
+constexpr int kAccRows = 2;
 
 __global__ void __launch_bounds__(256)
 accumulate_stats_kernel(SetView set, CbList cbs, int which, StatsView st, unsigned* err) {
@@ -114,26 +75,48 @@ accumulate_stats_kernel(SetView set, CbList cbs, int which, StatsView st, unsign
       for (int e = threadIdx.x; e < kSmemStatsK; e += blockDim.x) s_cnt[e] = 0;
       __syncthreads();
     }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < set.M;
-         i += (int64_t)gridDim.x * blockDim.x) {
-      const int32_t k = cw.codes[i * cw.ld + g];
-      if (k < 0 || k >= cw.K) {
-        raise_error(err, ERRBIT_INDEX);
-        continue;
-      }
-      float tau[kD], q[kD];
-      stats_target(set, cbs, which, i, g, tau, err);
-      stats_htau(set.Hb + g * kD * kD, tau, q);
-      if (smem) {
-        atomicAdd(&s_cnt[k], 1);
+    // the group's H block in registers: read once, not 64 loads per vector
+    float H[kD * kD];
 #pragma unroll
-        for (int j = 0; j < kD; ++j) {
-          const long long v = fix_rn_small(q[j], sscale);
-          atomicAdd(&s_b32[(2 * j) * kSmemStatsK + k], (int)(v >> 15));
-          atomicAdd(&s_b32[(2 * j + 1) * kSmemStatsK + k], (int)(v & 0x7fff));
+    for (int e = 0; e < kD * kD; e += 4) {
+      const float4 h = __ldg(reinterpret_cast<const float4*>(set.Hb + g * kD * kD + e));
+      H[e] = h.x;
+      H[e + 1] = h.y;
+      H[e + 2] = h.z;
+      H[e + 3] = h.w;
+    }
+    // kAccRows rows per step, their codes and vectors loaded before any is used
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < set.M;
+         i0 += kAccRows * stride) {
+      int32_t k[kAccRows];
+      float tau[kAccRows][kD];
+#pragma unroll
+      for (int u = 0; u < kAccRows; ++u) {
+        const int64_t i = i0 + u * stride;
+        k[u] = i < set.M ? cw.codes[i * cw.ld + g] : 0;
+        if (i < set.M) stats_target(set, cbs, which, i, g, tau[u], err);
+      }
+#pragma unroll
+      for (int u = 0; u < kAccRows; ++u) {
+        if (i0 + u * stride >= set.M) break;
+        if (k[u] < 0 || k[u] >= cw.K) {
+          raise_error(err, ERRBIT_INDEX);
+          continue;
         }
-      } else {
-        stats_add(st, sscale, g, k, q);
+        float q[kD];
+        stats_htau(H, tau[u], q);
+        if (smem) {
+          atomicAdd(&s_cnt[k[u]], 1);
+#pragma unroll
+          for (int j = 0; j < kD; ++j) {
+            const long long v = fix_rn_small(q[j], sscale);
+            atomicAdd(&s_b32[(2 * j) * kSmemStatsK + k[u]], (int)(v >> 15));
+            atomicAdd(&s_b32[(2 * j + 1) * kSmemStatsK + k[u]], (int)(v & 0x7fff));
+          }
+        } else {
+          stats_add(st, sscale, g, k[u], q);
+        }
       }
     }
     if (smem) {
@@ -464,7 +447,18 @@ crvq_status stats_alloc(Scratch& mem, int64_t G_cov, int K, StatsView* st, cudaS
 
 crvq_status stats_zero(const StatsView& st, cudaStream_t s) {
   const StatsLayout L = stats_layout(st.G_cov, st.K);
-  CRVQ_CUDA(cudaMemsetAsync(st.cnt, 0, L.cnt + L.bacc, s));
+  CRVQ_CUDA(cudaMemsetAsync(st.cnt, 0, L.total, s));
+  return CRVQ_OK;
+}
+
+static crvq_status launch_maxabs(const SetView& set, const CbList& cbs, int which,
+                                 const StatsView& st, unsigned* err, cudaStream_t stream) {
+  const int64_t n = set.M * cbs.cb[which].G_cov;
+  ProfScope ps("update_bound", stream, (double)n * kD * 4.0);
+  maxabs_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256),
+                                                                   4 * sm_count())),
+                  256, 0, stream>>>(set, cbs, which, st, std::max<int64_t>(1, n), err);
+  CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
 
@@ -472,20 +466,7 @@ crvq_status launch_stats_prepare(const SetView& set, const CbList& cbs, int whic
                                  const StatsView& st, cudaStream_t stream) {
   unsigned* err = nullptr;
   CRVQ_TRY(device_error_word(&err));
-  const CbView& cw = cbs.cb[which];
-  // maxbits live right after the scale (same 256-byte block).
-  unsigned* maxbits = reinterpret_cast<unsigned*>(st.scale + 1);
-  CRVQ_CUDA(cudaMemsetAsync(maxbits, 0, (2 + kMaxCodebooks) * sizeof(unsigned), stream));
-  const int64_t n = set.M * cw.G_cov;
-  const int nsm = sm_count();
-  ProfScope ps("update_bound", stream, (double)n * kD * 4.0);
-  maxabs_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), 4 * nsm)),
-                  256, 0, stream>>>(set, cw.G_cov, cbs, which, maxbits);
-  CRVQ_LAUNCHED();
-  stats_scale_kernel<<<1, 1, 0, stream>>>(maxbits, cbs.n, which, std::max<int64_t>(1, n),
-                                          st.scale, err);
-  CRVQ_LAUNCHED();
-  return CRVQ_OK;
+  return launch_maxabs(set, cbs, which, st, err, stream);
 }
 
 crvq_status launch_stats_solve(const SetView& set, const StatsView& st, const float* C_old,
@@ -542,16 +523,10 @@ crvq_status launch_update_codebook_on(const SetView& set, const CbList& cbs, int
   const StatsLayout L = stats_layout(cw.G_cov, cw.K);
   StatsView st;
   stats_bind(scratch, cw.G_cov, cw.K, &st);
-  unsigned* maxbits = reinterpret_cast<unsigned*>(st.scale + 1);
   // The scratch keeps the previous call's contents: clear counts, sums and maxima.
-  CRVQ_CUDA(cudaMemsetAsync(scratch, 0, L.cnt + L.bacc + L.head, stream));
+  CRVQ_CUDA(cudaMemsetAsync(scratch, 0, L.total, stream));
   const int nsm = sm_count();
-  maxabs_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), 4 * nsm)),
-                  256, 0, stream>>>(set, cw.G_cov, cbs, which, maxbits);
-  CRVQ_LAUNCHED();
-  stats_scale_kernel<<<1, 1, 0, stream>>>(maxbits, cbs.n, which, std::max<int64_t>(1, n),
-                                          st.scale, err);
-  CRVQ_LAUNCHED();
+  CRVQ_TRY(launch_maxabs(set, cbs, which, st, err, stream));
   if (n > 0) {
     accumulate_stats_kernel<<<accumulate_grid(set.M, cw.G_cov, nsm), 256, 0, stream>>>(
         set, cbs, which, st, err);

@@ -75,6 +75,13 @@ __global__ void extract_blocks_kernel(const float* __restrict__ H, int64_t N, in
 
 }  // namespace
 
+crvq_status launch_hessian_delta(const float* xsq, int64_t N, float damp_rel, float* delta,
+                                 double* delta64, cudaStream_t stream) {
+  hessian_delta_kernel<<<1, 1024, 0, stream>>>(xsq, N, damp_rel, delta, delta64);
+  CRVQ_LAUNCHED();
+  return CRVQ_OK;
+}
+
 crvq_status launch_hessian(const float* X, int64_t n, int64_t N, int d, float damp_rel,
                            float* H, float* xsq, float* H_blocks, float* delta,
                            cudaStream_t stream) {
@@ -83,8 +90,7 @@ crvq_status launch_hessian(const float* X, int64_t n, int64_t N, int d, float da
   CRVQ_TRY(launch_tc_syrk(X, n, N, H, xsq, stream));
   {
     ProfScope ps("hessian_finalize", stream, 0.0);
-    hessian_delta_kernel<<<1, 1024, 0, stream>>>(xsq, N, damp_rel, delta, mem.as<double>());
-    CRVQ_LAUNCHED();
+    CRVQ_TRY(launch_hessian_delta(xsq, N, damp_rel, delta, mem.as<double>(), stream));
     const int blocks = (int)std::min<int64_t>(ceil_div(N * kD, 256), 4 * sm_count());
     hessian_damp_kernel<<<blocks, 256, 0, stream>>>(H, N, mem.as<double>(), H_blocks);
     CRVQ_LAUNCHED();

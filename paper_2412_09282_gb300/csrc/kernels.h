@@ -23,6 +23,10 @@ crvq_status launch_hessian(const float* X, int64_t n, int64_t N, int d, float da
 crvq_status launch_extract_blocks(const float* H, int64_t N, int d, const int32_t* perm,
                                   float* H_blocks, cudaStream_t stream);
 
+// delta = damp_rel * mean(xsq) in fp64 (fixed order) to delta64 and, rounded, to delta (may be null).
+crvq_status launch_hessian_delta(const float* xsq, int64_t N, float damp_rel, float* delta,
+                                 double* delta64, cudaStream_t stream);
+
 // Tensor-core (tcgen05, 3xTF32) products.
 // S = X^T X / n for X n x N row-major (S N x N, both triangles) and its diagonal.
 crvq_status launch_tc_syrk(const float* X, int64_t n, int64_t N, float* S, float* diag,

@@ -38,36 +38,25 @@ sum_partials_kernel(const float* __restrict__ P, int64_t N, int chunks, float sc
   }
 }
 
-// Original-order blocks, one CTA: xsq[i] = the undamped diagonal, delta = damp_rel * mean(xsq)
-// by the dense path's fixed-order fp64 reduction (1024 strided partials, then a tree), and the
-// blocks with delta added on their diagonals (rounded once from fp64, as the dense path does).
-__global__ void __launch_bounds__(1024)
-blocks_finalize_kernel(const float* __restrict__ P, int chunks, int64_t stride, float scale,
-                       int64_t N, float damp_rel, float* __restrict__ xsq,
-                       float* __restrict__ delta_out, double* __restrict__ delta64,
-                       float* __restrict__ Hb) {
-  __shared__ double part[1024];
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < N; i += blockDim.x) {
-    const float v = chunk_sum(P, chunks, stride, i * 8 + (i & 7), scale);
-    xsq[i] = v;
-    s += (double)v;
-  }
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
-    __syncthreads();
-  }
-  const double delta = (double)damp_rel * (part[0] / (double)N);
-  for (int64_t e = threadIdx.x; e < N * 8; e += blockDim.x) {
+// Original-order blocks without the damping, and their diagonal xsq.
+__global__ void __launch_bounds__(256)
+blocks_sum_kernel(const float* __restrict__ P, int chunks, int64_t stride, float scale, int64_t N,
+                  float* __restrict__ xsq, float* __restrict__ Hb) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < N * 8;
+       e += (int64_t)gridDim.x * blockDim.x) {
     const float v = chunk_sum(P, chunks, stride, e, scale);
-    Hb[e] = ((e >> 3) & 7) == (e & 7) ? (float)((double)v + delta) : v;
+    Hb[e] = v;
+    if (((e >> 3) & 7) == (e & 7)) xsq[e >> 3] = v;
   }
-  if (threadIdx.x == 0) {
-    if (delta_out) *delta_out = (float)delta;
-    *delta64 = delta;
-  }
+}
+
+// Adds delta to the diagonals of the original-order blocks (rounded once from fp64, as the dense path
+// does).
+__global__ void __launch_bounds__(256)
+blocks_add_delta_kernel(const float* __restrict__ xsq, int64_t N, const double* __restrict__ delta64,
+                        float* __restrict__ Hb) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < N) Hb[i * 8 + (i & 7)] = (float)((double)xsq[i] + *delta64);
 }
 
 // Blocks of a given channel order with a known delta.
@@ -624,8 +613,12 @@ crvq_status launch_tc_hessian_blocks(const float* Xt, int64_t ldt, int64_t n, in
   ProfScope ps("hessian_blocks_finalize", stream, (double)chunks * stride * 4.0);
   if (!delta_known) {
     if (perm) return fail(CRVQ_ERR_UNSUPPORTED, "hessian blocks: delta needs the stored order");
-    blocks_finalize_kernel<<<1, 1024, 0, stream>>>(mem.as<float>(), (int)chunks, stride, scale,
-                                                   N, damp_rel, xsq, delta, delta64, Hb);
+    const int blocks = (int)std::min<int64_t>(ceil_div(stride, 256), 4 * sm_count());
+    blocks_sum_kernel<<<blocks, 256, 0, stream>>>(mem.as<float>(), (int)chunks, stride, scale, N, xsq,
+                                                  Hb);
+    CRVQ_LAUNCHED();
+    CRVQ_TRY(launch_hessian_delta(xsq, N, damp_rel, delta, delta64, stream));
+    blocks_add_delta_kernel<<<(unsigned)ceil_div(N, 256), 256, 0, stream>>>(xsq, N, delta64, Hb);
   } else {
     const int blocks = (int)std::min<int64_t>(ceil_div(stride, 256), 4 * sm_count());
     blocks_damp_kernel<<<blocks, 256, 0, stream>>>(mem.as<float>(), (int)chunks, stride, scale,

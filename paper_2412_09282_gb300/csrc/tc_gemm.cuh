@@ -6,7 +6,7 @@
 // lo parts are ~2^-22 relative), accumulated in fp32 by the tensor core.
 //
 // K is staged 16 at a time through two shared-memory stages. All 128 threads split and store a
-// stage while the tensor core works on the previous one, with the global loads of the next stage
+// stage while the tensor core works on the previous one, with the global loads of the next stages
 // already in flight in registers (software pipeline); thread 0 issues the MMAs and commits them to
 // the stage's mbarrier. Operands sit in shared memory in the canonical K-major layout
 // without swizzle: 8-row x 16-byte core matrices, consecutive along K (LBO = 128 B), 8-row
@@ -111,6 +111,7 @@ constexpr int kDiagStageBytes = 2 * kAStageBytes;                      // hi + l
 constexpr int kDiagSmemBytes = kStages * kDiagStageBytes + 1024 + 128;  // + alignment + barriers
 constexpr int kDiagTmemCols = kBM;
 constexpr uint32_t kIdescDiag = idesc_tf32(kBM, kBM);
+constexpr int kDiagAhead = 4;
 
 struct DiagArgs {
   Operand A;            // rows = channels (A.idx: the order, NULL = stored order)
@@ -159,36 +160,46 @@ __global__ void __launch_bounds__(kThreads, 1) syrk_diag_kernel(DiagArgs a) {
   const int64_t nkt = (kend - kbeg + kBK - 1) / kBK;
   uint32_t par = 0;
   bool ok = true;
-  float va[kBM / kThreads][kBK];
-  if (nkt > 0) load_tile<kBM>(a.A, m0, kbeg, kend, va);
-  for (int64_t kt = 0; kt < nkt; ++kt) {
-    const int s = (int)(kt & 1);
-    char* a_hi = smem + s * kDiagStageBytes;
-    char* a_lo = a_hi + kAStageBytes;
-    if (kt >= kStages) {
-      if (ok) ok = mbar_wait(smem_u32(&bars[s]), (par >> s) & 1u, a.err);
-      par ^= 1u << s;
-    }
-    ok = __syncthreads_and(ok);
-    if (!ok) break;
-    split_store<kBM>(va, a_hi, a_lo);
-    if (kt + 1 < nkt) load_tile<kBM>(a.A, m0, kbeg + (kt + 1) * kBK, kend, va);
-    fence_async_smem();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      tc_fence_after();
-      const uint32_t sbo = (kBK / 4) * 128;
+  // The tile's values come kDiagAhead steps ahead of their use, in registers (with one step ahead the
+  // loads' latency was most of a step: 58 us for 1024 tokens).
+  float va[kDiagAhead][kBM / kThreads][kBK];
 #pragma unroll
-      for (int ks = 0; ks < kBK / 8; ++ks) {
-        const uint32_t koff = ks * 256;
-        const uint64_t dh = smem_desc(smem_u32(a_hi) + koff, 128, sbo);
-        const uint64_t dl = smem_desc(smem_u32(a_lo) + koff, 128, sbo);
-        // same order as the dense tile: hi.hi, hi.lo, lo.hi
-        mma_tf32(tmem, dh, dh, kIdescDiag, (kt > 0 || ks > 0) ? 1u : 0u);
-        mma_tf32(tmem, dh, dl, kIdescDiag, 1u);
-        mma_tf32(tmem, dl, dh, kIdescDiag, 1u);
+  for (int u = 0; u < kDiagAhead; ++u)
+    if (u < nkt) load_tile<kBM>(a.A, m0, kbeg + u * kBK, kend, va[u]);
+  for (int64_t k0 = 0; k0 < nkt && ok; k0 += kDiagAhead) {
+#pragma unroll
+    for (int u = 0; u < kDiagAhead; ++u) {
+      const int64_t kt = k0 + u;
+      if (kt >= nkt) break;
+      const int s = (int)(kt & 1);
+      char* a_hi = smem + s * kDiagStageBytes;
+      char* a_lo = a_hi + kAStageBytes;
+      if (kt >= kStages) {
+        if (ok) ok = mbar_wait(smem_u32(&bars[s]), (par >> s) & 1u, a.err);
+        par ^= 1u << s;
       }
-      mma_commit(smem_u32(&bars[s]));
+      ok = __syncthreads_and(ok);
+      if (!ok) break;
+      split_store<kBM>(va[u], a_hi, a_lo);
+      if (kt + kDiagAhead < nkt)
+        load_tile<kBM>(a.A, m0, kbeg + (kt + kDiagAhead) * kBK, kend, va[u]);
+      fence_async_smem();
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        tc_fence_after();
+        const uint32_t sbo = (kBK / 4) * 128;
+#pragma unroll
+        for (int ks = 0; ks < kBK / 8; ++ks) {
+          const uint32_t koff = ks * 256;
+          const uint64_t dh = smem_desc(smem_u32(a_hi) + koff, 128, sbo);
+          const uint64_t dl = smem_desc(smem_u32(a_lo) + koff, 128, sbo);
+          // same order as the dense tile: hi.hi, hi.lo, lo.hi
+          mma_tf32(tmem, dh, dh, kIdescDiag, (kt > 0 || ks > 0) ? 1u : 0u);
+          mma_tf32(tmem, dh, dl, kIdescDiag, 1u);
+          mma_tf32(tmem, dl, dh, kIdescDiag, 1u);
+        }
+        mma_commit(smem_u32(&bars[s]));
+      }
     }
   }
   if (ok && nkt > 0) {

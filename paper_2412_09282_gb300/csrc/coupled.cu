@@ -38,23 +38,61 @@ namespace {
 constexpr int kBlockCols = 256;                 // channels per lazy block (32 groups)
 constexpr int kBlockG = kBlockCols / kD;
 
+// (rh + rl) = vector (i, g) of W minus the codewords of every covering codebook but `which`.
+__device__ __forceinline__ void others_target(const SetView& set, const CbList& cbs, int which,
+                                              int64_t i, int64_t g, float rh[kD], float rl[kD],
+                                              unsigned* err) {
+  load_vec(set.T + i * set.ldT + g * kD, rh);
+#pragma unroll
+  for (int j = 0; j < kD; ++j) rl[j] = 0.f;
+  for (int s = 0; s < cbs.n; ++s) {
+    const CbView& cb = cbs.cb[s];
+    if (s == which || g >= cb.G_cov) continue;
+    const int32_t k = cb.codes[i * cb.ld + g];
+    if (!code_ok(k, cb.K, err)) continue;
+    float c[kD];
+    load_vec(cb.C + (int64_t)k * kD, c);
+#pragma unroll
+    for (int j = 0; j < kD; ++j) {
+      float sj, ej;
+      dfl::two_sum(rh[j], -c[j], sj, ej);
+      rh[j] = sj;
+      rl[j] = __fadd_rn(rl[j], ej);
+    }
+  }
+}
+
+// (rh + rl) - c, rounded once.
+__device__ __forceinline__ float pair_minus(float rh, float rl, float c) {
+  float s, e;
+  dfl::two_sum(rh, -c, s, e);
+  return __fadd_rn(s, __fadd_rn(rl, e));
+}
+
 // D = W - sum over the covering codebooks of C[code] (fp32 pairs, rounded once), M x N.
 __global__ void __launch_bounds__(256)
-residual_kernel(const float* __restrict__ W, int64_t M, int64_t N, CbList cbs,
+residual_kernel(const float* __restrict__ W, int64_t M, int64_t N, CbList cbs, int which,
                 float* __restrict__ D, unsigned* err) {
   const int64_t G = N / kD;
   const SetView set{W, N, M, G, nullptr};
+  const CbView cw = cbs.cb[which];
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < M * G;
        v += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = v / G, g = v % G;
-    float rh[kD], rl[kD];
-    dfl::target(set, cbs, cbs.n, i, g, rh, rl, err);
+    float rh[kD], rl[kD], c[kD];
+    others_target(set, cbs, which, i, g, rh, rl, err);
+#pragma unroll
+    for (int j = 0; j < kD; ++j) c[j] = 0.f;
+    if (g < cw.G_cov) {
+      const int32_t k = cw.codes[i * cw.ld + g];
+      if (code_ok(k, cw.K, err)) load_vec(cw.C + (int64_t)k * kD, c);
+    }
+    float d[kD];
+#pragma unroll
+    for (int j = 0; j < kD; ++j) d[j] = pair_minus(rh[j], rl[j], c[j]);
     float* o = D + i * N + g * kD;
-    *reinterpret_cast<float4*>(o) = make_float4(__fadd_rn(rh[0], rl[0]), __fadd_rn(rh[1], rl[1]),
-                                                __fadd_rn(rh[2], rl[2]), __fadd_rn(rh[3], rl[3]));
-    *reinterpret_cast<float4*>(o + 4) =
-        make_float4(__fadd_rn(rh[4], rl[4]), __fadd_rn(rh[5], rl[5]), __fadd_rn(rh[6], rl[6]),
-                    __fadd_rn(rh[7], rl[7]));
+    *reinterpret_cast<float4*>(o) = make_float4(d[0], d[1], d[2], d[3]);
+    *reinterpret_cast<float4*>(o + 4) = make_float4(d[4], d[5], d[6], d[7]);
   }
 }
 
@@ -94,20 +132,23 @@ block_factor_kernel(const float* __restrict__ H, int64_t N, int64_t G_cov,
   }
 }
 
-// The group steps g = g0 .. g1 - 1 of one block for up to kCplRows rows per CTA. Per group:
+// The group steps g = g0 .. g1 - 1 of one block for up to kCplRows rows per CTA. What a step needs from
+// global memory is loaded before the steps, all at once: the rows' slice of B^T, their targets
+// without codebook `which` (fp32 pairs), their codes, the codebook when it has at most 256 codewords.
+// Per group:
 //  1. shifted targets, a thread per row: t' = t + H_gg^-1 b_g, t = D_g + C[code_g], b_g = the row's
-//     columns of B^T (shared memory, the block's earlier changes included) - H_gg D_g, the solve a
-//     forward and a back substitution in fp32 with the group's factor;
+//     columns of B^T (the block's earlier changes included) - H_gg D_g, the solve a forward and a back
+//     substitution in fp32 with the group's factor;
 //  2. scores, a thread per codeword (chunks of 256): the fp32 lower bound low_k = s_k - Et_k of every
 //     row (8 FMAs), the two smallest of a warp's 32 by integer minima over order-preserving keys
 //     (redux), the two smallest of all by the row's eight lanes;
 //  3. certificate low_2nd - low_j > 2 Et_j; rows without it are decided exactly, a warp per row: every
 //     codeword with low_k <= low_j + 2 Et_j in fp32 pairs, smallest (err, index);
-//  4. the new code, D_g from W, and its change dD_g H[g, g'] added to the later columns, a thread per
-//     column.
-// Bound: latency of the serial group steps (six barriers and about 3 k cycles each at 32 rows).
+//  4. the new code, D_g, and its change dD_g H[g, g'] added to the later columns, a thread per column.
+// Bound: latency of the serial group steps (a 4096 x 4096 sweep has 512 of them, eight warps per SM).
 // 4096 x 4096, 256 codewords, one sweep with both losses: 40.2 ms with a kernel per step and group, 13.3
-// ms with this one.
+// ms with the steps in this kernel, 7.9 ms with the block products and the losses from operand
+// images; loading what the steps need up front, and E's entries ahead in the loss: 5.4 ms.
 constexpr int kCplRows = 32;
 constexpr int kCplThreads = 256;
 constexpr int kCplPad = kBlockCols + 1;  // row stride of the B^T slice in shared memory
@@ -139,69 +180,113 @@ struct CplArgs {
   CbList cbs;
 };
 
+// A warp's two smallest keys of a row, the smallest one's codeword and its 2 Et.
+struct __align__(16) CplBest {
+  uint32_t v1, v2;
+  int k1;
+  float e2;
+};
+
+struct CplShared {
+  float B[kCplRows * kCplPad];               // [row][column of the block]
+  float2 R[kBlockG][kCplRows][kD];           // targets without `which`: (hi, lo)
+  float C[kCplThreads * kD];                 // the codebook (K <= 256)
+  int32_t code[kBlockG][kCplRows];
+  CplBest best[kCplRows][8];                 // per row and warp
+  float H[2][kD * kD], L[2][kD * kD], inv[2][kD];  // the group's and the next one's
+  float T[kCplRows][kD];                     // t'
+  float Q[kCplRows][kD];                     // -2 H t'
+  float beta[kCplRows];                      // -2 u C Pmax
+  float DD[kCplRows][kD];                    // D_g, then its change
+  float thr[kCplRows];
+  int open[kCplRows];
+  int n_open;
+};
+constexpr size_t kCplSmem = sizeof(CplShared) + 16;
+
 __global__ void __launch_bounds__(kCplThreads)
 coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
-  __shared__ float sB[kCplRows * kCplPad];            // [row][column of the block]
-  __shared__ __align__(16) float sH[kD * kD];
-  __shared__ float sL[kD * kD], sInv[kD];
-  __shared__ __align__(16) float sT[kCplRows][kD];    // t'
-  __shared__ __align__(16) float sQ[kCplRows][kD];    // -2 H t'
-  __shared__ float sPmax[kCplRows];
-  __shared__ __align__(16) float sDD[kCplRows][kD];   // change of D_g
-  __shared__ uint32_t sV1[kCplRows][8], sV2[kCplRows][8];  // per warp: smallest, second smallest key
-  __shared__ int sK1[kCplRows][8];
-  __shared__ float sE1[kCplRows][8];                  // 2 Et of the smallest
-  __shared__ int sCode[kCplRows];
-  __shared__ float sThr[kCplRows];
-  __shared__ int sOpen[kCplRows];
-  __shared__ int n_open;
+  extern __shared__ __align__(16) char cpl_raw[];
+  CplShared& s = *reinterpret_cast<CplShared*>(cpl_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t i0 = (int64_t)blockIdx.x * a.rows;
   const int nr = (int)min((int64_t)a.rows, a.M - i0);
-  const int ncol = (int)(a.g1 - a.g0) * kD;
+  const int ng = (int)(a.g1 - a.g0), ncol = ng * kD;
   const CbView cw = a.cbs.cb[a.which];
   const SetView wset{a.W, a.N, a.M, a.N / kD, nullptr};
   const float cmul = bound_mult(0);
   const int row8 = tid >> 3, j8 = tid & 7;  // (row, component) threads
+  const bool resident = cw.K <= kCplThreads;
+  const float* C = resident ? s.C : cw.C;
   for (int e = tid; e < nr * ncol; e += kCplThreads) {
     const int c = e / nr, r = e - c * nr;
-    float s = 0.f;
-    for (int q = 0; q < a.chunks; ++q) s += __ldg(a.P + ((int64_t)q * ncol + c) * a.M + i0 + r);
-    sB[r * kCplPad + c] = s;
+    float v = 0.f;
+    for (int q = 0; q < a.chunks; ++q) v += __ldg(a.P + ((int64_t)q * ncol + c) * a.M + i0 + r);
+    s.B[r * kCplPad + c] = v;
   }
+  for (int e = tid; e < nr * ng; e += kCplThreads) {
+    const int r = e / ng, gl = e - r * ng;
+    float rh[kD], rl[kD];
+    others_target(wset, a.cbs, a.which, i0 + r, a.g0 + gl, rh, rl, err);
+#pragma unroll
+    for (int j = 0; j < kD; ++j) s.R[gl][r][j] = make_float2(rh[j], rl[j]);
+    s.code[gl][r] = cw.codes[(i0 + r) * cw.ld + a.g0 + gl];
+  }
+  if (resident)
+    for (int e = tid; e < cw.K * kD; e += kCplThreads) s.C[e] = __ldg(cw.C + e);
+  auto load_group = [&](int64_t g, int buf) {  // the group's H block and factor
+    if (tid < kD * kD) {
+      s.H[buf][tid] = a.Hb[g * kD * kD + tid];
+    } else if (tid < 2 * kD * kD) {
+      s.L[buf][tid - kD * kD] = a.Lf[g * kD * kD + tid - kD * kD];
+    } else if (tid < 2 * kD * kD + kD) {
+      s.inv[buf][tid - 2 * kD * kD] = a.Linv[g * kD + tid - 2 * kD * kD];
+    }
+  };
+  load_group(a.g0, 0);
+  if (tid == 0) s.n_open = 0;
+  __syncthreads();
   for (int64_t g = a.g0; g < a.g1; ++g) {
-    const int col0 = (int)(g - a.g0) * kD;
-    // loads that do not depend on the previous group's decision
-    float hcol[kD];  // H[g][this thread's column of the block]
+    const int gl = (int)(g - a.g0), col0 = gl * kD, buf = gl & 1;
+    const float* sH = s.H[buf];
+    const float* sL = s.L[buf];
+    const float* sInv = s.inv[buf];
+    float hcol[kD];  // H[g][this thread's column of the block], used at the step's end
     const int col = tid;
     if (col < ncol)
 #pragma unroll
       for (int q = 0; q < kD; ++q) hcol[q] = __ldg(a.H + (g * kD + q) * a.N + a.g0 * kD + col);
-    float dold = 0.f;
-    if (row8 < nr) dold = a.D[(i0 + row8) * a.N + g * kD + j8];
-    if (tid < kD * kD) {
-      sH[tid] = a.Hb[g * kD * kD + tid];
-      sL[tid] = a.Lf[g * kD * kD + tid];
-    }
-    if (tid < kD) sInv[tid] = a.Linv[g * kD + tid];
-    if (tid == 0) n_open = 0;
-    if (row8 < nr) sDD[row8][j8] = dold;  // D_g until the decision
-    __syncthreads();  // (and the previous group's changes of sB are visible)
+    if (g + 1 < a.g1) load_group(g + 1, buf ^ 1);
     const bool factor = sInv[0] != 0.f;  // no factor (reported): the code stays
+    // this thread's codeword of the first chunk
+    float c[kD], n = 0.f, na = 0.f, l1 = 0.f;
+#pragma unroll
+    for (int j = 0; j < kD; ++j) c[j] = 0.f;
+    if (tid < cw.K) {
+      load_vec(C + tid * kD, c);
+      codeword_terms(c, sH, n, na, l1);
+    }
     // 1. shifted targets
     if (tid < nr) {
-      const int64_t i = i0 + tid;
-      float dg[kD], b[kD];
+      const int32_t k = s.code[gl][tid];
+      float dg[kD], ck[kD], b[kD];
 #pragma unroll
-      for (int j = 0; j < kD; ++j) dg[j] = sDD[tid][j];
+      for (int j = 0; j < kD; ++j) ck[j] = 0.f;
+      if (code_ok(k, cw.K, err)) load_vec(C + (int64_t)k * kD, ck);
+#pragma unroll
+      for (int j = 0; j < kD; ++j) {
+        const float2 r = s.R[gl][tid][j];
+        dg[j] = pair_minus(r.x, r.y, ck[j]);
+        s.DD[tid][j] = dg[j];
+      }
 #pragma unroll
       for (int q = 0; q < kD; ++q) {
         float hd = 0.f;
 #pragma unroll
-        for (int c = 0; c < kD; ++c) hd = fmaf(sH[q * kD + c], dg[c], hd);
-        b[q] = sB[tid * kCplPad + col0 + q] - hd;
+        for (int m = 0; m < kD; ++m) hd = fmaf(sH[q * kD + m], dg[m], hd);
+        b[q] = s.B[tid * kCplPad + col0 + q] - hd;
       }
-      // H_gg s = b: L y = b, L^T s = y
+      // H_gg x = b: L y = b, L^T x = y
       float y[kD], sv[kD];
 #pragma unroll
       for (int r = 0; r < kD; ++r) {
@@ -217,49 +302,44 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
         for (int m = r + 1; m < kD; ++m) acc = fmaf(-sL[m * kD + r], sv[m], acc);
         sv[r] = acc * sInv[r];
       }
-      const int32_t k = cw.codes[i * cw.ld + g];
-      const bool kok = code_ok(k, cw.K, err);
-      float c[kD];
 #pragma unroll
-      for (int j = 0; j < kD; ++j) c[j] = 0.f;
-      if (kok) load_vec(cw.C + (int64_t)k * kD, c);
-#pragma unroll
-      for (int j = 0; j < kD; ++j) sT[tid][j] = (dg[j] + c[j]) + sv[j];
-      sCode[tid] = k;
+      for (int j = 0; j < kD; ++j) s.T[tid][j] = (dg[j] + ck[j]) + sv[j];
     }
     __syncthreads();
-    if (row8 < kCplRows) {  // -2 H t' and Pmax, a thread per component
+    {  // -2 H t' and Pmax, a thread per component
       float q = 0.f, pa = 0.f;
       if (row8 < nr)
 #pragma unroll
         for (int j = 0; j < kD; ++j) {
-          q = fmaf(sH[j8 * kD + j], sT[row8][j], q);
-          pa = fmaf(fabsf(sH[j8 * kD + j]), fabsf(sT[row8][j]), pa);
+          q = fmaf(sH[j8 * kD + j], s.T[row8][j], q);
+          pa = fmaf(fabsf(sH[j8 * kD + j]), fabsf(s.T[row8][j]), pa);
         }
 #pragma unroll
       for (int off = 4; off > 0; off >>= 1)
         pa = fmaxf(pa, __shfl_xor_sync(0xffffffffu, pa, off));
-      sQ[row8][j8] = -2.f * q;
-      if (j8 == 0) sPmax[row8] = pa;
+      s.Q[row8][j8] = -2.f * q;
+      if (j8 == 0) s.beta[row8] = -2.f * kU * cmul * pa;
     }
     __syncthreads();
     // 2. scores, 256 codewords at a time; each warp keeps its two smallest per row
     for (int k0 = 0; k0 < cw.K; k0 += kCplThreads) {
       const int k = k0 + tid;
-      float c[kD], n = 0.f, na = 0.f, l1 = 0.f;
+      if (k0 > 0) {
 #pragma unroll
-      for (int j = 0; j < kD; ++j) c[j] = 0.f;
-      if (k < cw.K) {
-        load_vec(cw.C + (int64_t)k * kD, c);
-        codeword_terms(c, sH, n, na, l1);
+        for (int j = 0; j < kD; ++j) c[j] = 0.f;
+        n = na = l1 = 0.f;
+        if (k < cw.K) {
+          load_vec(cw.C + (int64_t)k * kD, c);
+          codeword_terms(c, sH, n, na, l1);
+        }
       }
-      const float nlow = fmaf(-kU * cmul, na, n);
+      const float nlow = k < cw.K ? fmaf(-kU * cmul, na, n) : __int_as_float(0x7fffffff);
 #pragma unroll 4
       for (int r = 0; r < nr; ++r) {
-        const float4 q0 = *reinterpret_cast<const float4*>(&sQ[r][0]);
-        const float4 q1 = *reinterpret_cast<const float4*>(&sQ[r][4]);
-        const float pmax = sPmax[r];
-        float sc = nlow;
+        const float4 q0 = *reinterpret_cast<const float4*>(&s.Q[r][0]);
+        const float4 q1 = *reinterpret_cast<const float4*>(&s.Q[r][4]);
+        const float beta = s.beta[r];
+        float sc = nlow;  // (NaN past the codebook: the largest key)
         sc = fmaf(q0.x, c[0], sc);
         sc = fmaf(q0.y, c[1], sc);
         sc = fmaf(q0.z, c[2], sc);
@@ -268,138 +348,126 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
         sc = fmaf(q1.y, c[5], sc);
         sc = fmaf(q1.z, c[6], sc);
         sc = fmaf(q1.w, c[7], sc);
-        sc = fmaf(-2.f * kU * cmul * pmax, l1, sc);
-        const uint32_t key = k < cw.K ? order_key(sc) : 0xffffffffu;
+        sc = fmaf(beta, l1, sc);
+        const uint32_t key = order_key(sc);
         const uint32_t m1 = __reduce_min_sync(0xffffffffu, key);
         const int src = __ffs(__ballot_sync(0xffffffffu, key == m1)) - 1;
         const uint32_t m2 = __reduce_min_sync(0xffffffffu, lane == src ? 0xffffffffu : key);
-        if (lane == src) {
-          const float e2 = 2.f * kU * cmul * (na + 2.f * pmax * l1);
-          if (k0 == 0) {
-            sV1[r][warp] = m1;
-            sV2[r][warp] = m2;
-            sK1[r][warp] = k;
-            sE1[r][warp] = e2;
-          } else {  // (the warp's earlier chunks; strictly below: ties keep the smaller index)
-            const uint32_t v1 = sV1[r][warp];
-            if (m1 < v1) {
-              sV2[r][warp] = min(v1, m2);
-              sV1[r][warp] = m1;
-              sK1[r][warp] = k;
-              sE1[r][warp] = e2;
-            } else {
-              sV2[r][warp] = min(sV2[r][warp], m1);
-            }
+        CplBest b{m1, m2, k, 2.f * kU * cmul * na - 2.f * beta * l1};
+        if (k0 > 0) {  // with the warp's earlier chunks; strictly below: ties keep the smaller index
+          const CplBest o = s.best[r][warp];
+          if (m1 < o.v1) {
+            b.v2 = min(o.v1, m2);
+          } else {
+            b = o;
+            b.v2 = min(o.v2, m1);
           }
         }
+        __syncwarp();
+        if (lane == src) s.best[r][warp] = b;
+        if (k0 + kCplThreads < cw.K) __syncwarp();
       }
-      __syncwarp();
     }
     __syncthreads();
     // 3. the row's smallest over its eight lanes (warps' entries), certificate
-    if (row8 < kCplRows) {
-      uint32_t v1 = 0xffffffffu, v2 = 0xffffffffu;
-      int k1 = 0;
-      float e2 = 0.f;
-      if (row8 < nr) {
-        v1 = sV1[row8][j8];
-        v2 = sV2[row8][j8];
-        k1 = sK1[row8][j8];
-        e2 = sE1[row8][j8];
-      }
+    {
+      CplBest b{0xffffffffu, 0xffffffffu, 0, 0.f};
+      if (row8 < nr) b = s.best[row8][j8];
 #pragma unroll
       for (int off = 4; off > 0; off >>= 1) {
-        const uint32_t o1 = __shfl_xor_sync(0xffffffffu, v1, off);
-        const uint32_t o2 = __shfl_xor_sync(0xffffffffu, v2, off);
-        const int ok = __shfl_xor_sync(0xffffffffu, k1, off);
-        const float oe = __shfl_xor_sync(0xffffffffu, e2, off);
-        const bool take = o1 < v1 || (o1 == v1 && ok < k1);
-        v2 = min(min(v2, o2), max(v1, o1));
-        if (take) {
-          v1 = o1;
-          k1 = ok;
-          e2 = oe;
-        }
+        CplBest o;
+        o.v1 = __shfl_xor_sync(0xffffffffu, b.v1, off);
+        o.v2 = __shfl_xor_sync(0xffffffffu, b.v2, off);
+        o.k1 = __shfl_xor_sync(0xffffffffu, b.k1, off);
+        o.e2 = __shfl_xor_sync(0xffffffffu, b.e2, off);
+        const bool take = o.v1 < b.v1 || (o.v1 == b.v1 && o.k1 < b.k1);
+        const uint32_t v2 = min(min(b.v2, o.v2), max(b.v1, o.v1));
+        if (take) b = o;
+        b.v2 = v2;
       }
       if (j8 == 0 && row8 < nr && factor) {
-        const float low1 = order_val(v1);
-        const bool cert = cw.K == 1 || (v1 != 0xffffffffu && order_val(v2) - low1 > e2) ||
-                          (v1 != 0xffffffffu && v2 == 0xffffffffu && isfinite(e2));
+        const float low1 = order_val(b.v1);
+        const bool cert = cw.K == 1 || (b.v1 != 0xffffffffu && order_val(b.v2) - low1 > b.e2) ||
+                          (b.v1 != 0xffffffffu && b.v2 == 0xffffffffu && isfinite(b.e2));
         if (cert) {
-          sCode[row8] = k1;
+          s.code[gl][row8] = b.k1;
         } else {
-          sThr[row8] = v1 != 0xffffffffu ? __fadd_ru(low1, e2) : INFINITY;
-          sOpen[atomicAdd(&n_open, 1)] = row8;
+          s.thr[row8] = b.v1 != 0xffffffffu ? __fadd_ru(low1, b.e2) : INFINITY;
+          s.open[atomicAdd(&s.n_open, 1)] = row8;
         }
       }
     }
     __syncthreads();
-    for (int q = warp; q < n_open; q += kCplThreads / 32) {  // exact decisions, a warp per row
-      const int r = sOpen[q];
-      const float thr = sThr[r];
-      float t[kD], zero[kD], m2q[kD];
+    if (s.n_open > 0) {  // exact decisions, a warp per row
+      for (int q = warp; q < s.n_open; q += kCplThreads / 32) {
+        const int r = s.open[q];
+        const float thr = s.thr[r], nbeta = s.beta[r];
+        float t[kD], zero[kD], m2q[kD];
 #pragma unroll
-      for (int j = 0; j < kD; ++j) {
-        t[j] = sT[r][j];
-        zero[j] = 0.f;
-        m2q[j] = sQ[r][j];
-      }
-      const float nbeta = -2.f * kU * cmul * sPmax[r];
-      float bh = INFINITY, bl = 0.f;
-      int bk = 0x7fffffff;
-      for (int k = lane; k < cw.K; k += 32) {
-        float c[kD], n, na, l1;
-        load_vec(cw.C + (int64_t)k * kD, c);
-        codeword_terms(c, sH, n, na, l1);
-        if (low_from(n, na, l1, c, m2q, nbeta, cmul) <= thr) {
-          float eh, el;
-          dfl::quad_err(t, zero, c, sH, eh, el);
-          if (dfl::less(eh, el, k, bh, bl, bk)) {
-            bh = eh;
-            bl = el;
-            bk = k;
+        for (int j = 0; j < kD; ++j) {
+          t[j] = s.T[r][j];
+          zero[j] = 0.f;
+          m2q[j] = s.Q[r][j];
+        }
+        float bh = INFINITY, bl = 0.f;
+        int bk = 0x7fffffff;
+        for (int k = lane; k < cw.K; k += 32) {
+          float cv[kD], kn, kna, kl1;
+          load_vec(C + (int64_t)k * kD, cv);
+          codeword_terms(cv, sH, kn, kna, kl1);
+          if (low_from(kn, kna, kl1, cv, m2q, nbeta, cmul) <= thr) {
+            float eh, el;
+            dfl::quad_err(t, zero, cv, sH, eh, el);
+            if (dfl::less(eh, el, k, bh, bl, bk)) {
+              bh = eh;
+              bl = el;
+              bk = k;
+            }
           }
         }
-      }
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float oh = __shfl_xor_sync(0xffffffffu, bh, off);
-        const float ol = __shfl_xor_sync(0xffffffffu, bl, off);
-        const int ok = __shfl_xor_sync(0xffffffffu, bk, off);
-        if (dfl::less(oh, ol, ok, bh, bl, bk)) {
-          bh = oh;
-          bl = ol;
-          bk = ok;
+        for (int off = 16; off > 0; off >>= 1) {
+          const float oh = __shfl_xor_sync(0xffffffffu, bh, off);
+          const float ol = __shfl_xor_sync(0xffffffffu, bl, off);
+          const int ok = __shfl_xor_sync(0xffffffffu, bk, off);
+          if (dfl::less(oh, ol, ok, bh, bl, bk)) {
+            bh = oh;
+            bl = ol;
+            bk = ok;
+          }
+        }
+        if (lane == 0) {
+          if (bk == 0x7fffffff)
+            raise_error(err, ERRBIT_NUMERIC);  // no candidate: non-finite scores (the code stays)
+          else
+            s.code[gl][r] = bk;
         }
       }
-      if (lane == 0) {
-        if (bk == 0x7fffffff)
-          raise_error(err, ERRBIT_NUMERIC);  // no candidate: non-finite scores (the code stays)
-        else
-          sCode[r] = bk;
-      }
+      __syncthreads();
+      if (tid == 0) s.n_open = 0;
     }
-    __syncthreads();
-    // 4. the decision: code, D_g from W, the change of D_g
-    if (tid < nr && factor) {
+    // 4. the decision: code, D_g and its operand images, the change of D_g
+    if (tid < nr) {
       const int64_t i = i0 + tid;
-      const int32_t kn = sCode[tid];
-      if (code_ok(kn, cw.K, err)) {
+      const int32_t kn = s.code[gl][tid];
+      if (factor && code_ok(kn, cw.K, err)) {
         cw.codes[i * cw.ld + g] = kn;
-        float rh[kD], rl[kD];
-        dfl::target(wset, a.cbs, a.cbs.n, i, g, rh, rl, err);  // (reads the code just written)
-        float* d = a.D + i * a.N + g * kD;
+        float ck[kD], nv[kD];
+        load_vec(C + (int64_t)kn * kD, ck);
         uint32_t hi[kD], lo[kD];
 #pragma unroll
         for (int j = 0; j < kD; ++j) {
-          const float nv = __fadd_rn(rh[j], rl[j]);
-          d[j] = nv;
-          sDD[tid][j] = nv - sDD[tid][j];
-          hi[j] = tc::to_tf32(nv);
-          lo[j] = tc::to_tf32(nv - __uint_as_float(hi[j]));
+          const float2 r = s.R[gl][tid][j];
+          nv[j] = pair_minus(r.x, r.y, ck[j]);
+          s.DD[tid][j] = nv[j] - s.DD[tid][j];
+          hi[j] = tc::to_tf32(nv[j]);
+          lo[j] = tc::to_tf32(nv[j] - __uint_as_float(hi[j]));
         }
+        float* d = a.D + i * a.N + g * kD;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
+          *reinterpret_cast<float4*>(d + 4 * q) =
+              make_float4(nv[4 * q], nv[4 * q + 1], nv[4 * q + 2], nv[4 * q + 3]);
           const int64_t off = img::img_off(i, g * kD + 4 * q, a.nslab);
           *reinterpret_cast<uint4*>(a.d_hi + off) =
               make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
@@ -408,16 +476,16 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < kD; ++j) sDD[tid][j] = 0.f;
+        for (int j = 0; j < kD; ++j) s.DD[tid][j] = 0.f;
       }
     }
     __syncthreads();
-    if (factor && col >= col0 + kD && col < ncol) {
+    if (col >= col0 + kD && col < ncol) {
 #pragma unroll 4
       for (int r = 0; r < nr; ++r) {
-        const float4 d0 = *reinterpret_cast<const float4*>(&sDD[r][0]);
-        const float4 d1 = *reinterpret_cast<const float4*>(&sDD[r][4]);
-        float acc = sB[r * kCplPad + col];
+        const float4 d0 = *reinterpret_cast<const float4*>(&s.DD[r][0]);
+        const float4 d1 = *reinterpret_cast<const float4*>(&s.DD[r][4]);
+        float acc = s.B[r * kCplPad + col];
         acc = fmaf(d0.x, hcol[0], acc);
         acc = fmaf(d0.y, hcol[1], acc);
         acc = fmaf(d0.z, hcol[2], acc);
@@ -426,7 +494,7 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
         acc = fmaf(d1.y, hcol[5], acc);
         acc = fmaf(d1.z, hcol[6], acc);
         acc = fmaf(d1.w, hcol[7], acc);
-        sB[r * kCplPad + col] = acc;
+        s.B[r * kCplPad + col] = acc;
       }
     }
     __syncthreads();
@@ -480,7 +548,7 @@ crvq_status launch_coupled_sweep(const float* W, int64_t M, int64_t N, const flo
   {
     ProfScope ps("coupled_residual", stream, (double)M * N * 8.0);
     residual_kernel<<<(unsigned)std::min<int64_t>(ceil_div(M * (N / kD), 256), 16 * nsm), 256, 0,
-                      stream>>>(W, M, N, cbs, D, err);
+                      stream>>>(W, M, N, cbs, which, D, err);
     CRVQ_LAUNCHED();
     block_factor_kernel<<<(unsigned)ceil_div(std::max<int64_t>(G_cov, 1), 128), 128, 0,
                           stream>>>(H, N, G_cov, Hb, Lf, Linv, err);
@@ -508,7 +576,8 @@ crvq_status launch_coupled_sweep(const float* W, int64_t M, int64_t N, const flo
       const CplArgs ca{W, D, H, Hb, Lf, Linv, mB.as<float>(), (int)chunks, d_hi, d_lo,
                        ceil_div(N, (int64_t)img::kSlabK), M, N, b0, b1, rows, which, cbs};
       ProfScope ps("coupled_block", stream, (double)M * (b1 - b0) * cw.K);
-      coupled_block_kernel<<<(unsigned)ceil_div(M, rows), kCplThreads, 0, stream>>>(ca, err);
+      CRVQ_TRY(smem_limit((const void*)coupled_block_kernel, kCplSmem));
+      coupled_block_kernel<<<(unsigned)ceil_div(M, rows), kCplThreads, kCplSmem, stream>>>(ca, err);
       CRVQ_LAUNCHED();
     }
     if (loss_dev) CRVQ_TRY(loss_into(loss_dev + 1 + sw));

@@ -317,6 +317,12 @@ __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
 #pragma unroll 1
       for (int c0 = 0; c0 < 256; c0 += 32) {
         uint32_t v[32], w[32];
+        float e[EPI == kDot ? 32 : 1];  // E's entries of this lane's column, all in flight at once
+        if (EPI == kDot && last) {
+          const int64_t n = min((int64_t)bn * 256 + c0 + lane, a.rows_n - 1);
+#pragma unroll
+          for (int r = 0; r < 32; ++r) e[r & (EPI == kDot ? 31 : 0)] = __ldg(a.E + min(m0 + r, a.rows_m - 1) * a.ldc + n);
+        }
         tc::tmem_ld32_nowait(tmem + lane_base + (uint32_t)c0, v);
         tc::tmem_wait_ld_dep(v);
         if (c > 0) {
@@ -341,20 +347,20 @@ __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
             if (EPI == kSymmetric && a.diag && n0 + j == m && m < a.rows_m) a.diag[m] = x;
           }
           __syncwarp();
-          if (n < a.rows_n) {
+          if (EPI == kDot) {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) {  // (operand padding makes x zero past the rows of A and B)
+              const float x = so[r * 33 + lane], er = e[r & (EPI == kDot ? 31 : 0)];
+              const float p = __fmul_rn(x, er);
+              pair_acc(sq, sl, p);
+              sl = __fadd_rn(sl, __fmaf_rn(x, er, -p));
+            }
+          } else if (n < a.rows_n) {
 #pragma unroll 8
             for (int r = 0; r < 32; ++r) {
               const int64_t mr = m0 + r;
               if (mr >= a.rows_m) break;
-              const float x = so[r * 33 + lane];
-              if (EPI == kDot) {
-                const float e = __ldg(a.E + mr * a.ldc + n);
-                const float p = __fmul_rn(x, e);
-                pair_acc(sq, sl, p);
-                sl = __fadd_rn(sl, __fmaf_rn(x, e, -p));
-              } else if (EPI == kPlain || n >= mr) {
-                C[mr * a.ldc + n] = x;
-              }
+              if (EPI == kPlain || n >= mr) C[mr * a.ldc + n] = so[r * 33 + lane];
             }
           }
           __syncwarp();

@@ -273,36 +273,46 @@ __device__ void cbmax_block(const float* __restrict__ C, int K, float* __restric
 constexpr int kTcCols = 128;                     // codewords per chunk (MMA N)
 constexpr int kTcBTile = kTcCols * tcenc::kK * 4;  // 16 KB
 
-// B operand images of the codebook for groups [g_begin, g_begin + G_range): block
-// (g, chunk) holds 128 rows in the canonical shared-memory layout, ready for a bulk copy.
-// terms[(g - g_begin) K + k] = (n, Na, L1, 0) of codeword k in group g (codeword_terms).
+// B operand images of the codebook for the groups g_begin + blockIdx.y: block (g, chunk) holds 128
+// rows in the canonical shared-memory layout, ready for a bulk copy. terms[g_rel K + k] = (n, Na, L1, 0)
+// of codeword k in the group (codeword_terms). A CTA stays in its group, whose H block it reads once.
 __global__ void __launch_bounds__(128)
-prep_b_kernel(SetView set, int64_t g_begin, int64_t G_range, const float* __restrict__ C,
-              int K, int nchunk, float uc, char* __restrict__ out, float4* __restrict__ terms,
-              float* __restrict__ cbmax, unsigned* __restrict__ flag_count) {
+prep_b_kernel(SetView set, int64_t g_begin, const float* __restrict__ C, int K, int nchunk, float uc,
+              char* __restrict__ out, float4* __restrict__ terms, float* __restrict__ cbmax,
+              unsigned* __restrict__ flag_count) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
   // The open lists of the arg-min pass that follows start empty. The previous pass's exact
   // kernels, which read the counts, completed before the wait above returned.
-  if (blockIdx.x == 0 && threadIdx.x < 2) flag_count[threadIdx.x] = 0u;
-  if (blockIdx.x == gridDim.x - 1) {  // the last CTA: the codebook maxima
-    cbmax_block(C, K, cbmax);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) flag_count[threadIdx.x] = 0u;
+  if (blockIdx.x == gridDim.x - 1) {  // the last column of CTAs: the codebook maxima (its first)
+    if (blockIdx.y == 0) cbmax_block(C, K, cbmax);
     return;
   }
-  const int64_t total = G_range * nchunk * (int64_t)kTcCols;
-  const int64_t nth = (int64_t)(gridDim.x - 1) * blockDim.x;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += nth) {
-    const int row = (int)(e % kTcCols);
-    const int64_t blk = e / kTcCols;  // g_rel * nchunk + chunk
-    const int chunk = (int)(blk % nchunk);
-    const int64_t g = g_begin + blk / nchunk;
-    uint32_t v[tcenc::kK];
-    const int kk = chunk * kTcCols + row;
-    float tk[3];
-    build_b_row(C, K, kk, set.Hb + g * kD * kD, uc, v, tk);
-    tcenc::put_row(out + blk * kTcBTile, row, v);
-    if (kk < K) terms[(g - g_begin) * K + kk] = make_float4(tk[0], tk[1], tk[2], 0.f);
+  const int64_t g = g_begin + blockIdx.y;
+  float H[kD * kD];
+#pragma unroll
+  for (int e = 0; e < kD * kD; e += 4) {
+    const float4 h = __ldg(reinterpret_cast<const float4*>(set.Hb + g * kD * kD + e));
+    H[e] = h.x;
+    H[e + 1] = h.y;
+    H[e + 2] = h.z;
+    H[e + 3] = h.w;
   }
+  for (int chunk = blockIdx.x; chunk < nchunk; chunk += gridDim.x - 1) {
+    const int kk = chunk * kTcCols + threadIdx.x;
+    uint32_t v[tcenc::kK];
+    float tk[3];
+    build_b_row(C, K, kk, H, uc, v, tk);
+    tcenc::put_row(out + ((int64_t)blockIdx.y * nchunk + chunk) * kTcBTile, threadIdx.x, v);
+    if (kk < K) terms[(int64_t)blockIdx.y * K + kk] = make_float4(tk[0], tk[1], tk[2], 0.f);
+  }
+}
+
+// Grid of prep_b_kernel: about 16 CTAs per SM in all, and the column that takes the maxima.
+dim3 prep_b_grid(int64_t G_range, int nchunk, int nsm) {
+  const int64_t x = std::max<int64_t>(1, std::min<int64_t>(nchunk, ceil_div(16 * (int64_t)nsm, G_range)));
+  return dim3((unsigned)x + 1, (unsigned)G_range);
 }
 
 // Per-vector terms of the arg-min's A rows that do not change while one codebook's Lloyd
@@ -873,8 +883,11 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
 // --------------------------------------------------------------------------- arg-min pass,
 // codebooks of more than 256 codewords: a CTA walks `tiles` consecutive row tiles of one group
 // (thread = row = tensor-memory lane), streaming the codebook's precomputed B images in chunks of 128
-// codewords by bulk copy through four buffers. Two 128-column accumulators: the MMA of the next chunk
-// runs while the threads sweep this one, one block barrier per chunk. 128 threads, two CTAs per SM.
+// codewords by bulk copy. Two halves of 128 threads share the tile's A rows and take alternate chunks,
+// each with its own accumulator, two chunk buffers, barriers and MMA issue; half 1 hands its minima to
+// half 0 at the tile's end. Two CTAs per SM: four pipelines of four warps whose waits (copy, MMA,
+// accumulator loads) overlap. (128 threads with two accumulators, so eight warps per SM, took 0.95 us
+// per chunk: one warp per scheduler and CTA cannot hide its own load and dependence latency.)
 //
 // Sweep, as in argmin_small_kernel but over 32-column granules and 32 classes (column % 32): a
 // granule's minimum and the class minima, 0.5 + 0.5 instructions per score, and the three smallest
@@ -897,12 +910,13 @@ struct NarrowList {
 };
 
 constexpr int kGran = 32;      // columns per granule
-constexpr int kBRing = 4;      // B chunk buffers
+constexpr int kBRing = 2;      // B chunk buffers of a half
 
-constexpr size_t kArgminStreamSmem = (size_t)tcenc::kATile + kBRing * (size_t)kTcBTile +
-                                     (size_t)tcenc::kRows * kD * 4 + 1024;
+constexpr int kHandWords = 5 + kGran;  // half 1's minima of a row
+constexpr size_t kArgminStreamSmem = (size_t)tcenc::kATile + 2 * kBRing * (size_t)kTcBTile +
+                                     (size_t)tcenc::kRows * (kD + kHandWords) * 4 + 1024;
 
-__global__ void __launch_bounds__(128, 2)
+__global__ void __launch_bounds__(256, 2)
 argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_idx,
                  int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
                  FlagList wide, NarrowList narrow, StatsView st, const float* __restrict__ cbmax,
@@ -915,15 +929,18 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   // 1024-byte aligned base, derived from the shared array (keeps the shared address space)
   char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
   char* Atile = smem;                     // 16 KB
-  char* Bbuf = smem + kATile;             // kBRing x 16 KB
-  float* sQ = reinterpret_cast<float*>(Bbuf + kBRing * kTcBTile);  // [128][8]: H r of a row
+  const int tid = threadIdx.x, warp = tid >> 5, half = tid >> 7, rrow = tid & (kRows - 1);
+  char* Bbuf = smem + kATile + half * kBRing * kTcBTile;  // this half's kBRing x 16 KB
+  float* sQ = reinterpret_cast<float*>(smem + kATile + 2 * kBRing * kTcBTile);  // [128][8]: H r
+  uint32_t* hand = reinterpret_cast<uint32_t*>(sQ + kRows * kD);  // [kHandWords][128]
   __shared__ __align__(16) float sH[kD * kD];
-  __shared__ __align__(8) uint64_t bar_mma[2], bar_b[kBRing];
+  __shared__ __align__(8) uint64_t bar_mma_s[2], bar_b_s[2][kBRing];
   __shared__ uint32_t tmem_slot;
+  uint64_t& bar_mma = bar_mma_s[half];
+  uint64_t* bar_b = bar_b_s[half];
 
   const int64_t g = g_begin + blockIdx.y;
   const int64_t G_range = gridDim.y;
-  const int tid = threadIdx.x, warp = tid >> 5;
   const CbView cw = cbs.cb[s_idx];
   const float cmul = kCmul + 4.f * n_fixed;
   const float uc = kU * cmul;
@@ -934,15 +951,17 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   if (tid < kD * kD) sH[tid] = set.Hb[g * kD * kD + tid];
   if (warp == 0) tc::tmem_alloc(&tmem_slot, 2 * kTcCols);
   if (tid == 0) {
-    for (int b = 0; b < 2; ++b) tc::mbar_init(tc::smem_u32(&bar_mma[b]), 1);
-    for (int b = 0; b < kBRing; ++b) tc::mbar_init(tc::smem_u32(&bar_b[b]), 1);
+    for (int h = 0; h < 2; ++h) {
+      tc::mbar_init(tc::smem_u32(&bar_mma_s[h]), 1);
+      for (int b = 0; b < kBRing; ++b) tc::mbar_init(tc::smem_u32(&bar_b_s[h][b]), 1);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
-  const uint32_t tmem = tmem_slot;
-  const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+  const uint32_t tmem = tmem_slot + (uint32_t)(half * kTcCols);  // this half's accumulator
+  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
   const float sscale = st.cnt ? stats_scale_f(st) : 1.f;
 
   // Bound on Na_k over the codebook for this group: (max row sum |H_g|) L1max cinfmax.
@@ -960,49 +979,49 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   // this CTA's row tiles (the last CTA of a column may have fewer)
   const int64_t row_tiles = (set.M + kRows - 1) / kRows;
   const int steps = (int)min((int64_t)tiles, row_tiles - (int64_t)blockIdx.x * tiles);
-  // Chunk uses are numbered u = t * nchunk + c. Use u reads buffer u % kBRing; thread 0 fetches,
-  // waits for and multiplies them in order (fetched: uses whose copy has started, issued: uses
-  // whose MMA has).
-  const int64_t n_uses = (int64_t)steps * nchunk;
+  // A half's chunk uses are numbered over its tiles: use u is its chunk u % nch, codebook chunk
+  // 2 (u % nch) + half, in buffer u % kBRing. The half's thread 0 fetches, waits for and multiplies
+  // them in order (fetched: uses whose copy has started, issued: uses whose MMA has).
+  const int nch = (nchunk + 1 - half) >> 1;
+  const int64_t n_uses = (int64_t)steps * nch;
   int64_t fetched = 0, issued = 0;
-  auto fetch = [&]() {  // thread 0: the next chunk, into the buffer of the use kBRing before it
+  auto fetch = [&]() {  // the next chunk, into the buffer of the use kBRing before it
     const int b = (int)(fetched % kBRing);
     tc::mbar_expect_tx(tc::smem_u32(&bar_b[b]), kTcBTile);
     tc::bulk_copy_g2s(tc::smem_u32(Bbuf + b * kTcBTile),
-                      bimg + (size_t)(fetched % nchunk) * kTcBTile, kTcBTile,
+                      bimg + (size_t)(2 * (fetched % nch) + half) * kTcBTile, kTcBTile,
                       tc::smem_u32(&bar_b[b]));
     ++fetched;
   };
-  // Thread 0: the next use's MMA into accumulator `acc`. After a timeout its waiters are released
-  // and the caller's ok turns false.
-  auto issue = [&](int acc) -> bool {
+  // The next use's MMA. After a timeout its waiters are released and the caller's ok turns false.
+  auto issue = [&]() -> bool {
     const int b = (int)(issued % kBRing);
     const bool ready = tc::mbar_wait(tc::smem_u32(&bar_b[b]), (uint32_t)((issued / kBRing) & 1), err);
     ++issued;
     if (!ready) {
-      tc::mbar_arrive(tc::smem_u32(&bar_mma[acc]));
+      tc::mbar_arrive(tc::smem_u32(&bar_mma));
       return false;
     }
     tc::tc_fence_after();
     const uint32_t a0 = tc::smem_u32(Atile), b0 = tc::smem_u32(Bbuf + b * kTcBTile);
 #pragma unroll
     for (int ks = 0; ks < kK / 8; ++ks)
-      tc::mma_tf32(tmem + (uint32_t)(acc * kTcCols), tc::smem_desc(a0 + ks * 256, 128, (kK / 4) * 128),
+      tc::mma_tf32(tmem, tc::smem_desc(a0 + ks * 256, 128, (kK / 4) * 128),
                    tc::smem_desc(b0 + ks * 256, 128, (kK / 4) * 128), idesc, ks > 0 ? 1u : 0u);
-    tc::mma_commit(tc::smem_u32(&bar_mma[acc]));
+    tc::mma_commit(tc::smem_u32(&bar_mma));
     return true;
   };
-  if (tid == 0)
+  if (rrow == 0)
     while (fetched < min((int64_t)kBRing, n_uses)) fetch();
   bool ok = true;
-  uint32_t mpar = 0;  // parity of the next wait per accumulator (bit = accumulator)
+  uint32_t mpar = 0;  // parity of the next MMA wait
 
   for (int t = 0; t < steps && ok; ++t) {
-    const int64_t i = ((int64_t)blockIdx.x * tiles + t) * kRows + tid;
+    const int64_t i = ((int64_t)blockIdx.x * tiles + t) * kRows + rrow;
     const bool row_ok = i < set.M;
-    // Prologue: this thread's A row.
-    float pmax, off;
-    {
+    // Prologue: the A rows, by half 0 (which also takes the rows' decisions).
+    float pmax = 0.f, off = 0.f;
+    if (half == 0) {
       float m2q[kD], rr, ra;
       if (rowterms) {  // precomputed for this Lloyd loop (row_terms_kernel)
         float4 q0 = make_float4(0.f, 0.f, 0.f, 0.f), q1 = q0, t2 = q0;
@@ -1031,9 +1050,9 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
                 (1.f + 4.f * uc) + 1e-30f;
       const float beta = -2.f * uc * pmax;
       if (st.cnt) {  // H r of this row, kept for the statistics (-m2q / 2, exact)
-        *reinterpret_cast<float4*>(sQ + tid * kD) =
+        *reinterpret_cast<float4*>(sQ + rrow * kD) =
             make_float4(-0.5f * m2q[0], -0.5f * m2q[1], -0.5f * m2q[2], -0.5f * m2q[3]);
-        *reinterpret_cast<float4*>(sQ + tid * kD + 4) =
+        *reinterpret_cast<float4*>(sQ + rrow * kD + 4) =
             make_float4(-0.5f * m2q[4], -0.5f * m2q[5], -0.5f * m2q[6], -0.5f * m2q[7]);
       }
       uint32_t row[kK];
@@ -1052,14 +1071,11 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
       row[27] = row[26];
       split(off * (1.f - uc), row[29], row[30]);
       row[31] = 0u;
-      put_row(Atile, tid, row);
+      put_row(Atile, rrow, row);
+      tc::fence_async_smem();
     }
-    tc::fence_async_smem();
     __syncthreads();
-    if (tid == 0) {
-      ok = issue(0);
-      if (ok && nchunk > 1) ok = issue(1);
-    }
+    if (rrow == 0) ok = issue();
 
     // fp32 bits: the three smallest granule minima, the first two's granules; the class minima
     uint32_t v1 = 0xffffffffu, v2 = 0xffffffffu, v3 = 0xffffffffu;
@@ -1067,21 +1083,20 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
     uint32_t mc[kGran];
 #pragma unroll
     for (int e = 0; e < kGran; ++e) mc[e] = 0xffffffffu;
-    for (int c = 0; c < nchunk; ++c) {
-      const int acc = c & 1;
-      const bool done = tc::mbar_wait(tc::smem_u32(&bar_mma[acc]), (mpar >> acc) & 1u, err);
-      mpar ^= 1u << acc;
+    for (int c = 0; c < nch; ++c) {
+      const bool done = tc::mbar_wait(tc::smem_u32(&bar_mma), mpar, err);
+      mpar ^= 1u;
       ok = __all_sync(0xffffffffu, ok && done);
       tc::tc_fence_after();
       if (ok) {
 #pragma unroll
         for (int rnd = 0; rnd < 2; ++rnd) {
           uint32_t v[64];
-          tc::tmem_ld64_wait(trow + (uint32_t)(acc * kTcCols + 64 * rnd), v);
+          tc::tmem_ld64_wait(trow + (uint32_t)(64 * rnd), v);
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             const uint32_t m = min(min16_bits(v + kGran * q), min16_bits(v + kGran * q + 16));
-            const int gr = c * (kTcCols / kGran) + 2 * rnd + q;
+            const int gr = (2 * c + half) * (kTcCols / kGran) + 2 * rnd + q;
             const bool lt1 = m < v1, lt2 = m < v2;
             v3 = min(v3, max(v2, m));
             b2 = lt1 ? b1 : (lt2 ? gr : b2);
@@ -1095,15 +1110,41 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
       }
       tc::tc_fence_before();
       // the accumulator has been read and its MMA is done with its buffer
-      ok = __syncthreads_and(ok);
+      ok = half_sync_and(half, ok);
       if (!ok) break;
-      if (tid == 0) {
+      if (rrow == 0) {
         if (fetched < n_uses) fetch();
-        if (c + 2 < nchunk) ok = issue(acc);
+        if (c + 1 < nch) ok = issue();
       }
+    }
+    if (half == 1 && ok) {
+      hand[0 * kRows + rrow] = v1;
+      hand[1 * kRows + rrow] = v2;
+      hand[2 * kRows + rrow] = v3;
+      hand[3 * kRows + rrow] = (uint32_t)b1;
+      hand[4 * kRows + rrow] = (uint32_t)b2;
+#pragma unroll
+      for (int e = 0; e < kGran; ++e) hand[(5 + e) * kRows + rrow] = mc[e];
     }
     ok = __syncthreads_and(ok);
     if (!ok) break;
+    if (half == 1) continue;  // (the next barrier is the next tile's, after its A rows)
+    {  // half 1's granules and classes
+      const uint32_t hv[3] = {hand[rrow], hand[kRows + rrow], hand[2 * kRows + rrow]};
+      const int hb[3] = {(int)hand[3 * kRows + rrow], (int)hand[4 * kRows + rrow], 0};
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const uint32_t m = hv[q];
+        const bool lt1 = m < v1, lt2 = m < v2;
+        v3 = min(v3, max(v2, m));
+        b2 = lt1 ? b1 : (lt2 ? hb[q] : b2);
+        b1 = lt1 ? hb[q] : b1;
+        v2 = min(v2, max(v1, m));
+        v1 = min(v1, m);
+      }
+#pragma unroll
+      for (int e = 0; e < kGran; ++e) mc[e] = min(mc[e], hand[(5 + e) * kRows + rrow]);
+    }
 
     // Certificate, code, open row and statistics of this thread's row.
     if (row_ok) {
@@ -1154,8 +1195,8 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
       if (cert && st.cnt) {
         // H r from the prologue (bit-identical to the standalone update's H tau)
         float q[kD];
-        const float4 q0 = *reinterpret_cast<const float4*>(sQ + tid * kD);
-        const float4 q1 = *reinterpret_cast<const float4*>(sQ + tid * kD + 4);
+        const float4 q0 = *reinterpret_cast<const float4*>(sQ + rrow * kD);
+        const float4 q1 = *reinterpret_cast<const float4*>(sQ + rrow * kD + 4);
         q[0] = q0.x; q[1] = q0.y; q[2] = q0.z; q[3] = q0.w;
         q[4] = q1.x; q[5] = q1.y; q[6] = q1.z; q[7] = q1.w;
         stats_add(st, sscale, g, j, q);
@@ -1163,7 +1204,7 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
     }
   }
   // After a timeout: let copies still in flight into this CTA's shared memory land (bounded).
-  if (tid == 0)
+  if (rrow == 0)
     for (; issued < fetched; ++issued)
       tc::mbar_wait(tc::smem_u32(&bar_b[issued % kBRing]), (uint32_t)((issued / kBRing) & 1), err);
   tc::tc_fence_before();
@@ -1192,24 +1233,28 @@ argmin_narrow_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int 
   }
 }
 
-// Exact decision of rows open over the whole codebook (argmin_tc_kernel's wide list): one CTA per row. The
-// threads stride over the codebook for U = min(fast-pass threshold, smallest fp32 upper
+// Exact decision of rows open over the whole codebook (argmin_tc_kernel's wide list): one CTA per row.
+// The threads stride over the codebook for U = min(fast-pass threshold, smallest fp32 upper
 // bound); every codeword whose fp32 lower bound is at most U is a candidate (the exact
-// arg-min always is) and is re-scored exactly in fp32 pairs (dfl) by one thread; the
-// smallest (err, index) wins. Adds the statistics of the decided code when requested.
-__global__ void __launch_bounds__(128)
+// arg-min always is) and is re-scored exactly in fp32 pairs (dfl) by the thread that holds it; the
+// smallest (err, index) wins. Adds the statistics of the decided code when requested. A launch with a
+// single such row takes as long as its scan: kExactThreads threads with kWideBatch codewords in
+// flight each (128 threads with one took 0.75 ms for 65536 codewords).
+constexpr int kExactThreads = 512;
+constexpr int kWideBatch = 4;  // codewords a thread loads before using them
+
+__global__ void __launch_bounds__(kExactThreads)
 argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, int n_fixed,
                     int s_idx, int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
                     FlagList flags, StatsView st, const float4* __restrict__ terms,
                     unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
+  constexpr int kWarps = kExactThreads / 32;
   __shared__ float sH[kD * kD];
-  __shared__ float redf[4];
-  __shared__ int cand[256];
-  __shared__ int ncand;
-  __shared__ float bh_s[4], bl_s[4];
-  __shared__ int bk_s[4];
+  __shared__ float redf[kWarps];
+  __shared__ float bh_s[kWarps], bl_s[kWarps];
+  __shared__ int bk_s[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned cnt = min((unsigned long long)*flags.count, (unsigned long long)flags.cap);
   if (flags.total && blockIdx.x == 0 && tid == 0) atomicAdd(flags.total, cnt);
@@ -1218,55 +1263,47 @@ argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
   for (unsigned f = blockIdx.x; f < cnt; f += gridDim.x) {
     const int64_t vi = flags.vec[f];
     const int64_t i = vi / G_range, grel = vi % G_range, g = g_begin + grel;
-    const float thr = flags.thr[f];
     __syncthreads();
     if (tid < kD * kD) sH[tid] = set.Hb[g * kD * kD + tid];
-    if (tid == 0) ncand = 0;
     __syncthreads();
     float rv[kD], av[kD], m2q[kD], pmax;
     target32(set, cbs, n_fixed, i, g, rv, av, err);
     vector_terms(rv, av, sH, m2q, pmax);
     const float nbeta = -2.f * kU * cmul * pmax;
-    const float4* gt = terms ? terms + grel * cw.K : nullptr;
-    auto terms_of = [&](int k, const float cv[kD], float& nn, float& na, float& l1) {
-      if (gt) {
-        const float4 t = gt[k];
-        nn = t.x;
-        na = t.y;
-        l1 = t.z;
-      } else {
-        codeword_terms(cv, sH, nn, na, l1);
+    const float4* gt = terms + grel * cw.K;
+    // two passes over the codebook: f(k, codeword, n, Na, L1)
+    auto sweep = [&](auto f) {
+      for (int k0 = tid; k0 < cw.K; k0 += kExactThreads * kWideBatch) {
+        float cv[kWideBatch][kD];
+        float4 tt[kWideBatch];
+#pragma unroll
+        for (int u = 0; u < kWideBatch; ++u) {
+          const int k = min(k0 + u * kExactThreads, cw.K - 1);  // (the last one again past the end)
+          load_vec(cw.C + (int64_t)k * kD, cv[u]);
+          tt[u] = gt[k];
+        }
+#pragma unroll
+        for (int u = 0; u < kWideBatch; ++u)
+          f(min(k0 + u * kExactThreads, cw.K - 1), cv[u], tt[u].x, tt[u].y, tt[u].z);
       }
     };
-    float U = thr;
-    for (int k = tid; k < cw.K; k += blockDim.x) {
-      float cv[kD], nn, na, l1;
-      load_vec(cw.C + (int64_t)k * kD, cv);
-      terms_of(k, cv, nn, na, l1);
+    float U = flags.thr[f];
+    sweep([&](int, const float cv[kD], float nn, float na, float l1) {
       U = fminf(U, up_from(nn, na, l1, cv, m2q, pmax, cmul));
-    }
+    });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) U = fminf(U, __shfl_xor_sync(0xffffffffu, U, o));
     if (lane == 0) redf[warp] = U;
     __syncthreads();
-    U = fminf(fminf(redf[0], redf[1]), fminf(redf[2], redf[3]));
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) U = fminf(U, redf[w]);
     float rh[kD], rl[kD];
     dfl::target(set, cbs, n_fixed, i, g, rh, rl, err);
     float bh = INFINITY, bl = 0.f;
     int bk = 0x7fffffff;
-    for (int k0 = 0; k0 < cw.K; k0 += 256) {
-      for (int k = k0 + tid; k < min(cw.K, k0 + 256); k += blockDim.x) {
-        float cv[kD], nn, na, l1;
-        load_vec(cw.C + (int64_t)k * kD, cv);
-        terms_of(k, cv, nn, na, l1);
-        if (low_from(nn, na, l1, cv, m2q, nbeta, cmul) <= U) cand[atomicAdd(&ncand, 1)] = k;
-      }
-      __syncthreads();
-      const int nc = ncand;
-      for (int q = tid; q < nc; q += blockDim.x) {
-        const int k = cand[q];
-        float cv[kD], eh, el;
-        load_vec(cw.C + (int64_t)k * kD, cv);
+    sweep([&](int k, const float cv[kD], float nn, float na, float l1) {
+      if (low_from(nn, na, l1, cv, m2q, nbeta, cmul) <= U) {
+        float eh, el;
         dfl::quad_err(rh, rl, cv, sH, eh, el);
         if (dfl::less(eh, el, k, bh, bl, bk)) {
           bh = eh;
@@ -1274,10 +1311,7 @@ argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
           bk = k;
         }
       }
-      __syncthreads();
-      if (tid == 0) ncand = 0;
-      __syncthreads();
-    }
+    });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const float oh = __shfl_xor_sync(0xffffffffu, bh, o);
@@ -1296,7 +1330,7 @@ argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
     }
     __syncthreads();
     if (tid == 0) {
-      for (int w = 1; w < 4; ++w)
+      for (int w = 1; w < kWarps; ++w)
         if (dfl::less(bh_s[w], bl_s[w], bk_s[w], bh, bl, bk)) {
           bh = bh_s[w];
           bl = bl_s[w];
@@ -2482,12 +2516,8 @@ crvq_status launch_beam_stage_tc(const SetView& set, int64_t g_begin, int64_t G_
   const float uc = kU * bound_mult(n_fixed + sd.s);
   {
     ProfScope pb("encode_prep_b", stream, (double)G_range * nchunk * kTcCols);
-    const int64_t rows = G_range * nchunk * kTcCols;
-    CRVQ_CUDA(launch_pdl(prep_b_kernel,
-                         dim3((unsigned)std::min<int64_t>(ceil_div(rows, 128), 16 * sm_count()) +
-                              1),
-                         dim3(128), 0, stream, set, g_begin, G_range, cw.C, cw.K, nchunk, uc,
-                         bimg, tout, cbmax, fl.count));
+    CRVQ_CUDA(launch_pdl(prep_b_kernel, prep_b_grid(G_range, nchunk, sm_count()), dim3(128), 0, stream,
+                         set, g_begin, cw.C, cw.K, nchunk, uc, bimg, tout, cbmax, fl.count));
     CRVQ_LAUNCHED();
   }
   // the list length L = Bs + 1, rounded up to an instantiated size
@@ -2604,11 +2634,8 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
     fl.thr = reinterpret_cast<float*>(fl.vec + nv);  // the count is cleared by prep_b
     {
       ProfScope pb("encode_prep_b", stream, (double)gn * nchunk * kTcCols);
-      const int64_t rows = gn * nchunk * kTcCols;
-      CRVQ_CUDA(launch_pdl(prep_b_kernel,
-                           dim3((unsigned)std::min<int64_t>(ceil_div(rows, 128), 16 * nsm) + 1),
-                           dim3(128), 0, stream, set, gs, gn, cw.C, cw.K, nchunk, uc, bimg,
-                           tout, cbmax, fl.count));
+      CRVQ_CUDA(launch_pdl(prep_b_kernel, prep_b_grid(gn, nchunk, nsm), dim3(128), 0, stream, set, gs,
+                           cw.C, cw.K, nchunk, uc, bimg, tout, cbmax, fl.count));
       CRVQ_LAUNCHED();
     }
     {
@@ -2619,7 +2646,7 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
       const dim3 grid((unsigned)ceil_div(row_tiles, tiles), (unsigned)gn);
       ProfScope ps(st.cnt ? "encode_argmin_lloyd" : "encode_argmin", stream,
                    (double)nv * cw.K);
-      CRVQ_CUDA(launch_pdl(argmin_tc_kernel, grid, dim3(128), kArgminStreamSmem, stream, set, gs,
+      CRVQ_CUDA(launch_pdl(argmin_tc_kernel, grid, dim3(256), kArgminStreamSmem, stream, set, gs,
                            cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, nl, st, cbmax, bimg, tout,
                            ex.rowterms, tiles, err));
       CRVQ_LAUNCHED();
@@ -2637,7 +2664,7 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
                              out_ld, out_g0, fl, st, tout, err));
       } else {
         CRVQ_CUDA(launch_pdl(argmin_exact_kernel,
-                             dim3((unsigned)std::min<int64_t>(nv, 16 * nsm)), dim3(128), 0,
+                             dim3((unsigned)std::min<int64_t>(nv, 2 * nsm)), dim3(kExactThreads), 0,
                              stream, set, gs, gn, cbs, n_fixed, s_idx, out, out_ld, out_g0, fl,
                              st, tout, err));
       }

@@ -51,6 +51,17 @@ def test_codebook_and_row_edges(M, G, K):
     _check(W, _blocks(rng, G), C)
 
 
+@pytest.mark.parametrize("K", [15, 16, 17, 129, 200, 241])
+def test_block_and_class_edges(K):
+    """Codebook sizes around the 16-column blocks of the sweep, whose two smallest minima carry their
+    block's number in their low bits; several groups per CTA and an odd number of row tiles."""
+    rng = np.random.default_rng(K)
+    M, G = 385, 260
+    W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
+    C = (0.02 * rng.standard_normal((K, D))).astype(np.float32)
+    _check(W, _blocks(rng, G), C)
+
+
 @pytest.mark.parametrize("K", [64, 256, 600])
 def test_open_rows_more_than_a_list_holds(K):
     """Every codeword twice, the copy one unit in the last place off: no row is certified."""

@@ -1604,130 +1604,162 @@ __device__ __forceinline__ void hyp_terms_pair(const float rh[kD], const float r
   }
 }
 
-// The end of a fast stage for one vector, given its sorted top-L list (topv, topi) of fp32
-// lower bounds low = approx_err - Et built in (h, k) order: bounds of the listed entries, the
-// fast certificate, the fp32-pair exact path, the flag for the fallback, and the kept tuples.
+// The end of a fast stage, given each thread's sorted top-L list (topv, topi) of fp32 lower bounds
+// low = approx_err - Et built in (h, k) order: bounds of the listed entries, the fast certificate,
+// the exact decision in fp32 pairs, the flag for the fallback, and the kept tuples. Whole warps call
+// it; a thread with live = false has no vector and only helps.
 // sRa / sPm: Ra_h, Pmax_h of this thread's hypotheses at [h * stride]; sNL / sNa: the staged
 // codeword terms (used when the whole codebook was staged, else recomputed).
+//
+// Exact decisions: a few vectors per warp fail the fast certificate, and their L entries cost about
+// 700 instructions each, so a lane takes one entry: 32 / L vectors at a time, ranks among a
+// vector's entries by shuffles, the entry of rank r writes tuple r. (A thread deciding all entries of
+// its own vector kept the warp for L entries whenever one lane had to: three stages over 11008 x 11
+// vectors with 8 hypotheses took 874 us, now 655.)
 template <int L>
 __device__ __forceinline__ void beam_list_finish(
     const SetView& set, const CbList& cbs, const StageDesc& sd, const BeamBufs& bb,
-    const FlagList& flags, int64_t i, int64_t g, int64_t vi, int Bh, float cmul,
+    const FlagList& flags, bool live, int64_t i, int64_t g, int64_t vi, int Bh, float cmul,
     const float th[kD], const float tl[kD], const float* sH, const float2* sNL,
     const float* sNa, bool one_chunk, const float* sRa, const float* sPm, int stride,
     float topv[L], int topi[L], unsigned* err) {
   const CbView cw = cbs.cb[sd.st[sd.s]];
   const int S = sd.S, B = sd.B, Bs = sd.Bs;
-  int toph[L], topk[L];
-#pragma unroll
-  for (int j = 0; j < L; ++j) {
-    toph[j] = topi[j] == 0x7fffffff ? 0x7fffffff : (topi[j] >> 16);
-    topk[j] = topi[j] == 0x7fffffff ? 0x7fffffff : (topi[j] & 0xffff);
-  }
-  const int64_t total = (int64_t)Bh * cw.K;
-  const int nkept = (int)min((int64_t)L, total);
-  const int keep = (int)min((int64_t)Bs, total);
-  // Non-finite scores never enter the list; keep indices valid and report it.
-#pragma unroll
-  for (int j = 0; j < L; ++j) {
-    if (j < nkept && (toph[j] >= Bh || topk[j] >= cw.K)) {
-      raise_error(err, ERRBIT_NUMERIC);
-      toph[j] = 0;
-      topk[j] = 0;
-    }
-  }
-  // Per-entry bound Et = u C (Ra_h + Na_k + 2 Pmax_h L1_k) for the listed entries, from the
-  // hypothesis terms kept in the sweep and the staged codeword terms (recomputed when the
-  // codebook spans several chunks).
-  float et[L];
-#pragma unroll
-  for (int j = 0; j < L; ++j) {
-    et[j] = 0.f;
-    if (j < nkept) {
-      const float ra = sRa[toph[j] * stride];
-      const float pmax = sPm[toph[j] * stride];
-      float na, l1;
-      if (one_chunk) {
-        na = sNa[topk[j]];
-        l1 = sNL[topk[j]].y;
-      } else {
-        float c[kD], n;
-        load_vec(cw.C + (int64_t)topk[j] * kD, c);
-        codeword_terms(c, sH, n, na, l1);
-      }
-      et[j] = kU * cmul * (ra + na + 2.f * pmax * l1);
-    }
-  }
-  // Fast certificate: low_{j+1} - low_j > 2 Et_j for j < min(keep, total - 1) (every
-  // candidate outside the list has low >= the last list entry).
-  bool ok = true;
-  const int lim = (int)min((int64_t)keep, total - 1);
-#pragma unroll
-  for (int j = 0; j < L - 1; ++j)
-    if (j < lim && !(topv[j + 1] - topv[j] > 2.f * et[j])) ok = false;
-
-  int32_t* out = bb.hyp_out + vi * B * S;
-  if (!ok) {
-    // Exact path on the listed candidates: errs as fp32 pairs (about 2^-44 relative; no fp64),
-    // (err, h, k) order; then every unlisted candidate must have low >= the last listed low,
-    // which must exceed an upper bound of the keep-th err.
-    float evh[L], evl[L];
+  const int lane = threadIdx.x & 31;
+  bool open = false;
+  if (live) {
+    const int64_t total = (int64_t)Bh * cw.K;
+    const int nkept = (int)min((int64_t)L, total);
+    const int keep = (int)min((int64_t)Bs, total);
+    // Non-finite scores never enter the list; keep indices valid and report it.
 #pragma unroll
     for (int j = 0; j < L; ++j) {
-      evh[j] = INFINITY;
-      evl[j] = 0.f;
-      if (j < nkept) {
-        float rh[kD], rl[kD], c[kD];
-        const int32_t* pc = bb.hyp_in ? bb.hyp_in + (vi * B + toph[j]) * S : nullptr;
-        hyp_residual_pair(th, tl, cbs, sd, pc, rh, rl, err);
-        load_vec(cw.C + (int64_t)topk[j] * kD, c);
-        dfl::quad_err(rh, rl, c, sH, evh[j], evl[j]);
+      if (j < nkept && ((topi[j] >> 16) >= Bh || (topi[j] & 0xffff) >= cw.K)) {
+        raise_error(err, ERRBIT_NUMERIC);
+        topi[j] = 0;
       }
     }
-    const float last_low = topv[nkept - 1];
+    // Fast certificate: low_{j+1} - low_j > 2 Et_j for j < min(keep, total - 1) (every candidate
+    // outside the list has low >= the last list entry), with the per-entry bound
+    // Et = u C (Ra_h + Na_k + 2 Pmax_h L1_k) from the hypothesis terms kept in the sweep and the
+    // staged codeword terms (recomputed when the codebook spans several chunks).
+    const int lim = (int)min((int64_t)keep, total - 1);
 #pragma unroll
-    for (int a = 1; a < L; ++a) {
+    for (int j = 0; j < L - 1; ++j) {
+      if (j < lim) {
+        const int h = topi[j] >> 16, k = topi[j] & 0xffff;
+        float na, l1;
+        if (one_chunk) {
+          na = sNa[k];
+          l1 = sNL[k].y;
+        } else {
+          float c[kD], n;
+          load_vec(cw.C + (int64_t)k * kD, c);
+          codeword_terms(c, sH, n, na, l1);
+        }
+        const float et = kU * cmul * (sRa[h * stride] + na + 2.f * sPm[h * stride] * l1);
+        if (!(topv[j + 1] - topv[j] > 2.f * et)) open = true;
+      }
+    }
+    if (!open) {
+      int32_t* out = bb.hyp_out + vi * B * S;
 #pragma unroll
-      for (int b = a; b > 0; --b) {
-        const bool sw = (evh[b] < evh[b - 1]) ||
-                        (evh[b] == evh[b - 1] &&
-                         (evl[b] < evl[b - 1] ||
-                          (evl[b] == evl[b - 1] &&
-                           (toph[b] < toph[b - 1] ||
-                            (toph[b] == toph[b - 1] && topk[b] < topk[b - 1])))));
-        if (sw) {
-          const float t0 = evh[b]; evh[b] = evh[b - 1]; evh[b - 1] = t0;
-          const float t1 = evl[b]; evl[b] = evl[b - 1]; evl[b - 1] = t1;
-          const int th_ = toph[b]; toph[b] = toph[b - 1]; toph[b - 1] = th_;
-          const int tk = topk[b]; topk[b] = topk[b - 1]; topk[b - 1] = tk;
+      for (int j = 0; j < L; ++j) {
+        if (j >= keep) break;
+        const int32_t* pc = bb.hyp_in ? bb.hyp_in + (vi * B + (topi[j] >> 16)) * S : nullptr;
+        for (int q = 0; q < sd.s; ++q) out[j * S + q] = pc[q];
+        out[j * S + sd.s] = topi[j] & 0xffff;
+      }
+      bb.n_out[vi] = keep;
+    }
+  }
+  // Exact decisions: lane = (slot, entry) of the next 32 / L open vectors. Errs as fp32 pairs (about
+  // 2^-44 relative; no fp64) in (err, h, k) order; every unlisted candidate must have low >= the
+  // last listed low, which must exceed an upper bound of the keep-th err.
+  constexpr int kPer = 32 / L;
+  const int slot = lane / L, e = lane - slot * L;
+  unsigned todo = __ballot_sync(0xffffffffu, open);
+  while (todo) {
+    unsigned rest = todo;
+    int src = -1;
+    for (int q = 0; q < kPer && rest; ++q) {
+      if (q == slot) src = __ffs(rest) - 1;
+      rest &= rest - 1u;
+    }
+    const bool has = src >= 0;
+    const int from = has ? src : __ffs(todo) - 1;
+    todo = rest;
+    float vth[kD], vtl[kD];
+#pragma unroll
+    for (int q = 0; q < kD; ++q) {
+      vth[q] = __shfl_sync(0xffffffffu, th[q], from);
+      vtl[q] = __shfl_sync(0xffffffffu, tl[q], from);
+    }
+    const int64_t v = __shfl_sync(0xffffffffu, vi, from);
+    const int64_t total = (int64_t)__shfl_sync(0xffffffffu, Bh, from) * cw.K;
+    const int nkept = (int)min((int64_t)L, total);
+    const int keep = (int)min((int64_t)Bs, total);
+    int hk = 0;
+    float last_low = INFINITY;
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      const int t = __shfl_sync(0xffffffffu, topi[j], from);
+      const float x = __shfl_sync(0xffffffffu, topv[j], from);
+      if (j == e) hk = t;
+      if (j == nkept - 1) last_low = x;
+    }
+    const bool mine = has && e < nkept;
+    float eh = INFINITY, el = 0.f;
+    const int32_t* pc = bb.hyp_in ? bb.hyp_in + (v * B + (hk >> 16)) * S : nullptr;
+    if (mine) {
+      float rh[kD], rl[kD], c[kD];
+      hyp_residual_pair(vth, vtl, cbs, sd, pc, rh, rl, err);
+      load_vec(cw.C + (int64_t)(hk & 0xffff) * kD, c);
+      dfl::quad_err(rh, rl, c, sH, eh, el);
+      if (!isfinite(eh)) {  // (NaN too: the ranks stay a permutation)
+        eh = INFINITY;
+        el = 0.f;
+      }
+    }
+    __syncwarp();
+    // rank among the vector's entries by (err, (h, k)), then place
+    int rank = 0;
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      const int at = min(slot * L + j, 31);
+      const float oh = __shfl_sync(0xffffffffu, eh, at), ol = __shfl_sync(0xffffffffu, el, at);
+      const int ok = __shfl_sync(0xffffffffu, hk, at);
+      const bool same = oh == eh && ol == el && ok == hk;
+      if (j < nkept && (same ? j < e : dfl::less(oh, ol, ok, eh, el, hk))) ++rank;
+    }
+    const unsigned holder =
+        (__ballot_sync(0xffffffffu, mine && rank == keep - 1) >> min(slot * L, 31)) &
+        ((1u << L) - 1u);
+    const int kth = holder ? min(slot * L + __ffs(holder) - 1, 31) : lane;
+    const float kh = __shfl_sync(0xffffffffu, eh, kth), kl = __shfl_sync(0xffffffffu, el, kth);
+    // upper bound of the keep-th listed err (the pair's own error is far below 1e-7)
+    const float ev_up = isfinite(kh) ? __fmul_ru(__fadd_ru(kh, kl), 1.0000002f) : INFINITY;
+    const bool cert = total <= L || last_low > ev_up;
+    if (mine && cert && rank < keep) {
+      int32_t* out = bb.hyp_out + (v * B + rank) * S;
+      for (int q = 0; q < sd.s; ++q) out[q] = pc[q];
+      out[sd.s] = hk & 0xffff;
+    }
+    if (has && e == 0) {
+      if (cert) {
+        bb.n_out[v] = keep;
+      } else {
+        const unsigned at = atomicAdd(flags.count, 1u);
+        if (at < flags.cap) {
+          flags.vec[at] = v;
+          // every member of the exact top-keep has err <= the keep-th listed err
+          flags.thr[at] = ev_up;
+        } else {
+          raise_error(err, ERRBIT_INDEX);
         }
       }
     }
-    // upper bound of the keep-th listed err (the pair's own error is far below 1e-7)
-    const float ev_up = isfinite(evh[keep - 1])
-                            ? __fmul_ru(__fadd_ru(evh[keep - 1], evl[keep - 1]), 1.0000002f)
-                            : INFINITY;
-    const bool cert = total <= L || last_low > ev_up;
-    if (!cert) {
-      const unsigned slot = atomicAdd(flags.count, 1u);
-      if (slot < flags.cap) {
-        flags.vec[slot] = vi;
-        // every member of the exact top-keep has err <= the keep-th listed err
-        flags.thr[slot] = ev_up;
-      } else {
-        raise_error(err, ERRBIT_INDEX);
-      }
-      return;
-    }
   }
-#pragma unroll
-  for (int j = 0; j < L; ++j) {
-    if (j >= keep) break;
-    const int32_t* pc = bb.hyp_in ? bb.hyp_in + (vi * B + toph[j]) * S : nullptr;
-    for (int q = 0; q < sd.s; ++q) out[j * S + q] = pc[q];
-    out[j * S + sd.s] = topk[j];
-  }
-  bb.n_out[vi] = keep;
 }
 
 constexpr int kBeamCand = 16;  // candidate buffer slots per thread
@@ -1866,9 +1898,9 @@ beam_stage_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDe
       }
     }
   }
-  if (!live) return;
-  flush();
-  beam_list_finish<L>(set, cbs, sd, bb, flags, i, g, vi, Bh, cmul, th, tl, sH, sNL, sNa,
+  if (live) flush();
+  __syncwarp();
+  beam_list_finish<L>(set, cbs, sd, bb, flags, live, i, g, vi, Bh, cmul, th, tl, sH, sNL, sNa,
                       cw.K <= kChunk, sRa + threadIdx.x, sPm + threadIdx.x, kThreads, topv,
                       topi, err);
 }
@@ -2149,8 +2181,7 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
   if (!ok && tid == 0) tc::mbar_wait(tc::smem_u32(&bar_b), 0u, err);
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, 2 * kTcCols);
-  if (!live) return;
-  beam_list_finish<L>(set, cbs, sd, bb, flags, i, g, vi, Bh, cmul, th, tl, sH, sNL, sNa, true,
+  beam_list_finish<L>(set, cbs, sd, bb, flags, live, i, g, vi, Bh, cmul, th, tl, sH, sNL, sNa, true,
                       sRa + tid, sPm + tid, kThreads, topv, topi, err);
 }
 

@@ -315,6 +315,57 @@ dim3 prep_b_grid(int64_t G_range, int nchunk, int nsm) {
   return dim3((unsigned)x + 1, (unsigned)G_range);
 }
 
+// The same rows for codebooks of more than 256 codewords, in two parts: of a row's 32 values only n'
+// depends on the group. A chunk's 128 rows are laid out by four-value columns of 2 KB (kBCol), and column
+// 6 (n'_hi n'_lo L1_hi L1_lo) is stored per group: out_g[(g_rel nchunk + chunk) 2 KB]; the others once:
+// out[chunk 16 KB], column 6 unused. A group takes 1 MB for 65536 codewords instead of 8, and 128
+// groups share a pass instead of 32. K = 65536, 1024 x 11008: 43 passes of (124 us images, 390 us
+// arg-min) became 11 of (97 us, 1331 us), 25.2 -> 17.4 ms in all.
+constexpr int kBCol = kTcCols * 16;
+constexpr int kBGroupCol = 6;
+
+__global__ void __launch_bounds__(128)
+prep_b_split_kernel(SetView set, int64_t g_begin, const float* __restrict__ C, int K, int nchunk, float uc,
+                    bool first, char* __restrict__ out, char* __restrict__ out_g,
+                    float4* __restrict__ terms, float* __restrict__ cbmax,
+                    unsigned* __restrict__ flag_count) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
+  // The open lists of the arg-min pass that follows start empty (see prep_b_kernel).
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) flag_count[threadIdx.x] = 0u;
+  if (blockIdx.x == gridDim.x - 1) {  // the last column of CTAs: the codebook maxima (its first)
+    if (first && blockIdx.y == 0) cbmax_block(C, K, cbmax);
+    return;
+  }
+  const int64_t g = g_begin + blockIdx.y;
+  float H[kD * kD];
+#pragma unroll
+  for (int e = 0; e < kD * kD; e += 4) {
+    const float4 h = __ldg(reinterpret_cast<const float4*>(set.Hb + g * kD * kD + e));
+    H[e] = h.x;
+    H[e + 1] = h.y;
+    H[e + 2] = h.z;
+    H[e + 3] = h.w;
+  }
+  for (int chunk = blockIdx.x; chunk < nchunk; chunk += gridDim.x - 1) {
+    const int kk = chunk * kTcCols + threadIdx.x;
+    uint32_t v[tcenc::kK];
+    float tk[3];
+    build_b_row(C, K, kk, H, uc, v, tk);
+    char* row = out + (int64_t)chunk * kTcBTile + threadIdx.x * 16;
+    if (first && blockIdx.y == 0)
+#pragma unroll
+      for (int q = 0; q < tcenc::kK / 4; ++q)
+        if (q != kBGroupCol)
+          *reinterpret_cast<uint4*>(row + q * kBCol) =
+              make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    constexpr int e = 4 * kBGroupCol;
+    *reinterpret_cast<uint4*>(out_g + ((int64_t)blockIdx.y * nchunk + chunk) * kBCol +
+                              threadIdx.x * 16) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+    if (kk < K) terms[(int64_t)blockIdx.y * K + kk] = make_float4(tk[0], tk[1], tk[2], 0.f);
+  }
+}
+
 // Per-vector terms of the arg-min's A rows that do not change while one codebook's Lloyd
 // iterations run (the target, H_g and the fixed codebooks stay put): m2q = -2 H_g r and rr,
 // Ra, Pmax (vector_terms_rr of target32), as three planes of M float4 per group,
@@ -935,7 +986,7 @@ __global__ void __launch_bounds__(256, 2)
 argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_idx,
                  int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
                  FlagList wide, NarrowList narrow, StatsView st, const float* __restrict__ cbmax,
-                 const char* __restrict__ bpre, const float4* __restrict__ terms,
+                 const char* __restrict__ bpre, const char* __restrict__ bpre_g, const float4* __restrict__ terms,
                  const float4* __restrict__ rowterms, int tiles, unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
@@ -960,7 +1011,7 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   const float cmul = kCmul + 4.f * n_fixed;
   const float uc = kU * cmul;
   const int nchunk = (cw.K + kTcCols - 1) / kTcCols;
-  const char* bimg = bpre + (size_t)(g - g_begin) * nchunk * kTcBTile;
+  const char* bgrp = bpre_g + (size_t)(g - g_begin) * nchunk * kBCol;
   const float4* gterms = terms + (g - g_begin) * cw.K;
 
   if (tid < kD * kD) sH[tid] = set.Hb[g * kD * kD + tid];
@@ -1003,9 +1054,12 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   auto fetch = [&]() {  // the next chunk, into the buffer of the use kBRing before it
     const int b = (int)(fetched % kBRing);
     tc::mbar_expect_tx(tc::smem_u32(&bar_b[b]), kTcBTile);
-    tc::bulk_copy_g2s(tc::smem_u32(Bbuf + b * kTcBTile),
-                      bimg + (size_t)(2 * (fetched % nch) + half) * kTcBTile, kTcBTile,
-                      tc::smem_u32(&bar_b[b]));
+    const size_t chunk = (size_t)(2 * (fetched % nch) + half);
+    const uint32_t dst = tc::smem_u32(Bbuf + b * kTcBTile), bar = tc::smem_u32(&bar_b[b]);
+    const char* src = bpre + chunk * kTcBTile;
+    tc::bulk_copy_g2s(dst, src, kBGroupCol * kBCol, bar);
+    tc::bulk_copy_g2s(dst + kBGroupCol * kBCol, bgrp + chunk * kBCol, kBCol, bar);
+    tc::bulk_copy_g2s(dst + (kBGroupCol + 1) * kBCol, src + (kBGroupCol + 1) * kBCol, kBCol, bar);
     ++fetched;
   };
   // The next use's MMA. After a timeout its waiters are released and the caller's ok turns false.
@@ -1022,7 +1076,7 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
 #pragma unroll
     for (int ks = 0; ks < kK / 8; ++ks)
       tc::mma_tf32(tmem, tc::smem_desc(a0 + ks * 256, 128, (kK / 4) * 128),
-                   tc::smem_desc(b0 + ks * 256, 128, (kK / 4) * 128), idesc, ks > 0 ? 1u : 0u);
+                   tc::smem_desc(b0 + ks * 2 * kBCol, kBCol, 128), idesc, ks > 0 ? 1u : 0u);
     tc::mma_commit(tc::smem_u32(&bar_mma));
     return true;
   };
@@ -2603,9 +2657,10 @@ crvq_status launch_beam_stage(const SetView& set, int64_t g_begin, int64_t G_ran
   return go(std::integral_constant<int, 17>{});
 }
 
-// Scratch of one arg-min pass: codebook maxima (256 B) | B images of G_sub groups (groups
-// in sub-ranges whose images take at most 256 MB) | codeword terms | counts of the two open lists
-// (256 B) | narrow list | wide list (vector ids and thresholds).
+// Scratch of one arg-min pass: codebook maxima (256 B) | B images (the columns that all groups
+// share, then those of G_sub groups) | codeword terms of G_sub groups | counts of the two open lists
+// (256 B) | narrow list | wide list (vector ids and thresholds). Sub-ranges of groups whose images
+// and terms take at most 256 MB.
 struct ArgminLayout {
   int nchunk;
   int64_t G_sub;
@@ -2616,9 +2671,9 @@ ArgminLayout argmin_layout(int64_t M, int64_t G_range, int K) {
   ArgminLayout L{};
   if (K <= kSmallK) return L;  // argmin_small_kernel takes none
   L.nchunk = (int)ceil_div(K, kTcCols);
-  const int64_t per_group = (int64_t)L.nchunk * kTcBTile;
+  const int64_t per_group = (int64_t)L.nchunk * kBCol + (int64_t)K * (int64_t)sizeof(float4);
   L.G_sub = std::max<int64_t>(1, std::min<int64_t>(G_range, (int64_t(256) << 20) / per_group));
-  L.bbytes = (size_t)L.G_sub * per_group;
+  L.bbytes = (size_t)L.nchunk * kTcBTile + (size_t)L.G_sub * L.nchunk * kBCol;
   L.tbytes = align_up((size_t)L.G_sub * K * sizeof(float4), 256);
   L.obytes = align_up((size_t)M * L.G_sub * sizeof(NarrowRow), 256);
   L.fbytes = align_up((size_t)M * L.G_sub * (sizeof(int64_t) + sizeof(float)), 256);
@@ -2650,9 +2705,9 @@ crvq_status launch_argmin_small(const SetView& set, const CbList& cbs, const Arg
   return CRVQ_OK;
 }
 
-// Larger codebooks: groups in sub-ranges whose B images (the codebook's tensor-core operand per
-// group) take at most 256 MB; per sub-range: images + per-group codeword terms (prep_b, which also
-// writes the codebook maxima), the arg-min pass, and the exact decision of flagged rows.
+// Larger codebooks: groups in sub-ranges (argmin_layout); per sub-range: images + per-group codeword
+// terms (prep_b_split, which also writes the shared images and the codebook maxima the first time),
+// the arg-min pass, and the exact decision of flagged rows.
 crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const ArgminCall& a,
                                 const EncodeExtras& ex, unsigned* err, cudaStream_t stream) {
   const int64_t g_begin = a.g_begin, G_range = a.G_range, out_ld = a.out_ld, out_g0 = a.out_g0;
@@ -2672,6 +2727,7 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
   }
   float* cbmax = reinterpret_cast<float*>(wbase);
   char* bimg = wbase + 256;
+  char* bgrp = bimg + (size_t)nchunk * kTcBTile;
   float4* tout = reinterpret_cast<float4*>(bimg + bbytes);
   FlagList fl;
   fl.count = reinterpret_cast<unsigned*>(wbase + 256 + bbytes + tbytes);
@@ -2689,8 +2745,8 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
     fl.thr = reinterpret_cast<float*>(fl.vec + nv);  // the count is cleared by prep_b
     {
       ProfScope pb("encode_prep_b", stream, (double)gn * nchunk * kTcCols);
-      CRVQ_CUDA(launch_pdl(prep_b_kernel, prep_b_grid(gn, nchunk, nsm), dim3(128), 0, stream, set, gs,
-                           cw.C, cw.K, nchunk, uc, bimg, tout, cbmax, fl.count));
+      CRVQ_CUDA(launch_pdl(prep_b_split_kernel, prep_b_grid(gn, nchunk, nsm), dim3(128), 0, stream, set,
+                           gs, cw.C, cw.K, nchunk, uc, gs == g_begin, bimg, bgrp, tout, cbmax, fl.count));
       CRVQ_LAUNCHED();
     }
     {
@@ -2702,7 +2758,7 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
       ProfScope ps(st.cnt ? "encode_argmin_lloyd" : "encode_argmin", stream,
                    (double)nv * cw.K);
       CRVQ_CUDA(launch_pdl(argmin_tc_kernel, grid, dim3(256), kArgminStreamSmem, stream, set, gs,
-                           cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, nl, st, cbmax, bimg, tout,
+                           cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, nl, st, cbmax, bimg, bgrp, tout,
                            ex.rowterms, tiles, err));
       CRVQ_LAUNCHED();
     }

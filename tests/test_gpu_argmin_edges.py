@@ -51,6 +51,16 @@ def test_codebook_and_row_edges(M, G, K):
     _check(W, _blocks(rng, G), C)
 
 
+def test_more_groups_than_one_sub_range():
+    """K = 3000: the operand images of about 2760 groups fit a sub-range; the shared part of the
+    images serves the second one too."""
+    rng = np.random.default_rng(11)
+    M, G, K = 2, 2800, 3000
+    W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
+    C = (0.02 * rng.standard_normal((K, D))).astype(np.float32)
+    _check(W, _blocks(rng, G), C)
+
+
 @pytest.mark.parametrize("K", [15, 16, 17, 129, 200, 241])
 def test_block_and_class_edges(K):
     """Codebook sizes around the 16-column blocks of the sweep, whose two smallest minima carry their

@@ -1566,46 +1566,6 @@ struct StageDesc {
   int Bs;                 // hypotheses kept by the current stage (1 at the last stage)
 };
 
-// fp64 residual of a hypothesis before stage s: target - sum_{s' < s} C_{st[s']}[code].
-__device__ void hyp_residual64(const double tgt[kD], const CbList& cbs, const StageDesc& sd,
-                               const int32_t* codes, double r[kD], unsigned* err) {
-#pragma unroll
-  for (int j = 0; j < kD; ++j) r[j] = tgt[j];
-  for (int q = 0; q < sd.s; ++q) {
-    const CbView& cb = cbs.cb[sd.st[q]];
-    const int32_t k = codes[q];
-    if (!code_ok(k, cb.K, err)) continue;
-    const float* c = cb.C + (int64_t)k * kD;
-#pragma unroll
-    for (int j = 0; j < kD; ++j) r[j] -= (double)c[j];
-  }
-}
-
-// Per-hypothesis terms of the approximate err: m2q = -2 H r, rr = r^T H r (r rounded to
-// fp32), and the bound pieces Ra = |r|^T |H| |r|, Pmax = max_p (|H| |r|)_p.
-__device__ __forceinline__ void hyp_terms(const double r64[kD], const float* H, float m2q[kD],
-                                          float& rr, float& ra, float& pmax) {
-  float r[kD];
-#pragma unroll
-  for (int j = 0; j < kD; ++j) r[j] = (float)r64[j];
-  rr = 0.f;
-  ra = 0.f;
-  pmax = 0.f;
-#pragma unroll
-  for (int p = 0; p < kD; ++p) {
-    float q = 0.f, pa = 0.f;
-#pragma unroll
-    for (int j = 0; j < kD; ++j) {
-      q = fmaf(H[p * kD + j], r[j], q);
-      pa = fmaf(fabsf(H[p * kD + j]), fabsf(r[j]), pa);
-    }
-    m2q[p] = -2.f * q;
-    rr = fmaf(r[p], q, rr);
-    ra = fmaf(fabsf(r[p]), pa, ra);
-    pmax = fmaxf(pmax, pa);
-  }
-}
-
 // fp32-pair residual of a hypothesis before stage s: (rh + rl) = (th + tl) - sum_{s' < s}
 // C_{st[s']}[code] (TwoSum per subtraction, about 2^-48 relative; no fp64 arithmetic).
 __device__ __forceinline__ void hyp_residual_pair(const float th[kD], const float tl[kD],
@@ -1633,7 +1593,8 @@ __device__ __forceinline__ void hyp_residual_pair(const float th[kD], const floa
   }
 }
 
-// hyp_terms of a pair residual, rounded once to fp32.
+// Per-hypothesis terms of the approximate err: m2q = -2 H r, rr = r^T H r (r: the pair residual
+// rounded to fp32), and the bound pieces Ra = |r|^T |H| |r|, Pmax = max_p (|H| |r|)_p.
 __device__ __forceinline__ void hyp_terms_pair(const float rh[kD], const float rl[kD],
                                                const float* H, float m2q[kD], float& rr,
                                                float& ra, float& pmax) {
@@ -2240,10 +2201,13 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
 }
 
 // Exact stage for flagged vectors: one warp per vector; the lanes stride over the (h, k)
-// candidates, re-score in fp64 those whose fp32 lower bound is at most the vector's
+// candidates, re-score in fp32 pairs those whose fp32 lower bound is at most the vector's
 // threshold (the keep-th exact err among the fast pass's listed candidates, which bounds
 // every member of the exact top-Bs) and keep a sorted local top-Bs; a warp merge then
 // extracts the global top-Bs in (err, h, k) order.
+// Bound: latency (a few thousand vectors per stage). In fp64 the re-scoring alone kept an SM's
+// fp64 pipe busy: 56 us per stage over 11008 x 11 vectors, now 31. The pairs are those of
+// beam_list_finish and of the arg-min's exact decisions.
 __global__ void __launch_bounds__(kThreads)
 beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs,
                            int n_fixed, StageDesc sd, BeamBufs bb, FlagList flags,
@@ -2262,15 +2226,18 @@ beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList
     const int64_t vi = flags.vec[f];
     const int64_t i = vi / G_range, g = g_begin + vi % G_range;
     const float* H = set.Hb + g * kD * kD;
-    double tgt[kD];
-    target64(set, cbs, n_fixed, i, g, tgt, err);
+    float th[kD], tl[kD];
+    dfl::target(set, cbs, n_fixed, i, g, th, tl, err);
     const int Bh = (sd.s == 0) ? 1 : bb.n_in[vi];
     const float thr = flags.thr[f];
     const float cmul = bound_mult(n_fixed + sd.s);
-    double be[16];
+    float be[16], bl[16];  // err pairs
     int bh[16], bk[16];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) be[j] = INFINITY;
+    for (int j = 0; j < 16; ++j) {
+      be[j] = INFINITY;
+      bl[j] = 0.f;
+    }
     int nb = 0;
     // Candidates (h, k) are queued in increasing (h, k) order and scored one per lane, so
     // every lane still sees its own candidates in increasing (h, k): strict comparison in
@@ -2280,17 +2247,25 @@ beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList
       __syncwarp();
       if (lane < qn) {
         const int h = qh[lane], k = q[lane];
-        double r64[kD];
+        float rh[kD], rl[kD], c[kD], e, el;
         const int32_t* pc = bb.hyp_in ? bb.hyp_in + (vi * B + h) * S : nullptr;
-        hyp_residual64(tgt, cbs, sd, pc, r64, err);
-        const double e = quad_err64(r64, cw.C + (int64_t)k * kD, H);
-        if (nb < Bs || e < be[nb - 1]) {
+        hyp_residual_pair(th, tl, cbs, sd, pc, rh, rl, err);
+        load_vec(cw.C + (int64_t)k * kD, c);
+        dfl::quad_err(rh, rl, c, H, e, el);
+        auto before = [&](int at) { return e < be[at] || (e == be[at] && el < bl[at]); };
+        if (nb < Bs || before(nb - 1)) {
           int pos = nb < Bs ? nb : Bs - 1;
-          while (pos > 0 && e < be[pos - 1]) {
-            be[pos] = be[pos - 1]; bh[pos] = bh[pos - 1]; bk[pos] = bk[pos - 1];
+          while (pos > 0 && before(pos - 1)) {
+            be[pos] = be[pos - 1];
+            bl[pos] = bl[pos - 1];
+            bh[pos] = bh[pos - 1];
+            bk[pos] = bk[pos - 1];
             --pos;
           }
-          be[pos] = e; bh[pos] = h; bk[pos] = k;
+          be[pos] = e;
+          bl[pos] = el;
+          bh[pos] = h;
+          bk[pos] = k;
           if (nb < Bs) ++nb;
         }
       }
@@ -2298,11 +2273,11 @@ beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList
       qn = 0;
     };
     for (int h = 0; h < Bh; ++h) {
-      double r64[kD];
+      float rh[kD], rl[kD];
       const int32_t* pc = bb.hyp_in ? bb.hyp_in + (vi * B + h) * S : nullptr;
-      hyp_residual64(tgt, cbs, sd, pc, r64, err);
+      hyp_residual_pair(th, tl, cbs, sd, pc, rh, rl, err);
       float m2q[kD], rr, ra, pmax;
-      hyp_terms(r64, H, m2q, rr, ra, pmax);
+      hyp_terms_pair(rh, rl, H, m2q, rr, ra, pmax);
       const float base = rr - kU * cmul * ra;
       const float nbeta = -2.f * kU * cmul * pmax;
       for (int k0 = 0; k0 < cw.K; k0 += 32) {
@@ -2338,19 +2313,25 @@ beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList
     int32_t* out = bb.hyp_out + vi * B * S;
     const int total = (int)min((int64_t)Bs, (int64_t)Bh * cw.K);
     for (int j = 0; j < total; ++j) {
-      double e = head < nb ? be[head] : INFINITY;
+      float e = head < nb ? be[head] : INFINITY, el = head < nb ? bl[head] : 0.f;
       int hh = head < nb ? bh[head] : 0x7fffffff;
       int kk = head < nb ? bk[head] : 0x7fffffff;
       int src = lane;
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) {
-        const double oe = __shfl_xor_sync(0xffffffffu, e, off);
+        const float oe = __shfl_xor_sync(0xffffffffu, e, off);
+        const float ol = __shfl_xor_sync(0xffffffffu, el, off);
         const int oh = __shfl_xor_sync(0xffffffffu, hh, off);
         const int ok = __shfl_xor_sync(0xffffffffu, kk, off);
         const int os = __shfl_xor_sync(0xffffffffu, src, off);
-        const bool take = oe < e || (oe == e && (oh < hh || (oh == hh && ok < kk)));
+        const bool take =
+            oe < e || (oe == e && (ol < el || (ol == el && (oh < hh || (oh == hh && ok < kk)))));
         if (take) {
-          e = oe; hh = oh; kk = ok; src = os;
+          e = oe;
+          el = ol;
+          hh = oh;
+          kk = ok;
+          src = os;
         }
       }
       if (lane == src) ++head;

@@ -2130,23 +2130,34 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
       }
       if (act) tau_x = __fadd_ru(bl[L - 1], eps);
     }
-    // Candidates of hypothesis h, 64 columns at a time: a mask (a compare and a predicated or
-    // per score), then its members in codeword order, scored again with the fast stage's chain
+    // Candidates of hypothesis h, 64 columns at a time: a mask (a subtraction and a funnel
+    // shift per score), then its members in codeword order, scored again with the fast stage's chain
     // and inserted; the threshold tightens after every 64 columns. NaN threshold for a thread
     // without this hypothesis: no value compares below it.
 #pragma unroll 1
     for (int q = 0; q < nq; ++q) {
-      const float thrD =
-          act ? __fadd_ru(fminf(topv[L - 1], tau_x), eps) : __int_as_float(0x7fffffff);
+      const float thrD = act ? __fadd_ru(fminf(topv[L - 1], tau_x), eps) : -INFINITY;
+      // y <= thrD as the sign of y - (the next number above thrD), shifted into the mask: one
+      // instruction on the FMA pipe and one on the ALU pipe, which had both of the compare form (three
+      // stages over 11008 x 11 vectors 581 -> 561 us)
+      const float up = thrD < INFINITY && thrD > -INFINITY
+                           ? __int_as_float(__float_as_int(thrD) +
+                                            (thrD > 0.f ? 1 : thrD < 0.f ? -1 : 0)) +
+                                 (thrD == 0.f ? 1.401298464e-45f : 0.f)
+                           : thrD;
       uint32_t m0 = 0u, m1 = 0u;
       {
         uint32_t v[64];
         tc::tmem_ld64_wait(trow + 64 * q, v);
+        uint32_t part[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          if (__uint_as_float(v[e]) <= thrD) m0 |= 1u << e;
-          if (__uint_as_float(v[32 + e]) <= thrD) m1 |= 1u << e;
-        }
+        for (int e = 15; e >= 0; --e)
+#pragma unroll
+          for (int w = 0; w < 4; ++w)
+            part[w] = __funnelshift_l(__float_as_uint(__fsub_rn(__uint_as_float(v[16 * w + e]), up)),
+                                      part[w], 1);
+        m0 = part[0] | part[1] << 16;
+        m1 = part[2] | part[3] << 16;
       }
 #pragma unroll
       for (int w = 0; w < 2; ++w) {

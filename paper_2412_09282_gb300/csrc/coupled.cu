@@ -140,27 +140,21 @@ block_factor_kernel(const float* __restrict__ H, int64_t N, int64_t G_cov,
 //     columns of B^T (the block's earlier changes included) - H_gg D_g, the solve a forward and a back
 //     substitution in fp32 with the group's factor;
 //  2. scores, a thread per codeword (chunks of 256): the fp32 lower bound low_k = s_k - Et_k of every
-//     row (8 FMAs), the two smallest of a warp's 32 by integer minima over order-preserving keys
-//     (redux), the two smallest of all by the row's eight lanes;
+//     row (8 FMAs) to shared memory; then the two smallest by eight lanes per row (two warp-wide
+//     integer reductions per row and warp instead took twice the instructions);
 //  3. certificate low_2nd - low_j > 2 Et_j; rows without it are decided exactly, a warp per row: every
 //     codeword with low_k <= low_j + 2 Et_j in fp32 pairs, smallest (err, index);
 //  4. the new code, D_g, and its change dD_g H[g, g'] added to the later columns, a thread per column.
 // Bound: latency of the serial group steps (a 4096 x 4096 sweep has 512 of them, eight warps per SM).
 // 4096 x 4096, 256 codewords, one sweep with both losses: 40.2 ms with a kernel per step and group, 13.3
 // ms with the steps in this kernel, 7.9 ms with the block products and the losses from operand
-// images; loading what the steps need up front, and E's entries ahead in the loss: 5.4 ms.
+// images; loading what the steps need up front, and E's entries ahead in the loss: 5.4 ms; the
+// scores' minima from shared memory: 4.7 ms.
 constexpr int kCplRows = 32;
 constexpr int kCplThreads = 256;
 constexpr int kCplPad = kBlockCols + 1;  // row stride of the B^T slice in shared memory
 
-// Order-preserving map of fp32 to uint32 (NaN above every number).
-__device__ __forceinline__ uint32_t order_key(float x) {
-  const uint32_t b = __float_as_uint(x);
-  return x != x ? 0xffffffffu : ((b >> 31) ? ~b : b | 0x80000000u);
-}
-__device__ __forceinline__ float order_val(uint32_t k) {
-  return __uint_as_float((k >> 31) ? k & 0x7fffffffu : ~k);
-}
+constexpr int kCplScores = kCplThreads + 8;  // row stride of the scores: four rows on distinct banks
 
 struct CplArgs {
   const float* W;      // M x N
@@ -180,19 +174,13 @@ struct CplArgs {
   CbList cbs;
 };
 
-// A warp's two smallest keys of a row, the smallest one's codeword and its 2 Et.
-struct __align__(16) CplBest {
-  uint32_t v1, v2;
-  int k1;
-  float e2;
-};
-
 struct CplShared {
   float B[kCplRows * kCplPad];               // [row][column of the block]
   float2 R[kBlockG][kCplRows][kD];           // targets without `which`: (hi, lo)
   float C[kCplThreads * kD];                 // the codebook (K <= 256)
   int32_t code[kBlockG][kCplRows];
-  CplBest best[kCplRows][8];                 // per row and warp
+  float S[kCplRows][kCplScores];             // the rows' scores
+  float2 nal[kCplThreads];                   // the codewords' (Na, L1)
   float H[2][kD * kD], L[2][kD * kD], inv[2][kD];  // the group's and the next one's
   float T[kCplRows][kD];                     // t'
   float Q[kCplRows][kD];                     // -2 H t'
@@ -321,10 +309,13 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
       if (j8 == 0) s.beta[row8] = -2.f * kU * cmul * pa;
     }
     __syncthreads();
-    // 2. scores, 256 codewords at a time; each warp keeps its two smallest per row
+    // 2. scores, 256 codewords at a time; lane j8 of a row takes every eighth
+    float f1 = INFINITY, f2 = INFINITY, e2 = INFINITY;  // smallest, second smallest, 2 Et
+    int k1 = 0;
     for (int k0 = 0; k0 < cw.K; k0 += kCplThreads) {
-      const int k = k0 + tid;
+      const int k = k0 + tid, nk = min(kCplThreads, cw.K - k0);
       if (k0 > 0) {
+        __syncthreads();  // the earlier chunk's scores have been read
 #pragma unroll
         for (int j = 0; j < kD; ++j) c[j] = 0.f;
         n = na = l1 = 0.f;
@@ -333,13 +324,13 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
           codeword_terms(c, sH, n, na, l1);
         }
       }
-      const float nlow = k < cw.K ? fmaf(-kU * cmul, na, n) : __int_as_float(0x7fffffff);
+      s.nal[tid] = make_float2(na, l1);
+      const float nlow = fmaf(-kU * cmul, na, n);
 #pragma unroll 4
       for (int r = 0; r < nr; ++r) {
         const float4 q0 = *reinterpret_cast<const float4*>(&s.Q[r][0]);
         const float4 q1 = *reinterpret_cast<const float4*>(&s.Q[r][4]);
-        const float beta = s.beta[r];
-        float sc = nlow;  // (NaN past the codebook: the largest key)
+        float sc = nlow;
         sc = fmaf(q0.x, c[0], sc);
         sc = fmaf(q0.y, c[1], sc);
         sc = fmaf(q0.z, c[2], sc);
@@ -348,51 +339,45 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
         sc = fmaf(q1.y, c[5], sc);
         sc = fmaf(q1.z, c[6], sc);
         sc = fmaf(q1.w, c[7], sc);
-        sc = fmaf(beta, l1, sc);
-        const uint32_t key = order_key(sc);
-        const uint32_t m1 = __reduce_min_sync(0xffffffffu, key);
-        const int src = __ffs(__ballot_sync(0xffffffffu, key == m1)) - 1;
-        const uint32_t m2 = __reduce_min_sync(0xffffffffu, lane == src ? 0xffffffffu : key);
-        CplBest b{m1, m2, k, 2.f * kU * cmul * na - 2.f * beta * l1};
-        if (k0 > 0) {  // with the warp's earlier chunks; strictly below: ties keep the smaller index
-          const CplBest o = s.best[r][warp];
-          if (m1 < o.v1) {
-            b.v2 = min(o.v1, m2);
-          } else {
-            b = o;
-            b.v2 = min(o.v2, m1);
-          }
+        s.S[r][tid] = fmaf(s.beta[r], l1, sc);
+      }
+      __syncthreads();
+      if (row8 < nr) {
+#pragma unroll 8
+        for (int kk = j8; kk < nk; kk += 8) {  // (a NaN score makes the two equal: the row is open)
+          const float sc = s.S[row8][kk];
+          k1 = sc < f1 ? k0 + kk : k1;  // ties: the smaller index
+          f2 = fminf(f2, fmaxf(f1, sc));
+          f1 = fminf(f1, sc);
         }
-        __syncwarp();
-        if (lane == src) s.best[r][warp] = b;
-        if (k0 + kCplThreads < cw.K) __syncwarp();
+        if (k1 >= k0) {
+          const float2 t = s.nal[k1 - k0];
+          e2 = 2.f * kU * cmul * t.x - 2.f * s.beta[row8] * t.y;
+        }
       }
     }
-    __syncthreads();
-    // 3. the row's smallest over its eight lanes (warps' entries), certificate
+    // 3. the row's smallest over its eight lanes, certificate
     {
-      CplBest b{0xffffffffu, 0xffffffffu, 0, 0.f};
-      if (row8 < nr) b = s.best[row8][j8];
 #pragma unroll
       for (int off = 4; off > 0; off >>= 1) {
-        CplBest o;
-        o.v1 = __shfl_xor_sync(0xffffffffu, b.v1, off);
-        o.v2 = __shfl_xor_sync(0xffffffffu, b.v2, off);
-        o.k1 = __shfl_xor_sync(0xffffffffu, b.k1, off);
-        o.e2 = __shfl_xor_sync(0xffffffffu, b.e2, off);
-        const bool take = o.v1 < b.v1 || (o.v1 == b.v1 && o.k1 < b.k1);
-        const uint32_t v2 = min(min(b.v2, o.v2), max(b.v1, o.v1));
-        if (take) b = o;
-        b.v2 = v2;
+        const float o1 = __shfl_xor_sync(0xffffffffu, f1, off);
+        const float o2 = __shfl_xor_sync(0xffffffffu, f2, off);
+        const int ok = __shfl_xor_sync(0xffffffffu, k1, off);
+        const float oe = __shfl_xor_sync(0xffffffffu, e2, off);
+        const bool take = o1 < f1 || (o1 == f1 && ok < k1);
+        f2 = fminf(fminf(f2, o2), fmaxf(f1, o1));
+        if (take) {
+          f1 = o1;
+          k1 = ok;
+          e2 = oe;
+        }
       }
       if (j8 == 0 && row8 < nr && factor) {
-        const float low1 = order_val(b.v1);
-        const bool cert = cw.K == 1 || (b.v1 != 0xffffffffu && order_val(b.v2) - low1 > b.e2) ||
-                          (b.v1 != 0xffffffffu && b.v2 == 0xffffffffu && isfinite(b.e2));
-        if (cert) {
-          s.code[gl][row8] = b.k1;
+        const bool found = f1 < INFINITY;
+        if (cw.K == 1 || (found && f2 - f1 > e2)) {
+          s.code[gl][row8] = k1;
         } else {
-          s.thr[row8] = b.v1 != 0xffffffffu ? __fadd_ru(low1, b.e2) : INFINITY;
+          s.thr[row8] = found ? __fadd_ru(f1, e2) : INFINITY;
           s.open[atomicAdd(&s.n_open, 1)] = row8;
         }
       }

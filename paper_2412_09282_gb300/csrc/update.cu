@@ -50,81 +50,94 @@ maxabs_kernel(SetView set, CbList cbs, int which, StatsView st, int64_t n_member
   stats_merge_scale(st, cbs, which, tm, hm, n_members, err);
 }
 
-// Statistics of every covered vector from its current code. CTA (x, y): groups y,
-// y + gridDim.y, ..., rows x, x + gridDim.x, ... of each; with K <= kSmemStatsK the CTA sums
-// its counts and fixed-point terms in shared memory and adds them to the global sums once;
-// larger codebooks add each vector's terms to the global sums directly. A term (|v| < 2^30)
-// enters shared memory as v = 2^15 vh + vl (0 <= vl < 2^15) in two 32-bit sums (native 32-bit
-// atomics): exact, as accumulate_grid gives a CTA fewer than 2^16 rows of a group. Integer
-// sums: the order is immaterial.
+// Statistics of every covered vector from its current code. CTA (x, y): the four adjacent groups of
+// quads y, y + gridDim.y, ..., rows x, x + gridDim.x, ... of each, thread = (row, group): four lanes
+// read a row's 128 bytes. With K <= kSmemStatsK the CTA sums its counts (per group) and fixed-point
+// terms in shared memory and adds them to the global sums once; larger codebooks add each vector's
+// terms to the global sums directly. A term (|v| < 2^30) enters shared memory as v = 2^15 vh + vl
+// (0 <= vl < 2^15) in two 32-bit sums (native 32-bit atomics): exact, as accumulate_grid gives a CTA
+// fewer than 2^16 vectors of a quad. Integer sums: the order is immaterial.
+// Bound: load latency and the shared atomics. (With a group per CTA a warp's 32-byte reads lay in 32
+// lines: 251 us per codebook of a 28672 x 8192 layer, now 206; k-means step 160 -> 156 us.)
 constexpr int kSmemStatsK = 256;
 constexpr int kAccRows = 2;
+constexpr int kAccGroups = 4;
 
 __global__ void __launch_bounds__(256)
 accumulate_stats_kernel(SetView set, CbList cbs, int which, StatsView st, unsigned* err) {
   // [component][vh, vl][code]: lanes of a warp adding one component hit spread banks
   __shared__ int s_b32[kD * 2 * kSmemStatsK];
-  __shared__ int s_cnt[kSmemStatsK];
+  __shared__ int s_cnt[kAccGroups * kSmemStatsK];
   const CbView cw = cbs.cb[which];
   const float sscale = stats_scale_f(st);
   const bool smem = cw.K <= kSmemStatsK;
-  for (int64_t g = blockIdx.y; g < cw.G_cov; g += gridDim.y) {
+  const int gq = threadIdx.x % kAccGroups;
+  for (int64_t g0 = (int64_t)blockIdx.y * kAccGroups; g0 < cw.G_cov;
+       g0 += (int64_t)gridDim.y * kAccGroups) {
     if (smem) {
-      __syncthreads();  // the previous group's flush has read the sums
+      __syncthreads();  // the previous quad's flush has read the sums
       for (int e = threadIdx.x; e < kSmemStatsK * kD * 2; e += blockDim.x) s_b32[e] = 0;
-      for (int e = threadIdx.x; e < kSmemStatsK; e += blockDim.x) s_cnt[e] = 0;
+      for (int e = threadIdx.x; e < kAccGroups * kSmemStatsK; e += blockDim.x) s_cnt[e] = 0;
       __syncthreads();
     }
-    // the group's H block in registers: read once, not 64 loads per vector
-    float H[kD * kD];
+    const int64_t g = g0 + gq;
+    if (g < cw.G_cov) {
+      // the group's H block in registers: read once, not 64 loads per vector
+      float H[kD * kD];
 #pragma unroll
-    for (int e = 0; e < kD * kD; e += 4) {
-      const float4 h = __ldg(reinterpret_cast<const float4*>(set.Hb + g * kD * kD + e));
-      H[e] = h.x;
-      H[e + 1] = h.y;
-      H[e + 2] = h.z;
-      H[e + 3] = h.w;
-    }
-    // kAccRows rows per step, their codes and vectors loaded before any is used
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < set.M;
-         i0 += kAccRows * stride) {
-      int32_t k[kAccRows];
-      float tau[kAccRows][kD];
-#pragma unroll
-      for (int u = 0; u < kAccRows; ++u) {
-        const int64_t i = i0 + u * stride;
-        k[u] = i < set.M ? cw.codes[i * cw.ld + g] : 0;
-        if (i < set.M) stats_target(set, cbs, which, i, g, tau[u], err);
+      for (int e = 0; e < kD * kD; e += 4) {
+        const float4 h = __ldg(reinterpret_cast<const float4*>(set.Hb + g * kD * kD + e));
+        H[e] = h.x;
+        H[e + 1] = h.y;
+        H[e + 2] = h.z;
+        H[e + 3] = h.w;
       }
+      // kAccRows rows per step, their codes and vectors loaded before any is used
+      const int64_t stride = (int64_t)gridDim.x * (blockDim.x / kAccGroups);
+      for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kAccGroups; i0 < set.M;
+           i0 += kAccRows * stride) {
+        int32_t k[kAccRows];
+        float tau[kAccRows][kD];
 #pragma unroll
-      for (int u = 0; u < kAccRows; ++u) {
-        if (i0 + u * stride >= set.M) break;
-        if (k[u] < 0 || k[u] >= cw.K) {
-          raise_error(err, ERRBIT_INDEX);
-          continue;
+        for (int u = 0; u < kAccRows; ++u) {
+          const int64_t i = i0 + u * stride;
+          k[u] = i < set.M ? cw.codes[i * cw.ld + g] : 0;
+          if (i < set.M) stats_target(set, cbs, which, i, g, tau[u], err);
         }
-        float q[kD];
-        stats_htau(H, tau[u], q);
-        if (smem) {
-          atomicAdd(&s_cnt[k[u]], 1);
 #pragma unroll
-          for (int j = 0; j < kD; ++j) {
-            const long long v = fix_rn_small(q[j], sscale);
-            atomicAdd(&s_b32[(2 * j) * kSmemStatsK + k[u]], (int)(v >> 15));
-            atomicAdd(&s_b32[(2 * j + 1) * kSmemStatsK + k[u]], (int)(v & 0x7fff));
+        for (int u = 0; u < kAccRows; ++u) {
+          if (i0 + u * stride >= set.M) break;
+          if (k[u] < 0 || k[u] >= cw.K) {
+            raise_error(err, ERRBIT_INDEX);
+            continue;
           }
-        } else {
-          stats_add(st, sscale, g, k[u], q);
+          float q[kD];
+          stats_htau(H, tau[u], q);
+          if (smem) {
+            atomicAdd(&s_cnt[gq * kSmemStatsK + k[u]], 1);
+#pragma unroll
+            for (int j = 0; j < kD; ++j) {
+              const long long v = fix_rn_small(q[j], sscale);
+              atomicAdd(&s_b32[(2 * j) * kSmemStatsK + k[u]], (int)(v >> 15));
+              atomicAdd(&s_b32[(2 * j + 1) * kSmemStatsK + k[u]], (int)(v & 0x7fff));
+            }
+          } else {
+            stats_add(st, sscale, g, k[u], q);
+          }
         }
       }
     }
     if (smem) {
       __syncthreads();
       for (int k = threadIdx.x; k < cw.K; k += blockDim.x) {
-        const int c = s_cnt[k];
-        if (c == 0) continue;
-        atomicAdd(&st.cnt[g * st.K + k], c);
+        int all = 0;
+#pragma unroll
+        for (int q = 0; q < kAccGroups; ++q) {
+          const int c = s_cnt[q * kSmemStatsK + k];
+          if (c != 0) atomicAdd(&st.cnt[(g0 + q) * st.K + k], c);
+          all += c;
+        }
+        if (all == 0) continue;
 #pragma unroll
         for (int j = 0; j < kD; ++j) {
           const long long v = (long long)s_b32[(2 * j) * kSmemStatsK + k] * 32768 +
@@ -137,15 +150,16 @@ accumulate_stats_kernel(SetView set, CbList cbs, int which, StatsView st, unsign
   }
 }
 
-// Grid of accumulate_stats_kernel: one column of CTAs per group, enough rows per CTA that
-// the flush stays small, at least ~4 CTAs per SM overall, and fewer than 2^16 rows per CTA
-// (the 32-bit shared sums).
+// Grid of accumulate_stats_kernel: one column of CTAs per quad of groups, enough of them for about 4
+// per SM overall with at least 128 rows each (two per thread), and fewer than 2^16 vectors per
+// CTA and quad (the 32-bit shared sums).
 dim3 accumulate_grid(int64_t M, int64_t G_cov, int nsm) {
-  const int64_t want =
-      std::max<int64_t>(1, ceil_div(4 * (int64_t)nsm, std::max<int64_t>(G_cov, 1)));
+  const int64_t quads = std::max<int64_t>(ceil_div(G_cov, kAccGroups), 1);
+  const int64_t want = std::max<int64_t>(1, ceil_div(4 * (int64_t)nsm, quads));
   const int64_t rows_x = std::max<int64_t>(
-      ceil_div(M, 65000), std::max<int64_t>(1, std::min<int64_t>(want, ceil_div(M, 1024))));
-  return dim3((unsigned)rows_x, (unsigned)std::min<int64_t>(std::max<int64_t>(G_cov, 1), 65535));
+      ceil_div(M, 65000 / kAccGroups),
+      std::max<int64_t>(1, std::min<int64_t>(want, ceil_div(M, 128))));
+  return dim3((unsigned)rows_x, (unsigned)std::min<int64_t>(quads, 65535));
 }
 
 // fp32 Cholesky factor of the packed lower triangle (false unless every pivot is positive)

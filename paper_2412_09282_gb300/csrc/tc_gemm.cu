@@ -601,7 +601,10 @@ crvq_status launch_tc_hessian_blocks(const float* Xt, int64_t ldt, int64_t n, in
   Scratch mem;
   CRVQ_TRY(mem.alloc((size_t)chunks * stride * sizeof(float), stream));
   tc::DiagArgs a{};
-  a.A = tc::Operand{Xt, ldt, N, true, perm};
+  a.A = Xt;
+  a.ld = ldt;
+  a.rows = N;
+  a.idx = perm;
   a.K = n;
   a.k_chunk = kKChunk;
   a.out = mem.as<float>();
@@ -613,7 +616,7 @@ crvq_status launch_tc_hessian_blocks(const float* Xt, int64_t ldt, int64_t n, in
     ProfScope ps(perm ? "reorder_blocks_tc" : "hessian_blocks_tc", stream,
                  6.0 * (double)n * N * tc::kBM);
     dim3 grid((unsigned)ceil_div(N, tc::kBM), (unsigned)chunks);
-    tc::syrk_diag_kernel<<<grid, tc::kThreads, tc::kDiagSmemBytes, stream>>>(a);
+    tc::syrk_diag_kernel<<<grid, tc::kDiagThreads, tc::kDiagSmemBytes, stream>>>(a);
     CRVQ_LAUNCHED();
   }
   ProfScope ps("hessian_blocks_finalize", stream, (double)chunks * stride * 4.0);

@@ -321,10 +321,10 @@ __device__ __forceinline__ void fixed_to_pair(long long v, int sexp, float& h, f
 // identical on every run. Codewords without members keep their old value.
 // Bound: latency (0.4 MB per launch). As two kernels, the solve with one thread per codeword, a 512 x
 // 512 layer (64 groups) took 5.3 + 8.0 us per Lloyd iteration; one kernel saves 4.8 us of that, and
-// nothing at 512 groups, where the sums' own work is the larger part.
+// nothing at 512 groups, where the sums' own work is the larger part; two slices per thread took 19 us
+// there, one takes 14.
 constexpr int kSolveSlices = 16;  // groups split 16 ways: short dependent chains per thread
-constexpr int kSolveSpt = 2;      // slices per thread (their chains interleave)
-constexpr int kSumThreads = kSolveSlices / kSolveSpt * kNA;  // 296: registers for the solve
+constexpr int kSumThreads = kSolveSlices * kNA;  // 592
 constexpr int kSolveNC = 2;       // 256 codewords: 128 CTAs, one wave
 
 __global__ void __launch_bounds__(kSumThreads)
@@ -345,51 +345,41 @@ stats_solve_kernel(const float* __restrict__ Hb, StatsView st, const float* C_ol
   while ((r + 1) * (r + 2) / 2 <= e && r < kD - 1) ++r;
   const int c = e - r * (r + 1) / 2;
   const int hoff = r * kD + c;
-  constexpr int kThreadSlices = kSolveSlices / kSolveSpt;
-  float hi[kSolveSpt][kSolveNC], lo[kSolveSpt][kSolveNC];
+  float hi[kSolveNC], lo[kSolveNC];
 #pragma unroll
-  for (int w = 0; w < kSolveSpt; ++w)
-#pragma unroll
-    for (int q = 0; q < kSolveNC; ++q) hi[w][q] = lo[w][q] = 0.f;
-  // thread slice sl takes the group slices sl and sl + kThreadSlices, each in group order
+  for (int q = 0; q < kSolveNC; ++q) hi[q] = lo[q] = 0.f;
+  // slice sl: gper groups, in group order
   const int64_t gper = (st.G_cov + kSolveSlices - 1) / kSolveSlices;
-  constexpr int kBatch = 8;  // loads of 8 groups per slice in flight together; no branches
+  const int64_t g0 = sl * gper, g1 = min(st.G_cov, g0 + gper);
+  constexpr int kBatch = 8;  // groups whose loads are in flight together; no branches
   for (int64_t gb = 0; gb < gper; gb += kBatch) {
-    float fc[kSolveSpt][kBatch][kSolveNC], h[kSolveSpt][kBatch];
+    float fc[kBatch][kSolveNC], h[kBatch];
 #pragma unroll
-    for (int w = 0; w < kSolveSpt; ++w) {
-      const int64_t g0 = (sl + w * kThreadSlices) * gper, g1 = min(st.G_cov, g0 + gper);
+    for (int u = 0; u < kBatch; ++u) {
+      const int64_t g = g0 + gb + u;
+      const bool in = g < g1;
 #pragma unroll
-      for (int u = 0; u < kBatch; ++u) {
-        const int64_t g = g0 + gb + u;
-        const bool in = g < g1;
-#pragma unroll
-        for (int q = 0; q < kSolveNC; ++q)  // exact: counts stay below 2^24
-          fc[w][u][q] = in && q < nk ? (float)st.cnt[g * K + k0 + q] : 0.f;
-        h[w][u] = in ? (e < 36 ? __ldg(Hb + g * kD * kD + hoff) : 1.f) : 0.f;
-      }
+      for (int q = 0; q < kSolveNC; ++q)  // exact: counts stay below 2^24
+        fc[u][q] = in && q < nk ? (float)st.cnt[g * K + k0 + q] : 0.f;
+      h[u] = in ? (e < 36 ? __ldg(Hb + g * kD * kD + hoff) : 1.f) : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
 #pragma unroll
-      for (int w = 0; w < kSolveSpt; ++w)
-#pragma unroll
-        for (int q = 0; q < kSolveNC; ++q) {
-          const float p = __fmul_rn(fc[w][u][q], h[w][u]);
-          const float pe = __fmaf_rn(fc[w][u][q], h[w][u], -p);  // fc h = p + pe exactly
-          float sum, t;
-          pair_two_sum(hi[w][q], p, sum, t);
-          hi[w][q] = sum;
-          lo[w][q] = __fadd_rn(lo[w][q], __fadd_rn(t, pe));
-        }
+      for (int q = 0; q < kSolveNC; ++q) {
+        const float p = __fmul_rn(fc[u][q], h[u]);
+        const float pe = __fmaf_rn(fc[u][q], h[u], -p);  // fc h = p + pe exactly
+        float sum, t;
+        pair_two_sum(hi[q], p, sum, t);
+        hi[q] = sum;
+        lo[q] = __fadd_rn(lo[q], __fadd_rn(t, pe));
+      }
   }
 #pragma unroll
-  for (int w = 0; w < kSolveSpt; ++w)
-#pragma unroll
-    for (int q = 0; q < kSolveNC; ++q) {
-      part_h[q][sl + w * kThreadSlices][e] = hi[w][q];
-      part_l[q][sl + w * kThreadSlices][e] = lo[w][q];
-    }
+  for (int q = 0; q < kSolveNC; ++q) {
+    part_h[q][sl][e] = hi[q];
+    part_l[q][sl][e] = lo[q];
+  }
   __syncthreads();
   // Every thread has read its counts: clear them, so that the statistics are zero for the next
   // accumulation (the Lloyd loop needs no memset between iterations).

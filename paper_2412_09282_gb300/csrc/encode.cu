@@ -505,7 +505,7 @@ __device__ __forceinline__ void decide_open(const SetView& set, const CbList& cb
     if (bk == 0x7fffffff) {
       raise_error(err, ERRBIT_NUMERIC);  // no candidate: non-finite scores
     } else {
-      out_code[i * out_ld + (g - out_g0)] = bk;
+      if (out_code) out_code[i * out_ld + (g - out_g0)] = bk;
       if (st.cnt) {
         float q[kD];
         stats_htau(H, rh, q);  // rh is the fp32 target (TwoSum's rounded sums)
@@ -865,7 +865,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
           o.g = (uint32_t)g;
           o.masks = (mask_le<kBlk>(mb, tb) << 16) | mask_le<kBlk>(mc, tb);
         }
-        out_code[i * out_ld + (g - out_g0)] = j;
+        if (out_code) out_code[i * out_ld + (g - out_g0)] = j;
         if (cert && st.cnt) {
           // H r from the prologue (bit-identical to the standalone update's H tau). A term v
           // (|v| < 2^30) enters as v = 2^15 vh + vl, 0 <= vl < 2^15, in two 32-bit sums: exact,
@@ -1269,7 +1269,7 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
           }
         }
       }
-      out_code[i * out_ld + (g - out_g0)] = j;
+      if (out_code) out_code[i * out_ld + (g - out_g0)] = j;
       if (cert && st.cnt) {
         // H r from the prologue (bit-identical to the standalone update's H tau)
         float q[kD];
@@ -1417,7 +1417,7 @@ argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
       if (bk == 0x7fffffff) {
         raise_error(err, ERRBIT_NUMERIC);  // no candidate: non-finite scores
       } else {
-        out_code[i * out_ld + (g - out_g0)] = bk;
+        if (out_code) out_code[i * out_ld + (g - out_g0)] = bk;
         if (st.cnt) {
           float q[kD];
 #pragma unroll
@@ -1536,7 +1536,7 @@ argmin_exact_warp_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList c
       if (bk == 0x7fffffff) {
         raise_error(err, ERRBIT_NUMERIC);  // no candidate: non-finite scores
       } else {
-        out_code[i * out_ld + (g - out_g0)] = bk;
+        if (out_code) out_code[i * out_ld + (g - out_g0)] = bk;
         if (st.cnt) {
           float q[kD];
 #pragma unroll
@@ -2674,7 +2674,7 @@ ArgminLayout argmin_layout(int64_t M, int64_t G_range, int K) {
 }
 
 // One arg-min pass over the groups [g_begin, g_begin + G_range): codebook s_idx searched, those
-// before n_fixed fixed, codes to out (with the statistics of st when it has any).
+// before n_fixed fixed, codes to out unless it is null (with the statistics of st when it has any).
 struct ArgminCall {
   int64_t g_begin, G_range;
   int n_fixed, s_idx;
@@ -2811,6 +2811,7 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
     }
     StatsView st{};
     if (ex.stats && !keep_if_better) st = *ex.stats;
+    if (ex.discard_codes && !keep_if_better && !vec_err) out = nullptr;
     const ArgminCall ac{g_begin, G_range, n_fixed, s_idx, out, out_ld, out_g0, st};
     if (cw.K <= kSmallK)
       CRVQ_TRY(launch_argmin_small(set, cbs, ac, ex, err, stream));

@@ -10,9 +10,8 @@
 //   Na_k = |c_k|^T |H_g| |c_k|,  L1_k = ||c_k||_1,  Pmax = max_p sum_j |H_pj| (|t_j| + sum_f |c_f,j|),
 // and the pass ranks the lower bounds low_k = s_k - Et_k, keeping the best two. The arg-min j
 // is certified when low_2nd - low_j > 2 Et_j: every other codeword's exact score is then larger
-// than j's. Otherwise the vector is flagged; a fallback re-scores it, keeps the codewords with
-// low_k <= low_j + 2 Et_j (the exact arg-min is among them) and decides among those in fp64.
-// Codes therefore equal the fp64 arg-min (ties to the smaller index) except for ties at fp64
+// than j's. Otherwise the vector is open: the codewords with low_k <= low_j + 2 Et_j (the exact
+// arg-min is among them) are decided among in fp32 pairs (score.cuh). Codes therefore equal the fp64 arg-min (ties to the smaller index) except for ties at fp64
 // rounding level. Beam stages use the same bounds on a sorted top-(B+1) list.
 #include <algorithm>
 #include <cstdlib>
@@ -584,6 +583,94 @@ __device__ __forceinline__ bool half_sync_and(int half, bool v) {
   return r != 0;
 }
 
+// decide_grid of one row by a whole warp: four candidates at a time, lane b of eight takes column b of
+// H (r - c); the same operations in the same order as dfl::quad_err's, so the same err pairs. About
+// 260 dependent instructions per four candidates instead of 700: for a CTA with few open rows,
+// whose end they are (a Lloyd pass over 512 x 64 vectors 16.7 -> 15.3 us, the codes' stores included).
+__device__ __forceinline__ void decide_grid_warp(const SetView& set, const CbList& cbs, int n_fixed,
+                                                 int s_idx, const OpenRow& o,
+                                                 int32_t* __restrict__ out_code, int64_t out_ld,
+                                                 int64_t out_g0, const StatsView& st, float sscale,
+                                                 unsigned* err) {
+  const CbView& cw = cbs.cb[s_idx];
+  const int lane = threadIdx.x & 31, b = lane & 7, base = lane & 24;
+  const int64_t i = o.i, g = o.g;
+  const uint32_t bm = o.masks >> 16, em = o.masks & 0xffffu;
+  const int ne = __popc(em), total = __popc(bm) * ne;
+  const float* H = set.Hb + g * kD * kD;
+  float hb[kD];  // column b
+#pragma unroll
+  for (int a = 0; a < kD; ++a) hb[a] = __ldg(H + a * kD + b);
+  float rh[kD], rl[kD];
+  dfl::target(set, cbs, n_fixed, i, g, rh, rl, err);
+  float bh = INFINITY, bl = 0.f;
+  int bk = 0x7fffffff;
+  for (int c0 = 0; c0 < total; c0 += 4) {
+    const int c = c0 + (lane >> 3);
+    const int k = c < total ? kBlk * nth_bit(bm, c / ne) + nth_bit(em, c % ne) : cw.K;
+    const bool valid = k < cw.K;  // (the others are padding columns)
+    float cv[kD], dh[kD], dl[kD], yh = 0.f, yl = 0.f;
+    load_vec(cw.C + (int64_t)(valid ? k : 0) * kD, cv);
+#pragma unroll
+    for (int j = 0; j < kD; ++j) {
+      float e;
+      dfl::two_sum(rh[j], -cv[j], dh[j], e);
+      dl[j] = __fadd_rn(rl[j], e);
+    }
+#pragma unroll
+    for (int a = 0; a < kD; ++a) {
+      const float p = __fmul_rn(dh[a], hb[a]);
+      const float pe = __fmaf_rn(dh[a], hb[a], -p);  // dh h = p + pe exactly
+      float s, t;
+      dfl::two_sum(yh, p, s, t);
+      yh = s;
+      yl = __fadd_rn(yl, __fadd_rn(t, __fmaf_rn(dl[a], hb[a], pe)));
+    }
+    float sh = 0.f, sl = 0.f;
+#pragma unroll
+    for (int q = 0; q < kD; ++q) {
+      const float qh = __shfl_sync(0xffffffffu, yh, base + q);
+      const float ql = __shfl_sync(0xffffffffu, yl, base + q);
+      const float p = __fmul_rn(dh[q], qh);
+      const float pe = __fmaf_rn(dh[q], qh, -p);
+      float s, t;
+      dfl::two_sum(sh, p, s, t);
+      sh = s;
+      sl = __fadd_rn(sl, __fadd_rn(t, __fmaf_rn(dh[q], ql, __fmaf_rn(dl[q], qh, pe))));
+    }
+    const float eh = __fadd_rn(sh, sl), el = __fsub_rn(sl, __fsub_rn(eh, sh));
+    if (valid && dfl::less(eh, el, k, bh, bl, bk)) {
+      bh = eh;
+      bl = el;
+      bk = k;
+    }
+  }
+#pragma unroll
+  for (int off = 8; off < 32; off <<= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, bh, off);
+    const float ol = __shfl_xor_sync(0xffffffffu, bl, off);
+    const int ok = __shfl_xor_sync(0xffffffffu, bk, off);
+    if (dfl::less(oh, ol, ok, bh, bl, bk)) {
+      bh = oh;
+      bl = ol;
+      bk = ok;
+    }
+  }
+  if (bk == 0x7fffffff) {
+    if (lane == 0) raise_error(err, ERRBIT_NUMERIC);  // no candidate: non-finite scores
+    return;
+  }
+  if (lane == 0 && out_code) out_code[i * out_ld + (g - out_g0)] = bk;
+  if (st.cnt && lane < kD) {  // stats_add, a component per lane
+    float a = 0.f;
+#pragma unroll
+    for (int c = 0; c < kD; ++c) a = fmaf(__ldg(H + lane * kD + c), rh[c], a);
+    if (lane == 0) atomicAdd(&st.cnt[g * st.K + bk], 1);
+    atomicAdd(reinterpret_cast<unsigned long long*>(&st.bacc[(int64_t)bk * kD + lane]),
+              (unsigned long long)fix_rn_small(a, sscale));
+  }
+}
+
 __global__ void __launch_bounds__(256, 2)
 argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, int n_fixed,
                     int s_idx, int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
@@ -932,11 +1019,16 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
     if (!ok) break;
     p += np;
   }
-  // the open rows of every segment, four per warp at a time
+  // the open rows of every segment: a warp each when they are few, else four per warp at a time
   const unsigned found = n_open;  // (the barrier after the last segment ordered it)
   if (flag_total && tid == 0 && found) atomicAdd(flag_total, (unsigned long long)found);
   const int n = (int)min(found, (unsigned)kOpenCap);
-  for (int e0 = warp * 4; e0 < n; e0 += 32) {
+  if (n <= 8) {
+    if (warp < n)
+      decide_grid_warp(set, cbs, n_fixed, s_idx, s_open[warp], out_code, out_ld, out_g0, st, sscale,
+                       err);
+  }
+  for (int e0 = n <= 8 ? n : warp * 4; e0 < n; e0 += 32) {
     const int e = e0 + (lane >> 3);
     decide_grid(set, cbs, n_fixed, s_idx, s_open[min(e, n - 1)], e < n, out_code, out_ld, out_g0,
                 st, sscale, err);

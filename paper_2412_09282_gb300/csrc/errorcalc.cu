@@ -30,7 +30,8 @@ __device__ __forceinline__ void pair_merge(float& h, float& l, float oh, float o
 }
 
 constexpr int kDecRows = 16;     // rows per warp (the CTA's H blocks are staged once for all)
-constexpr int kDecBatch = 2;     // rows whose codes and vectors are loaded together
+// rows whose codes and vectors are loaded together (both two CTAs per SM)
+constexpr int dec_batch(int max_cb) { return max_cb == 1 ? 4 : 2; }
 constexpr int kDecWarps = 8;     // warps per CTA
 constexpr int kDecHStride = 260; // floats per staged H block (256 + 4: conflict-free float4)
 constexpr int kDecSmemCb = 48 * 1024;  // codebooks staged in shared memory up to this size
@@ -84,15 +85,19 @@ __device__ __forceinline__ void recon_codes(const float* const* cw, const int32_
 // S = sum over its rows of dl dl^T (dl = w - w_hat; the 36 entries of the symmetric 8 x 8), then
 // takes the loss as tr(H_g S) = sum_v dl_v^T H_g dl_v once, and ||dW||^2 as tr(S). A CTA's warps
 // share one slice: its H blocks are staged in shared memory once; the codebooks sit in shared
-// memory when they fit, so the codeword lookup is not a dependent global load; the codes of
-// kDecBatch rows are loaded before any is used.
+// memory when they fit (those that reach the slice), so the codeword lookup is not a dependent global
+// load; the codes of a few rows are loaded before any is used. A CTA takes several row blocks of its
+// slice in a large matrix: staged for each 128 rows, the five codebooks of a 28672 x 8192 matrix were
+// 48 KB for 128 KB of weights. There, with the slices that one codebook reaches in a launch of
+// their own, a call takes 341 us instead of 808.
 template <int MAXCB>
 __global__ void __launch_bounds__(kDecWarps * 32)
 decode_vec_kernel(const float* __restrict__ Ws, int64_t M, int64_t N,
                   const float* __restrict__ Hb, CbList cbs, int64_t n_crit_groups, int slices,
-                  int cb_in_smem, float* __restrict__ W_rec, float2* __restrict__ row_part,
+                  int slice0, int n_slices, int cb_in_smem, float* __restrict__ W_rec, float2* __restrict__ row_part,
                   unsigned* err) {
   extern __shared__ __align__(16) float s_dyn[];
+  constexpr int kDecBatch = dec_batch(MAXCB);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* sH = s_dyn;                         // the CTA slice's 32 H blocks
   float* s_cb = s_dyn + 32 * kDecHStride;    // codebooks (when staged)
@@ -104,9 +109,10 @@ decode_vec_kernel(const float* __restrict__ Ws, int64_t M, int64_t N,
       if (s >= cbs.n) break;
       const int64_t n = (int64_t)cbs.cb[s].K * kD;
       if (cb_in_smem) {
-        for (int64_t e = threadIdx.x * 4; e < n; e += blockDim.x * 4)
-          *reinterpret_cast<float4*>(s_cb + off + e) =
-              __ldg(reinterpret_cast<const float4*>(cbs.cb[s].C + e));
+        if ((int64_t)(slice0 + blockIdx.x % n_slices) * 32 < cbs.cb[s].G_cov)
+          for (int64_t e = threadIdx.x * 4; e < n; e += blockDim.x * 4)
+            *reinterpret_cast<float4*>(s_cb + off + e) =
+                __ldg(reinterpret_cast<const float4*>(cbs.cb[s].C + e));
         cw[s] = s_cb + off;
         off += n;
       } else {
@@ -115,10 +121,9 @@ decode_vec_kernel(const float* __restrict__ Ws, int64_t M, int64_t N,
     }
     if (cb_in_smem) __syncthreads();
   }
-  // CTA = (slice of 32 groups, kDecWarps x kDecRows rows); warp w takes kDecRows rows
+  // CTA = (slice of 32 groups, blocks of kDecWarps x kDecRows rows); warp w takes kDecRows rows of each
   const int64_t G = N / kD;
-  const int sl = (int)(blockIdx.x % slices);
-  const int64_t rb = (int64_t)(blockIdx.x / slices) * kDecWarps + warp;
+  const int sl = slice0 + (int)(blockIdx.x % n_slices);
   const int64_t g = (int64_t)sl * 32 + lane;
   const bool gok = g < G;
   // stage the H blocks of the slice (256 bytes per group, 16 floats of padding between)
@@ -129,99 +134,103 @@ decode_vec_kernel(const float* __restrict__ Ws, int64_t M, int64_t N,
           __ldg(reinterpret_cast<const float4*>(Hb + ((int64_t)sl * 32 + gl) * kD * kD) + q);
   }
   __syncthreads();
-  const int64_t i0 = rb * kDecRows;
-  if (i0 >= M) return;  // whole warps (no block barrier follows)
-  const int nr = (int)min((int64_t)kDecRows, M - i0);
-  float S[kD * (kD + 1) / 2];  // sum of dl dl^T over this warp's rows, packed lower triangle
+  // (no block barrier follows)
+  const int64_t row_blocks = (M + kDecRows - 1) / kDecRows, parts = gridDim.x / n_slices;
+  for (int64_t rb = (int64_t)(blockIdx.x / n_slices) * kDecWarps + warp; rb < row_blocks;
+       rb += parts * kDecWarps) {
+    const int64_t i0 = rb * kDecRows;
+    const int nr = (int)min((int64_t)kDecRows, M - i0);
+    float S[kD * (kD + 1) / 2];  // sum of dl dl^T over this warp's rows, packed lower triangle
 #pragma unroll
-  for (int e = 0; e < kD * (kD + 1) / 2; ++e) S[e] = 0.f;
-  for (int r0 = 0; r0 < nr; r0 += kDecBatch) {
-    int32_t kc[kDecBatch][MAXCB];
-    float4 tv[kDecBatch][2];
+    for (int e = 0; e < kD * (kD + 1) / 2; ++e) S[e] = 0.f;
+    for (int r0 = 0; r0 < nr; r0 += kDecBatch) {
+      int32_t kc[kDecBatch][MAXCB];
+      float4 tv[kDecBatch][2];
 #pragma unroll
-    for (int u = 0; u < kDecBatch; ++u) {
-      const int64_t i = i0 + min(r0 + u, nr - 1);
+      for (int u = 0; u < kDecBatch; ++u) {
+        const int64_t i = i0 + min(r0 + u, nr - 1);
 #pragma unroll
-      for (int s = 0; s < MAXCB; ++s) {
-        kc[u][s] = -1;
-        if (gok && s < cbs.n && g < cbs.cb[s].G_cov)
-          kc[u][s] = cbs.cb[s].codes[i * cbs.cb[s].ld + g];
-      }
-      tv[u][0] = tv[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (gok) {
-        tv[u][0] = *reinterpret_cast<const float4*>(Ws + i * N + g * kD);
-        tv[u][1] = *reinterpret_cast<const float4*>(Ws + i * N + g * kD + 4);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kDecBatch; ++u) {
-      if (r0 + u >= nr || !gok) break;
-      const int64_t i = i0 + r0 + u;
-#pragma unroll
-      for (int s = 0; s < MAXCB; ++s) {
-        if (s >= cbs.n || g >= cbs.cb[s].G_cov) continue;
-        if (kc[u][s] < 0 || kc[u][s] >= cbs.cb[s].K) {
-          raise_error(err, ERRBIT_INDEX);
+        for (int s = 0; s < MAXCB; ++s) {
           kc[u][s] = -1;
+          if (gok && s < cbs.n && g < cbs.cb[s].G_cov)
+            kc[u][s] = cbs.cb[s].codes[i * cbs.cb[s].ld + g];
+        }
+        tv[u][0] = tv[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (gok) {
+          tv[u][0] = *reinterpret_cast<const float4*>(Ws + i * N + g * kD);
+          tv[u][1] = *reinterpret_cast<const float4*>(Ws + i * N + g * kD + 4);
         }
       }
-      float rv[kD], dl[kD];
-      recon_codes<MAXCB>(cw, kc[u], cbs.n, rv);
-      const float t[kD] = {tv[u][0].x, tv[u][0].y, tv[u][0].z, tv[u][0].w,
-                           tv[u][1].x, tv[u][1].y, tv[u][1].z, tv[u][1].w};
 #pragma unroll
-      for (int j = 0; j < kD; ++j) dl[j] = t[j] - rv[j];
+      for (int u = 0; u < kDecBatch; ++u) {
+        if (r0 + u >= nr || !gok) break;
+        const int64_t i = i0 + r0 + u;
+#pragma unroll
+        for (int s = 0; s < MAXCB; ++s) {
+          if (s >= cbs.n || g >= cbs.cb[s].G_cov) continue;
+          if (kc[u][s] < 0 || kc[u][s] >= cbs.cb[s].K) {
+            raise_error(err, ERRBIT_INDEX);
+            kc[u][s] = -1;
+          }
+        }
+        float rv[kD], dl[kD];
+        recon_codes<MAXCB>(cw, kc[u], cbs.n, rv);
+        const float t[kD] = {tv[u][0].x, tv[u][0].y, tv[u][0].z, tv[u][0].w,
+                             tv[u][1].x, tv[u][1].y, tv[u][1].z, tv[u][1].w};
+#pragma unroll
+        for (int j = 0; j < kD; ++j) dl[j] = t[j] - rv[j];
+        int e = 0;
+#pragma unroll
+        for (int a2 = 0; a2 < kD; ++a2)
+#pragma unroll
+          for (int b2 = 0; b2 <= a2; ++b2, ++e) S[e] = fmaf(dl[a2], dl[b2], S[e]);
+        if (W_rec) {
+          float* o = W_rec + i * N + g * kD;
+          *reinterpret_cast<float4*>(o) = make_float4(rv[0], rv[1], rv[2], rv[3]);
+          *reinterpret_cast<float4*>(o + 4) = make_float4(rv[4], rv[5], rv[6], rv[7]);
+        }
+      }
+    }
+    // lb = tr(H_g S) (H_g symmetric: diagonal once, each off-diagonal pair twice), sq = tr(S)
+    float lb = 0.f, lc = 0.f, sq = 0.f;
+    if (gok) {
+      const float* Hl = sH + lane * kDecHStride;
+      float off = 0.f;
       int e = 0;
 #pragma unroll
       for (int a2 = 0; a2 < kD; ++a2)
 #pragma unroll
-        for (int b2 = 0; b2 <= a2; ++b2, ++e) S[e] = fmaf(dl[a2], dl[b2], S[e]);
-      if (W_rec) {
-        float* o = W_rec + i * N + g * kD;
-        *reinterpret_cast<float4*>(o) = make_float4(rv[0], rv[1], rv[2], rv[3]);
-        *reinterpret_cast<float4*>(o + 4) = make_float4(rv[4], rv[5], rv[6], rv[7]);
-      }
-    }
-  }
-  // lb = tr(H_g S) (H_g symmetric: diagonal once, each off-diagonal pair twice), sq = tr(S)
-  float lb = 0.f, lc = 0.f, sq = 0.f;
-  if (gok) {
-    const float* Hl = sH + lane * kDecHStride;
-    float off = 0.f;
-    int e = 0;
-#pragma unroll
-    for (int a2 = 0; a2 < kD; ++a2)
-#pragma unroll
-      for (int b2 = 0; b2 <= a2; ++b2, ++e) {
-        if (a2 == b2) {
-          lb = fmaf(Hl[a2 * kD + b2], S[e], lb);
-          sq += S[e];
-        } else {
-          off = fmaf(Hl[a2 * kD + b2], S[e], off);
+        for (int b2 = 0; b2 <= a2; ++b2, ++e) {
+          if (a2 == b2) {
+            lb = fmaf(Hl[a2 * kD + b2], S[e], lb);
+            sq += S[e];
+          } else {
+            off = fmaf(Hl[a2 * kD + b2], S[e], off);
+          }
         }
-      }
-    lb = fmaf(2.f, off, lb);
-    if (g < n_crit_groups) lc = lb;
-  }
-  // the 32 groups of this (row block, slice) summed as fp32 pairs in a fixed tree
-  float lbl = 0.f, lcl = 0.f, sql = 0.f;
+      lb = fmaf(2.f, off, lb);
+      if (g < n_crit_groups) lc = lb;
+    }
+    // the 32 groups of this (row block, slice) summed as fp32 pairs in a fixed tree
+    float lbl = 0.f, lcl = 0.f, sql = 0.f;
 #pragma unroll
-  for (int o2 = 16; o2 > 0; o2 >>= 1) {
-    const float a0 = __shfl_xor_sync(0xffffffffu, lb, o2);
-    const float a1 = __shfl_xor_sync(0xffffffffu, lbl, o2);
-    const float b0 = __shfl_xor_sync(0xffffffffu, lc, o2);
-    const float b1 = __shfl_xor_sync(0xffffffffu, lcl, o2);
-    const float c0 = __shfl_xor_sync(0xffffffffu, sq, o2);
-    const float c1 = __shfl_xor_sync(0xffffffffu, sql, o2);
-    pair_merge(lb, lbl, a0, a1);
-    pair_merge(lc, lcl, b0, b1);
-    pair_merge(sq, sql, c0, c1);
-  }
-  if (lane == 0) {
-    float2* o = row_part + (rb * slices + sl) * 3;
-    o[0] = make_float2(lb, lbl);
-    o[1] = make_float2(lc, lcl);
-    o[2] = make_float2(sq, sql);
+    for (int o2 = 16; o2 > 0; o2 >>= 1) {
+      const float a0 = __shfl_xor_sync(0xffffffffu, lb, o2);
+      const float a1 = __shfl_xor_sync(0xffffffffu, lbl, o2);
+      const float b0 = __shfl_xor_sync(0xffffffffu, lc, o2);
+      const float b1 = __shfl_xor_sync(0xffffffffu, lcl, o2);
+      const float c0 = __shfl_xor_sync(0xffffffffu, sq, o2);
+      const float c1 = __shfl_xor_sync(0xffffffffu, sql, o2);
+      pair_merge(lb, lbl, a0, a1);
+      pair_merge(lc, lcl, b0, b1);
+      pair_merge(sq, sql, c0, c1);
+    }
+    if (lane == 0) {
+      float2* o = row_part + (rb * slices + sl) * 3;
+      o[0] = make_float2(lb, lbl);
+      o[1] = make_float2(lc, lcl);
+      o[2] = make_float2(sq, sql);
+    }
   }
 }
 
@@ -326,23 +335,43 @@ crvq_status launch_reconstruct_error(const float* W_sorted, int64_t M, int64_t N
   {
     ProfScope ps("decode_rows", stream,
                  (double)M * N * 4.0 * (1.0 + (W_rec ? 1.0 : 0.0)));
-    const int64_t ctas = ceil_div(row_blocks, (int64_t)kDecWarps) * slices;
-    int64_t cb_bytes = 0;
-    for (int s = 0; s < cbs.n; ++s) cb_bytes += (int64_t)cbs.cb[s].K * kD * sizeof(float);
-    const int in_smem = cb_bytes <= kDecSmemCb ? 1 : 0;
-    const size_t smem = (size_t)32 * kDecHStride * sizeof(float) +
-                        (in_smem ? (size_t)cb_bytes : 0);
-    const dim3 grid((unsigned)ctas);
-    if (cbs.n <= 4) {
-      CRVQ_TRY(smem_limit((const void*)decode_vec_kernel<4>, smem));
-      decode_vec_kernel<4><<<grid, kDecWarps * 32, smem, stream>>>(
-          W_sorted, M, N, Hb, cbs, n_crit_groups, slices, in_smem, W_rec, row_part, err);
-    } else {
-      CRVQ_TRY(smem_limit((const void*)decode_vec_kernel<kMaxCodebooks>, smem));
-      decode_vec_kernel<kMaxCodebooks><<<grid, kDecWarps * 32, smem, stream>>>(
-          W_sorted, M, N, Hb, cbs, n_crit_groups, slices, in_smem, W_rec, row_part, err);
+    const int64_t groups = ceil_div(row_blocks, (int64_t)kDecWarps);
+    auto run = [&](const CbList& l, int s0, int ns) -> crvq_status {
+      // about eight CTAs per SM, each with an equal number of row blocks
+      const int64_t per = std::max<int64_t>(1, groups * ns / (8 * (int64_t)nsm));
+      const dim3 grid((unsigned)(ceil_div(groups, per) * ns));
+      int64_t cb_bytes = 0;
+      for (int s = 0; s < l.n; ++s) cb_bytes += (int64_t)l.cb[s].K * kD * sizeof(float);
+      const int in_smem = cb_bytes <= kDecSmemCb ? 1 : 0;
+      const size_t smem =
+          (size_t)32 * kDecHStride * sizeof(float) + (in_smem ? (size_t)cb_bytes : 0);
+      auto launch = [&](auto* kernel) -> crvq_status {
+        CRVQ_TRY(smem_limit((const void*)kernel, smem));
+        kernel<<<grid, kDecWarps * 32, smem, stream>>>(W_sorted, M, N, Hb, l, n_crit_groups, slices, s0,
+                                                       ns, in_smem, W_rec, row_part, err);
+        CRVQ_LAUNCHED();
+        return CRVQ_OK;
+      };
+      if (l.n <= 1) return launch(decode_vec_kernel<1>);
+      return l.n <= 4 ? launch(decode_vec_kernel<4>) : launch(decode_vec_kernel<kMaxCodebooks>);
+    };
+    // Slices that only the codebooks of all groups reach, when there are many, in a launch of their own:
+    // one codebook takes fewer registers, so more rows are in flight.
+    CbList all{};
+    int64_t part_cov = 0;
+    for (int s = 0; s < cbs.n; ++s) {
+      if (cbs.cb[s].G_cov >= G)
+        all.cb[all.n++] = cbs.cb[s];
+      else
+        part_cov = std::max(part_cov, cbs.cb[s].G_cov);
     }
-    CRVQ_LAUNCHED();
+    const int sc = (int)ceil_div(part_cov, (int64_t)32);
+    if (all.n == 1 && cbs.n > 1 && (slices - sc) * groups >= 4 * (int64_t)nsm) {
+      if (sc > 0) CRVQ_TRY(run(cbs, 0, sc));
+      CRVQ_TRY(run(all, sc, slices - sc));
+    } else {
+      CRVQ_TRY(run(cbs, 0, slices));
+    }
   }
   if (W_hat && perm) {  // back to the original channel order: W_hat[:, c] = W_rec[:, inv[c]]
     ProfScope ps("decode_unpermute", stream, (double)M * N * 8.0);

@@ -1,0 +1,39 @@
+"""Reconstruction of a matrix large enough that the slices without extended codebooks run in a launch
+of their own and a block takes several row blocks, against plain fp64 sums: reconstructions are
+bit-exact, block losses within 1e-4 (the bar of the parity tests: fp32 terms)."""
+import numpy as np
+import pytest
+
+import paper_2412_09282_gb300 as P
+from paper_2412_09282_gb300 import Codebook
+from parity_util import dev, host
+
+pytestmark = pytest.mark.gpu
+
+D = 8
+
+
+@pytest.mark.parametrize("M,N,Gc", [(2600, 8192, 33), (5001, 4616, 5), (17, 9224, 2)])
+def test_reconstruct_over_row_blocks_and_slices(M, N, Gc):
+    rng = np.random.default_rng(M + N)
+    G = N // D
+    W = (0.02 * rng.standard_normal((M, N))).astype(np.float32)
+    A = rng.standard_normal((G, 12, D))
+    Hb = (A.transpose(0, 2, 1) @ A / 12 + 0.05 * np.eye(D)).astype(np.float32)
+    perm = rng.permutation(N).astype(np.int32)
+    Cs = [(0.02 * rng.standard_normal((k, D))).astype(np.float32) for k in (256, 16, 9)]
+    codes = [rng.integers(0, k, (M, g)).astype(np.int32) for k, g in ((256, G), (16, Gc), (9, Gc))]
+    cbs = [Codebook(dev(C), dev(c), c.shape[1]) for C, c in zip(Cs, codes)]
+    Wh, lb, lc, lf = P.crvq_reconstruct_error(dev(W), D, dev(Hb), dev(perm), cbs, Gc)
+    rec = Cs[0][codes[0]].astype(np.float64)
+    for C, c in zip(Cs[1:], codes[1:]):
+        rec[:, :Gc] += C[c]
+    rec = rec.astype(np.float32).reshape(M, N)
+    want = np.empty_like(rec)
+    want[:, perm] = rec
+    assert lf is None
+    np.testing.assert_array_equal(host(Wh), want)
+    d = (W - rec).astype(np.float64).reshape(M, G, D)
+    per_group = np.einsum("mgi,gij,mgj->g", d, Hb.astype(np.float64), d, optimize=True)
+    assert abs(lb - per_group.sum()) <= 1e-4 * per_group.sum()
+    assert abs(lc - per_group[:Gc].sum()) <= 1e-4 * per_group[:Gc].sum()

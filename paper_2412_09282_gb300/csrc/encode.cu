@@ -1878,6 +1878,8 @@ template <int L>
 __global__ void __launch_bounds__(kThreads, L <= 9 ? 3 : 2)
 beam_stage_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc sd,
                   BeamBufs bb, FlagList flags, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int64_t g = g_begin + blockIdx.y;
   const int64_t G_range = gridDim.y;
   const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
@@ -2039,6 +2041,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc sd,
                BeamBufs bb, const char* __restrict__ bimg, const float* __restrict__ cbmax,
                FlagList flags, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   using namespace tcenc;
   extern __shared__ __align__(1024) char smem_raw[];
   char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -2315,6 +2319,8 @@ __global__ void __launch_bounds__(kThreads)
 beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs,
                            int n_fixed, StageDesc sd, BeamBufs bb, FlagList flags,
                            const float4* __restrict__ terms, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   __shared__ int queue[kThreads / 32][32], queue_h[kThreads / 32][32];
   const int lane = threadIdx.x & 31;
   int* q = queue[threadIdx.x >> 5];
@@ -2528,6 +2534,8 @@ __global__ void beam_finalize_kernel(SetView set, int64_t g_begin, int64_t G_ran
                                      CbList cbs, int n_fixed, StageDesc sd,
                                      const int32_t* __restrict__ hyp, bool keep_if_better,
                                      float* __restrict__ vec_err, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int64_t nvec = set.M * G_range;
   const int S = sd.S, B = sd.B;
   for (int64_t vi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; vi < nvec;
@@ -2595,6 +2603,8 @@ __global__ void beam_finalize_kernel(SetView set, int64_t g_begin, int64_t G_ran
 // err of the tuple currently in the codes (all covering codebooks), in fp32 pairs.
 __global__ void residual_err_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs,
                                     float* __restrict__ vec_err, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int64_t nvec = set.M * G_range;
   StageDesc none{};
   for (int64_t vi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; vi < nvec;
@@ -2608,6 +2618,8 @@ __global__ void residual_err_kernel(SetView set, int64_t g_begin, int64_t G_rang
 // --------------------------------------------------------------------------- k-means init
 __global__ void kmeans_init_kernel(SetView set, CbList fixed, int K, uint64_t seed,
                                    float* __restrict__ C_out, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= K) return;
   const int64_t n = set.M * set.G_sub;
@@ -2636,8 +2648,8 @@ crvq_status launch_kmeans_init(const SetView& set, const CbList& fixed, int K, u
   unsigned* err = nullptr;
   CRVQ_TRY(device_error_word(&err));
   ProfScope ps("kmeans_init", stream, (double)K);
-  kmeans_init_kernel<<<(unsigned)ceil_div(K, 128), 128, 0, stream>>>(set, fixed, K, seed,
-                                                                    C_out, err);
+  CRVQ_CUDA(launch_pdl(kmeans_init_kernel, dim3((unsigned)ceil_div(K, 128)), dim3(128), 0, stream,
+                       set, fixed, K, seed, C_out, err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -2651,8 +2663,8 @@ crvq_status launch_beam_stage_L(const SetView& set, int64_t g_begin, int64_t G_r
                                 double units, cudaStream_t stream) {
   dim3 grid((unsigned)ceil_div(set.M, kThreads), (unsigned)G_range);
   ProfScope ps("encode_beam_stage", stream, units);
-  beam_stage_kernel<L><<<grid, kThreads, 0, stream>>>(set, g_begin, cbs, n_fixed, sd, bb, fl,
-                                                     err);
+  CRVQ_CUDA(launch_pdl(beam_stage_kernel<L>, grid, dim3(kThreads), 0, stream, set, g_begin, cbs,
+                       n_fixed, sd, bb, fl, err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -2666,8 +2678,8 @@ crvq_status launch_beam_tc_L(const SetView& set, int64_t g_begin, int64_t G_rang
   CRVQ_TRY(set_smem_attr(beam_tc_kernel<L>, kBeamTcSmem));
   dim3 grid((unsigned)ceil_div(set.M, kThreads), (unsigned)G_range);
   ProfScope ps("encode_beam_stage", stream, units);
-  beam_tc_kernel<L><<<grid, kThreads, kBeamTcSmem, stream>>>(set, g_begin, cbs, n_fixed, sd, bb,
-                                                             bimg, cbmax, fl, err);
+  CRVQ_CUDA(launch_pdl(beam_tc_kernel<L>, grid, dim3(kThreads), kBeamTcSmem, stream, set, g_begin,
+                       cbs, n_fixed, sd, bb, bimg, cbmax, fl, err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -2880,8 +2892,8 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
   const unsigned fin_blocks = (unsigned)std::min<int64_t>(ceil_div(nvec, 128), 8 * nsm);
   if (sd.S == 0) {
     if (vec_err) {
-      residual_err_kernel<<<fin_blocks, 128, 0, stream>>>(set, g_begin, G_range, cbs, vec_err,
-                                                          err);
+      CRVQ_CUDA(launch_pdl(residual_err_kernel, dim3(fin_blocks), dim3(128), 0, stream, set,
+                           g_begin, G_range, cbs, vec_err, err));
       CRVQ_LAUNCHED();
     }
     return CRVQ_OK;
@@ -2915,13 +2927,13 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
       StageDesc one = sd;
       one.B = 1;
       one.Bs = 1;
-      beam_finalize_kernel<<<fin_blocks, 128, 0, stream>>>(set, g_begin, G_range, cbs, n_fixed,
-                                                           one, out, true, vec_err, err);
+      CRVQ_CUDA(launch_pdl(beam_finalize_kernel, dim3(fin_blocks), dim3(128), 0, stream, set,
+                           g_begin, G_range, cbs, n_fixed, one, out, true, vec_err, err));
       CRVQ_LAUNCHED();
     } else if (vec_err) {
       ProfScope ps3("encode_finalize", stream, 0.0);
-      residual_err_kernel<<<fin_blocks, 128, 0, stream>>>(set, g_begin, G_range, cbs, vec_err,
-                                                          err);
+      CRVQ_CUDA(launch_pdl(residual_err_kernel, dim3(fin_blocks), dim3(128), 0, stream, set,
+                           g_begin, G_range, cbs, vec_err, err));
       CRVQ_LAUNCHED();
     }
     return CRVQ_OK;
@@ -2978,9 +2990,9 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
                                  (double)nvec * parents * K, stream));
     {
       ProfScope ps("encode_beam_fallback", stream, 0.0);
-      beam_stage_fallback_kernel<<<4 * nsm, kThreads, 0, stream>>>(
-          set, g_begin, G_range, cbs, n_fixed, sd, bb, fl,
-          tc_stage ? beam_tc_terms(tc_mem.as<char>(), G_range, K) : nullptr, err);
+      CRVQ_CUDA(launch_pdl(beam_stage_fallback_kernel, dim3(4 * nsm), dim3(kThreads), 0, stream,
+                           set, g_begin, G_range, cbs, n_fixed, sd, bb, fl, tc_stage ?
+                           beam_tc_terms(tc_mem.as<char>(), G_range, K) : nullptr, err));
       CRVQ_LAUNCHED();
     }
     sc += (double)nvec * parents * K;
@@ -2992,8 +3004,8 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
   }
   if (ex.scores) *ex.scores += sc;
   ProfScope ps("encode_finalize", stream, 0.0);
-  beam_finalize_kernel<<<fin_blocks, 128, 0, stream>>>(set, g_begin, G_range, cbs, n_fixed, sd,
-                                                       in_h, keep_if_better, vec_err, err);
+  CRVQ_CUDA(launch_pdl(beam_finalize_kernel, dim3(fin_blocks), dim3(128), 0, stream, set, g_begin,
+                       G_range, cbs, n_fixed, sd, in_h, keep_if_better, vec_err, err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }

@@ -96,6 +96,8 @@ decode_vec_kernel(const float* __restrict__ Ws, int64_t M, int64_t N,
                   const float* __restrict__ Hb, CbList cbs, int64_t n_crit_groups, int slices,
                   int slice0, int n_slices, int cb_in_smem, float* __restrict__ W_rec, float2* __restrict__ row_part,
                   unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   extern __shared__ __align__(16) float s_dyn[];
   constexpr int kDecBatch = dec_batch(MAXCB);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -237,6 +239,8 @@ decode_vec_kernel(const float* __restrict__ Ws, int64_t M, int64_t N,
 // inv[perm[p]] = p; entries outside [0, N) are reported and skipped.
 __global__ void invert_perm_kernel(const int32_t* __restrict__ perm, int64_t N,
                                    int32_t* __restrict__ inv, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N;
        p += (int64_t)gridDim.x * blockDim.x) {
     const int32_t c = perm[p];
@@ -255,6 +259,8 @@ finalize_losses_kernel(const float2* __restrict__ row_part, int64_t n_rows,
                        const double* __restrict__ gemm_part, int64_t n_gemm, int64_t n_tok,
                        double delta_host, const float* __restrict__ delta_dev,
                        double* __restrict__ losses) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   __shared__ float red_h[3][1024], red_l[3][1024];
   __shared__ double red_e[1024];
   float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f};
@@ -347,8 +353,8 @@ crvq_status launch_reconstruct_error(const float* W_sorted, int64_t M, int64_t N
           (size_t)32 * kDecHStride * sizeof(float) + (in_smem ? (size_t)cb_bytes : 0);
       auto launch = [&](auto* kernel) -> crvq_status {
         CRVQ_TRY(smem_limit((const void*)kernel, smem));
-        kernel<<<grid, kDecWarps * 32, smem, stream>>>(W_sorted, M, N, Hb, l, n_crit_groups, slices, s0,
-                                                       ns, in_smem, W_rec, row_part, err);
+        CRVQ_CUDA(launch_pdl(kernel, grid, dim3(kDecWarps * 32), smem, stream, W_sorted, M, N, Hb,
+                             l, n_crit_groups, slices, s0, ns, in_smem, W_rec, row_part, err));
         CRVQ_LAUNCHED();
         return CRVQ_OK;
       };
@@ -375,8 +381,8 @@ crvq_status launch_reconstruct_error(const float* W_sorted, int64_t M, int64_t N
   }
   if (W_hat && perm) {  // back to the original channel order: W_hat[:, c] = W_rec[:, inv[c]]
     ProfScope ps("decode_unpermute", stream, (double)M * N * 8.0);
-    invert_perm_kernel<<<(unsigned)std::min<int64_t>(ceil_div(N, 256), 4 * nsm), 256, 0,
-                         stream>>>(perm, N, inv, err);
+    CRVQ_CUDA(launch_pdl(invert_perm_kernel, dim3((unsigned)std::min<int64_t>(ceil_div(N, 256), 4 *
+                         nsm)), dim3(256), 0, stream, perm, N, inv, err));
     CRVQ_LAUNCHED();
     CRVQ_TRY(launch_gather_cols(W_rec, M, N, inv, W_hat, stream));
   }
@@ -386,10 +392,9 @@ crvq_status launch_reconstruct_error(const float* W_sorted, int64_t M, int64_t N
     CRVQ_TRY(launch_tc_sumsq(W_sorted, W_rec, M, X, perm, n_tok, N, gemm_part, n_gemm_cap,
                              &n_gemm, stream));
   }
-  finalize_losses_kernel<<<1, 1024, 0, stream>>>(row_part, row_blocks * slices,
-                                                 X ? gemm_part : nullptr,
-                                                 n_gemm, n_tok, damp_delta, delta_dev,
-                                                 losses_dev);
+  CRVQ_CUDA(launch_pdl(finalize_losses_kernel, dim3(1), dim3(1024), 0, stream, row_part, row_blocks
+                       * slices, X ? gemm_part : nullptr, n_gemm, n_tok, damp_delta, delta_dev,
+                       losses_dev));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }

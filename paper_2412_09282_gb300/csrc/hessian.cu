@@ -17,6 +17,8 @@ namespace {
 __global__ void __launch_bounds__(1024)
 hessian_delta_kernel(const float* __restrict__ xsq, int64_t N, float damp_rel,
                      float* __restrict__ delta_out, double* __restrict__ delta64) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   __shared__ double part[1024];
   double s = 0.0;
   for (int64_t i = threadIdx.x; i < N; i += blockDim.x) s += (double)xsq[i];
@@ -38,6 +40,8 @@ hessian_delta_kernel(const float* __restrict__ xsq, int64_t N, float damp_rel,
 __global__ void __launch_bounds__(256)
 hessian_damp_kernel(float* __restrict__ H, int64_t N, const double* __restrict__ delta64,
                     float* __restrict__ Hb) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const double delta = *delta64;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N * kD;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -54,6 +58,8 @@ hessian_damp_kernel(float* __restrict__ H, int64_t N, const double* __restrict__
 __global__ void extract_blocks_kernel(const float* __restrict__ H, int64_t N, int d,
                                       const int32_t* __restrict__ perm,
                                       float* __restrict__ Hb, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int64_t G = N / d;
   const int64_t total = G * d * d;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
@@ -77,7 +83,8 @@ __global__ void extract_blocks_kernel(const float* __restrict__ H, int64_t N, in
 
 crvq_status launch_hessian_delta(const float* xsq, int64_t N, float damp_rel, float* delta,
                                  double* delta64, cudaStream_t stream) {
-  hessian_delta_kernel<<<1, 1024, 0, stream>>>(xsq, N, damp_rel, delta, delta64);
+  CRVQ_CUDA(launch_pdl(hessian_delta_kernel, dim3(1), dim3(1024), 0, stream, xsq, N, damp_rel,
+                       delta, delta64));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -92,7 +99,8 @@ crvq_status launch_hessian(const float* X, int64_t n, int64_t N, int d, float da
     ProfScope ps("hessian_finalize", stream, 0.0);
     CRVQ_TRY(launch_hessian_delta(xsq, N, damp_rel, delta, mem.as<double>(), stream));
     const int blocks = (int)std::min<int64_t>(ceil_div(N * kD, 256), 4 * sm_count());
-    hessian_damp_kernel<<<blocks, 256, 0, stream>>>(H, N, mem.as<double>(), H_blocks);
+    CRVQ_CUDA(launch_pdl(hessian_damp_kernel, dim3(blocks), dim3(256), 0, stream, H, N,
+                         mem.as<double>(), H_blocks));
     CRVQ_LAUNCHED();
   }
   return CRVQ_OK;
@@ -105,7 +113,8 @@ crvq_status launch_extract_blocks(const float* H, int64_t N, int d, const int32_
   const int64_t total = (N / d) * d * d;
   const int blocks = (int)std::min<int64_t>(ceil_div(total, 256), 4096);
   ProfScope ps("extract_blocks", stream, (double)total * 8.0);
-  extract_blocks_kernel<<<blocks, 256, 0, stream>>>(H, N, d, perm, H_blocks, err);
+  CRVQ_CUDA(launch_pdl(extract_blocks_kernel, dim3(blocks), dim3(256), 0, stream, H, N, d, perm,
+                       H_blocks, err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }

@@ -23,6 +23,8 @@ __global__ void __launch_bounds__(kColThreads * kRowThreads)
 colmax_kernel(const float* __restrict__ W, const float* __restrict__ W_pre, int64_t M,
               int64_t N, int64_t rows_per_block, unsigned* __restrict__ maxbits,
               unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   __shared__ float part[kRowThreads][kColThreads * 4];
   const int cx = threadIdx.x % kColThreads, ry = threadIdx.x / kColThreads;
   const int64_t c0 = ((int64_t)blockIdx.x * kColThreads + cx) * 4;
@@ -64,6 +66,8 @@ __global__ void importance_kernel(const unsigned* __restrict__ maxbits,
                                   const float* __restrict__ xsq,
                                   const double* __restrict__ hinv, int64_t N, int mode,
                                   uint64_t seed, float* __restrict__ I) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
        i += (int64_t)gridDim.x * blockDim.x) {
     float v;
@@ -86,6 +90,8 @@ __global__ void importance_kernel(const unsigned* __restrict__ maxbits,
 // ties to the smaller index). One warp per channel: the lanes count over j, a warp sum.
 __global__ void __launch_bounds__(256)
 rank_kernel(const float* __restrict__ I, int64_t N, int32_t* __restrict__ perm) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (i >= N) return;  // whole warps
@@ -102,6 +108,8 @@ rank_kernel(const float* __restrict__ I, int64_t N, int32_t* __restrict__ perm) 
 __global__ void __launch_bounds__(256)
 gather_cols_kernel(const float* __restrict__ W, int64_t M, int64_t N,
                    const int32_t* __restrict__ perm, float* __restrict__ Ws, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   extern __shared__ __align__(16) float row[];
   for (int64_t r = blockIdx.x; r < M; r += gridDim.x) {
     __syncthreads();
@@ -156,16 +164,17 @@ crvq_status launch_select_reorder(const float* W, int64_t M, int64_t N, int d,
     const int64_t rows_per = ceil_div(M, row_blocks);
     dim3 grid((unsigned)col_blocks, (unsigned)ceil_div(M, rows_per));
     ProfScope ps("reorder_colmax", stream, (double)M * N * 4.0 * (with_pre ? 2.0 : 1.0));
-    colmax_kernel<<<grid, kColThreads * kRowThreads, 0, stream>>>(
-        W, with_pre ? W_pre : nullptr, M, N, rows_per, maxbits, err);
+    CRVQ_CUDA(launch_pdl(colmax_kernel, grid, dim3(kColThreads * kRowThreads), 0, stream, W,
+                         with_pre ? W_pre : nullptr, M, N, rows_per, maxbits, err));
     CRVQ_LAUNCHED();
   }
-  importance_kernel<<<(unsigned)ceil_div(N, 256), 256, 0, stream>>>(maxbits, xsq, hinv, N, mode,
-                                                                     seed, I);
+  CRVQ_CUDA(launch_pdl(importance_kernel, dim3((unsigned)ceil_div(N, 256)), dim3(256), 0, stream,
+                       maxbits, xsq, hinv, N, mode, seed, I));
   CRVQ_LAUNCHED();
   {
     ProfScope ps("reorder_rank", stream, (double)N * N);
-    rank_kernel<<<(unsigned)ceil_div(N, 8), 256, 0, stream>>>(I, N, perm);
+    CRVQ_CUDA(launch_pdl(rank_kernel, dim3((unsigned)ceil_div(N, 8)), dim3(256), 0, stream, I, N,
+                         perm));
     CRVQ_LAUNCHED();
   }
   {
@@ -185,7 +194,8 @@ crvq_status launch_gather_cols(const float* src, int64_t M, int64_t N, const int
     CRVQ_CUDA(cudaFuncSetAttribute(gather_cols_kernel,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int blocks = (int)std::min<int64_t>(M, (int64_t)8 * sm_count());
-  gather_cols_kernel<<<blocks, 256, smem, stream>>>(src, M, N, idx, dst, err);
+  CRVQ_CUDA(launch_pdl(gather_cols_kernel, dim3(blocks), dim3(256), smem, stream, src, M, N, idx,
+                       dst, err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }

@@ -30,6 +30,8 @@ __device__ __forceinline__ float chunk_sum(const float* __restrict__ P, int chun
 __global__ void __launch_bounds__(256)
 sum_partials_kernel(const float* __restrict__ P, int64_t N, int chunks, float scale,
                     float* __restrict__ S, float* __restrict__ diag) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < N * N;
        e += (int64_t)gridDim.x * blockDim.x) {
     const float v = chunk_sum(P, chunks, N * N, e, scale);
@@ -42,6 +44,8 @@ sum_partials_kernel(const float* __restrict__ P, int64_t N, int chunks, float sc
 __global__ void __launch_bounds__(256)
 blocks_sum_kernel(const float* __restrict__ P, int chunks, int64_t stride, float scale, int64_t N,
                   float* __restrict__ xsq, float* __restrict__ Hb) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < N * 8;
        e += (int64_t)gridDim.x * blockDim.x) {
     const float v = chunk_sum(P, chunks, stride, e, scale);
@@ -55,6 +59,8 @@ blocks_sum_kernel(const float* __restrict__ P, int chunks, int64_t stride, float
 __global__ void __launch_bounds__(256)
 blocks_add_delta_kernel(const float* __restrict__ xsq, int64_t N, const double* __restrict__ delta64,
                         float* __restrict__ Hb) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < N) Hb[i * 8 + (i & 7)] = (float)((double)xsq[i] + *delta64);
 }
@@ -63,6 +69,8 @@ blocks_add_delta_kernel(const float* __restrict__ xsq, int64_t N, const double* 
 __global__ void __launch_bounds__(256)
 blocks_damp_kernel(const float* __restrict__ P, int chunks, int64_t stride, float scale,
                    int64_t N, const double* __restrict__ delta64, float* __restrict__ Hb) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const double delta = *delta64;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < N * 8;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -75,6 +83,8 @@ blocks_damp_kernel(const float* __restrict__ P, int chunks, int64_t stride, floa
 __global__ void __launch_bounds__(256)
 transpose_kernel(const float* __restrict__ X, int64_t n, int64_t N, float* __restrict__ out,
                  int64_t ldt) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   __shared__ float t[32][33];
   const int64_t k0 = (int64_t)blockIdx.x * 32, a0 = (int64_t)blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
@@ -145,6 +155,8 @@ __global__ void __launch_bounds__(512)
 image_gather_kernel(const float* __restrict__ src, const int32_t* __restrict__ cols, int64_t rows,
                     int64_t K, int64_t rows_pad, int64_t nslab, char* __restrict__ hi,
                     char* __restrict__ lo) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   extern __shared__ __align__(16) float staged[];  // [kGatherRows][K]
   const bool vec = (K & 3) == 0 && ((uintptr_t)src & 15) == 0;
   const int r = threadIdx.x % kGatherRows;
@@ -182,6 +194,8 @@ __global__ void __launch_bounds__(256)
 image_kernel(const float* __restrict__ src, const float* __restrict__ sub,
              const int32_t* __restrict__ cols, int64_t rows, int64_t K, int64_t ld,
              int64_t rows_pad, int64_t nslab, char* __restrict__ hi, char* __restrict__ lo) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t r = (int64_t)blockIdx.x * 8 + (lane & 7);
   const int64_t sl = (int64_t)blockIdx.y * 8 + warp;
@@ -218,6 +232,8 @@ image_kernel(const float* __restrict__ src, const float* __restrict__ sub,
 __global__ void __launch_bounds__(256)
 image_t_kernel(const float* __restrict__ X, int64_t rows, int64_t K, int64_t rows_pad,
                int64_t nslab, char* __restrict__ hi, char* __restrict__ lo) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int64_t r = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
   if (r >= rows_pad) return;
   for (int64_t k = ((int64_t)blockIdx.y * 8 + (threadIdx.x >> 5)) * 4; k < nslab * kSlabK;
@@ -261,6 +277,8 @@ __device__ __forceinline__ void pair_acc(float& h, float& l, float x) {  // (h, 
 
 template <int EPI>
 __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   extern __shared__ __align__(1024) char smem_raw[];
   char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
   float* stage_out = reinterpret_cast<float*>(smem + kStages * kStageBytes);
@@ -440,8 +458,8 @@ __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
 template <int EPI>
 crvq_status launch(const ImgArgs& a, int64_t tiles_m, int64_t chunks, cudaStream_t stream) {
   CRVQ_TRY(smem_limit((const void*)img_gemm_kernel<EPI>, kSmem));
-  img_gemm_kernel<EPI><<<dim3((unsigned)(tiles_m * a.tiles_n), (unsigned)chunks), kThreads, kSmem,
-                         stream>>>(a);
+  CRVQ_CUDA(launch_pdl(img_gemm_kernel<EPI>, dim3((unsigned)(tiles_m * a.tiles_n),
+                       (unsigned)chunks), dim3(kThreads), kSmem, stream, a));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -464,13 +482,14 @@ crvq_status launch_images(const float* src, const float* sub, const int32_t* col
   if (cols && staged <= img::kGatherSmem) {
     CRVQ_TRY(smem_limit((const void*)img::image_gather_kernel, img::kGatherSmem));
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(220 * 1024 / (staged + 1024))));
-    img::image_gather_kernel<<<(unsigned)std::min<int64_t>(pad / img::kGatherRows, per_sm * sm_count()), 512,
-                               staged, stream>>>(src, cols, rows, K, pad, nslab, hi, lo);
+    CRVQ_CUDA(launch_pdl(img::image_gather_kernel, dim3((unsigned)std::min<int64_t>(pad /
+                         img::kGatherRows, per_sm * sm_count())), dim3(512), staged, stream, src,
+                         cols, rows, K, pad, nslab, hi, lo));
     CRVQ_LAUNCHED();
     return CRVQ_OK;
   }
-  img::image_kernel<<<dim3((unsigned)(pad / 8), (unsigned)ceil_div(nslab, 8)), 256, 0, stream>>>(
-      src, sub, cols, rows, K, K, pad, nslab, hi, lo);
+  CRVQ_CUDA(launch_pdl(img::image_kernel, dim3((unsigned)(pad / 8), (unsigned)ceil_div(nslab, 8)),
+                       dim3(256), 0, stream, src, sub, cols, rows, K, K, pad, nslab, hi, lo));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -491,8 +510,8 @@ crvq_status launch_tc_syrk(const float* X, int64_t n, int64_t N, float* S, float
   {
     ProfScope ps("hessian_images", stream, 12.0 * (double)n * N);
     const unsigned gy = (unsigned)std::min<int64_t>(ceil_div(nslab * 4, 8), 65535);
-    img::image_t_kernel<<<dim3((unsigned)(pad / 32), gy), 256, 0, stream>>>(X, N, n, pad, nslab, hi,
-                                                                            lo);
+    CRVQ_CUDA(launch_pdl(img::image_t_kernel, dim3((unsigned)(pad / 32), gy), dim3(256), 0, stream,
+                         X, N, n, pad, nslab, hi, lo));
     CRVQ_LAUNCHED();
   }
   // Few tiles (small N): each K chunk in its own CTA, the partials added afterwards in chunk order;
@@ -523,7 +542,8 @@ crvq_status launch_tc_syrk(const float* X, int64_t n, int64_t N, float* S, float
   if (split) {
     ProfScope ps("hessian_sum_partials", stream, (double)chunks * N * N * 4.0);
     const int blocks = (int)std::min<int64_t>(ceil_div(N * N, 256), 16 * sm_count());
-    sum_partials_kernel<<<blocks, 256, 0, stream>>>(pmem.as<float>(), N, (int)chunks, scale, S, diag);
+    CRVQ_CUDA(launch_pdl(sum_partials_kernel, dim3(blocks), dim3(256), 0, stream, pmem.as<float>(),
+                         N, (int)chunks, scale, S, diag));
     CRVQ_LAUNCHED();
   }
   return CRVQ_OK;
@@ -626,8 +646,8 @@ crvq_status launch_img_dot(const char* a_hi, const char* a_lo, int64_t M, const 
 crvq_status launch_transpose(const float* X, int64_t n, int64_t N, float* Xt, int64_t ldt,
                              cudaStream_t stream) {
   ProfScope ps("hessian_transpose", stream, 8.0 * (double)n * N);
-  transpose_kernel<<<dim3((unsigned)ceil_div(ldt, 32), (unsigned)ceil_div(N, 32)), 256, 0,
-                     stream>>>(X, n, N, Xt, ldt);
+  CRVQ_CUDA(launch_pdl(transpose_kernel, dim3((unsigned)ceil_div(ldt, 32), (unsigned)ceil_div(N,
+                       32)), dim3(256), 0, stream, X, n, N, Xt, ldt));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -671,22 +691,24 @@ crvq_status launch_tc_hessian_blocks(const float* Xt, int64_t ldt, int64_t n, in
     ProfScope ps(perm ? "reorder_blocks_tc" : "hessian_blocks_tc", stream,
                  6.0 * (double)n * N * tc::kBM);
     dim3 grid((unsigned)ceil_div(N, tc::kBM), (unsigned)chunks);
-    tc::syrk_diag_kernel<<<grid, tc::kDiagThreads, tc::kDiagSmemBytes, stream>>>(a);
+    CRVQ_CUDA(launch_pdl(tc::syrk_diag_kernel, grid, dim3(tc::kDiagThreads), tc::kDiagSmemBytes,
+                         stream, a));
     CRVQ_LAUNCHED();
   }
   ProfScope ps("hessian_blocks_finalize", stream, (double)chunks * stride * 4.0);
   if (!delta_known) {
     if (perm) return fail(CRVQ_ERR_UNSUPPORTED, "hessian blocks: delta needs the stored order");
     const int blocks = (int)std::min<int64_t>(ceil_div(stride, 256), 4 * sm_count());
-    blocks_sum_kernel<<<blocks, 256, 0, stream>>>(mem.as<float>(), (int)chunks, stride, scale, N, xsq,
-                                                  Hb);
+    CRVQ_CUDA(launch_pdl(blocks_sum_kernel, dim3(blocks), dim3(256), 0, stream, mem.as<float>(),
+                         (int)chunks, stride, scale, N, xsq, Hb));
     CRVQ_LAUNCHED();
     CRVQ_TRY(launch_hessian_delta(xsq, N, damp_rel, delta, delta64, stream));
-    blocks_add_delta_kernel<<<(unsigned)ceil_div(N, 256), 256, 0, stream>>>(xsq, N, delta64, Hb);
+    CRVQ_CUDA(launch_pdl(blocks_add_delta_kernel, dim3((unsigned)ceil_div(N, 256)), dim3(256), 0,
+                         stream, xsq, N, delta64, Hb));
   } else {
     const int blocks = (int)std::min<int64_t>(ceil_div(stride, 256), 4 * sm_count());
-    blocks_damp_kernel<<<blocks, 256, 0, stream>>>(mem.as<float>(), (int)chunks, stride, scale,
-                                                   N, delta64, Hb);
+    CRVQ_CUDA(launch_pdl(blocks_damp_kernel, dim3(blocks), dim3(256), 0, stream, mem.as<float>(),
+                         (int)chunks, stride, scale, N, delta64, Hb));
   }
   CRVQ_LAUNCHED();
   return CRVQ_OK;

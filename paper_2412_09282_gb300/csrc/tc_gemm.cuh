@@ -92,6 +92,8 @@ struct DiagArgs {
 };
 
 __global__ void __launch_bounds__(kDiagThreads, 1) syrk_diag_kernel(DiagArgs a) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   extern __shared__ __align__(1024) char smem_raw[];
   char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   __shared__ __align__(8) uint64_t full[kDiagStages], empty[kDiagStages], done;

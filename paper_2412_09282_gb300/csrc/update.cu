@@ -25,6 +25,8 @@ namespace {
 // The maxima behind the fixed-point scale, and the scale (stats_merge_scale).
 __global__ void __launch_bounds__(256)
 maxabs_kernel(SetView set, CbList cbs, int which, StatsView st, int64_t n_members, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   const int64_t G_cov = st.G_cov;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nth = (int64_t)gridDim.x * blockDim.x;
@@ -65,6 +67,8 @@ constexpr int kAccGroups = 4;
 
 __global__ void __launch_bounds__(256)
 accumulate_stats_kernel(SetView set, CbList cbs, int which, StatsView st, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
   // [component][vh, vl][code]: lanes of a warp adding one component hit spread banks
   __shared__ int s_b32[kD * 2 * kSmemStatsK];
   __shared__ int s_cnt[kAccGroups * kSmemStatsK];
@@ -459,9 +463,9 @@ static crvq_status launch_maxabs(const SetView& set, const CbList& cbs, int whic
                                  const StatsView& st, unsigned* err, cudaStream_t stream) {
   const int64_t n = set.M * cbs.cb[which].G_cov;
   ProfScope ps("update_bound", stream, (double)n * kD * 4.0);
-  maxabs_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256),
-                                                                   4 * sm_count())),
-                  256, 0, stream>>>(set, cbs, which, st, std::max<int64_t>(1, n), err);
+  CRVQ_CUDA(launch_pdl(maxabs_kernel, dim3((unsigned)std::max<int64_t>(1,
+                       std::min<int64_t>(ceil_div(n, 256), 4 * sm_count()))), dim3(256), 0, stream,
+                       set, cbs, which, st, std::max<int64_t>(1, n), err));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }
@@ -493,8 +497,8 @@ crvq_status launch_update_codebook(const SetView& set, const CbList& cbs, int wh
   if (n > 0) {
     ProfScope ps("update_accumulate", stream, (double)n);
     const int nsm = sm_count();
-    accumulate_stats_kernel<<<accumulate_grid(set.M, cw.G_cov, nsm), 256, 0, stream>>>(
-        set, cbs, which, st, err);
+    CRVQ_CUDA(launch_pdl(accumulate_stats_kernel, accumulate_grid(set.M, cw.G_cov, nsm), dim3(256),
+                         0, stream, set, cbs, which, st, err));
     CRVQ_LAUNCHED();
   }
   return launch_stats_solve(set, st, cw.C, C_out, counts, stream);
@@ -532,8 +536,8 @@ crvq_status launch_update_codebook_on(const SetView& set, const CbList& cbs, int
   const int nsm = sm_count();
   CRVQ_TRY(launch_maxabs(set, cbs, which, st, err, stream));
   if (n > 0) {
-    accumulate_stats_kernel<<<accumulate_grid(set.M, cw.G_cov, nsm), 256, 0, stream>>>(
-        set, cbs, which, st, err);
+    CRVQ_CUDA(launch_pdl(accumulate_stats_kernel, accumulate_grid(set.M, cw.G_cov, nsm), dim3(256),
+                         0, stream, set, cbs, which, st, err));
     CRVQ_LAUNCHED();
   }
   return launch_solve_kernels(set.Hb, st, cw.C, C_out, counts, err, stream);

@@ -2034,7 +2034,7 @@ beam_stage_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDe
 // at least L pairs have y <= tau, so the L-th smallest x is at most tau + eps_0.
 constexpr size_t kBeamTcSmem = 1024 + (size_t)tcenc::kATile + 2 * (size_t)kTcBTile +
                                (size_t)kChunk * kD * 4 + (size_t)kChunk * 8 + (size_t)kChunk * 4 +
-                               2 * 16 * (size_t)kThreads * 4;
+                               2 * 16 * (size_t)kThreads * 4 + 8 * (size_t)kThreads * 4;
 
 template <int L>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -2053,6 +2053,7 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
   float* sNa = reinterpret_cast<float*>(sNL + kChunk);
   float* sRa = sNa + kChunk;  // [h][thread]
   float* sPm = sRa + 16 * kThreads;
+  uint32_t* sMask = reinterpret_cast<uint32_t*>(sPm + 16 * kThreads);  // [32-column word][thread]
   __shared__ __align__(16) float sH[kD * kD];
   __shared__ __align__(8) uint64_t bar_b, bar_mma;
   __shared__ uint32_t tmem_slot;
@@ -2226,69 +2227,77 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
       }
       if (act) tau_x = __fadd_ru(bl[L - 1], eps);
     }
-    // Candidates of hypothesis h, 64 columns at a time: a mask (a subtraction and a funnel
-    // shift per score), then its members in codeword order, scored again with the fast stage's chain
-    // and inserted; the threshold tightens after every 64 columns. NaN threshold for a thread
-    // without this hypothesis: no value compares below it.
+    // Candidates of hypothesis h: masks of all its columns first (a subtraction and a funnel shift per
+    // score), then their members in codeword order, scored again with the fast stage's chain and
+    // inserted. A warp's lanes walk their own masks side by side: it takes as many rounds as its longest
+    // list of about five, where rounds per 32 columns took three times as many (three stages over 11008 x
+    // 11 vectors 548 -> 512 us). The threshold is that of the pass's start (-inf for a thread without this hypothesis).
+    const float thrD = act ? __fadd_ru(fminf(topv[L - 1], tau_x), eps) : -INFINITY;
+    // y <= thrD as the sign of y - (the next number above thrD): one instruction on the FMA pipe and
+    // one on the ALU pipe, which had both of the compare form
+    const float up = thrD < INFINITY && thrD > -INFINITY
+                         ? __int_as_float(__float_as_int(thrD) +
+                                          (thrD > 0.f ? 1 : thrD < 0.f ? -1 : 0)) +
+                               (thrD == 0.f ? 1.401298464e-45f : 0.f)
+                         : thrD;
+    uint32_t words = 0u;  // the mask words with members
 #pragma unroll 1
     for (int q = 0; q < nq; ++q) {
-      const float thrD = act ? __fadd_ru(fminf(topv[L - 1], tau_x), eps) : -INFINITY;
-      // y <= thrD as the sign of y - (the next number above thrD), shifted into the mask: one
-      // instruction on the FMA pipe and one on the ALU pipe, which had both of the compare form (three
-      // stages over 11008 x 11 vectors 581 -> 561 us)
-      const float up = thrD < INFINITY && thrD > -INFINITY
-                           ? __int_as_float(__float_as_int(thrD) +
-                                            (thrD > 0.f ? 1 : thrD < 0.f ? -1 : 0)) +
-                                 (thrD == 0.f ? 1.401298464e-45f : 0.f)
-                           : thrD;
-      uint32_t m0 = 0u, m1 = 0u;
-      {
-        uint32_t v[64];
-        tc::tmem_ld64_wait(trow + 64 * q, v);
-        uint32_t part[4] = {0u, 0u, 0u, 0u};
+      uint32_t v[64];
+      tc::tmem_ld64_wait(trow + 64 * q, v);
+      uint32_t part[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-        for (int e = 15; e >= 0; --e)
+      for (int e = 15; e >= 0; --e)
 #pragma unroll
-          for (int w = 0; w < 4; ++w)
-            part[w] = __funnelshift_l(__float_as_uint(__fsub_rn(__uint_as_float(v[16 * w + e]), up)),
-                                      part[w], 1);
-        m0 = part[0] | part[1] << 16;
-        m1 = part[2] | part[3] << 16;
-      }
+        for (int w = 0; w < 4; ++w)
+          part[w] = __funnelshift_l(__float_as_uint(__fsub_rn(__uint_as_float(v[16 * w + e]), up)),
+                                    part[w], 1);
 #pragma unroll
       for (int w = 0; w < 2; ++w) {
-        uint32_t m = w ? m1 : m0;
-        while (m) {
-          const int k = 64 * q + 32 * w + __ffs(m) - 1;
-          m &= m - 1u;
-          if (k >= cw.K) break;  // padding columns (only with an unbounded threshold)
-          const float4 c0 = *reinterpret_cast<const float4*>(sC + k * kD);
-          const float4 c1 = *reinterpret_cast<const float4*>(sC + k * kD + 4);
-          const float2 nl = sNL[k];
-          float sv = base + nl.x;
-          sv = fmaf(m2q[0], c0.x, sv);
-          sv = fmaf(m2q[1], c0.y, sv);
-          sv = fmaf(m2q[2], c0.z, sv);
-          sv = fmaf(m2q[3], c0.w, sv);
-          sv = fmaf(m2q[4], c1.x, sv);
-          sv = fmaf(m2q[5], c1.y, sv);
-          sv = fmaf(m2q[6], c1.z, sv);
-          sv = fmaf(m2q[7], c1.w, sv);
-          sv = fmaf(nbeta, nl.y, sv);
-          if (sv < topv[L - 1]) {  // insert before the first entry strictly above sv
-            const int si = (h << 16) | k;
+        const int k0 = 64 * q + 32 * w;
+        uint32_t m = part[2 * w] | part[2 * w + 1] << 16;
+        if (k0 + 32 > cw.K)  // padding columns (only with an unbounded threshold)
+          m &= k0 < cw.K ? (1u << (cw.K - k0)) - 1u : 0u;
+        sMask[(2 * q + w) * kThreads + tid] = m;
+        words |= m ? 1u << (2 * q + w) : 0u;
+      }
+    }
+    int kw = 0;
+    uint32_t m = 0u;
+    while (m | words) {
+      if (m == 0u) {
+        const int w = __ffs(words) - 1;
+        words &= words - 1u;
+        m = sMask[w * kThreads + tid];
+        kw = 32 * w;
+      }
+      const int k = kw + __ffs(m) - 1;
+      m &= m - 1u;
+      const float4 c0 = *reinterpret_cast<const float4*>(sC + k * kD);
+      const float4 c1 = *reinterpret_cast<const float4*>(sC + k * kD + 4);
+      const float2 nl = sNL[k];
+      float sv = base + nl.x;
+      sv = fmaf(m2q[0], c0.x, sv);
+      sv = fmaf(m2q[1], c0.y, sv);
+      sv = fmaf(m2q[2], c0.z, sv);
+      sv = fmaf(m2q[3], c0.w, sv);
+      sv = fmaf(m2q[4], c1.x, sv);
+      sv = fmaf(m2q[5], c1.y, sv);
+      sv = fmaf(m2q[6], c1.z, sv);
+      sv = fmaf(m2q[7], c1.w, sv);
+      sv = fmaf(nbeta, nl.y, sv);
+      if (sv < topv[L - 1]) {  // insert before the first entry strictly above sv
+        const int si = (h << 16) | k;
 #pragma unroll
-            for (int j = L - 1; j >= 0; --j) {
-              const bool below = j > 0 && sv < topv[j > 0 ? j - 1 : 0];
-              const bool here = sv < topv[j];
-              topi[j] = below ? topi[j > 0 ? j - 1 : 0] : (here ? si : topi[j]);
-              topv[j] = below ? topv[j > 0 ? j - 1 : 0] : (here ? sv : topv[j]);
-            }
-          }
+        for (int j = L - 1; j >= 0; --j) {
+          const bool below = j > 0 && sv < topv[j > 0 ? j - 1 : 0];
+          const bool here = sv < topv[j];
+          topi[j] = below ? topi[j > 0 ? j - 1 : 0] : (here ? si : topi[j]);
+          topv[j] = below ? topv[j > 0 ? j - 1 : 0] : (here ? sv : topv[j]);
         }
       }
-      __syncwarp();
     }
+    __syncwarp();
     tc::tc_fence_before();
     if (h + 1 < Bmax) {  // the pass of h has completed: its A tile is free
       write_a(nm2q, nbase, nnbeta);

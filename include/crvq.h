@@ -17,7 +17,8 @@
  *    CRVQ_ERR_INVALID_ARG for a host pointer; crvq_quantize_layer accepts either.
  *  - Calls enqueue work on `stream` and return without waiting, except calls that return a
  *    value in host memory (their documentation says so): those synchronize `stream`.
- *  - Scratch memory is taken with stream-ordered cudaMallocAsync/cudaFreeAsync on `stream`.
+ *  - Scratch memory is stream-ordered on `stream`, from a memory pool of the library's own (one
+ *    per device) that keeps at most 1 GiB between calls.
  *  - Arguments are validated before any launch: a bad argument returns
  *    CRVQ_ERR_INVALID_ARG, an unsupported size CRVQ_ERR_UNSUPPORTED, and nothing is
  *    enqueued. crvq_last_error() then describes the problem (per host thread).
@@ -227,7 +228,8 @@ crvq_status crvq_kmeans_init(const float* T, int64_t ldT, int64_t M, int64_t G_s
  * With one searched stage this is the arg-min assignment step of k-means.
  *   keep_if_better  nonzero: the searched codes hold a tuple on entry, which is kept when
  *                   its err is strictly smaller than the beam's best.
- *   vec_err         [M x G_sub] out or NULL: err of the written tuple (fp64, rounded).
+ *   vec_err         [M x G_sub] out or NULL: err of the written tuple (an fp32 pair, about
+ *                   2^-44 relative, rounded).
  * Requires 1 <= B <= 16, 0 <= n_fixed < n_cb <= 8. Sets of more than 65535 groups return
  * CRVQ_ERR_UNSUPPORTED (a beam stage launches one grid row per group).
  * Beam stages over codebooks of at most 256 codewords with B <= 8 score on the tensor cores and
@@ -315,7 +317,7 @@ crvq_status crvq_reconstruct_error(const float* W_sorted, int64_t M, int64_t N, 
  *             and rewritten in place.
  *   sweeps    >= 0 passes over the groups.
  *   loss      HOST out [sweeps + 1] or NULL: tr(dW H dW^T) before the first sweep and after
- *             each (3xTF32 products, fp64 sums). Synchronizes `stream` when given.
+ *             each (3xTF32 products, summed in fp32 pairs and fp64). Synchronizes `stream` when given.
  * b_g comes from tensor-core products of H with D^T taken per block of 256 channels at the
  * block's start plus the block's own earlier changes; the shift is solved in fp32 with a
  * Cholesky factor of H_gg computed in fp64. A block without a factor is reported as

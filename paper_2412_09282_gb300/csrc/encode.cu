@@ -11,8 +11,9 @@
 // and the pass ranks the lower bounds low_k = s_k - Et_k, keeping the best two. The arg-min j
 // is certified when low_2nd - low_j > 2 Et_j: every other codeword's exact score is then larger
 // than j's. Otherwise the vector is open: the codewords with low_k <= low_j + 2 Et_j (the exact
-// arg-min is among them) are decided among in fp32 pairs (score.cuh). Codes therefore equal the fp64 arg-min (ties to the smaller index) except for ties at fp64
-// rounding level. Beam stages use the same bounds on a sorted top-(B+1) list.
+// arg-min is among them) are decided among in fp32 pairs (score.cuh). Codes therefore equal the fp64
+// arg-min (ties to the smaller index) except for ties at fp64 rounding level. Beam stages use the same
+// bounds on a sorted top-(B+1) list.
 #include <algorithm>
 #include <cstdlib>
 #include <type_traits>
@@ -444,9 +445,10 @@ constexpr int kBlk = 16;  // columns per block of the arg-min sweep
 // column whose exact score could be the smallest has D <= top, so its block and its class have
 // minima <= top, and the two 16-bit masks of those name all candidates (two to four columns as a
 // rule, instead of the whole codebook). They go to a list in shared memory, and after its last tile
-// the CTA decides its open rows exactly (dfl, fp32 pairs), eight lanes per row. A row that finds
-// the list full is decided at once by its warp. This replaces a kernel that gave every open row a
-// warp and scanned the codebook twice (21 us per pass of a 4096 x 4096 matrix, 9 us of a 512 x 512).
+// the CTA decides its open rows exactly (dfl, fp32 pairs), eight lanes per row (a warp each when they
+// are at most eight). A row that finds the list full is decided at once by its warp. This replaces a
+// kernel that gave every open row a warp and scanned the codebook twice (21 us per pass of a 4096 x
+// 4096 matrix, 9 us of a 512 x 512).
 constexpr int kOpenCap = 256;  // open rows a CTA keeps for its end
 
 struct OpenRow {
@@ -2231,7 +2233,8 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
     // score), then their members in codeword order, scored again with the fast stage's chain and
     // inserted. A warp's lanes walk their own masks side by side: it takes as many rounds as its longest
     // list of about five, where rounds per 32 columns took three times as many (three stages over 11008 x
-    // 11 vectors 548 -> 512 us). The threshold is that of the pass's start (-inf for a thread without this hypothesis).
+    // 11 vectors 548 -> 512 us). The threshold is that of the pass's start (-inf for a thread without
+    // this hypothesis).
     const float thrD = act ? __fadd_ru(fminf(topv[L - 1], tau_x), eps) : -INFINITY;
     // y <= thrD as the sign of y - (the next number above thrD): one instruction on the FMA pipe and
     // one on the ALU pipe, which had both of the compare form

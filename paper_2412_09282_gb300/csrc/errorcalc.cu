@@ -94,8 +94,8 @@ template <int MAXCB>
 __global__ void __launch_bounds__(kDecWarps * 32)
 decode_vec_kernel(const float* __restrict__ Ws, int64_t M, int64_t N,
                   const float* __restrict__ Hb, CbList cbs, int64_t n_crit_groups, int slices,
-                  int slice0, int n_slices, int cb_in_smem, float* __restrict__ W_rec, float2* __restrict__ row_part,
-                  unsigned* err) {
+                  int slice0, int n_slices, int cb_in_smem, float* __restrict__ W_rec,
+                  float2* __restrict__ row_part, unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
   extern __shared__ __align__(16) float s_dyn[];

@@ -497,7 +497,7 @@ crvq_status launch_images(const float* src, const float* sub, const int32_t* col
 // S = X^T X / n (X: n x N row-major) into S (N x N), both triangles, and its diagonal: the images of X^T, then one
 // product over the tiles that reach the upper triangle, chunk sums kept in tensor memory. (Splitting
 // the operands in the product's own shared-memory stages bound it by the L1TEX pipe: 765 us at
-// N = n = 4096, with 57 us more for adding chunk partials kept in memory; now 325 us in all.)
+// N = n = 4096, with 57 us more for adding chunk partials kept in memory; now 317 us in all.)
 crvq_status launch_tc_syrk(const float* X, int64_t n, int64_t N, float* S, float* diag,
                            cudaStream_t stream) {
   unsigned* err = nullptr;

@@ -37,10 +37,12 @@ constexpr int kDecHStride = 260; // floats per staged H block (256 + 4: conflict
 constexpr int kDecSmemCb = 48 * 1024;  // codebooks staged in shared memory up to this size
 
 // Reconstruction of a vector from its codes (k[s] < 0: codebook s does not cover it), with the
-// codewords read from `cw[s]` (shared memory or global): the sum in codebook order, correctly
-// rounded to fp32 like the fp64 sum rounded once (two terms in fp32 give that value exactly;
-// three or more are summed as an fp32 pair: in fp64 the few CTAs with the critical groups took
-// four times as long as the others, 145 us for a kernel of 37 us on a 4096 x 4096 matrix).
+// codewords read from `cw[s]` (shared memory or global): the sum in codebook order, rounded to fp32.
+// Up to two terms are added in fp32, which rounds their sum correctly. Three or more are summed as an
+// fp32 pair, known to about 2^-48 of the terms before its one rounding (in fp64 the few CTAs with the
+// critical groups took four times as long as the others, 145 us for a kernel of 37 us on a 4096 x 4096
+// matrix); a pair that has left fp32's range, for good (an infinite codeword) or on the way (large terms
+// of both signs), is no number any more, and the sum is taken in fp64.
 template <int MAXCB>
 __device__ __forceinline__ void recon_codes(const float* const* cw, const int32_t* k, int ncb,
                                             float r[kD]) {
@@ -73,8 +75,24 @@ __device__ __forceinline__ void recon_codes(const float* const* cw, const int32_
 #pragma unroll
       for (int j = 0; j < kD; ++j) pair_add(r[j], l[j], c[j]);
     }
+    bool bad = false;
 #pragma unroll
-    for (int j = 0; j < kD; ++j) r[j] = __fadd_rn(r[j], l[j]);
+    for (int j = 0; j < kD; ++j) {
+      r[j] = __fadd_rn(r[j], l[j]);
+      bad = bad || !isfinite(r[j]);
+    }
+    if (bad) {
+#pragma unroll 1
+      for (int j = 0; j < kD; ++j) {
+        double d = 0.0;
+#pragma unroll
+        for (int s = 0; s < MAXCB; ++s)
+          if (s < ncb && k[s] >= 0) d += (double)cw[s][(int64_t)k[s] * kD + j];
+#pragma unroll
+        for (int q = 0; q < kD; ++q)
+          if (q == j && !isfinite(r[q])) r[q] = (float)d;
+      }
+    }
   }
 }
 

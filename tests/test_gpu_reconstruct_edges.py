@@ -1,6 +1,7 @@
 """Reconstruction of a matrix large enough that the slices without extended codebooks run in a launch
 of their own and a block takes several row blocks, against plain fp64 sums: reconstructions are
-bit-exact, block losses within 1e-4 (the bar of the parity tests: fp32 terms)."""
+bit-exact, block losses within 1e-4 (the bar of the parity tests: fp32 terms). Sums that leave fp32's
+range, for good or on the way, are those of fp64 rounded."""
 import numpy as np
 import pytest
 
@@ -37,3 +38,31 @@ def test_reconstruct_over_row_blocks_and_slices(M, N, Gc):
     per_group = np.einsum("mgi,gij,mgj->g", d, Hb.astype(np.float64), d, optimize=True)
     assert abs(lb - per_group.sum()) <= 1e-4 * per_group.sum()
     assert abs(lc - per_group[:Gc].sum()) <= 1e-4 * per_group[:Gc].sum()
+
+
+@pytest.mark.parametrize("n_cb", [3, 6])
+def test_reconstruct_sums_beyond_fp32(n_cb):
+    """An infinite codeword gives an infinite element, and large terms of both signs their sum, whatever
+    the partial sums did."""
+    M, N = 40, 16
+    G = N // D
+    rng = np.random.default_rng(n_cb)
+    Cs = [(0.02 * rng.standard_normal((4, D))).astype(np.float32) for _ in range(n_cb)]
+    Cs[0][0, 3], Cs[1][1, 5] = np.inf, -np.inf
+    for C, v in zip(Cs, (3e38, 3e38, -3e38)):
+        C[2, 1] = v
+        C[3, 6] = -v
+    codes = [rng.integers(0, 2 if s < 3 else 4, (M, G)).astype(np.int32) for s in range(n_cb)]
+    for c in codes[:3]:
+        c[:10] = 2
+        c[10:20] = 3
+    codes[1][(codes[0] == 0) & (codes[1] == 1)] = 0
+    cbs = [Codebook(dev(C), dev(c), G) for C, c in zip(Cs, codes)]
+    W = np.zeros((M, N), np.float32)
+    Hb = np.stack([np.eye(D, dtype=np.float32)] * G)
+    Wh, _, _, _ = P.crvq_reconstruct_error(dev(W), D, dev(Hb), None, cbs, 0)
+    rec = sum(C.astype(np.float64)[c] for C, c in zip(Cs, codes))
+    with np.errstate(over="ignore"):
+        want = rec.astype(np.float32).reshape(M, N)
+    assert np.isinf(want).any() and not np.isnan(want).any() and (np.abs(want) > 1e38).any()
+    np.testing.assert_array_equal(host(Wh), want)

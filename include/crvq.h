@@ -41,10 +41,10 @@
  * part of the Alg. 1 loss ||W X - W_enc X||^2 written with H = X^T X / n + delta I. With
  * H_g = c I it is the squared L2 distance of Sec. 3.1 Eq. (2)-(3). Code indices are decided
  * exactly: scores are computed in fp32 (on the tensor cores for one searched codebook) with
- * a rigorous error bound, and any decision closer than that bound is re-taken exactly (errs
- * as unevaluated fp32 pairs, about 2^-44 relative, or in fp64), so codes equal those of an
- * fp64 evaluation except for ties at rounding level (ties go to the smaller index / earlier
- * tuple).
+ * a rigorous error bound, and any decision closer than that bound is re-taken with errs in
+ * unevaluated fp32 pairs (within a few 2^-48 of |r|^T |H_g| |r|, as long as the products in it stay
+ * above about 2^-102, where a pair is exact) or in fp64, so codes equal those of an fp64 evaluation
+ * except for ties at that level (ties go to the smaller index / earlier tuple).
  */
 #ifndef CRVQ_H
 #define CRVQ_H
@@ -228,8 +228,10 @@ crvq_status crvq_kmeans_init(const float* T, int64_t ldT, int64_t M, int64_t G_s
  * With one searched stage this is the arg-min assignment step of k-means.
  *   keep_if_better  nonzero: the searched codes hold a tuple on entry, which is kept when
  *                   its err is strictly smaller than the beam's best.
- *   vec_err         [M x G_sub] out or NULL: err of the written tuple (an fp32 pair, about
- *                   2^-44 relative, rounded).
+ *   vec_err         [M x G_sub] out or NULL: err of the written tuple, evaluated in fp32 pairs
+ *                   (within a few 2^-48 of |r|^T |H_g| |r| for the residual r, which is known to 2^-48
+ *                   of the terms that it is left over from) and rounded; in fp64 above fp32's range
+ *                   (Inf results) and below 2^-100.
  * Requires 1 <= B <= 16, 0 <= n_fixed < n_cb <= 8. Sets of more than 65535 groups return
  * CRVQ_ERR_UNSUPPORTED (a beam stage launches one grid row per group).
  * Beam stages over codebooks of at most 256 codewords with B <= 8 score on the tensor cores and

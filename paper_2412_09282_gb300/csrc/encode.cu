@@ -1783,7 +1783,7 @@ __device__ __forceinline__ void beam_list_finish(
     }
   }
   // Exact decisions: lane = (slot, entry) of the next 32 / L open vectors. Errs as fp32 pairs (about
-  // 2^-44 relative; no fp64) in (err, h, k) order; every unlisted candidate must have low >= the
+  // 2^-44 of their terms; no fp64) in (err, h, k) order; every unlisted candidate must have low >= the
   // last listed low, which must exceed an upper bound of the keep-th err.
   constexpr int kPer = 32 / L;
   const int slot = lane / L, e = lane - slot * L;
@@ -2325,8 +2325,7 @@ beam_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, StageDesc 
 // every member of the exact top-Bs) and keep a sorted local top-Bs; a warp merge then
 // extracts the global top-Bs in (err, h, k) order.
 // Bound: latency (a few thousand vectors per stage). In fp64 the re-scoring alone kept an SM's
-// fp64 pipe busy: 56 us per stage over 11008 x 11 vectors, now 31. The pairs are those of
-// beam_list_finish and of the arg-min's exact decisions.
+// fp64 pipe busy: 56 us per stage over 11008 x 11 vectors, now 31.
 __global__ void __launch_bounds__(kThreads)
 beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs,
                            int n_fixed, StageDesc sd, BeamBufs bb, FlagList flags,
@@ -2372,7 +2371,7 @@ beam_stage_fallback_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList
         const int32_t* pc = bb.hyp_in ? bb.hyp_in + (vi * B + h) * S : nullptr;
         hyp_residual_pair(th, tl, cbs, sd, pc, rh, rl, err);
         load_vec(cw.C + (int64_t)k * kD, c);
-        dfl::quad_err(rh, rl, c, H, e, el);
+        dfl::quad_err<true>(rh, rl, c, H, e, el);
         auto before = [&](int at) { return e < be[at] || (e == be[at] && el < bl[at]); };
         if (nb < Bs || before(nb - 1)) {
           int pos = nb < Bs ? nb : Bs - 1;
@@ -2509,13 +2508,33 @@ __device__ void tuple_err32(const SetView& set, const CbList& cbs, int n_fixed,
   bnd = kU * bound_mult(n_fixed + sd.S + 1) * na;
 }
 
-// err of a whole tuple of vector (i, g) in fp32 pairs (a few 2^-44 relative, so the rounded value is
-// the one an fp64 evaluation gives; GB300's fp64 pipe made this most of the kernel's time): the
-// fixed codebooks' codes, then for each searched stage q the code sc[q] (with sc null: the code
-// already stored).
+// err of a whole tuple of vector (i, g) in fp64: the fixed codebooks' codes, then for each searched
+// stage q the code sc[q] (with sc null: the code already stored).
+__device__ double tuple_err64(const SetView& set, const CbList& cbs, int n_fixed,
+                              const StageDesc& sd, int64_t i, int64_t g, const int32_t* sc,
+                              const float* H, unsigned* err) {
+  double r[kD];
+  target64(set, cbs, n_fixed, i, g, r, err);
+  for (int q = 0; q < sd.S; ++q) {
+    const CbView& cb = cbs.cb[sd.st[q]];
+    const int32_t k = sc ? sc[q] : cb.codes[i * cb.ld + g];
+    if (!code_ok(k, cb.K, err)) continue;
+    const float* c = cb.C + (int64_t)k * kD;
+#pragma unroll
+    for (int j = 0; j < kD; ++j) r[j] -= (double)c[j];
+  }
+  return quad_err64(r, nullptr, H);
+}
+
+// The same err in fp32 pairs (GB300's fp64 pipe made it most of the kernel's time): within a few 2^-48
+// of |d|^T |H| |d| for the tuple's residual d, itself known to 2^-48 of the terms that it is left over
+// from, so its fp32 rounding is fp64's but for the last place now and then. An err beyond fp32, and one
+// so small that products lose their low parts (TwoProduct is exact above about 2^-102), are
+// evaluated in fp64.
 __device__ __forceinline__ float tuple_err_pair(const SetView& set, const CbList& cbs, int n_fixed,
                                                 const StageDesc& sd, int64_t i, int64_t g,
                                                 const int32_t* sc, const float* H, unsigned* err) {
+  constexpr float kSmallest = 7.8886091e-31f;  // 2^-100
   float rh[kD], rl[kD], zero[kD], eh, el;
   dfl::target(set, cbs, n_fixed, i, g, rh, rl, err);
 #pragma unroll
@@ -2534,8 +2553,13 @@ __device__ __forceinline__ float tuple_err_pair(const SetView& set, const CbList
       rl[j] = __fadd_rn(rl[j], ej);
     }
   }
-  dfl::quad_err(rh, rl, zero, H, eh, el);
-  return __fadd_rn(eh, el);
+  dfl::quad_err<true>(rh, rl, zero, H, eh, el);
+  const float e = __fadd_rn(eh, el);
+  if (e >= kSmallest && e <= 3.402823466e38f) return e;
+  bool exact = true;  // an exact tuple: the err is 0
+#pragma unroll
+  for (int j = 0; j < kD; ++j) exact = exact && rh[j] == 0.f && rl[j] == 0.f;
+  return exact ? 0.f : (float)tuple_err64(set, cbs, n_fixed, sd, i, g, sc, H, err);
 }
 
 // Final step of a multi-stage (or keep-if-better) encode: write the best tuple, or keep the
@@ -2575,30 +2599,8 @@ __global__ void beam_finalize_kernel(SetView set, int64_t g_begin, int64_t G_ran
       }
     }
     if (exact) {
-      double tgt[kD];
-      target64(set, cbs, n_fixed, i, g, tgt, err);
-      double r[kD];
-#pragma unroll
-      for (int j = 0; j < kD; ++j) r[j] = tgt[j];
-      for (int q = 0; q < S; ++q) {
-        const CbView& cb = cbs.cb[sd.st[q]];
-        if (!code_ok(best[q], cb.K, err)) continue;
-        const float* c = cb.C + (int64_t)best[q] * kD;
-#pragma unroll
-        for (int j = 0; j < kD; ++j) r[j] -= (double)c[j];
-      }
-      const double e_new = quad_err64(r, nullptr, H);
-#pragma unroll
-      for (int j = 0; j < kD; ++j) r[j] = tgt[j];
-      for (int q = 0; q < S; ++q) {
-        const CbView& cb = cbs.cb[sd.st[q]];
-        const int32_t k = cb.codes[i * cb.ld + g];
-        if (!code_ok(k, cb.K, err)) continue;
-        const float* c = cb.C + (int64_t)k * kD;
-#pragma unroll
-        for (int j = 0; j < kD; ++j) r[j] -= (double)c[j];
-      }
-      use_old = quad_err64(r, nullptr, H) < e_new;
+      const double e_new = tuple_err64(set, cbs, n_fixed, sd, i, g, best, H, err);
+      use_old = tuple_err64(set, cbs, n_fixed, sd, i, g, nullptr, H, err) < e_new;
     }
     if (vec_err)
       vec_err[i * set.G_sub + g] =

@@ -70,9 +70,10 @@ __device__ __forceinline__ float up_from(float n, float na, float l1, const floa
 // Exact scoring in unevaluated fp32 pairs ("double-float"): GB300's fp64 pipe is a small
 // fraction of its fp32 rate, so the few decisions that the certified bounds leave open are
 // settled with error-free transformations (Knuth's TwoSum, the FMA-based TwoProduct) on the
-// fp32 pipe instead. The residual r = t - sum of the fixed codewords is held exactly as
-// rh + rl; the err (r - c)^T H (r - c) comes out within a few 2^-48 of |r - c|^T |H| |r - c|,
-// far inside the near-tie margin at which fp64 itself stops deciding.
+// fp32 pipe instead. The residual r = t - sum of the fixed codewords is held as rh + rl (exactly for
+// one codeword, to 2^-48 of the terms for more); the err (r - c)^T H (r - c) comes out within a few 2^-48
+// of |r - c|^T |H| |r - c|: coarser than fp64's 2^-53, far finer than any margin that the data
+// determine. TwoProduct is exact above about 2^-102.
 namespace dfl {
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -105,7 +106,10 @@ __device__ __forceinline__ void target(const SetView& set, const CbList& cbs, in
   }
 }
 
-// err = (r - c)^T H (r - c) as a normalised pair (eh, el), r = rh + rl.
+// err = (r - c)^T H (r - c) as a normalised pair (eh, el), r = rh + rl. NORM: also where r and c cancel
+// to a difference below the rounding of the terms that r is left over from (dl would be the larger
+// part, and the products keep only its high one).
+template <bool NORM = false>
 __device__ __forceinline__ void quad_err(const float rh[kD], const float rl[kD],
                                          const float c[kD], const float* H, float& eh,
                                          float& el) {
@@ -115,6 +119,7 @@ __device__ __forceinline__ void quad_err(const float rh[kD], const float rl[kD],
     float e;
     two_sum(rh[j], -c[j], dh[j], e);
     dl[j] = __fadd_rn(rl[j], e);
+    if (NORM) two_sum(dh[j], dl[j], dh[j], dl[j]);
   }
   float yh[kD], yl[kD];
 #pragma unroll

@@ -98,6 +98,45 @@ def test_three_close_codewords_in_different_granules(K):
     _check(W, _blocks(rng, G), C)
 
 
+def _tail_errs(T, C0s, H):
+    """errs of one group that the searched codebook does not cover: T minus the fixed codebooks C0s (one
+    codeword each), from crvq_encode_beam."""
+    M = T.shape[0]
+    W = np.concatenate([np.zeros((M, D), np.float32), T], axis=1)
+    Hb = np.stack([np.eye(D, dtype=np.float32), H])
+    zeros = torch.zeros((M, 2), dtype=torch.int32, device="cuda")
+    cbs = [Codebook(dev(C.reshape(1, D)), zeros, 2) for C in C0s]
+    cbs.append(Codebook(dev(np.zeros((1, D), np.float32)), torch.zeros_like(zeros[:, :1]), 1))
+    err = P.crvq_encode_beam(dev(W), D, dev(Hb), cbs, len(C0s), 1, want_err=True)
+    P.crvq_sync()
+    r = T.astype(np.float64) - sum((C.astype(np.float64) for C in C0s), np.zeros(D))
+    H = H.astype(np.float64)
+    with np.errstate(over="ignore"):
+        return host(err)[:, 1], np.einsum("md,de,me->m", r, H, r).astype(np.float32)
+
+
+@pytest.mark.parametrize("scale", [1e20, 1.0, 1e-15, 1e-18, 1e-19, 3e-20, 1e-22])
+def test_errs_beyond_the_range_of_fp32_pairs(scale):
+    """Inf above fp32, and below 2^-100, where products of fp32 numbers lose their low parts, the fp64
+    value rounded, denormal ones included (one unit in the last place: the order of the fp64 sums)."""
+    rng = np.random.default_rng(3)
+    T = (scale * rng.standard_normal((500, D))).astype(np.float32)
+    err, want = _tail_errs(T, [], _blocks(rng, 1)[0])
+    assert np.isinf(want).all() == (scale == 1e20) and not np.isnan(err).any()
+    ok = np.abs(err.view(np.int32).astype(np.int64) - want.view(np.int32)) <= 1
+    assert ok.all(), (err[~ok][:4], want[~ok][:4])
+
+
+def test_errs_of_a_residual_that_is_the_rounding_of_its_terms():
+    """t - c0 - c1 with t = c1 = 1 and a tiny c0: the fp32 residual is 0, the exact one -c0."""
+    rng = np.random.default_rng(4)
+    c0 = (1e-9 * rng.standard_normal(D)).astype(np.float32)
+    one = np.ones(D, np.float32)
+    err, want = _tail_errs(np.ones((5, D), np.float32), [c0, one], _blocks(rng, 1)[0])
+    assert want.min() > 0
+    np.testing.assert_allclose(err, want, rtol=1e-6)  # c0's part in fp32 pairs: 2^-24 of it each
+
+
 def test_non_finite_codeword_and_target_are_reported_and_leave_the_rest():
     rng = np.random.default_rng(5)
     M, G, K = 200, 2, 100

@@ -112,7 +112,8 @@ transpose_kernel(const float* __restrict__ X, int64_t n, int64_t N, float* __res
 // partials: after every 1024-column chunk the accumulator is added, in chunk order and in fp32, to
 // a running sum kept in the other half of tensor memory. The last chunk's sum goes to the epilogue:
 //   kSumsq      the sum of its squares (the full loss of Alg. 1 QuantLoss);
-//   kDot        the sum of its products with E's entries in fp32 pairs (tr(D H D^T));
+//   kDot        the sum of its products with E's entries in fp32 pairs, in fp64 beyond fp32's range
+//               (tr(D H D^T));
 //   kSymmetric  C[m][n] = C[n][m] = alpha D[m][n] for n >= m (the Hessian; tiles below the
 //               diagonal do nothing);
 //   kPlain      C[m][n] = alpha D[m][n] (blockIdx.y: one K chunk each, to its own C).
@@ -371,6 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
     float* C = EPI == kPlain || EPI == kSymmetric ? a.C + blockIdx.y * a.c_stride : nullptr;
     float* so = stage_out + (warp & 3) * 32 * 33;
     float sq = 0.f, sl = 0.f;  // kSumsq: the sum of squares; kDot: a pair
+    double beyond = 0.0;       // kDot: runs of 32 products that leave fp32's range
     bool ok = true;
     for (int c = 0; c < nchunk && ok; ++c) {
       ok = tc::mbar_wait(tc::smem_u32(acc_full), (uint32_t)(c & 1), a.err);
@@ -412,12 +414,20 @@ __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
           }
           __syncwarp();
           if (EPI == kDot) {
+            const float sq0 = sq, sl0 = sl;
 #pragma unroll
             for (int r = 0; r < 32; ++r) {  // (operand padding makes x zero past the rows of A and B)
               const float x = so[r * 33 + lane], er = e[r & (EPI == kDot ? 31 : 0)];
               const float p = __fmul_rn(x, er);
               pair_acc(sq, sl, p);
               sl = __fadd_rn(sl, __fmaf_rn(x, er, -p));
+            }
+            if (!isfinite(sq) || !isfinite(sl)) {
+              sq = sq0;
+              sl = sl0;
+#pragma unroll
+              for (int r = 0; r < 32; ++r)
+                beyond += (double)so[r * 33 + lane] * (double)e[r & (EPI == kDot ? 31 : 0)];
             }
           } else if (n < a.rows_n) {
 #pragma unroll 8
@@ -436,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
       if (!last) tc::mbar_arrive(tc::smem_u32(acc_empty));
     }
     if (!ok) sq = sl = 0.f;
-    double sd = (double)sq + (double)sl;
+    double sd = (double)sq + (double)sl + (EPI == kDot && ok ? beyond : 0.0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sd += __shfl_xor_sync(0xffffffffu, sd, o);
     if (lane == 0) red[warp - 2] = sd;

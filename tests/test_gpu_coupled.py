@@ -164,3 +164,18 @@ def test_coupled_sweep_block_row_and_codebook_edges(M, G, K):
     after = [O.Codebook(cbs[0].C, codes, G), cbs[1]]
     assert loss[0] == pytest.approx(O.full_loss(W, H, cbs), rel=1e-5)
     assert loss[1] == pytest.approx(O.full_loss(W, H, after), rel=1e-5)
+
+
+def test_coupled_loss_of_products_beyond_fp32():
+    """Residuals of 1e14 under an H of 1e12: the terms of tr(D H D^T) are 1e40 and more, their sum is
+    that of fp64 (no sweep: the loss alone)."""
+    import paper_2412_09282_gb300 as P
+    from paper_2412_09282_gb300 import Codebook
+    W, H, cbs = _case(5, M=130, G=33)
+    W, H = (W * 5e15).astype(np.float32), (H * 1e12).astype(np.float32)
+    gcbs = [Codebook(dev(cb.C), dev(cb.codes.astype(np.int32)), cb.G_cov) for cb in cbs]
+    loss = P.crvq_coupled_sweep(dev(W), dev(H), gcbs, 0, sweeps=0)
+    P.crvq_sync()
+    want = O.full_loss(W, H, cbs)
+    assert want > 1e42
+    assert loss[0] == pytest.approx(want, rel=4e-5)  # 3xTF32 products

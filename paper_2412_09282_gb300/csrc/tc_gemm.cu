@@ -321,7 +321,8 @@ __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
       const int64_t b0 = ((int64_t)bn * a.nslab + slab0) * kSlabBytes;
       const char *ah = a.a_hi + a0, *al = a.a_lo + a0, *bh = a.b_hi + b0, *bl = a.b_lo + b0;
       bool ok = true;
-      for (int64_t it = 0; it < nslab && ok; ++it) {
+      int64_t it = 0;
+      for (; it < nslab; ++it) {
         const int s = (int)(it % kStages);
         if (it >= kStages)
           ok = tc::mbar_wait(tc::smem_u32(&empty[s]), (uint32_t)((it / kStages - 1) & 1), a.err);
@@ -334,6 +335,10 @@ __global__ void __launch_bounds__(kThreads, 1) img_gemm_kernel(ImgArgs a) {
         tc::bulk_copy_g2s(tc::smem_u32(st + kAStage), bh + it * kSlabBytes, kSlabBytes, fb);
         tc::bulk_copy_g2s(tc::smem_u32(st + kAStage + kSlabBytes), bl + it * kSlabBytes, kSlabBytes, fb);
       }
+      // No copy may land in this block's shared memory after its end: the last ones are waited for here
+      // (bounded), whether or not a timeout kept the MMAs from waiting for them.
+      for (int64_t u = it > kStages ? it - kStages : 0; u < it; ++u)
+        ok = tc::mbar_wait(tc::smem_u32(&full[u % kStages]), (uint32_t)((u / kStages) & 1), a.err) && ok;
       if (!ok) ok_s[0] = 0;
     }
   } else if (warp == 1) {

@@ -9,13 +9,15 @@
 // Layout. A unit is one (codebook, group) pair; a call has U = sum_s G_cov(s) of them. A cluster
 // of up to eight CTAs owns a block of rows: each CTA takes a consecutive share of the units for
 // all of the block's rows, and the shares meet in distributed shared memory, added in a fixed
-// tree. So a call is one launch with no scratch, no zeroed counters and no partials in global
-// memory, and its results are identical on every run. Two kernels form a share's row sums; both
-// read a row's codes 16 bytes at a time, a thread per row, and need no warp reduction:
-//   table_kernel (one or two inputs, codebooks of up to 1024 / b codewords): the CTA builds the
+// tree: no zeroed counters and no partials in global memory, and results that are identical on every run.
+// Two kernels form a share's row sums; both read a row's codes 16 bytes at a time and need no warp
+// reduction:
+//   table_kernel (one or two inputs, codebooks of up to 1024 / b codewords; a thread per row, one launch,
+//     no scratch): the CTA builds the
 //     tables lut[unit][k] = <C_s[k], xs[unit]> of 32 units at a time, a code is one entry.
 //     Entries are 4 b bytes at random banks, about 3.5 b bank passes per warp and unit.
-//   dot_kernel (the rest): a code's codeword is read and dotted with the unit's inputs. With
+//   dot_kernel (the rest; after sort_inputs_kernel, which writes the inputs in the sorted order to
+//     scratch): a code's codeword is read and dotted with the unit's inputs. With
 //     three or more inputs a table entry spans 16-32 bytes, costs as many random bank passes as
 //     the codeword itself, and 256 entries are built for the few hundred rows that use them, so
 //     tables lose. The codebook is held eight times, copy c in 16-byte bank group c: the eight
@@ -29,7 +31,7 @@
 // codebooks on 2% of the channels; before: tables built by a kernel of their own, a warp per row
 // with a shuffle reduction, partials in global memory):
 //   11008 x 4096, one input: 88 -> 16.6 us;  512 x 512, one input: 29 -> 6.4 us;
-//   4096 x 11008, eight inputs: 305 -> 47 us.
+//   4096 x 11008, eight inputs: 305 -> 49 us.
 // Copying the codes to shared memory asynchronously instead of loading them by row was slower
 // (21.9 / 8.3 / 65 us), and so were clusters of four for the tables (21.5 us: twice the row
 // blocks, so twice the table builds) and of eight for the dots (74 us: 16 clusters where 15 fit).
@@ -61,6 +63,12 @@ constexpr int kDotRows = 4;                 // rows per thread
 constexpr int kDotCopies = 8;               // one per 16-byte bank group
 constexpr int kDotStageK = 512;             // codebooks held in shared memory up to this size
 constexpr int kXUnits = 192;                // units whose inputs are resident at a time
+// dot_kernel adds a warp's units in runs of eight, or of kDotFold when it has more than 128 of them, and
+// then the runs: added one after another, the 268 units of a warp in a 28672 x 8192 product left three
+// times the error of a tree. Error against 64 bits (2-norm, three inputs) of a warp-wide tree per 32 units
+// / one chain / these runs: 512 x 512 8.5 / 8.9 / 8.5e-8, 4096 x 4096 1.11 / 1.20 / 1.06e-7, 28672 x 8192
+// 1.34 / 3.07 / 1.27e-7. The runs and dot8's second chain cost 4% (eight inputs) to 10% (three).
+constexpr int kDotFold = 16;
 
 struct MatvecArgs {
   const float* X;       // b x N, row stride ldx
@@ -75,6 +83,7 @@ struct MatvecArgs {
   int units_cta;        // units per CTA share (a multiple of 4)
   int lut_k;            // table stride: the largest K, at least 256 (table_kernel)
   int rows;             // rows per cluster
+  int fold;             // units per run of a sum, a power of two (dot_kernel)
   const float* xs;      // [N / 8][BP][8]: the inputs in the sorted order (dot_kernel)
   float* Y;             // b x M, row stride ldy
   int64_t ldy;
@@ -125,17 +134,15 @@ sort_inputs_kernel(const float* __restrict__ X, int64_t ldx, int64_t N,
     out[((e >> 3) * BP + bi) * kD + (e & 7)] = (src >= 0 && bi < b) ? __ldg(X + bi * ldx + src) : 0.f;
 }
 
-// <c, x>, an 8-term FMA chain.
+// <c, x>, two 4-term FMA chains (a single chain of eight rounds more; see kDotFold).
 __device__ __forceinline__ float dot8(const float4& c0, const float4& c1, const float4& x0,
                                       const float4& x1) {
-  float v = c0.x * x0.x;
+  float v = c0.x * x0.x, w = c1.x * x1.x;
   v = fmaf(c0.y, x0.y, v);
+  w = fmaf(c1.y, x1.y, w);
   v = fmaf(c0.z, x0.z, v);
-  v = fmaf(c0.w, x0.w, v);
-  v = fmaf(c1.x, x1.x, v);
-  v = fmaf(c1.y, x1.y, v);
-  v = fmaf(c1.z, x1.z, v);
-  return fmaf(c1.w, x1.w, v);
+  w = fmaf(c1.z, x1.z, w);
+  return fmaf(c0.w, x0.w, v) + fmaf(c1.w, x1.w, w);
 }
 
 // Y of this cluster's rows from its CTAs' shares part[row][BP] in distributed shared memory, in a
@@ -308,11 +315,21 @@ dot_kernel(const __grid_constant__ MatvecArgs a, int warps_r, unsigned* err) {
   const int U = a.u_begin[a.cbs.n];
   const int u0 = min(U, rank * a.units_cta), u1 = min(U, u0 + a.units_cta);
   const int row0 = wr * 32 * kDotRows + lane;       // this lane's first row in the block
-  float acc[kDotRows][BP];
+  // the sums of the present run of units, and of the runs before it
+  float acc[kDotRows][BP], tot[kDotRows][BP];
 #pragma unroll
   for (int q = 0; q < kDotRows; ++q)
 #pragma unroll
-    for (int bi = 0; bi < BP; ++bi) acc[q][bi] = 0.f;
+    for (int bi = 0; bi < BP; ++bi) acc[q][bi] = tot[q][bi] = 0.f;
+  auto fold = [&]() {
+#pragma unroll
+    for (int q = 0; q < kDotRows; ++q)
+#pragma unroll
+      for (int bi = 0; bi < BP; ++bi) {
+        tot[q][bi] += acc[q][bi];
+        acc[q][bi] = 0.f;
+      }
+  };
 
   for (int s = 0; s < a.cbs.n; ++s) {
     const int ra = max(u0, a.u_begin[s]), re = min(u1, a.u_begin[s + 1]);
@@ -396,7 +413,9 @@ dot_kernel(const __grid_constant__ MatvecArgs a, int warps_r, unsigned* err) {
             for (int q = 0; q < kDotRows; ++q) acc[q][bi] += dot8(c0[q], c1[q], x0, x1);
           }
         }
+        if (((ua - wa) & (a.fold - 1)) == a.fold - 4) fold();
       }
+      fold();
     }
   }
   // the warps along the units add their sums one after another
@@ -406,7 +425,7 @@ dot_kernel(const __grid_constant__ MatvecArgs a, int warps_r, unsigned* err) {
       for (int q = 0; q < kDotRows; ++q) {
         float* p = part + (row0 + 32 * q) * BP;
 #pragma unroll
-        for (int bi = 0; bi < BP; ++bi) p[bi] = w == 0 ? acc[q][bi] : p[bi] + acc[q][bi];
+        for (int bi = 0; bi < BP; ++bi) p[bi] = w == 0 ? tot[q][bi] : p[bi] + tot[q][bi];
       }
     __syncthreads();
   }
@@ -470,6 +489,7 @@ crvq_status launch_dot(MatvecArgs& a, int csize, int stage_k, unsigned* err, cud
   int warps_r = 1;
   while (warps_r < kDotThreads / 32 && warps_r * kWarpRows < rows) warps_r *= 2;
   a.rows = warps_r * kWarpRows;
+  a.fold = (int64_t)a.units_cta * warps_r <= 128 * (kDotThreads / 32) ? 8 : kDotFold;
   const size_t smem = (size_t)a.rows * BP * 4 + (size_t)kXUnits * BP * kD * 4 +
                       (size_t)stage_k * kDotCopies * kD * 4;
   Scratch mem;

@@ -147,3 +147,24 @@ def test_lut_matvec_units_rows_and_unaligned_code_rows(b, M, N, Ks, Gcs, aligned
     P.crvq_sync()
     assert torch.equal(Y, _check(X, perm, cbs, M)) or np.allclose(
         host(Y), host(_check(X, perm, cbs, M)), rtol=0, atol=1e-5 * float(np.abs(host(Y)).max()))
+
+
+@pytest.mark.parametrize("b", [2, 3, 8])
+def test_lut_matvec_long_shares_keep_the_precision_of_a_tree(b):
+    """A warp of a 19000 x 8192 product adds 256 units. In one chain their roundings (0.4 * 2^-24 rms of
+    each partial sum) come to 0.4 * sqrt(256 / 2) = 4.5 * 2^-24 of the result and more (3.1e-7 was
+    measured); in runs of 16 to 0.4 * sqrt(16 / 2 + 16 / 2), beside the products' own: 1.3e-7 was
+    measured, the error of a tree."""
+    import paper_2412_09282_gb300 as P
+    from paper_2412_09282_gb300 import Codebook
+    M, N = 19000, 8192
+    G = N // D
+    g = torch.Generator(device="cuda").manual_seed(b)
+    X = torch.randn((b, N), generator=g, device="cuda")
+    K = 1024 if b == 2 else 256                             # (two inputs: too large for tables)
+    C = 0.02 * torch.randn((K, D), generator=g, device="cuda")
+    codes = torch.randint(0, K, (M, G), generator=g, device="cuda", dtype=torch.int32)
+    Y = P.crvq_lut_matvec(X, None, [Codebook(C, codes, G)], M)
+    tab = torch.einsum("kd,bgd->bgk", C.double(), X.double().view(b, G, D))
+    ref = torch.stack([torch.gather(tab[i], 1, codes.t().long()).sum(0) for i in range(b)])
+    assert float((Y - ref).norm() / ref.norm()) < 2e-7

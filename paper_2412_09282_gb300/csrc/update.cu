@@ -52,38 +52,42 @@ maxabs_kernel(SetView set, CbList cbs, int which, StatsView st, int64_t n_member
   stats_merge_scale(st, cbs, which, tm, hm, n_members, err);
 }
 
-// Statistics of every covered vector from its current code. CTA (x, y): the four adjacent groups of
-// quads y, y + gridDim.y, ..., rows x, x + gridDim.x, ... of each, thread = (row, group): four lanes
-// read a row's 128 bytes. With K <= kSmemStatsK the CTA sums its counts (per group) and fixed-point
-// terms in shared memory and adds them to the global sums once; larger codebooks add each vector's
-// terms to the global sums directly. A term (|v| < 2^30) enters shared memory as v = 2^15 vh + vl
-// (0 <= vl < 2^15) in two 32-bit sums (native 32-bit atomics): exact, as accumulate_grid gives a CTA
-// fewer than 2^16 vectors of a quad. Integer sums: the order is immaterial.
+// Statistics of every covered vector from its current code, up to 1024 codewords. CTA (x, y): the four
+// adjacent groups of quads y, y + gridDim.y, ..., rows x, x + gridDim.x, ... of each, thread = (row,
+// group): four lanes read a row's 128 bytes. The CTA sums its counts (per group) and fixed-point
+// terms in shared memory (planes of KS entries, KS >= K) and adds them to the global sums once. A term
+// (|v| < 2^30) enters shared memory as v = 2^15 vh + vl (0 <= vl < 2^15) in two 32-bit sums (native 32-bit
+// atomics): exact, as accumulate_grid gives a CTA fewer than 2^16 vectors of a quad. Integer sums:
+// the order is immaterial.
 // Bound: load latency and the shared atomics. (With a group per CTA a warp's 32-byte reads lay in 32
 // lines: 251 us per codebook of a 28672 x 8192 layer, now 206; k-means step 160 -> 156 us.)
-constexpr int kSmemStatsK = 256;
+// 257 to 1024 codewords take 80 KB instead of 20, which still leaves two CTAs per SM. Straight to the
+// global sums, as larger codebooks go, the few addresses of a small codebook are contended: 12000 x
+// 512 vectors took 1.39 ms with 300 codewords and 0.70 with 1024, now 0.117 and 0.142; 64 x 8 vectors,
+// the smallest measured, lose 1 to 3 us of 9 to zeroing and flushing.
+constexpr int kSmemStatsK = 256, kSmemStatsKMax = 1024;
 constexpr int kAccRows = 2;
 constexpr int kAccGroups = 4;
 
+constexpr size_t acc_smem(int KS) { return (size_t)KS * (2 * kD + kAccGroups) * sizeof(int); }
+
+template <int KS>
 __global__ void __launch_bounds__(256)
 accumulate_stats_kernel(SetView set, CbList cbs, int which, StatsView st, unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
   // [component][vh, vl][code]: lanes of a warp adding one component hit spread banks
-  __shared__ int s_b32[kD * 2 * kSmemStatsK];
-  __shared__ int s_cnt[kAccGroups * kSmemStatsK];
+  extern __shared__ __align__(16) int s_b32[];
+  int* s_cnt = s_b32 + kD * 2 * KS;  // [group of the quad][code]
   const CbView cw = cbs.cb[which];
   const float sscale = stats_scale_f(st);
-  const bool smem = cw.K <= kSmemStatsK;
   const int gq = threadIdx.x % kAccGroups;
   for (int64_t g0 = (int64_t)blockIdx.y * kAccGroups; g0 < cw.G_cov;
        g0 += (int64_t)gridDim.y * kAccGroups) {
-    if (smem) {
-      __syncthreads();  // the previous quad's flush has read the sums
-      for (int e = threadIdx.x; e < kSmemStatsK * kD * 2; e += blockDim.x) s_b32[e] = 0;
-      for (int e = threadIdx.x; e < kAccGroups * kSmemStatsK; e += blockDim.x) s_cnt[e] = 0;
-      __syncthreads();
-    }
+    __syncthreads();  // the previous quad's flush has read the sums
+    for (int e = threadIdx.x * 4; e < (2 * kD + kAccGroups) * KS; e += blockDim.x * 4)
+      *reinterpret_cast<int4*>(s_b32 + e) = make_int4(0, 0, 0, 0);
+    __syncthreads();
     const int64_t g = g0 + gq;
     if (g < cw.G_cov) {
       // the group's H block in registers: read once, not 64 loads per vector
@@ -117,41 +121,60 @@ accumulate_stats_kernel(SetView set, CbList cbs, int which, StatsView st, unsign
           }
           float q[kD];
           stats_htau(H, tau[u], q);
-          if (smem) {
-            atomicAdd(&s_cnt[gq * kSmemStatsK + k[u]], 1);
+          atomicAdd(&s_cnt[gq * KS + k[u]], 1);
 #pragma unroll
-            for (int j = 0; j < kD; ++j) {
-              const long long v = fix_rn_small(q[j], sscale);
-              atomicAdd(&s_b32[(2 * j) * kSmemStatsK + k[u]], (int)(v >> 15));
-              atomicAdd(&s_b32[(2 * j + 1) * kSmemStatsK + k[u]], (int)(v & 0x7fff));
-            }
-          } else {
-            stats_add(st, sscale, g, k[u], q);
+          for (int j = 0; j < kD; ++j) {
+            const long long v = fix_rn_small(q[j], sscale);
+            atomicAdd(&s_b32[(2 * j) * KS + k[u]], (int)(v >> 15));
+            atomicAdd(&s_b32[(2 * j + 1) * KS + k[u]], (int)(v & 0x7fff));
           }
         }
       }
     }
-    if (smem) {
-      __syncthreads();
-      for (int k = threadIdx.x; k < cw.K; k += blockDim.x) {
-        int all = 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k < cw.K; k += blockDim.x) {
+      int all = 0;
 #pragma unroll
-        for (int q = 0; q < kAccGroups; ++q) {
-          const int c = s_cnt[q * kSmemStatsK + k];
-          if (c != 0) atomicAdd(&st.cnt[(g0 + q) * st.K + k], c);
-          all += c;
-        }
-        if (all == 0) continue;
+      for (int q = 0; q < kAccGroups; ++q) {
+        const int c = s_cnt[q * KS + k];
+        if (c != 0) atomicAdd(&st.cnt[(g0 + q) * st.K + k], c);
+        all += c;
+      }
+      if (all == 0) continue;
 #pragma unroll
-        for (int j = 0; j < kD; ++j) {
-          const long long v = (long long)s_b32[(2 * j) * kSmemStatsK + k] * 32768 +
-                              s_b32[(2 * j + 1) * kSmemStatsK + k];
-          atomicAdd(reinterpret_cast<unsigned long long*>(&st.bacc[(int64_t)k * kD + j]),
-                    (unsigned long long)v);
-        }
+      for (int j = 0; j < kD; ++j) {
+        const long long v =
+            (long long)s_b32[(2 * j) * KS + k] * 32768 + s_b32[(2 * j + 1) * KS + k];
+        atomicAdd(reinterpret_cast<unsigned long long*>(&st.bacc[(int64_t)k * kD + j]),
+                  (unsigned long long)v);
       }
     }
   }
+}
+
+// The same for larger codebooks: every vector's terms straight to the global sums. CTA (x, y): groups y,
+// y + gridDim.y, ..., thread = row. Bound: latency of the atomics, so it wants many warps: H is read
+// per vector (35 registers; with four groups per CTA and H in registers, two CTAs per SM, 12000 x 512
+// vectors and 300 codewords took 2.2 ms instead of 1.4).
+__global__ void __launch_bounds__(256)
+accumulate_global_kernel(SetView set, CbList cbs, int which, StatsView st, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
+  const CbView cw = cbs.cb[which];
+  const float sscale = stats_scale_f(st);
+  for (int64_t g = blockIdx.y; g < cw.G_cov; g += gridDim.y)
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < set.M;
+         i += (int64_t)gridDim.x * blockDim.x) {
+      const int32_t k = cw.codes[i * cw.ld + g];
+      if (k < 0 || k >= cw.K) {
+        raise_error(err, ERRBIT_INDEX);
+        continue;
+      }
+      float tau[kD], q[kD];
+      stats_target(set, cbs, which, i, g, tau, err);
+      stats_htau(set.Hb + g * kD * kD, tau, q);
+      stats_add(st, sscale, g, k, q);
+    }
 }
 
 // Grid of accumulate_stats_kernel: one column of CTAs per quad of groups, enough of them for about 4
@@ -164,6 +187,30 @@ dim3 accumulate_grid(int64_t M, int64_t G_cov, int nsm) {
       ceil_div(M, 65000 / kAccGroups),
       std::max<int64_t>(1, std::min<int64_t>(want, ceil_div(M, 128))));
   return dim3((unsigned)rows_x, (unsigned)std::min<int64_t>(quads, 65535));
+}
+
+// Accumulates the statistics of codebook `which` over its M * G_cov > 0 covered vectors.
+crvq_status launch_accumulate(const SetView& set, const CbList& cbs, int which, const StatsView& st,
+                              unsigned* err, cudaStream_t stream) {
+  const CbView& cw = cbs.cb[which];
+  const int nsm = sm_count();
+  const dim3 grid = accumulate_grid(set.M, cw.G_cov, nsm);
+  if (cw.K <= kSmemStatsK) {
+    CRVQ_CUDA(launch_pdl(accumulate_stats_kernel<kSmemStatsK>, grid, dim3(256), acc_smem(kSmemStatsK),
+                         stream, set, cbs, which, st, err));
+  } else if (cw.K <= kSmemStatsKMax) {
+    CRVQ_TRY(smem_limit((const void*)accumulate_stats_kernel<kSmemStatsKMax>,
+                        acc_smem(kSmemStatsKMax)));
+    CRVQ_CUDA(launch_pdl(accumulate_stats_kernel<kSmemStatsKMax>, grid, dim3(256),
+                         acc_smem(kSmemStatsKMax), stream, set, cbs, which, st, err));
+  } else {
+    const int64_t x = std::min<int64_t>(ceil_div(4 * (int64_t)nsm, cw.G_cov), ceil_div(set.M, 1024));
+    CRVQ_CUDA(launch_pdl(accumulate_global_kernel,
+                         dim3((unsigned)x, (unsigned)std::min<int64_t>(cw.G_cov, 65535)), dim3(256), 0,
+                         stream, set, cbs, which, st, err));
+  }
+  CRVQ_LAUNCHED();
+  return CRVQ_OK;
 }
 
 // fp32 Cholesky factor of the packed lower triangle (false unless every pivot is positive)
@@ -496,10 +543,7 @@ crvq_status launch_update_codebook(const SetView& set, const CbList& cbs, int wh
   CRVQ_TRY(launch_stats_prepare(set, cbs, which, st, stream));
   if (n > 0) {
     ProfScope ps("update_accumulate", stream, (double)n);
-    const int nsm = sm_count();
-    CRVQ_CUDA(launch_pdl(accumulate_stats_kernel, accumulate_grid(set.M, cw.G_cov, nsm), dim3(256),
-                         0, stream, set, cbs, which, st, err));
-    CRVQ_LAUNCHED();
+    CRVQ_TRY(launch_accumulate(set, cbs, which, st, err, stream));
   }
   return launch_stats_solve(set, st, cw.C, C_out, counts, stream);
 }
@@ -533,13 +577,8 @@ crvq_status launch_update_codebook_on(const SetView& set, const CbList& cbs, int
   stats_bind(scratch, cw.G_cov, cw.K, &st);
   // The scratch keeps the previous call's contents: clear counts, sums and maxima.
   CRVQ_CUDA(cudaMemsetAsync(scratch, 0, L.total, stream));
-  const int nsm = sm_count();
   CRVQ_TRY(launch_maxabs(set, cbs, which, st, err, stream));
-  if (n > 0) {
-    CRVQ_CUDA(launch_pdl(accumulate_stats_kernel, accumulate_grid(set.M, cw.G_cov, nsm), dim3(256),
-                         0, stream, set, cbs, which, st, err));
-    CRVQ_LAUNCHED();
-  }
+  if (n > 0) CRVQ_TRY(launch_accumulate(set, cbs, which, st, err, stream));
   return launch_solve_kernels(set.Hb, st, cw.C, C_out, counts, err, stream);
 }
 

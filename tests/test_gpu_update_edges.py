@@ -1,5 +1,6 @@
-"""Edges of the codebook update's accumulation (four adjacent groups per block) and of the
-keep-if-better step (only changed tuples are compared) against the fp64 oracle. Counts are exact;
+"""Edges of the codebook update's accumulation (four adjacent groups per block; sums in shared memory up
+to 1024 codewords), of its solve (codewords per block by their number) and of the keep-if-better step
+(only changed tuples are compared) against the fp64 oracle. Counts are exact;
 codebooks agree to fp32 rounding of the solve (1e-4 of the largest value, the bar of the parity
 tests); codes equal the oracle's up to fp64 near-ties."""
 import numpy as np
@@ -21,8 +22,10 @@ def _blocks(rng, G, n=64):
     return (Xb.transpose(0, 2, 1) @ Xb / n + 0.05 * np.eye(D)).astype(np.float32)
 
 
-@pytest.mark.parametrize("M,G,Gc,K", [(1, 1, 1, 3), (127, 3, 2, 256), (129, 4, 1, 256),
-                                      (400, 5, 4, 257), (700, 9, 6, 100)])
+@pytest.mark.parametrize("M,G,Gc,K", [
+    (1, 1, 1, 3), (127, 3, 2, 256), (129, 4, 1, 256), (400, 5, 4, 257), (700, 9, 6, 100),
+    # the larger shared sums, the global sums, and the solve's four and eight codewords per CTA
+    (500, 6, 5, 305), (900, 7, 3, 611), (1300, 5, 5, 1024), (1300, 9, 2, 1025), (257, 4, 3, 4099)])
 def test_update_over_group_quads(M, G, Gc, K):
     rng = np.random.default_rng(100 * G + K)
     W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
@@ -42,8 +45,8 @@ def test_update_over_group_quads(M, G, Gc, K):
 @pytest.mark.parametrize("share", [0.0, 0.05, 1.0])
 @pytest.mark.parametrize("M,G,Gc", [(1, 1, 1), (600, 5, 2)])
 def test_keep_if_better_over_changed_tuples(M, G, Gc, share):
-    """`share` of the old codes are random, the others the best ones: a few, none or all of the
-    tuples change, over several batches of compared vectors and a ragged last one."""
+    """`share` of the old codes are random, the others the best ones: none, a few or all of the
+    tuples change."""
     rng = np.random.default_rng(int(100 * share) + M)
     W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
     Hb = _blocks(rng, G)

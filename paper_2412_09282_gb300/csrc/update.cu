@@ -13,6 +13,7 @@
 // same statistics for the codes it writes.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -362,62 +363,64 @@ __device__ __forceinline__ void fixed_to_pair(long long v, int sexp, float& h, f
   l = ldexpf(__fadd_rn(t, t2), -sexp);
 }
 
-// The least-squares solve of every codeword, one kernel. CTA = kSolveNC codewords; thread = (entry
+// The least-squares solve of every codeword, one kernel. CTA = NC codewords; thread = (entry
 // e of A_k's packed lower triangle or the count, slice of the groups). Each thread sums
 // cnt[g][k] * H_g[e] over its slice as an unevaluated fp32 pair for each of the CTA's codewords
 // (every product is split exactly: cnt < 2^24; TwoSum for the high part), so no fp64 arithmetic
-// runs per group and an H entry is read once for both codewords; the slices are added in a fixed
+// runs per group and an H entry is read once for all NC codewords; the slices are added in a fixed
 // order as fp32 pairs, and then a warp per codeword solves A_k c_k = b_k (b_k from the fixed point)
 // by Cholesky with refinement in fp32 pairs. The fixed assignment and order make the result
 // identical on every run. Codewords without members keep their old value.
 // Bound: latency (0.4 MB per launch). As two kernels, the solve with one thread per codeword, a 512 x
 // 512 layer (64 groups) took 5.3 + 8.0 us per Lloyd iteration; one kernel saves 4.8 us of that, and
 // nothing at 512 groups, where the sums' own work is the larger part; two slices per thread took 19 us
-// there, one takes 14.
+// there, one takes 14. NC is the smallest of 2, 4 and 8 that makes a single wave (one CTA per SM), 8 beyond
+// that: with 2 always, two of a CTA's 18 warps solved while the next CTAs waited (371 groups: 65536
+// codewords 2.32 ms, now 1.17; 4096: 141 us, now 83; 1024: 43 us, now 25; 256 keep 2: 16 us, 24 with 8).
 constexpr int kSolveSlices = 16;  // groups split 16 ways: short dependent chains per thread
 constexpr int kSumThreads = kSolveSlices * kNA;  // 592
-constexpr int kSolveNC = 2;       // 256 codewords: 128 CTAs, one wave
 
+template <int NC>
 __global__ void __launch_bounds__(kSumThreads)
 stats_solve_kernel(const float* __restrict__ Hb, StatsView st, const float* C_old, float* C_out,
                    int32_t* __restrict__ counts_out, unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
-  __shared__ float part_h[kSolveNC][kSolveSlices][kNA], part_l[kSolveNC][kSolveSlices][kNA];
-  __shared__ float sAh[kSolveNC][kNA], sAl[kSolveNC][kNA];
+  __shared__ float part_h[NC][kSolveSlices][kNA], part_l[NC][kSolveSlices][kNA];
+  __shared__ float sAh[NC][kNA], sAl[NC][kNA];
   const int tid = threadIdx.x;
   const int sl = tid / kNA;
   const int e = tid % kNA;
   const int K = st.K;
-  const int k0 = blockIdx.x * kSolveNC;
-  const int nk = min(kSolveNC, K - k0);
+  const int k0 = blockIdx.x * NC;
+  const int nk = min(NC, K - k0);
   // entry e of the packed lower triangle: row r, column c (c <= r); e = 36 is the count
   int r = 0;
   while ((r + 1) * (r + 2) / 2 <= e && r < kD - 1) ++r;
   const int c = e - r * (r + 1) / 2;
   const int hoff = r * kD + c;
-  float hi[kSolveNC], lo[kSolveNC];
+  float hi[NC], lo[NC];
 #pragma unroll
-  for (int q = 0; q < kSolveNC; ++q) hi[q] = lo[q] = 0.f;
+  for (int q = 0; q < NC; ++q) hi[q] = lo[q] = 0.f;
   // slice sl: gper groups, in group order
   const int64_t gper = (st.G_cov + kSolveSlices - 1) / kSolveSlices;
   const int64_t g0 = sl * gper, g1 = min(st.G_cov, g0 + gper);
   constexpr int kBatch = 8;  // groups whose loads are in flight together; no branches
   for (int64_t gb = 0; gb < gper; gb += kBatch) {
-    float fc[kBatch][kSolveNC], h[kBatch];
+    float fc[kBatch][NC], h[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
       const int64_t g = g0 + gb + u;
       const bool in = g < g1;
 #pragma unroll
-      for (int q = 0; q < kSolveNC; ++q)  // exact: counts stay below 2^24
+      for (int q = 0; q < NC; ++q)  // exact: counts stay below 2^24
         fc[u][q] = in && q < nk ? (float)st.cnt[g * K + k0 + q] : 0.f;
       h[u] = in ? (e < 36 ? __ldg(Hb + g * kD * kD + hoff) : 1.f) : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
 #pragma unroll
-      for (int q = 0; q < kSolveNC; ++q) {
+      for (int q = 0; q < NC; ++q) {
         const float p = __fmul_rn(fc[u][q], h[u]);
         const float pe = __fmaf_rn(fc[u][q], h[u], -p);  // fc h = p + pe exactly
         float sum, t;
@@ -427,7 +430,7 @@ stats_solve_kernel(const float* __restrict__ Hb, StatsView st, const float* C_ol
       }
   }
 #pragma unroll
-  for (int q = 0; q < kSolveNC; ++q) {
+  for (int q = 0; q < NC; ++q) {
     part_h[q][sl][e] = hi[q];
     part_l[q][sl][e] = lo[q];
   }
@@ -437,9 +440,9 @@ stats_solve_kernel(const float* __restrict__ Hb, StatsView st, const float* C_ol
   for (int64_t v = tid; v < st.G_cov * nk; v += kSumThreads)
     st.cnt[(v / nk) * K + k0 + v % nk] = 0;
   // Slices are merged per entry by one thread in fp32 pairs (TwoSum of the high parts, low parts
-  // added), in slice order; codeword q by warps 2 q and 2 q + 1.
-  const int q = tid >> 6, eq = tid & 63;
-  if (q < kSolveNC && eq < kNA) {
+  // added), in slice order.
+  for (int v = tid; v < NC * kNA; v += kSumThreads) {
+    const int q = v / kNA, eq = v % kNA;
     float h = part_h[q][0][eq], l = part_l[q][0][eq];
 #pragma unroll
     for (int s2 = 1; s2 < kSolveSlices; ++s2) {
@@ -486,8 +489,15 @@ crvq_status launch_solve_kernels(const float* Hb, const StatsView& st, const flo
                                  float* C_out, int32_t* counts, unsigned* err,
                                  cudaStream_t stream) {
   ProfScope ps("update_solve", stream, (double)st.K);
-  CRVQ_CUDA(launch_pdl(stats_solve_kernel, dim3((unsigned)ceil_div(st.K, kSolveNC)),
-                       dim3(kSumThreads), 0, stream, Hb, st, C_old, C_out, counts, err));
+  auto run = [&](auto nc) -> cudaError_t {
+    constexpr int NC = decltype(nc)::value;
+    return launch_pdl(stats_solve_kernel<NC>, dim3((unsigned)ceil_div(st.K, NC)), dim3(kSumThreads), 0,
+                      stream, Hb, st, C_old, C_out, counts, err);
+  };
+  const int nsm = sm_count();
+  CRVQ_CUDA(st.K <= 2 * nsm   ? run(std::integral_constant<int, 2>{})
+            : st.K <= 4 * nsm ? run(std::integral_constant<int, 4>{})
+                              : run(std::integral_constant<int, 8>{}));
   CRVQ_LAUNCHED();
   return CRVQ_OK;
 }

@@ -1043,11 +1043,14 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
 // --------------------------------------------------------------------------- arg-min pass,
 // codebooks of more than 256 codewords: a CTA walks `tiles` consecutive row tiles of one group
 // (thread = row = tensor-memory lane), streaming the codebook's precomputed B images in chunks of 128
-// codewords by bulk copy. Two halves of 128 threads share the tile's A rows and take alternate chunks,
-// each with its own accumulator, two chunk buffers, barriers and MMA issue; half 1 hands its minima to
-// half 0 at the tile's end. Two CTAs per SM: four pipelines of four warps whose waits (copy, MMA,
-// accumulator loads) overlap. (128 threads with two accumulators, so eight warps per SM, took 0.95 us
-// per chunk: one warp per scheduler and CTA cannot hide its own load and dependence latency.)
+// codewords by bulk copy, in two halves of 128 threads with an accumulator, two chunk buffers, barriers
+// and MMA issue each. OWN: a half takes every second tile and all chunks. Otherwise the halves share a
+// tile's A rows and take alternate chunks; half 1 hands its minima to half 0 at the tile's end. Two CTAs
+// per SM: four pipelines of four warps whose waits (copy, MMA, accumulator loads) overlap. (128 threads
+// with two accumulators, so eight warps per SM, took 0.95 us per chunk: one warp per scheduler and CTA
+// cannot hide its own load and dependence latency. Shared tiles alone left half 1 idle for the rows,
+// certificate and statistics of every tile, most of the work with few chunks: 300 codewords over 12000
+// x 512 vectors took 841 us, 596 with a tile per half.)
 //
 // Sweep, as in argmin_small_kernel but over 32-column granules and 32 classes (column % 32): a
 // granule's minimum and the class minima, 0.5 + 0.5 instructions per score, and the three smallest
@@ -1073,9 +1076,12 @@ constexpr int kGran = 32;      // columns per granule
 constexpr int kBRing = 2;      // B chunk buffers of a half
 
 constexpr int kHandWords = 5 + kGran;  // half 1's minima of a row
-constexpr size_t kArgminStreamSmem = (size_t)tcenc::kATile + 2 * kBRing * (size_t)kTcBTile +
-                                     (size_t)tcenc::kRows * (kD + kHandWords) * 4 + 1024;
+constexpr size_t argmin_stream_smem(bool own) {
+  return (own ? 2 : 1) * (size_t)tcenc::kATile + 2 * kBRing * (size_t)kTcBTile +
+         (size_t)tcenc::kRows * (own ? 2 * kD : kD + kHandWords) * 4 + 1024;
+}
 
+template <bool OWN>
 __global__ void __launch_bounds__(256, 2)
 argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_idx,
                  int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
@@ -1088,11 +1094,13 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   extern __shared__ __align__(1024) char smem_raw[];
   // 1024-byte aligned base, derived from the shared array (keeps the shared address space)
   char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
-  char* Atile = smem;                     // 16 KB
   const int tid = threadIdx.x, warp = tid >> 5, half = tid >> 7, rrow = tid & (kRows - 1);
-  char* Bbuf = smem + kATile + half * kBRing * kTcBTile;  // this half's kBRing x 16 KB
-  float* sQ = reinterpret_cast<float*>(smem + kATile + 2 * kBRing * kTcBTile);  // [128][8]: H r
-  uint32_t* hand = reinterpret_cast<uint32_t*>(sQ + kRows * kD);  // [kHandWords][128]
+  constexpr int kTiles = OWN ? 2 : 1;                     // A tiles at a time
+  char* Atile = smem + (OWN ? half : 0) * kATile;         // kTiles x 16 KB
+  char* Bbuf = smem + kTiles * kATile + half * kBRing * kTcBTile;  // this half's kBRing x 16 KB
+  float* sQ = reinterpret_cast<float*>(smem + kTiles * kATile + 2 * kBRing * kTcBTile) +
+              (OWN ? half : 0) * kRows * kD;              // [128][8]: H r
+  uint32_t* hand = reinterpret_cast<uint32_t*>(sQ + kRows * kD);  // [kHandWords][128] (not OWN)
   __shared__ __align__(16) float sH[kD * kD];
   __shared__ __align__(8) uint64_t bar_mma_s[2], bar_b_s[2][kBRing];
   __shared__ uint32_t tmem_slot;
@@ -1136,19 +1144,20 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   const float l1max = cbmax[0], cinf = cbmax[1];
   constexpr uint32_t idesc = tc::idesc_tf32(kRows, kTcCols);
 
-  // this CTA's row tiles (the last CTA of a column may have fewer)
+  // this CTA's row tiles (the last CTA of a column may have fewer); OWN: half h takes h, h + 2, ...
   const int64_t row_tiles = (set.M + kRows - 1) / kRows;
-  const int steps = (int)min((int64_t)tiles, row_tiles - (int64_t)blockIdx.x * tiles);
-  // A half's chunk uses are numbered over its tiles: use u is its chunk u % nch, codebook chunk
-  // 2 (u % nch) + half, in buffer u % kBRing. The half's thread 0 fetches, waits for and multiplies
-  // them in order (fetched: uses whose copy has started, issued: uses whose MMA has).
-  const int nch = (nchunk + 1 - half) >> 1;
+  const int my_tiles = (int)min((int64_t)tiles, row_tiles - (int64_t)blockIdx.x * tiles);
+  const int steps = OWN ? (my_tiles + 1 - half) >> 1 : my_tiles;
+  // A half's chunk uses are numbered over its tiles: use u is chunk u % nch of its chunks (all of the
+  // codebook's, or every second one), in buffer u % kBRing. The half's thread 0 fetches, waits for and
+  // multiplies them in order (fetched: uses whose copy has started, issued: uses whose MMA has).
+  const int nch = OWN ? nchunk : (nchunk + 1 - half) >> 1;
   const int64_t n_uses = (int64_t)steps * nch;
   int64_t fetched = 0, issued = 0;
   auto fetch = [&]() {  // the next chunk, into the buffer of the use kBRing before it
     const int b = (int)(fetched % kBRing);
     tc::mbar_expect_tx(tc::smem_u32(&bar_b[b]), kTcBTile);
-    const size_t chunk = (size_t)(2 * (fetched % nch) + half);
+    const size_t chunk = (size_t)(OWN ? fetched % nch : 2 * (fetched % nch) + half);
     const uint32_t dst = tc::smem_u32(Bbuf + b * kTcBTile), bar = tc::smem_u32(&bar_b[b]);
     const char* src = bpre + chunk * kTcBTile;
     tc::bulk_copy_g2s(dst, src, kBGroupCol * kBCol, bar);
@@ -1180,11 +1189,11 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   uint32_t mpar = 0;  // parity of the next MMA wait
 
   for (int t = 0; t < steps && ok; ++t) {
-    const int64_t i = ((int64_t)blockIdx.x * tiles + t) * kRows + rrow;
+    const int64_t i = ((int64_t)blockIdx.x * tiles + (OWN ? 2 * t + half : t)) * kRows + rrow;
     const bool row_ok = i < set.M;
-    // Prologue: the A rows, by half 0 (which also takes the rows' decisions).
+    // Prologue: the A rows; of a shared tile by half 0 (which also takes the rows' decisions).
     float pmax = 0.f, off = 0.f;
-    if (half == 0) {
+    if (OWN || half == 0) {
       float m2q[kD], rr, ra;
       if (rowterms) {  // precomputed for this Lloyd loop (row_terms_kernel)
         float4 q0 = make_float4(0.f, 0.f, 0.f, 0.f), q1 = q0, t2 = q0;
@@ -1237,7 +1246,10 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
       put_row(Atile, rrow, row);
       tc::fence_async_smem();
     }
-    __syncthreads();
+    if constexpr (OWN)
+      half_sync_and(half, true);
+    else
+      __syncthreads();
     if (rrow == 0) ok = issue();
 
     // fp32 bits: the three smallest granule minima, the first two's granules; the class minima
@@ -1259,7 +1271,7 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             const uint32_t m = min(min16_bits(v + kGran * q), min16_bits(v + kGran * q + 16));
-            const int gr = (2 * c + half) * (kTcCols / kGran) + 2 * rnd + q;
+            const int gr = (OWN ? c : 2 * c + half) * (kTcCols / kGran) + 2 * rnd + q;
             const bool lt1 = m < v1, lt2 = m < v2;
             v3 = min(v3, max(v2, m));
             b2 = lt1 ? b1 : (lt2 ? gr : b2);
@@ -1280,19 +1292,22 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
         if (c + 1 < nch) ok = issue();
       }
     }
-    if (half == 1 && ok) {
-      hand[0 * kRows + rrow] = v1;
-      hand[1 * kRows + rrow] = v2;
-      hand[2 * kRows + rrow] = v3;
-      hand[3 * kRows + rrow] = (uint32_t)b1;
-      hand[4 * kRows + rrow] = (uint32_t)b2;
+    if constexpr (OWN) {
+      if (!ok) break;
+    } else {
+      if (half == 1 && ok) {
+        hand[0 * kRows + rrow] = v1;
+        hand[1 * kRows + rrow] = v2;
+        hand[2 * kRows + rrow] = v3;
+        hand[3 * kRows + rrow] = (uint32_t)b1;
+        hand[4 * kRows + rrow] = (uint32_t)b2;
 #pragma unroll
-      for (int e = 0; e < kGran; ++e) hand[(5 + e) * kRows + rrow] = mc[e];
-    }
-    ok = __syncthreads_and(ok);
-    if (!ok) break;
-    if (half == 1) continue;  // (the next barrier is the next tile's, after its A rows)
-    {  // half 1's granules and classes
+        for (int e = 0; e < kGran; ++e) hand[(5 + e) * kRows + rrow] = mc[e];
+      }
+      ok = __syncthreads_and(ok);
+      if (!ok) break;
+      if (half == 1) continue;  // (the next barrier is the next tile's, after its A rows)
+      // half 1's granules and classes
       const uint32_t hv[3] = {hand[rrow], hand[kRows + rrow], hand[2 * kRows + rrow]};
       const int hb[3] = {(int)hand[3 * kRows + rrow], (int)hand[4 * kRows + rrow], 0};
 #pragma unroll
@@ -2847,7 +2862,8 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
   fl.cap = set.M * G_sub;
   fl.thr = reinterpret_cast<float*>(fl.vec + fl.cap);
   const float uc = kU * (tcenc::kCmul + 4.f * n_fixed);
-  CRVQ_TRY(smem_limit((const void*)argmin_tc_kernel, kArgminStreamSmem));
+  CRVQ_TRY(smem_limit((const void*)argmin_tc_kernel<true>, argmin_stream_smem(true)));
+  CRVQ_TRY(smem_limit((const void*)argmin_tc_kernel<false>, argmin_stream_smem(false)));
   for (int64_t gs = g_begin; gs < g_begin + G_range; gs += G_sub) {
     const int64_t gn = std::min<int64_t>(G_sub, g_begin + G_range - gs);
     const int64_t nv = set.M * gn;
@@ -2860,14 +2876,21 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
       CRVQ_LAUNCHED();
     }
     {
-      // row tiles per CTA: about sixteen waves of two CTAs per SM (a fine-grained tail)
+      // A tile per half (OWN) for codebooks of few chunks when every half on the chip gets one, a shared
+      // tile otherwise. OWN / shared: 300 codewords, 12000 x 512 vectors 596 / 841 us, 1024 x 128 29 / 34;
+      // 1024, 3001 x 371 249 / 296; 2048, 300 x 1000 206 / 204; 65536, 1024 x 1376 19.2 / 17.5 ms; one
+      // tile per group (1024, 128 x 1024) 78 / 72 us; few groups (1024, 700 x 30) 36 / 33 us.
       const int64_t row_tiles = ceil_div(set.M, tcenc::kRows);
-      const int64_t per_group = std::max<int64_t>(1, 32 * (int64_t)nsm / std::max<int64_t>(1, gn));
-      const int tiles = (int)std::max<int64_t>(1, ceil_div(row_tiles, per_group));
+      const bool own = cw.K <= 2048 && row_tiles >= 2 && gn * row_tiles >= 4 * (int64_t)nsm;
+      // row tiles per CTA: about sixteen waves of two CTAs per SM (a fine-grained tail)
+      const int64_t per_group =
+          std::max<int64_t>(1, (own ? 16 : 32) * (int64_t)nsm / std::max<int64_t>(1, gn));
+      const int tiles = (int)std::max<int64_t>(own ? 2 : 1, ceil_div(row_tiles, per_group));
       const dim3 grid((unsigned)ceil_div(row_tiles, tiles), (unsigned)gn);
       ProfScope ps(st.cnt ? "encode_argmin_lloyd" : "encode_argmin", stream,
                    (double)nv * cw.K);
-      CRVQ_CUDA(launch_pdl(argmin_tc_kernel, grid, dim3(256), kArgminStreamSmem, stream, set, gs,
+      auto* kernel = own ? argmin_tc_kernel<true> : argmin_tc_kernel<false>;
+      CRVQ_CUDA(launch_pdl(kernel, grid, dim3(256), argmin_stream_smem(own), stream, set, gs,
                            cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, nl, st, cbmax, bimg, bgrp, tout,
                            ex.rowterms, tiles, err));
       CRVQ_LAUNCHED();

@@ -43,7 +43,8 @@ def _check(W, Hb, C):
 @pytest.mark.parametrize("M,G,K", [
     (1, 1, 1), (127, 3, 2), (128, 2, 127), (129, 2, 128), (255, 5, 129), (256, 1, 255),
     (257, 7, 256), (300, 650, 16),                                   # shares over several groups
-    (130, 2, 257), (1, 3, 384), (257, 2, 385), (129, 3, 1025), (64, 2, 3000)])
+    (130, 2, 257), (1, 3, 384), (257, 2, 385), (129, 3, 1025), (64, 2, 3000),
+    (300, 310, 257), (257, 210, 640), (130, 320, 1100)])             # a row tile per half of a block
 def test_codebook_and_row_edges(M, G, K):
     rng = np.random.default_rng(M * 1000 + K)
     W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)

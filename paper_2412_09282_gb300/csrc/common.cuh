@@ -55,7 +55,8 @@ void count_launch();
 // (pdl_wait) before it reads anything or allocates tensor memory. Both are no-ops in a kernel
 // launched without the attribute. Removes the launch gap between dependent kernels of a layer
 // (with every kernel of the encode, update, reorder and loss steps: a 512 x 512 layer 1.43 -> 1.38 ms,
-// a k-means step 149 -> 143 us). A kernel that is launched this way has both at its very top.
+// a k-means step 149 -> 143 us). A kernel that is launched this way waits before anything but work on its
+// own shared memory, and triggers, if it does, at its very top.
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -678,8 +678,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
                     int s_idx, int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
                     unsigned long long* flag_total, StatsView st,
                     const float4* __restrict__ rowterms, unsigned* err) {
-  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
-  pdl_wait();
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor below
   using namespace tcenc;
   extern __shared__ __align__(1024) char smem_raw[];
   // 1024-byte aligned base, derived from the shared array (keeps the shared address space)
@@ -695,7 +694,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
   __shared__ __align__(8) uint64_t bar_mma_s[2];
   __shared__ uint32_t tmem_slot;
   __shared__ float s_l1[8], s_cinf[8];
-  __shared__ unsigned n_open;
+  __shared__ unsigned n_open, s_repeated[8];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int half = tid >> 7, rrow = tid & (kRows - 1);
@@ -706,7 +705,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
   const float uc = kU * cmul;
   const int nchunk = cw.K > kTcCols ? 2 : 1;
 
-  if (warp == 0) tc::tmem_alloc(&tmem_slot, 2 * kTcCols);
+  // Before the wait only this block's shared memory is touched.
   if (tid == 0) {
     n_open = 0;
     tc::mbar_init(tc::smem_u32(&bar_mma_s[0]), 1);
@@ -715,16 +714,40 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
   }
   for (int e = tid; e < kTcSmemStatsK * kD * 2; e += 256) s_b32[e] = 0;
   s_cnt[tid] = 0;
+  // Repeated codewords. Only the first of equal ones can be a row's code, so the others get padding
+  // columns: scored, they would leave every row nearest to them open with all of them as candidates (a
+  // matrix whose vectors are zero by half, where most codewords are zero too: a pass over 4096 x 512
+  // vectors took 12.5 ms, now 0.13). Two hash tables (in sQ, not in use yet) keep the smallest codeword of
+  // each slot. A repeated one that finds another codeword first in both of its slots goes unnoticed, and
+  // costs time only.
+  constexpr int kSlots = 1024;
+  int* s_slot = reinterpret_cast<int*>(sQ);                             // [2][kSlots]
+  uint32_t* s_hash = reinterpret_cast<uint32_t*>(s_slot + 2 * kSlots);  // [256]
+  uint32_t hash = 0;
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    *reinterpret_cast<int4*>(s_slot + 4 * (tid + 256 * e)) = make_int4(256, 256, 256, 256);
+  __syncthreads();
+  pdl_wait();
+  if (warp == 0) tc::tmem_alloc(&tmem_slot, 2 * kTcCols);
+  float cv[kD];
+#pragma unroll
+  for (int j = 0; j < kD; ++j) cv[j] = 0.f;
+  if (tid < cw.K) load_vec(cw.C + (int64_t)tid * kD, cv);
   {  // codebook maxima: max_k ||c_k||_1 (raised by 1e-6 relative) and max |c|
     float l1 = 0.f, cm = 0.f;
     if (tid < cw.K) {
-      float c[kD];
-      load_vec(cw.C + (int64_t)tid * kD, c);
 #pragma unroll
       for (int j = 0; j < kD; ++j) {
-        l1 += fabsf(c[j]);
-        cm = fmaxf(cm, fabsf(c[j]));
+        l1 += fabsf(cv[j]);
+        cm = fmaxf(cm, fabsf(cv[j]));
+        hash += __float_as_uint(__fadd_rn(cv[j], 0.f)) * (0x9E3779B1u * (2 * j + 1));  // (-0 as 0)
       }
+      hash ^= hash >> 13;
+      hash *= 0x85EBCA6Bu;
+      atomicMin(&s_slot[hash >> 22], tid);
+      atomicMin(&s_slot[kSlots + ((hash >> 12) & (kSlots - 1))], tid);
+      s_hash[tid] = hash;
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -739,6 +762,23 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  {
+    bool repeated = false;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int first = s_slot[e == 0 ? hash >> 22 : kSlots + ((hash >> 12) & (kSlots - 1))];
+      if (first < tid && s_hash[first] == hash && tid < cw.K) {
+        float o[kD];
+        load_vec(cw.C + (int64_t)first * kD, o);
+        bool same = true;
+#pragma unroll
+        for (int j = 0; j < kD; ++j) same = same && cv[j] == o[j];
+        repeated = repeated || same;
+      }
+    }
+    const unsigned rep = __ballot_sync(0xffffffffu, repeated);
+    if (lane == 0) s_repeated[warp] = rep;  // (read by its own warp, after the first segment's barrier)
+  }
   // this half's accumulator: columns [128 half, 128 half + 128)
   const uint32_t tmem = tmem_slot + (uint32_t)(half * kTcCols);
   const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -771,7 +811,7 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
       uint32_t row[kK];
       float tk[3];
       if (tid < nchunk * kTcCols) {
-        build_b_row(cw.C, cw.K, tid, sH, uc, row, tk);
+        build_b_row(cw.C, (s_repeated[warp] >> lane) & 1u ? 0 : cw.K, tid, sH, uc, row, tk);
         put_row(Bbuf + (tid >> 7) * kTcBTile, tid & (kTcCols - 1), row);
         sNaL1[tid] = make_float2(tk[1], tk[2]);
       }

@@ -11,6 +11,7 @@ import paper_2412_09282_gb300 as P
 from paper_2412_09282_gb300 import Codebook
 from oracle import crvq_oracle as O
 from parity_util import check_codes_with_ties, dev, host
+from synthetic import LayerConfig
 
 pytestmark = pytest.mark.gpu
 
@@ -97,6 +98,29 @@ def test_three_close_codewords_in_different_granules(K):
     base = (0.02 * rng.standard_normal((K // 4, D))).astype(np.float32)
     C = np.concatenate([base * (1 + 1e-7 * t) for t in range(4)]).astype(np.float32)
     _check(W, _blocks(rng, G), C)
+
+
+@pytest.mark.parametrize("K", [40, 256])
+def test_repeated_codewords_do_not_open_rows(K):
+    """Half of the vectors and of the codewords zero (of both signs), others repeated: the smallest index of
+    equal codewords, and few rows that need an exact decision."""
+    rng = np.random.default_rng(K)
+    M, G = 300, 9
+    W = (0.02 * rng.standard_normal((M, G, D))).astype(np.float32)
+    W[rng.random((M, G)) < 0.5] = 0.0
+    W = W.reshape(M, G * D)
+    C = (0.02 * rng.standard_normal((K, D))).astype(np.float32)
+    C[rng.random(K) < 0.5] = 0.0
+    C[rng.random(K) < 0.2] *= -0.0
+    C[K - 4:] = C[:4]
+    codes = _check(W, _blocks(rng, G), C)
+    first = np.array([np.nonzero((C == c).all(1))[0][0] for c in C])
+    np.testing.assert_array_equal(first[codes], codes)
+
+    cfg = LayerConfig("zeros", M, G * D, 64, "plain", "lognormal", K_base=K, n_ext=0, B=1,
+                      kmeans_iters=2, refine_rounds=0)
+    out = P.crvq_quantize_layer(dev(W), dev(rng.standard_normal((64, G * D)).astype(np.float32)), cfg)
+    assert out.report["flagged"] < 0.1 * 6 * M * G  # six passes
 
 
 def _tail_errs(T, C0s, H):

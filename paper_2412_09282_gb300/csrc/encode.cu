@@ -1097,8 +1097,8 @@ argmin_small_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
 // granule minima with the first two's numbers (10 instructions per 32 scores). The winner is the
 // smallest granule's column of the smallest class; the runner-up is the second smallest granule or
 // class minimum. An open row whose third smallest granule lies above the bound has its candidates in
-// two granules and the classes below the bound (a few columns): the narrow list, decided by
-// argmin_narrow_kernel. The others (wide list) are decided over the whole codebook. Sending every
+// two granules and the classes below the bound (a few columns): the narrow list (decide_narrow).
+// The others (wide list) are decided over the whole codebook. Sending every
 // open row over the whole codebook took 60% of a K = 65536 pass (3% of the rows are open there).
 struct NarrowRow {
   uint32_t i, g;     // row, group (absolute)
@@ -1439,18 +1439,17 @@ argmin_tc_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_id
   if (warp == 0) tc::tmem_dealloc(tmem_slot, 2 * kTcCols);
 }
 
-// Exact decision of the narrow list, a quarter warp per row.
-__global__ void __launch_bounds__(128)
-argmin_narrow_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int s_idx,
-                     int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
-                     NarrowList list, StatsView st, unsigned* err) {
-  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
-  pdl_wait();
+// Exact decision of the narrow list, a quarter warp per row, by every warp of the grid.
+__device__ __forceinline__ void decide_narrow(const SetView& set, const CbList& cbs, int n_fixed,
+                                              int s_idx, int32_t* __restrict__ out_code,
+                                              int64_t out_ld, int64_t out_g0, const NarrowList& list,
+                                              const StatsView& st, unsigned* err) {
   const int n = (int)*list.count;
   if (list.total && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(list.total, (unsigned long long)n);
   const float sscale = st.cnt ? stats_scale_f(st) : 1.f;
   const int quarter = (threadIdx.x & 31) >> 3;
-  for (int e0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * 4; e0 < n; e0 += gridDim.x * 16) {
+  const int warps = (int)(blockDim.x >> 5);
+  for (int e0 = (blockIdx.x * warps + (threadIdx.x >> 5)) * 4; e0 < n; e0 += gridDim.x * warps * 4) {
     const int e = e0 + quarter;
     const NarrowRow o = list.row[min(e, n - 1)];
     const int ga = (int)(o.gran >> 16), gb = (int)(o.gran & 0xffffu), ne = __popc(o.classes);
@@ -1458,6 +1457,18 @@ argmin_narrow_kernel(SetView set, int64_t g_begin, CbList cbs, int n_fixed, int 
                 [&](int c) { return kGran * (c < ne ? ga : gb) + nth_bit(o.classes, c % ne); },
                 out_code, out_ld, out_g0, st, sscale, err);
   }
+}
+
+// Whether c equals codeword k (an index past the codebook: no). A thread's candidate that repeats its best so
+// far cannot win, and is not scored (see argmin_small_kernel on repeated codewords).
+__device__ __forceinline__ bool equals(const CbView& cw, int k, const float c[kD]) {
+  if (k >= cw.K) return false;
+  float o[kD];
+  load_vec(cw.C + (int64_t)k * kD, o);
+  bool same = true;
+#pragma unroll
+  for (int j = 0; j < kD; ++j) same = same && c[j] == o[j];
+  return same;
 }
 
 // Exact decision of rows open over the whole codebook (argmin_tc_kernel's wide list): one CTA per row.
@@ -1473,8 +1484,8 @@ constexpr int kWideBatch = 4;  // codewords a thread loads before using them
 __global__ void __launch_bounds__(kExactThreads)
 argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, int n_fixed,
                     int s_idx, int32_t* __restrict__ out_code, int64_t out_ld, int64_t out_g0,
-                    FlagList flags, StatsView st, const float4* __restrict__ terms,
-                    unsigned* err) {
+                    FlagList flags, unsigned many, StatsView st,
+                    const float4* __restrict__ terms, unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
   constexpr int kWarps = kExactThreads / 32;
@@ -1484,6 +1495,7 @@ argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
   __shared__ int bk_s[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned cnt = min((unsigned long long)*flags.count, (unsigned long long)flags.cap);
+  if (cnt > many) return;  // (argmin_exact_warp_kernel has taken them)
   if (flags.total && blockIdx.x == 0 && tid == 0) atomicAdd(flags.total, cnt);
   const CbView cw = cbs.cb[s_idx];
   const float cmul = bound_mult(n_fixed);
@@ -1529,7 +1541,7 @@ argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
     float bh = INFINITY, bl = 0.f;
     int bk = 0x7fffffff;
     sweep([&](int k, const float cv[kD], float nn, float na, float l1) {
-      if (low_from(nn, na, l1, cv, m2q, nbeta, cmul) <= U) {
+      if (low_from(nn, na, l1, cv, m2q, nbeta, cmul) <= U && !equals(cw, bk, cv)) {
         float eh, el;
         dfl::quad_err(rh, rl, cv, sH, eh, el);
         if (dfl::less(eh, el, k, bh, bl, bk)) {
@@ -1591,13 +1603,15 @@ constexpr int kExactBatch = 2;  // codewords a lane loads before using them
 __global__ void __launch_bounds__(128)
 argmin_exact_warp_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs,
                          int n_fixed, int s_idx, int32_t* __restrict__ out_code, int64_t out_ld,
-                         int64_t out_g0, FlagList flags, StatsView st,
+                         int64_t out_g0, NarrowList narrow, FlagList flags, unsigned many, StatsView st,
                          const float4* __restrict__ terms, unsigned* err) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
+  decide_narrow(set, cbs, n_fixed, s_idx, out_code, out_ld, out_g0, narrow, st, err);
   __shared__ float sHw[4][kD * kD];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned cnt = min((unsigned long long)*flags.count, (unsigned long long)flags.cap);
+  if (cnt <= many) return;  // (left to argmin_exact_kernel)
   if (flags.total && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(flags.total, cnt);
   const CbView cw = cbs.cb[s_idx];
   const float cmul = bound_mult(n_fixed);
@@ -1614,7 +1628,7 @@ argmin_exact_warp_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList c
     target32(set, cbs, n_fixed, i, g, rv, av, err);
     vector_terms(rv, av, sH, m2q, pmax);
     const float nbeta = -2.f * kU * cmul * pmax;
-    const float4* gt = terms ? terms + grel * cw.K : nullptr;
+    const float4* gt = terms + grel * cw.K;
     // a lane takes codewords lane, lane + 32, ...; kExactBatch of them are loaded before any is
     // used, so their L2 round trips overlap
     float U = thr;
@@ -1626,21 +1640,13 @@ argmin_exact_warp_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList c
         const int k = k0 + 32 * u;
         if (k < cw.K) {
           load_vec(cw.C + (int64_t)k * kD, cv[u]);
-          if (gt) tt[u] = gt[k];
+          tt[u] = gt[k];
         }
       }
 #pragma unroll
       for (int u = 0; u < kExactBatch; ++u) {
         if (k0 + 32 * u >= cw.K) break;
-        float nn, na, l1;
-        if (gt) {
-          nn = tt[u].x;
-          na = tt[u].y;
-          l1 = tt[u].z;
-        } else {
-          codeword_terms(cv[u], sH, nn, na, l1);
-        }
-        U = fminf(U, up_from(nn, na, l1, cv[u], m2q, pmax, cmul));
+        U = fminf(U, up_from(tt[u].x, tt[u].y, tt[u].z, cv[u], m2q, pmax, cmul));
       }
     }
 #pragma unroll
@@ -1650,17 +1656,10 @@ argmin_exact_warp_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList c
     float bh = INFINITY, bl = 0.f;
     int bk = 0x7fffffff;
     for (int k = lane; k < cw.K; k += 32) {
-      float cv[kD], nn, na, l1;
+      float cv[kD];
       load_vec(cw.C + (int64_t)k * kD, cv);
-      if (gt) {
-        const float4 t = gt[k];
-        nn = t.x;
-        na = t.y;
-        l1 = t.z;
-      } else {
-        codeword_terms(cv, sH, nn, na, l1);
-      }
-      if (low_from(nn, na, l1, cv, m2q, nbeta, cmul) <= U) {
+      const float4 t = gt[k];
+      if (low_from(t.x, t.y, t.z, cv, m2q, nbeta, cmul) <= U && !equals(cw, bk, cv)) {
         float eh, el;
         dfl::quad_err(rh, rl, cv, sH, eh, el);
         if (dfl::less(eh, el, k, bh, bl, bk)) {
@@ -2937,20 +2936,17 @@ crvq_status launch_argmin_large(const SetView& set, const CbList& cbs, const Arg
     }
     {
       ProfScope pf("encode_exact", stream, 0.0);
-      CRVQ_CUDA(launch_pdl(argmin_narrow_kernel,
-                           dim3((unsigned)std::min<int64_t>(ceil_div(nv, 16), 8 * nsm)), dim3(128), 0,
-                           stream, set, gs, cbs, n_fixed, s_idx, out, out_ld, out_g0, nl, st, err));
-      CRVQ_LAUNCHED();
-      if (cw.K <= kExactWarpK) {
-        CRVQ_CUDA(launch_pdl(argmin_exact_warp_kernel,
-                             dim3((unsigned)std::min<int64_t>(ceil_div(nv, 4), 16 * nsm)),
-                             dim3(128), 0, stream, set, gs, gn, cbs, n_fixed, s_idx, out,
-                             out_ld, out_g0, fl, st, tout, err));
-      } else {
-        CRVQ_CUDA(launch_pdl(argmin_exact_kernel,
-                             dim3((unsigned)std::min<int64_t>(nv, 2 * nsm)), dim3(kExactThreads), 0,
-                             stream, set, gs, gn, cbs, n_fixed, s_idx, out, out_ld, out_g0, fl,
-                             st, tout, err));
+      // few wide rows go to blocks, one each (eight per block of that grid at most)
+      const unsigned blocks = (unsigned)std::min<int64_t>(nv, 2 * nsm);
+      const unsigned many = cw.K <= kExactWarpK ? 0u : 8 * blocks;
+      CRVQ_CUDA(launch_pdl(argmin_exact_warp_kernel,
+                           dim3((unsigned)std::min<int64_t>(ceil_div(nv, 4), 16 * nsm)), dim3(128), 0,
+                           stream, set, gs, gn, cbs, n_fixed, s_idx, out, out_ld, out_g0, nl, fl, many,
+                           st, tout, err));
+      if (many) {
+        CRVQ_LAUNCHED();
+        CRVQ_CUDA(launch_pdl(argmin_exact_kernel, dim3(blocks), dim3(kExactThreads), 0, stream, set, gs,
+                             gn, cbs, n_fixed, s_idx, out, out_ld, out_g0, fl, many, st, tout, err));
       }
       CRVQ_LAUNCHED();
     }

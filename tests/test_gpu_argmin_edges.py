@@ -100,6 +100,21 @@ def test_three_close_codewords_in_different_granules(K):
     _check(W, _blocks(rng, G), C)
 
 
+@pytest.mark.parametrize("K,M", [(600, 300), (1100, 300), (1100, 40), (2500, 300)])
+def test_open_rows_by_repeated_codewords_of_a_large_codebook(K, M):
+    """Half of the vectors and of the codewords zero: thousands of rows open over most of the codebook
+    (with 40 rows: hundreds, which blocks take instead of warps above 1024 codewords)."""
+    rng = np.random.default_rng(K + M)
+    G = 40
+    W = (0.02 * rng.standard_normal((M, G, D))).astype(np.float32)
+    W[rng.random((M, G)) < 0.5] = 0.0
+    C = (0.02 * rng.standard_normal((K, D))).astype(np.float32)
+    C[rng.random(K) < 0.5] = 0.0
+    C[7] = 0.0
+    codes = _check(W.reshape(M, G * D), _blocks(rng, G), C)
+    assert codes[(W == 0).all(2)].max() <= 7
+
+
 @pytest.mark.parametrize("K", [40, 256])
 def test_repeated_codewords_do_not_open_rows(K):
     """Half of the vectors and of the codewords zero (of both signs), others repeated: the smallest index of

@@ -21,7 +21,10 @@
 // The rows do not see one another, so all 32 group steps of a block run in one kernel
 // (coupled_block_kernel), a CTA carrying up to 32 rows through them with its slice of B^T in shared
 // memory, and the launches between steps (five per group: target, operand images, arg-min, exact
-// decisions, update) and the round trips of B^T through L2 are gone.
+// decisions, update) and the round trips of B^T through L2 are gone. Its scores run on the fp32 pipe, and
+// a row that they leave open is a scan of the codebook by one warp, so for large codebooks and many rows
+// the steps go through the encode path's tensor-core arg-min instead (coupled_target_kernel,
+// launch_encode_beam on the shifted targets, coupled_apply_kernel): the same decisions, on the same t'.
 #include <algorithm>
 #include <vector>
 
@@ -129,6 +132,49 @@ block_factor_kernel(const float* __restrict__ H, int64_t N, int64_t G_cov,
       Lf[g * kD * kD + r * kD + c] = (ok && c <= r) ? (float)L[r * kD + c] : 0.f;
     }
     Linv[g * kD + r] = ok ? (float)(1.0 / L[r * kD + r]) : 0.f;
+  }
+}
+
+// x = H_gg^-1 b from the factor: L y = b, L^T x = y.
+__device__ __forceinline__ void factor_solve(const float* L, const float* inv, const float b[kD],
+                                             float x[kD]) {
+  float y[kD];
+#pragma unroll
+  for (int r = 0; r < kD; ++r) {
+    float acc = b[r];
+#pragma unroll
+    for (int m = 0; m < r; ++m) acc = fmaf(-L[r * kD + m], y[m], acc);
+    y[r] = acc * inv[r];
+  }
+#pragma unroll
+  for (int r = kD - 1; r >= 0; --r) {
+    float acc = y[r];
+#pragma unroll
+    for (int m = r + 1; m < kD; ++m) acc = fmaf(-L[m * kD + r], x[m], acc);
+    x[r] = acc * inv[r];
+  }
+}
+
+// Vector (i, g) of D and of its operand images.
+__device__ __forceinline__ void store_residual(float* D, int64_t N, char* d_hi, char* d_lo,
+                                               int64_t nslab, int64_t i, int64_t g,
+                                               const float nv[kD]) {
+  uint32_t hi[kD], lo[kD];
+#pragma unroll
+  for (int j = 0; j < kD; ++j) {
+    hi[j] = tc::to_tf32(nv[j]);
+    lo[j] = tc::to_tf32(nv[j] - __uint_as_float(hi[j]));
+  }
+  float* d = D + i * N + g * kD;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    *reinterpret_cast<float4*>(d + 4 * q) =
+        make_float4(nv[4 * q], nv[4 * q + 1], nv[4 * q + 2], nv[4 * q + 3]);
+    const int64_t off = img::img_off(i, g * kD + 4 * q, nslab);
+    *reinterpret_cast<uint4*>(d_hi + off) =
+        make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
+    *reinterpret_cast<uint4*>(d_lo + off) =
+        make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
   }
 }
 
@@ -274,22 +320,8 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
         for (int m = 0; m < kD; ++m) hd = fmaf(sH[q * kD + m], dg[m], hd);
         b[q] = s.B[tid * kCplPad + col0 + q] - hd;
       }
-      // H_gg x = b: L y = b, L^T x = y
-      float y[kD], sv[kD];
-#pragma unroll
-      for (int r = 0; r < kD; ++r) {
-        float acc = b[r];
-#pragma unroll
-        for (int m = 0; m < r; ++m) acc = fmaf(-sL[r * kD + m], y[m], acc);
-        y[r] = acc * sInv[r];
-      }
-#pragma unroll
-      for (int r = kD - 1; r >= 0; --r) {
-        float acc = y[r];
-#pragma unroll
-        for (int m = r + 1; m < kD; ++m) acc = fmaf(-sL[m * kD + r], sv[m], acc);
-        sv[r] = acc * sInv[r];
-      }
+      float sv[kD];
+      factor_solve(sL, sInv, b, sv);
 #pragma unroll
       for (int j = 0; j < kD; ++j) s.T[tid][j] = (dg[j] + ck[j]) + sv[j];
     }
@@ -439,26 +471,13 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
         cw.codes[i * cw.ld + g] = kn;
         float ck[kD], nv[kD];
         load_vec(C + (int64_t)kn * kD, ck);
-        uint32_t hi[kD], lo[kD];
 #pragma unroll
         for (int j = 0; j < kD; ++j) {
           const float2 r = s.R[gl][tid][j];
           nv[j] = pair_minus(r.x, r.y, ck[j]);
           s.DD[tid][j] = nv[j] - s.DD[tid][j];
-          hi[j] = tc::to_tf32(nv[j]);
-          lo[j] = tc::to_tf32(nv[j] - __uint_as_float(hi[j]));
         }
-        float* d = a.D + i * a.N + g * kD;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          *reinterpret_cast<float4*>(d + 4 * q) =
-              make_float4(nv[4 * q], nv[4 * q + 1], nv[4 * q + 2], nv[4 * q + 3]);
-          const int64_t off = img::img_off(i, g * kD + 4 * q, a.nslab);
-          *reinterpret_cast<uint4*>(a.d_hi + off) =
-              make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
-          *reinterpret_cast<uint4*>(a.d_lo + off) =
-              make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
-        }
+        store_residual(a.D, a.N, a.d_hi, a.d_lo, a.nslab, i, g, nv);
       } else {
 #pragma unroll
         for (int j = 0; j < kD; ++j) s.DD[tid][j] = 0.f;
@@ -486,6 +505,111 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
   }
 }
 
+// ---- the same step in three parts, for the tensor-core arg-min; B^T summed over the chunks first.
+
+// P[0] += P[1] + ... in order (n elements each).
+__global__ void __launch_bounds__(256)
+coupled_sum_chunks_kernel(float* __restrict__ P, int chunks, int64_t n) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    float v = P[e];
+    for (int q = 1; q < chunks; ++q) v += P[q * n + e];
+    P[e] = v;
+  }
+}
+
+// Shifted targets of group g (step 1 of coupled_block_kernel), a thread per row: Tp[i][8].
+__global__ void __launch_bounds__(128)
+coupled_target_kernel(const __grid_constant__ CplArgs a, int64_t g, const float* __restrict__ Bt,
+                      float* __restrict__ Tp, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
+  __shared__ float sH[kD * kD], sL[kD * kD], sInv[kD];
+  if (threadIdx.x < kD * kD) {
+    sH[threadIdx.x] = a.Hb[g * kD * kD + threadIdx.x];
+    sL[threadIdx.x] = a.Lf[g * kD * kD + threadIdx.x];
+  }
+  if (threadIdx.x < kD) sInv[threadIdx.x] = a.Linv[g * kD + threadIdx.x];
+  __syncthreads();
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= a.M) return;
+  const CbView cw = a.cbs.cb[a.which];
+  const int col0 = (int)(g - a.g0) * kD;
+  float dg[kD], ck[kD], b[kD], sv[kD];
+  load_vec(a.D + i * a.N + g * kD, dg);
+#pragma unroll
+  for (int j = 0; j < kD; ++j) ck[j] = 0.f;
+  const int32_t k = cw.codes[i * cw.ld + g];
+  if (code_ok(k, cw.K, err)) load_vec(cw.C + (int64_t)k * kD, ck);
+#pragma unroll
+  for (int q = 0; q < kD; ++q) {
+    float hd = 0.f;
+#pragma unroll
+    for (int m = 0; m < kD; ++m) hd = fmaf(sH[q * kD + m], dg[m], hd);
+    b[q] = Bt[(int64_t)(col0 + q) * a.M + i] - hd;
+  }
+  factor_solve(sL, sInv, b, sv);  // (no factor: zeros)
+#pragma unroll
+  for (int j = 0; j < kD; ++j) sv[j] = (dg[j] + ck[j]) + sv[j];
+  float* t = Tp + i * kD;
+  *reinterpret_cast<float4*>(t) = make_float4(sv[0], sv[1], sv[2], sv[3]);
+  *reinterpret_cast<float4*>(t + 4) = make_float4(sv[4], sv[5], sv[6], sv[7]);
+}
+
+// Applies the decisions of group g (step 4 of coupled_block_kernel): 32 rows per CTA, a lane each; the
+// first warp takes the code, D_g and its change, all eight the later columns of the block in turn.
+__global__ void __launch_bounds__(256)
+coupled_apply_kernel(const __grid_constant__ CplArgs a, int64_t g, const int32_t* __restrict__ code,
+                     float* __restrict__ Bt, unsigned* err) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
+  __shared__ float sDD[kD][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+  const CbView cw = a.cbs.cb[a.which];
+  if (a.Linv[g * kD] == 0.f) return;  // no factor (reported): the codes stay
+  if (warp == 0) {
+    float dd[kD];
+#pragma unroll
+    for (int j = 0; j < kD; ++j) dd[j] = 0.f;
+    if (i < a.M) {
+      const int32_t kn = code[i];
+      if (code_ok(kn, cw.K, err)) {
+        cw.codes[i * cw.ld + g] = kn;
+        const SetView wset{a.W, a.N, a.M, a.N / kD, nullptr};
+        float rh[kD], rl[kD], ck[kD], nv[kD];
+        others_target(wset, a.cbs, a.which, i, g, rh, rl, err);
+        load_vec(cw.C + (int64_t)kn * kD, ck);
+        load_vec(a.D + i * a.N + g * kD, dd);
+#pragma unroll
+        for (int j = 0; j < kD; ++j) {
+          nv[j] = pair_minus(rh[j], rl[j], ck[j]);
+          dd[j] = nv[j] - dd[j];
+        }
+        store_residual(a.D, a.N, a.d_hi, a.d_lo, a.nslab, i, g, nv);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kD; ++j) sDD[j][lane] = dd[j];
+  }
+  __syncthreads();
+  if (i >= a.M) return;
+  float dd[kD];
+#pragma unroll
+  for (int j = 0; j < kD; ++j) dd[j] = sDD[j][lane];
+  const int ncol = (int)(a.g1 - a.g0) * kD;
+#pragma unroll 4
+  for (int col = (int)(g + 1 - a.g0) * kD + warp; col < ncol; col += 8) {
+    float acc = Bt[(int64_t)col * a.M + i];
+#pragma unroll
+    for (int q = 0; q < kD; ++q)
+      acc = fmaf(dd[q], __ldg(a.H + (g * kD + q) * a.N + a.g0 * kD + col), acc);
+    Bt[(int64_t)col * a.M + i] = acc;
+  }
+}
+
 // *out = sum of part[0 .. n) (one CTA, strided sums and a tree: a fixed order).
 __global__ void __launch_bounds__(1024)
 sum_parts_kernel(const double* __restrict__ part, int64_t n, double* out) {
@@ -499,6 +623,18 @@ sum_parts_kernel(const double* __restrict__ part, int64_t n, double* out) {
     __syncthreads();
   }
   if (threadIdx.x == 0) *out = red[0];
+}
+
+// Whether a sweep's steps go through the tensor-core arg-min. coupled_block_kernel takes about 10 ns per
+// codeword and step (more above 16384 codewords, whose open rows are long scans) for each wave of blocks;
+// the arg-min takes about 30 us per step in its five launches, 4 ns more per codeword, and next to
+// nothing per row. Block kernel / arg-min, one sweep with both losses: 4096 x 1024, 4096 codewords 6.4 / 6.9
+// ms, 8192 13.2 / 10.9, 65536 142 / 64; 6000 x 1024 (two waves), 1024 codewords 3.6 / 4.2, 2048 6.2 / 5.4;
+// 9800 x 512 (three), 256 1.3 / 1.8, 1024 2.5 / 2.1; 16384 x 512 (four), 256 1.7 / 1.9, 600 2.7 / 2.2;
+// 28672 x 512 (six), 256 2.6 / 2.6, 4096 16 / 5.
+bool coupled_by_argmin(int64_t M, int K, int rows, int nsm) {
+  const int64_t waves = ceil_div(ceil_div(M, rows), nsm);
+  return K * waves * waves > 6000;
 }
 
 }  // namespace
@@ -551,6 +687,16 @@ crvq_status launch_coupled_sweep(const float* W, int64_t M, int64_t N, const flo
   if (loss_dev) CRVQ_TRY(loss_into(loss_dev));
   // rows per CTA: every SM gets rows, at least eight of them (a group step is mostly latency)
   const int rows = (int)std::min<int64_t>(kCplRows, std::max<int64_t>(8, ceil_div(M, nsm)));
+  const bool by_argmin = coupled_by_argmin(M, cw.K, rows, nsm);
+  Scratch mT, mW;
+  EncodeExtras ex;
+  if (by_argmin) {
+    CRVQ_TRY(mT.alloc((size_t)M * (kD + 1) * sizeof(float), stream));
+    const size_t wbytes = argmin_scratch_bytes(M, 1, cw.K);
+    CRVQ_TRY(mW.alloc(wbytes, stream));
+    ex.work = mW.as<char>();
+    ex.work_bytes = wbytes;
+  }
   for (int sw = 0; sw < sweeps; ++sw) {
     for (int64_t b0 = 0; b0 < G_cov; b0 += kBlockG) {
       const int64_t b1 = std::min<int64_t>(G_cov, b0 + kBlockG);
@@ -561,9 +707,34 @@ crvq_status launch_coupled_sweep(const float* W, int64_t M, int64_t N, const flo
       const CplArgs ca{W, D, H, Hb, Lf, Linv, mB.as<float>(), (int)chunks, d_hi, d_lo,
                        ceil_div(N, (int64_t)img::kSlabK), M, N, b0, b1, rows, which, cbs};
       ProfScope ps("coupled_block", stream, (double)M * (b1 - b0) * cw.K);
-      CRVQ_TRY(smem_limit((const void*)coupled_block_kernel, kCplSmem));
-      coupled_block_kernel<<<(unsigned)ceil_div(M, rows), kCplThreads, kCplSmem, stream>>>(ca, err);
-      CRVQ_LAUNCHED();
+      if (!by_argmin) {
+        CRVQ_TRY(smem_limit((const void*)coupled_block_kernel, kCplSmem));
+        coupled_block_kernel<<<(unsigned)ceil_div(M, rows), kCplThreads, kCplSmem, stream>>>(ca, err);
+        CRVQ_LAUNCHED();
+        continue;
+      }
+      float* Bt = mB.as<float>();
+      float* Tp = mT.as<float>();
+      int32_t* code = reinterpret_cast<int32_t*>(Tp + M * kD);
+      if (chunks > 1) {
+        const int64_t n = (int64_t)nc * M;
+        CRVQ_CUDA(launch_pdl(coupled_sum_chunks_kernel, dim3((unsigned)std::min<int64_t>(
+                             ceil_div(n, 256), 16 * nsm)), dim3(256), 0, stream, Bt, (int)chunks, n));
+        CRVQ_LAUNCHED();
+      }
+      CbList one{};
+      one.n = 1;
+      one.cb[0] = CbView{cw.C, code, 1, 1, cw.K};
+      for (int64_t g = b0; g < b1; ++g) {
+        CRVQ_CUDA(launch_pdl(coupled_target_kernel, dim3((unsigned)ceil_div(M, (int64_t)128)),
+                             dim3(128), 0, stream, ca, g, Bt, Tp, err));
+        CRVQ_LAUNCHED();
+        CRVQ_TRY(launch_encode_beam(SetView{Tp, kD, M, 1, Hb + g * kD * kD}, one, 0, 1, false,
+                                    nullptr, ex, stream));
+        CRVQ_CUDA(launch_pdl(coupled_apply_kernel, dim3((unsigned)ceil_div(M, (int64_t)32)), dim3(256),
+                             0, stream, ca, g, code, Bt, err));
+        CRVQ_LAUNCHED();
+      }
     }
     if (loss_dev) CRVQ_TRY(loss_into(loss_dev + 1 + sw));
   }

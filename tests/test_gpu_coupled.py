@@ -149,10 +149,14 @@ def test_coupled_sweep_on_a_quantized_q_proj_sampled_rows():
     _stepwise(host(Ws), host(Hs), ocbs, 0, host(out.codes_base), rows)
 
 
-@pytest.mark.parametrize("M,G,K", [(1, 1, 1), (33, 33, 300), (7, 65, 256), (1300, 3, 257)])
+@pytest.mark.parametrize("M,G,K", [
+    (1, 1, 1), (33, 33, 300), (7, 65, 256), (1300, 3, 257),
+    # steps by the tensor-core arg-min: a large codebook, and several waves of rows with a smaller one
+    (1, 2, 6100), (45, 34, 6500), (9001, 3, 1600), (20000, 2, 400), (30000, 2, 200)])
 def test_coupled_sweep_block_row_and_codebook_edges(M, G, K):
     """Rows around a CTA's share, groups around the 32-group blocks, codebooks around the 256 of a
-    score chunk; stepwise against the fp64 arg-min, losses against the oracle."""
+    score chunk and around the line between the two forms of a step; stepwise against the fp64 arg-min
+    (sampled rows of the large ones), losses against the oracle."""
     import paper_2412_09282_gb300 as P
     from paper_2412_09282_gb300 import Codebook
     W, H, cbs = _case(31, M=M, G=G, K=K, Ke=5, Gc=min(G, 2), n=8 * G + 100)
@@ -160,7 +164,8 @@ def test_coupled_sweep_block_row_and_codebook_edges(M, G, K):
     loss = P.crvq_coupled_sweep(dev(W), dev(H), gcbs, 0, sweeps=1)
     P.crvq_sync()
     codes = host(gcbs[0].codes)
-    _stepwise(W, H, cbs, 0, codes, np.arange(M))
+    rows = np.arange(M) if M <= 1300 else np.sort(np.random.default_rng(M).choice(M, 300, False))
+    _stepwise(W, H, cbs, 0, codes, rows)
     after = [O.Codebook(cbs[0].C, codes, G), cbs[1]]
     assert loss[0] == pytest.approx(O.full_loss(W, H, cbs), rel=1e-5)
     assert loss[1] == pytest.approx(O.full_loss(W, H, after), rel=1e-5)

@@ -18,7 +18,7 @@
  *  - Calls enqueue work on `stream` and return without waiting, except calls that return a
  *    value in host memory (their documentation says so): those synchronize `stream`.
  *  - Scratch memory is stream-ordered on `stream`, from a memory pool of the library's own (one
- *    per device) that keeps at most 1 GiB between calls.
+ *    per device) that keeps at most 1 GiB between calls (crvq_release_scratch gives it back).
  *  - Arguments are validated before any launch: a bad argument returns
  *    CRVQ_ERR_INVALID_ARG, an unsupported size CRVQ_ERR_UNSUPPORTED, and nothing is
  *    enqueued. crvq_last_error() then describes the problem (per host thread).
@@ -95,6 +95,11 @@ const char* crvq_last_error(void);
  * (the library's, and that of crvq_update_codebook_noalloc): CRVQ_OK, CRVQ_ERR_DEVICE,
  * CRVQ_ERR_NUMERIC or CRVQ_ERR_TIMEOUT (or CRVQ_ERR_CUDA). */
 crvq_status crvq_sync(crvq_stream_t stream);
+
+/* Gives the scratch memory that the library keeps on the current device back to the device, for
+ * other allocators to use; what calls still in flight hold stays (synchronize first to give back all
+ * of it). The next call that needs scratch maps it again. */
+crvq_status crvq_release_scratch(void);
 
 /* Library build string (compiler, architecture). Host memory, static. */
 const char* crvq_version(void);

@@ -10,7 +10,7 @@ from .api import (  # noqa: F401
     crvq_hessian_blocks, crvq_hessian_inverse_diag,
     crvq_kmeans_init, crvq_lut_matvec, crvq_n_crit_groups, crvq_quantize_layer,
     crvq_reconstruct_error,
-    crvq_select_reorder_channels, crvq_sync, crvq_update_codebook_noalloc, crvq_profile_begin,
+    crvq_release_scratch, crvq_select_reorder_channels, crvq_sync, crvq_update_codebook_noalloc, crvq_profile_begin,
     crvq_profile_end, crvq_profile_filter, crvq_launch_count, crvq_selftest_bounded_wait,
     crvq_update_codebook,
     crvq_version, CrvqError, IMPORTANCE_WA, IMPORTANCE_W_ONLY, IMPORTANCE_RANDOM,

@@ -51,6 +51,7 @@ SIGNATURES = {
     "crvq_last_error": (C.c_char_p, []),
     "crvq_version": (C.c_char_p, []),
     "crvq_sync": (C.c_int32, [c_vp]),
+    "crvq_release_scratch": (C.c_int32, []),
     "crvq_profile_begin": (C.c_int32, []),
     "crvq_profile_end": (C.c_int32, [C.POINTER(crvq_kernel_stat), C.c_int32, c_i32p]),
     "crvq_profile_filter": (C.c_int32, [C.c_char_p]),

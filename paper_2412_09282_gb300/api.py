@@ -99,6 +99,12 @@ def crvq_sync(stream=None, device=None):
     _check(_L().crvq_sync(_stream(stream, dev)))
 
 
+def crvq_release_scratch(device=None):
+    """Give the scratch memory that the library keeps on the device (at most 1 GiB) back to it."""
+    with torch.cuda.device(device if device is not None else torch.cuda.current_device()):
+        _check(_L().crvq_release_scratch())
+
+
 def crvq_selftest_bounded_wait(stream=None, device=None):
     """Enqueue the bounded-wait self-test: the next crvq_sync raises CRVQ_ERR_TIMEOUT."""
     dev = device if device is not None else torch.cuda.current_device()

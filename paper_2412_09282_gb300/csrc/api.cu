@@ -53,7 +53,8 @@ std::vector<int> g_sm;               // per device
 // whenever a stream is synchronized, so a call after a synchronization paid for mapping its scratch
 // again (0.25 ms for a few MB, 0.7 ms for the 330 MB of a 4096 x 4096 reconstruction). This pool keeps
 // at most kPoolKeep of what is free; the rest goes back at the next synchronization, and all of
-// it when an allocation fails. Freed memory is reused in stream order by any stream or thread.
+// it when an allocation fails or crvq_release_scratch asks for it. Freed memory is reused in stream order
+// by any stream or thread.
 namespace {
 constexpr uint64_t kPoolKeep = uint64_t(1) << 30;
 
@@ -342,6 +343,19 @@ const char* crvq_version(void) {
 }
 
 int64_t crvq_launch_count(void) { return (int64_t)g_launches.load(); }
+
+crvq_status crvq_release_scratch(void) {
+  clear_last_error();
+  int dev = 0;
+  CRVQ_CUDA(cudaGetDevice(&dev));
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    if ((int)g_pools.size() > dev) pool = g_pools[dev];
+  }
+  if (pool) CRVQ_CUDA(cudaMemPoolTrimTo(pool, 0));
+  return CRVQ_OK;
+}
 
 crvq_status crvq_profile_begin(void) {
   {

@@ -122,3 +122,24 @@ def test_noalloc_update_reports_device_errors_through_crvq_sync():
     P.crvq_sync()
     np.testing.assert_array_equal(out.cpu().numpy(), ref.cpu().numpy())
     np.testing.assert_array_equal(cnt.cpu().numpy(), ref_cnt.cpu().numpy())
+
+
+def test_kept_scratch_is_given_back_on_request():
+    """A reconstruction's scratch (over 200 MB) stays with the library until crvq_release_scratch; the
+    next call maps it again and gives the same results."""
+    import paper_2412_09282_gb300 as P
+    from paper_2412_09282_gb300 import Codebook
+    g = torch.Generator(device="cuda").manual_seed(0)
+    M = N = 4096
+    W = 0.02 * torch.randn((M, N), generator=g, device="cuda")
+    X = torch.randn((1024, N), generator=g, device="cuda")
+    Hb = torch.eye(8, device="cuda").expand(N // 8, 8, 8).contiguous()
+    cb = [Codebook(0.02 * torch.randn((256, 8), generator=g, device="cuda"),
+                   torch.randint(0, 256, (M, N // 8), generator=g, device="cuda", dtype=torch.int32),
+                   N // 8)]
+    a = P.crvq_reconstruct_error(W, 8, Hb, None, cb, 0, X=X, want_W_hat=False)
+    P.crvq_sync()
+    held = torch.cuda.mem_get_info()[0]
+    P.crvq_release_scratch()
+    assert torch.cuda.mem_get_info()[0] - held > 200 << 20
+    assert P.crvq_reconstruct_error(W, 8, Hb, None, cb, 0, X=X, want_W_hat=False) == a

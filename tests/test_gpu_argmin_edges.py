@@ -75,7 +75,7 @@ def test_block_and_class_edges(K):
 
 
 @pytest.mark.parametrize("K", [64, 256, 600])
-def test_open_rows_more_than_a_list_holds(K):
+def test_rows_open_by_close_codewords(K):
     """Every codeword twice, the copy one unit in the last place off: no row is certified."""
     rng = np.random.default_rng(K)
     M, G = 700, 4
@@ -98,6 +98,70 @@ def test_three_close_codewords_in_different_granules(K):
     base = (0.02 * rng.standard_normal((K // 4, D))).astype(np.float32)
     C = np.concatenate([base * (1 + 1e-7 * t) for t in range(4)]).astype(np.float32)
     _check(W, _blocks(rng, G), C)
+
+
+@pytest.mark.parametrize("K", [64, 256])
+def test_open_rows_more_than_a_list_holds(K):
+    """1950 tile pairs in at most a few hundred blocks, every row open (the copies are one unit in the last
+    place off): a block finds over a thousand open rows, four times what its list holds, so most are
+    decided inside the running pipeline. The same codes as four groups at a time, where a block has one
+    tile pair and its list holds every row; sampled groups against the oracle."""
+    rng = np.random.default_rng(K)
+    M, G = 700, 650
+    W = (0.02 * rng.standard_normal((M, G * D))).astype(np.float32)
+    C = (0.02 * rng.standard_normal((K // 2, D))).astype(np.float32)
+    C = np.concatenate([C, np.nextafter(C, np.float32(1))]).astype(np.float32)
+    Hb = _blocks(rng, G)
+    Wd, Hd, Cd = dev(W), dev(Hb), dev(C)
+
+    def run(g0, n):
+        codes = torch.full((M, n), -1, dtype=torch.int32, device="cuda")
+        P.crvq_encode_beam(Wd[:, g0 * D:(g0 + n) * D], D, Hd[g0:g0 + n], [Codebook(Cd, codes, n)], 0, 1)
+        P.crvq_sync()
+        return host(codes)
+
+    codes = run(0, G)
+    parts = np.concatenate([run(g0, min(4, G - g0)) for g0 in range(0, G, 4)], axis=1)
+    np.testing.assert_array_equal(codes, parts)
+    for g in (0, 317, 649):
+        T, cb = W[:, g * D:(g + 1) * D], [O.Codebook(C, None, 1)]
+        oc, _ = O.encode_beam(T, D, Hb[g:g + 1], cb, 0, 1)
+        check_codes_with_ties(T, D, Hb[g:g + 1], cb, 0, [codes[:, g:g + 1]], oc)
+
+
+def test_lloyd_statistics_of_open_rows_more_than_a_list_holds():
+    """A layer's base codebook after one Lloyd iteration from an initial codebook whose codewords come in
+    pairs one unit in the last place apart: every row of its pass is open, far more per block than the list
+    holds. Counts and sums of all of them: the same codebook and codes, bit for bit, as a separate
+    encode, update and encode."""
+    M, G, K = 700, 650, 64
+    N = G * D
+    rng = np.random.default_rng(9)
+    cfg = LayerConfig("open_rows", M, N, 64, "plain", "lognormal", K_base=K, n_ext=0, B=1,
+                      kmeans_iters=1, refine_rounds=0, importance_mode=2)
+    X = dev(rng.standard_normal((64, N)).astype(np.float32))
+    W = (0.02 * rng.standard_normal((M, N))).astype(np.float32)
+    perm = P.crvq_quantize_layer(dev(W), X, cfg).perm  # the random order depends on the seed alone
+    Ws = W[:, host(perm)].reshape(M * G, D)
+    at = O.kmeans_sample_indices(M * G, K, O.phase_seed(cfg.seed, O.PHASE_BASE, 0))
+    for a, b in zip(at[0::2], at[1::2]):
+        Ws[b] = np.nextafter(Ws[a], np.float32(1))
+    W[:, host(perm)] = Ws.reshape(M, N)
+    out = P.crvq_quantize_layer(dev(W), X, cfg)
+    assert torch.equal(out.perm, perm)
+    assert out.report["flagged"] > M * G // 2
+
+    T = dev(Ws.reshape(M, N))
+    Hb, _, _ = P.crvq_hessian_blocks(X, cfg.damp_rel, perm=perm)
+    C = P.crvq_kmeans_init(T, D, G, K, O.phase_seed(cfg.seed, O.PHASE_BASE, 0))
+    codes = torch.empty((M, G), dtype=torch.int32, device="cuda")
+    P.crvq_encode_beam(T, D, Hb, [Codebook(C, codes, G)], 0, 1)
+    C, counts = P.crvq_update_codebook(T, D, Hb, [Codebook(C, codes, G)], 0)
+    assert int(counts.sum()) == M * G
+    P.crvq_encode_beam(T, D, Hb, [Codebook(C, codes, G)], 0, 1)
+    P.crvq_sync()
+    assert torch.equal(out.C_base, C)
+    assert torch.equal(out.codes_base, codes)
 
 
 @pytest.mark.parametrize("K,M", [(600, 300), (1100, 300), (1100, 40), (2500, 300)])

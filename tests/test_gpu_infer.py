@@ -3,9 +3,11 @@ against the fp64 oracle's lookup-table product (O.lut_matvec, pinned on the CPU 
 explicit route W_hat x).
 
 Bar: |y_gpu - y_oracle| <= 1e-5 * sum over the terms of |<c, x>|, the sum taken with |C| and
-|x| (fp32 arithmetic: each codeword-input product is an 8-term FMA chain, a warp adds 32 group
-terms in a 5-level tree, the slices are added in order, so the rounding error is below about
-(8 + 5 + slices) * 2^-24 of that sum).
+|x|. fp32 arithmetic: a codeword-input product is two 4-term FMA chains and their sum (5 roundings).
+Tables add 32 units in a tree (5) and those sums in order, dots add up to 16 units in order, then
+those sums, then up to 8 warps' sums; the CTAs' shares meet in a tree (3). So with n units per
+share the error is below (5 + 16 + n / 16 + 8 + 3) * 2^-24 of that sum: 8e-6 for n = 1600, more than
+any case here has.
 """
 import numpy as np
 import pytest
@@ -123,7 +125,14 @@ def test_lut_matvec_is_deterministic_and_reports_bad_codes():
 @pytest.mark.parametrize("b,M,N,Ks,Gcs", [
     (1, 1, 8, [16], [1]),                               # one row, one group
     (8, 97, 16, [256, 3], [2, 1]),                      # fewer units than a cluster has CTAs
-    (5, 40, 8 * 261, [256, 256], [261, 7]),             # tables of several sub-ranges of units
+    (5, 40, 8 * 261, [256, 256], [261, 7]),             # shares with a remainder of four units
+    (1, 300, 8 * 70, [300, 1000], [70, 20]),            # tables with a stride of the largest codebook
+    (1, 129, 8 * 37, [1024], [37]),                     # the largest tables of one input
+    (2, 257, 8 * 65, [400, 512, 3], [65, 65, 2]),       # of two
+    (2, 50, 8 * 33, [513], [33]),                       # just too large for them
+    (1, 70, 8 * 1700, [256, 60], [1700, 30]),           # shares of more units than are resident: tables,
+    (8, 70, 8 * 1700, [256, 60], [1700, 30]),           # dots,
+    (3, 900, 8 * 1600, [700], [1600]),                  # and dots from L2
     (2, 20000, 8 * 9, [17, 5], [9, 2]),                 # more rows per cluster than threads
     (4, 130, 8 * 37, [5000, 64, 300], [37, 11, 10]),    # dotted and looked-up codebooks mixed
 ])

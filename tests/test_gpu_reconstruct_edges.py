@@ -1,9 +1,10 @@
-"""Reconstruction of a matrix large enough that the slices without extended codebooks run in a launch
-of their own and a block takes several row blocks, against plain fp64 sums: reconstructions are
+"""Reconstruction of matrices large enough that the slices without extended codebooks run in a launch
+of their own, and that a block takes several row blocks, against plain fp64 sums: reconstructions are
 bit-exact, block losses within 1e-4 (the bar of the parity tests: fp32 terms). Sums that leave fp32's
 range, for good or on the way, are those of fp64 rounded."""
 import numpy as np
 import pytest
+import torch
 
 import paper_2412_09282_gb300 as P
 from paper_2412_09282_gb300 import Codebook
@@ -38,6 +39,31 @@ def test_reconstruct_over_row_blocks_and_slices(M, N, Gc):
     per_group = np.einsum("mgi,gij,mgj->g", d, Hb.astype(np.float64), d, optimize=True)
     assert abs(lb - per_group.sum()) <= 1e-4 * per_group.sum()
     assert abs(lc - per_group[:Gc].sum()) <= 1e-4 * per_group[:Gc].sum()
+
+
+def test_reconstruct_with_several_row_blocks_per_block():
+    """158 row groups of 33 slices, more than sixteen blocks per SM: a block takes three or four row
+    groups, the last ones ragged. Against fp64 on the device."""
+    M, N, Gc = 20011, 8200, 40
+    G = N // D
+    g = torch.Generator(device="cuda").manual_seed(1)
+    W = 0.02 * torch.randn((M, N), generator=g, device="cuda")
+    A = torch.randn((G, 12, D), generator=g, device="cuda")
+    Hb = (A.transpose(1, 2) @ A / 12 + 0.05 * torch.eye(D, device="cuda")).contiguous()
+    perm = torch.randperm(N, generator=g, device="cuda").to(torch.int32)
+    cbs = [Codebook(0.02 * torch.randn((k, D), generator=g, device="cuda"),
+                    torch.randint(0, k, (M, c), generator=g, device="cuda", dtype=torch.int32), c)
+           for k, c in ((256, G), (16, Gc), (9, Gc))]
+    Wh, lb, lc, _ = P.crvq_reconstruct_error(W, D, Hb, perm, cbs, Gc)
+    rec = cbs[0].C.double()[cbs[0].codes.long()]
+    for cb in cbs[1:]:
+        rec[:, :Gc] += cb.C.double()[cb.codes.long()]
+    rec = rec.float().view(M, N)
+    assert torch.equal(Wh[:, perm.long()], rec)
+    d = (W - rec).double().view(M, G, D)
+    per_group = torch.stack([((d[:, i] @ Hb[i].double()) * d[:, i]).sum() for i in range(G)])
+    assert abs(lb - float(per_group.sum())) <= 1e-4 * float(per_group.sum())
+    assert abs(lc - float(per_group[:Gc].sum())) <= 1e-4 * float(per_group[:Gc].sum())
 
 
 @pytest.mark.parametrize("n_cb", [3, 6])

@@ -375,8 +375,9 @@ coupled_block_kernel(const __grid_constant__ CplArgs a, unsigned* err) {
       }
       __syncthreads();
       if (row8 < nr) {
+        // (a NaN score never wins; it takes f2 down to f1, which opens the row unless a smaller one follows)
 #pragma unroll 8
-        for (int kk = j8; kk < nk; kk += 8) {  // (a NaN score makes the two equal: the row is open)
+        for (int kk = j8; kk < nk; kk += 8) {
           const float sc = s.S[row8][kk];
           k1 = sc < f1 ? k0 + kk : k1;  // ties: the smaller index
           f2 = fminf(f2, fmaxf(f1, sc));

@@ -12,8 +12,8 @@
 // is certified when low_2nd - low_j > 2 Et_j: every other codeword's exact score is then larger
 // than j's. Otherwise the vector is open: the codewords with low_k <= low_j + 2 Et_j (the exact
 // arg-min is among them) are decided among in fp32 pairs (score.cuh). Codes therefore equal the fp64
-// arg-min (ties to the smaller index) except for ties at fp64 rounding level. Beam stages use the same
-// bounds on a sorted top-(B+1) list.
+// arg-min (ties to the smaller index) except for ties below the pairs' resolution, a few 2^-48 of
+// |r - c|^T |H| |r - c|. Beam stages use the same bounds on a sorted top-(B+1) list.
 #include <algorithm>
 #include <cstdlib>
 #include <type_traits>
@@ -164,13 +164,11 @@ __device__ __forceinline__ void stage_chunk(const float* __restrict__ C, int k0,
 //   A row (vector):   [q_hi x8 | q_hi x8 | q_lo x8 | 1 1 | beta_hi beta_hi beta_lo | off_hi off_lo | 0]
 //   B row (codeword): [c_hi x8 | c_lo x8 | c_hi x8 | n'_hi n'_lo | L1_hi L1_lo L1_hi | 1 1 | 0]
 // One tcgen05.mma M = 128 vectors x N = 128 codewords x K = 8, four per chunk (K = 32), fp32
-// accumulator in tensor memory. The epilogue reads each row's scores in blocks of 16: per block
-// its minimum (integer minima of the non-negative fp32 bit patterns); per row the block with the
-// smallest minimum, kept whole, and the second smallest block minimum. The row's winner and
-// second smallest score come from those 17 values, exact (no packed index). The certificate and
-// the fp64 fallback are those of the fp32 pass, with the bound multiplier raised to cover the
-// tensor-core products and accumulation (about 2^-22 per split product and fp32 accumulation
-// over 32 terms).
+// accumulator in tensor memory. The epilogue takes minima of the non-negative scores as integer minima
+// of their bit patterns, along the columns in two ways, so that the smallest of each name the winner's
+// column (argmin_small_kernel, argmin_tc_kernel). The certificate is that of the fp32 pass, with the bound
+// multiplier raised to cover the tensor-core products and accumulation (about 2^-22 per split product
+// and fp32 accumulation over 32 terms); rows without it are decided in fp32 pairs.
 namespace tcenc {
 
 constexpr int kRows = 128;        // vectors per row tile (TMEM lanes)
@@ -282,9 +280,9 @@ prep_b_kernel(SetView set, int64_t g_begin, const float* __restrict__ C, int K, 
               unsigned* __restrict__ flag_count) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
-  // The open lists of the arg-min pass that follows start empty. The previous pass's exact
-  // kernels, which read the counts, completed before the wait above returned.
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) flag_count[threadIdx.x] = 0u;
+  // The flag list of the beam stage that follows starts empty. The previous stage's fallback, which
+  // read the count, completed before the wait above returned.
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *flag_count = 0u;
   if (blockIdx.x == gridDim.x - 1) {  // the last column of CTAs: the codebook maxima (its first)
     if (blockIdx.y == 0) cbmax_block(C, K, cbmax);
     return;
@@ -331,7 +329,8 @@ prep_b_split_kernel(SetView set, int64_t g_begin, const float* __restrict__ C, i
                     unsigned* __restrict__ flag_count) {
   pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
   pdl_wait();
-  // The open lists of the arg-min pass that follows start empty (see prep_b_kernel).
+  // The open lists of the arg-min pass that follows start empty. The previous pass's exact kernels,
+  // which read the counts, completed before the wait above returned.
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) flag_count[threadIdx.x] = 0u;
   if (blockIdx.x == gridDim.x - 1) {  // the last column of CTAs: the codebook maxima (its first)
     if (first && blockIdx.y == 0) cbmax_block(C, K, cbmax);
@@ -1591,12 +1590,14 @@ argmin_exact_kernel(SetView set, int64_t g_begin, int64_t G_range, CbList cbs, i
 }
 
 
-// Exact decision of flagged rows, one warp per row, for codebooks of up to kExactWarpK
-// entries: the bounds and fp32-pair scores of argmin_exact_kernel without block barriers.
-// Lane l takes codewords l, l + 32, ...; the fp32 upper bounds give U, every codeword whose
-// lower bound reaches U is scored in fp32 pairs by the lane that holds it, and the best
-// (value, index) is reduced across the warp with the same total order, so the decision is the
-// one argmin_exact_kernel makes.
+// Exact decision of both open lists: the narrow one, then the wide one with a warp per row, by the bounds
+// and fp32-pair scores of argmin_exact_kernel without block barriers. Lane l takes codewords l, l + 32,
+// ...; the fp32 upper bounds give U, every codeword whose lower bound reaches U is scored in fp32 pairs
+// by the lane that holds it, and the best (value, index) is reduced across the warp with the same total
+// order, so the decision is the one argmin_exact_kernel makes. Wide lists of at most `many` rows are left
+// to that kernel: above kExactWarpK codewords a lone row is a long scan for a warp, but with thousands of
+// them (a matrix full of repeated vectors) a block each wastes its barriers and most of its threads
+// (4096 codewords, half of 1024 x 512 vectors open: 38 ms by blocks, 14 by warps).
 constexpr int kExactWarpK = 1024;
 constexpr int kExactBatch = 2;  // codewords a lane loads before using them
 
@@ -3051,10 +3052,11 @@ crvq_status encode_range(const SetView& set, int64_t g_begin, int64_t G_range,
   for (int s = 0; s < S; ++s) {
     sd.s = s;
     sd.Bs = (s == S - 1) ? 1 : B;  // only the best tuple of the last stage is used
-    CRVQ_CUDA(cudaMemsetAsync(fl.count, 0, sizeof(unsigned), stream));
     BeamBufs bb{in_h, in_n, out_h, out_n};
     const int K = cbs.cb[sd.st[s]].K;
     const bool tc_stage = beam_tc_applies(sd, cbs, G_range);
+    if (!tc_stage)  // (prep_b_kernel clears it for the tensor-core stages)
+      CRVQ_CUDA(cudaMemsetAsync(fl.count, 0, sizeof(unsigned), stream));
     if (tc_stage)
       CRVQ_TRY(launch_beam_stage_tc(set, g_begin, G_range, cbs, n_fixed, sd, bb, fl, err,
                                     tc_mem.as<char>(), (double)nvec * parents * K, stream));

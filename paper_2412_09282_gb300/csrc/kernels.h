@@ -90,7 +90,7 @@ struct EncodeExtras {
   // The codes are not wanted (a Lloyd iteration that needs only their statistics): an arg-min pass
   // over one codebook leaves the codebook's codes as they are.
   bool discard_codes = false;
-  unsigned long long* flag_total = nullptr;  // device: += vectors sent to the fp64 fallback
+  unsigned long long* flag_total = nullptr;  // device: += vectors decided exactly
   // Scratch of the arg-min pass provided by the caller (e.g. once for a whole Lloyd loop, so
   // that its iterations allocate nothing); used when at least argmin_scratch_bytes long.
   char* work = nullptr;

@@ -65,6 +65,44 @@ blocks_add_delta_kernel(const float* __restrict__ xsq, int64_t N, const double* 
   if (i < N) Hb[i * 8 + (i & 7)] = (float)((double)xsq[i] + *delta64);
 }
 
+// blocks_sum_kernel, hessian_delta_kernel and blocks_add_delta_kernel in one block, the same values, for
+// up to kSmallRows channels and kSmallTerms chunk terms: there two launches more are most of the difference
+// (16 x 128: 32 us as three kernels, 28 as one; 1024 x 512 44 us either way; with 32768 terms, 4096 x
+// 1024, one block is slower, 54 us instead of 51).
+constexpr int kSmallRows = 1024;
+constexpr int64_t kSmallTerms = 8192;
+
+__global__ void __launch_bounds__(kSmallRows)
+blocks_small_kernel(const float* __restrict__ P, int chunks, int64_t stride, float scale, int N,
+                    float damp_rel, float* __restrict__ xsq, float* __restrict__ delta_out,
+                    double* __restrict__ delta64, float* __restrict__ Hb) {
+  pdl_trigger();  // dependents may launch; this grid waits for its predecessor first
+  pdl_wait();
+  __shared__ double part[kSmallRows];
+  __shared__ float sx[kSmallRows];
+  const int t = threadIdx.x;
+  for (int e = t; e < N * 8; e += kSmallRows) {
+    const float v = chunk_sum(P, chunks, stride, e, scale);
+    if (((e >> 3) & 7) == (e & 7))
+      xsq[e >> 3] = sx[e >> 3] = v;
+    else
+      Hb[e] = v;
+  }
+  __syncthreads();
+  part[t] = t < N ? (double)sx[t] : 0.0;
+  __syncthreads();
+  for (int w = kSmallRows / 2; w > 0; w >>= 1) {
+    if (t < w) part[t] += part[t + w];
+    __syncthreads();
+  }
+  const double delta = (double)damp_rel * (part[0] / (double)N);
+  if (t == 0) {
+    if (delta_out) *delta_out = (float)delta;
+    *delta64 = delta;
+  }
+  if (t < N) Hb[t * 8 + (t & 7)] = (float)((double)sx[t] + delta);
+}
+
 // Blocks of a given channel order with a known delta.
 __global__ void __launch_bounds__(256)
 blocks_damp_kernel(const float* __restrict__ P, int chunks, int64_t stride, float scale,
@@ -713,6 +751,12 @@ crvq_status launch_tc_hessian_blocks(const float* Xt, int64_t ldt, int64_t n, in
   ProfScope ps("hessian_blocks_finalize", stream, (double)chunks * stride * 4.0);
   if (!delta_known) {
     if (perm) return fail(CRVQ_ERR_UNSUPPORTED, "hessian blocks: delta needs the stored order");
+    if (N <= kSmallRows && chunks * stride <= kSmallTerms) {
+      CRVQ_CUDA(launch_pdl(blocks_small_kernel, dim3(1), dim3(kSmallRows), 0, stream, mem.as<float>(),
+                           (int)chunks, stride, scale, (int)N, damp_rel, xsq, delta, delta64, Hb));
+      CRVQ_LAUNCHED();
+      return CRVQ_OK;
+    }
     const int blocks = (int)std::min<int64_t>(ceil_div(stride, 256), 4 * sm_count());
     CRVQ_CUDA(launch_pdl(blocks_sum_kernel, dim3(blocks), dim3(256), 0, stream, mem.as<float>(),
                          (int)chunks, stride, scale, N, xsq, Hb));

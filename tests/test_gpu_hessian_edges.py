@@ -29,3 +29,19 @@ def test_dense_hessian_edges(n, N):
     G = N // 8
     i = np.arange(G)
     np.testing.assert_array_equal(Hb, H.reshape(G, 8, G, 8)[i, :, i, :])
+
+
+@pytest.mark.parametrize("n,N", [(1, 8), (16, 128), (17, 136), (8000, 128), (8200, 128), (1024, 1016),
+                                 (100, 1024), (100, 1032), (1025, 512), (1025, 520)])
+def test_hessian_blocks_small_sizes(n, N):
+    """On both sides of the line up to which one block sums, damps and writes the blocks (1024 channels,
+    8192 terms): the same bits as the dense call, and as the blocks of the identity order."""
+    rng = np.random.default_rng(n * N)
+    X = dev((rng.standard_normal((n, N)) * rng.lognormal(0.0, 0.5, N)).astype(np.float32))
+    _, xsq, Hb, delta = P.crvq_hessian(X, 0.01)
+    Hb2, xsq2, delta2 = P.crvq_hessian_blocks(X, 0.01)
+    P.crvq_sync()
+    for a, b in ((xsq, xsq2), (Hb, Hb2), (delta, delta2)):
+        np.testing.assert_array_equal(host(a), host(b))
+    order = dev(np.arange(N, dtype=np.int32))
+    np.testing.assert_array_equal(host(P.crvq_hessian_blocks(X, 0.01, perm=order)[0]), host(Hb2))
